@@ -287,11 +287,10 @@ EpiArgs base_epi(esp_handle* h, int n_out, int s0, int nb) {
 }
 
 int run_gemm(esp_handle* h, TcGemm* plan, int epi, int n_tiles, const void* const w[3], const int32_t rows_w[3],
-             const void* x, int K, const EpiArgs& a, bool tc, bool pdl, int nq = 1, int b_row0 = 0) {
+             const void* x, int K, const EpiArgs& a, bool tc, bool pdl, int rows_cap, int nq = 1, int b_row0 = 0) {
     h->launches++;
     if (tc) return tc_gemm_launch(plan, a, h->stream, pdl, nq, b_row0);
-    launch_gemm_simt(h->dtype, epi, n_tiles, h->D.batch, w, rows_w, x, K, a, h->stream, pdl);
-    return ESP_OK;
+    return launch_gemm_simt(h->dtype, epi, n_tiles, h->D.batch, w, rows_w, x, K, a, rows_cap, h->stream, pdl);
 }
 
 // One decoder forward over the block every active sequence of [s0, s0 + nb) has in its row table.
@@ -336,7 +335,7 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
     }
     for (int l = 0; l < D.n_layers && !fused; ++l) {
         if (tc) launch_resid_norm(st0, b.hres, pending, h->na[l], b.xn, b.xn_lo, D.d, D.rms_eps, nullptr, nb, s, pdl, rc_rows);
-        else launch_rmsnorm(h->dtype, st0, b.hres, h->na[l], b.xn, D.d, D.rms_eps, nb, nullptr, s, pdl);
+        else launch_rmsnorm(h->dtype, st0, b.hres, h->na[l], b.xn, D.d, D.rms_eps, nb, nullptr, s, pdl, rc_rows);
         h->launches++;
         mark(h, KIND_MISC);
         {
@@ -348,7 +347,7 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.k_norm = D.qk_norm ? h->kn[l] : nullptr;
             const void* w[3] = {h->wq[l], h->wk[l], h->wv[l]};
             const int32_t rows[3] = {dq, dkv, dkv};
-            int rc = run_gemm(h, tc ? plan(h->p_qkv, h->p_qkv_w, l) : nullptr, EPI_QKV, (dq + 2 * dkv) / TILE_N, w, rows, b.xn, D.d, a, tc, pdl, tc ? nb : 1);
+            int rc = run_gemm(h, tc ? plan(h->p_qkv, h->p_qkv_w, l) : nullptr, EPI_QKV, (dq + 2 * dkv) / TILE_N, w, rows, b.xn, D.d, a, tc, pdl, rc_rows, tc ? nb : 1);
             if (rc) return rc;
             mark(h, KIND_QKV);
             if (tc) {
@@ -387,12 +386,12 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.hres = b.hres;
             const void* w[3] = {h->wo[l], nullptr, nullptr};
             const int32_t rows[3] = {D.d, 0, 0};
-            int rc = run_gemm(h, tc ? plan(h->p_o, h->p_o_w, l) : nullptr, EPI_RESID, (D.d + TILE_N - 1) / TILE_N, w, rows, b.attn_out, dq, a, tc, pdl, tc ? nb : 1);
+            int rc = run_gemm(h, tc ? plan(h->p_o, h->p_o_w, l) : nullptr, EPI_RESID, (D.d + TILE_N - 1) / TILE_N, w, rows, b.attn_out, dq, a, tc, pdl, rc_rows, tc ? nb : 1);
             if (rc) return rc;
             mark(h, KIND_O);
         }
         if (tc) launch_resid_norm(st0, b.hres, tc_gemm_streamk(plan(h->p_o, h->p_o_w, l), nb), h->nf[l], b.xn, b.xn_lo, D.d, D.rms_eps, nullptr, nb, s, pdl, rc_rows);
-        else launch_rmsnorm(h->dtype, st0, b.hres, h->nf[l], b.xn, D.d, D.rms_eps, nb, nullptr, s, pdl);
+        else launch_rmsnorm(h->dtype, st0, b.hres, h->nf[l], b.xn, D.d, D.rms_eps, nb, nullptr, s, pdl, rc_rows);
         h->launches++;
         mark(h, KIND_MISC);
         {
@@ -400,7 +399,7 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.act_out = b.act;
             const void* w[3] = {h->wg[l], h->wu[l], nullptr};
             const int32_t rows[3] = {D.F, D.F, 0};
-            int rc = run_gemm(h, tc ? plan(h->p_gu, h->p_gu_w, l) : nullptr, EPI_SWIGLU, (D.F + 63) / 64, w, rows, b.xn, D.d, a, tc, pdl, tc ? nb : 1);
+            int rc = run_gemm(h, tc ? plan(h->p_gu, h->p_gu_w, l) : nullptr, EPI_SWIGLU, (D.F + 63) / 64, w, rows, b.xn, D.d, a, tc, pdl, rc_rows, tc ? nb : 1);
             if (rc) return rc;
             mark(h, KIND_GATEUP);
             if (tc) {
@@ -414,7 +413,7 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.hres = b.hres;
             const void* w[3] = {h->wd[l], nullptr, nullptr};
             const int32_t rows[3] = {D.d, 0, 0};
-            int rc = run_gemm(h, tc ? plan(h->p_down, h->p_down_w, l) : nullptr, EPI_RESID, (D.d + TILE_N - 1) / TILE_N, w, rows, b.act, D.F, a, tc, pdl, tc ? nb : 1);
+            int rc = run_gemm(h, tc ? plan(h->p_down, h->p_down_w, l) : nullptr, EPI_RESID, (D.d + TILE_N - 1) / TILE_N, w, rows, b.act, D.F, a, tc, pdl, rc_rows, tc ? nb : 1);
             if (rc) return rc;
             if (tc) pending = tc_gemm_streamk(plan(h->p_down, h->p_down_w, l), nb);
             mark(h, KIND_DOWN);
@@ -423,7 +422,7 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
     if (with_lm) {
         float* dbg_hidden = h->dbg_hidden ? h->dbg_hidden + (size_t)s0 * RT * D.d : nullptr;
         if (tc) launch_resid_norm(st0, b.hres, pending, h->final_norm, b.xn, nullptr, D.d, D.rms_eps, dbg_hidden, nb, s, pdl, rc_rows);   // the LM head reads one plane
-        else launch_rmsnorm(h->dtype, st0, b.hres, h->final_norm, b.xn, D.d, D.rms_eps, nb, dbg_hidden, s, pdl);
+        else launch_rmsnorm(h->dtype, st0, b.hres, h->final_norm, b.xn, D.d, D.rms_eps, nb, dbg_hidden, s, pdl, rc_rows);
         h->launches++;
         mark(h, KIND_MISC);
         const int n_tiles = (D.V + TILE_N - 1) / TILE_N;
@@ -436,7 +435,7 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.logits_dump = h->dbg_logits ? h->dbg_logits + (size_t)sq * RT * D.V : nullptr;
             const void* w[3] = {h->lm_head, nullptr, nullptr};
             const int32_t rows[3] = {D.V, 0, 0};
-            int rc = run_gemm(h, wide ? h->p_lm_w : h->p_lm, EPI_LOGITS, n_tiles, w, rows, b.xn, D.d, a, tc, pdl, 1, q);
+            int rc = run_gemm(h, wide ? h->p_lm_w : h->p_lm, EPI_LOGITS, n_tiles, w, rows, b.xn, D.d, a, tc, pdl, rc_rows, 1, q);
             if (rc) return rc;
             mark(h, KIND_LMHEAD);
             launch_topk_merge(b.states + sq, b.cand, b.cand_ms, n_tiles, D.KP, per, b.topk + (size_t)sq * RT * KP_MAX, b.lse + (size_t)sq * RT, s, pdl, rc_rows, b.cand_floor);
@@ -1127,8 +1126,8 @@ int esp_gemm_bf16(int32_t impl, int32_t rows, int32_t n_out, int32_t k_in, const
     const int32_t rw[3] = {n_out, 0, 0};
     const int n_tiles = (n_out + TILE_N - 1) / TILE_N;
     if (impl == 1) {
-        launch_gemm_simt(1, EPI_STORE_F32, n_tiles, 1, wv, rw, x, k_in, a, s, false);
-        return cuda_ok(cudaGetLastError());
+        const int rc = launch_gemm_simt(1, EPI_STORE_F32, n_tiles, 1, wv, rw, x, k_in, a, rows, s, false);
+        return rc ? rc : cuda_ok(cudaGetLastError());
     }
     if (impl != 0) return ESP_E_ARG;
     int dev = 0, n_sm = 0;

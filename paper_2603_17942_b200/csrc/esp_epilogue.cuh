@@ -1,11 +1,8 @@
-// Epilogues of the small-M GEMMs.  Both GEMM implementations (tcgen05 and
-// CUDA-core) finish a 128-feature tile by placing the fp32 accumulators in
-// shared memory as s_acc[row][feature] and calling run_epilogue with exactly
-// 128 threads (thread f owns feature f of the tile).  The fused work is what
-// follows the matrix product in the decoder layer: rotary embedding at the
-// tree-depth position and the KV-cache write (QKV), the residual add (O,
-// down), SiLU(gate)*up (gate/up) and per-row argmax / Top-K' / max+sum-exp
-// over the vocabulary tile (LM head).
+// Epilogues of the small-M GEMMs that work on a whole 128-feature tile.  Both GEMM implementations (tcgen05 and
+// CUDA-core) place the tile's fp32 accumulators in shared memory as s_acc[row][feature] and call run_epilogue (the
+// rows of a block) or run_epilogue_rows (some of them) with exactly 128 threads (thread f owns feature f of the
+// tile): rotary embedding at the tree-depth position and the KV-cache write (QKV), per-row argmax / Top-K' /
+// max+sum-exp over the vocabulary tile (LM head), a plain store.
 #pragma once
 
 #include "esp_common.cuh"
@@ -30,34 +27,19 @@ __device__ __forceinline__ void epi_bar(int bar_id) {
     asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
 }
 
-// s_acc: [RT][ACC_LD] fp32.  s_aux: >= RT*4 floats of scratch.  tid in [0,128).
+// s_acc: [rows][ACC_LD] fp32, rows r0 .. r1-1 of the block (r1 <= n_rows).  s_aux: >= RT*4 floats of scratch.
+// tid in [0,128).  A row's result does not depend on which rows share the call.
 template <typename T, int EPI>
-__device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, const EpiArgs& a, int tid, int bar_id) {
+__device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, int tile, int seq, const EpiArgs& a, int tid, int bar_id,
+                                                  const SeqState* st, int n_rows, const int r0, const int r1) {
     const int f = tid;
     const int n0 = tile * TILE_N;
-    const SeqState* st = a.st ? a.st + seq : nullptr;
-    const int n_rows = st ? st->n_rows : a.rows_fixed;
     const int grow0 = seq * RT;
+    s_acc -= r0 * ACC_LD;       // addressed by block row below
 
     if constexpr (EPI == EPI_STORE_F32) {
         if (n0 + f < a.n_out)
-            for (int r = 0; r < n_rows; ++r) a.y_f32[(size_t)(grow0 + r) * a.n_out + n0 + f] = s_acc[r * ACC_LD + f];
-    } else if constexpr (EPI == EPI_RESID) {
-        if (n0 + f < a.n_out)
-            for (int r = 0; r < n_rows; ++r) {
-                size_t i = (size_t)(grow0 + r) * a.n_out + n0 + f;
-                a.hres[i] = a.hres[i] + s_acc[r * ACC_LD + f];
-            }
-    } else if constexpr (EPI == EPI_SWIGLU) {
-        // tile rows 0..63 hold gate features [64*tile, 64*tile+64), rows 64..127 the matching up features
-        if (f < 64 && tile * 64 + f < a.n_out) {
-            T* out = reinterpret_cast<T*>(a.act_out);
-            for (int r = 0; r < n_rows; ++r) {
-                float g = s_acc[r * ACC_LD + f], u = s_acc[r * ACC_LD + f + 64];
-                float v = (g / (1.0f + expf(-g))) * u;
-                out[(size_t)(grow0 + r) * a.n_out + tile * 64 + f] = from_f32<T>(v);
-            }
-        }
+            for (int r = r0; r < r1; ++r) a.y_f32[(size_t)(grow0 + r) * a.n_out + n0 + f] = s_acc[r * ACC_LD + f];
     } else if constexpr (EPI == EPI_QKV) {
         const int h = a.h, dq = a.Hq * h, dkv = a.Hkv * h;
         const int feat = n0 + f;  // index in the concatenated [q | k | v] feature space
@@ -69,7 +51,7 @@ __device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, cons
         if (which != 2) {
             if (a.qk_norm) {
                 // per-head RMSNorm: sum of squares over the head's h features, per row
-                for (int r = 0; r < n_rows; ++r) {
+                for (int r = r0; r < r1; ++r) {
                     float v = s_acc[r * ACC_LD + f];
                     float ss = warp_sum(v * v);
                     if ((f & 31) == 0) s_aux[r * 4 + warp] = ss;
@@ -79,7 +61,7 @@ __device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, cons
                 const float gain = to_f32(g[fl]);
                 const int wpw = h / 32;                    // warps per head
                 const int w0 = (f / h) * wpw;              // first warp of this thread's head
-                for (int r = 0; r < n_rows; ++r) {
+                for (int r = r0; r < r1; ++r) {
                     float ss = 0.f;
                     for (int w = 0; w < wpw; ++w) ss += s_aux[r * 4 + w0 + w];
                     float rinv = 1.0f / sqrtf(ss / (float)h + a.rms_eps);
@@ -89,7 +71,7 @@ __device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, cons
             epi_bar(bar_id);
             // rotary embedding at position L + depth, rotate-half pairing (i, i + h/2)
             const int partner = fl < half ? f + half : f - half;
-            for (int r = 0; r < n_rows; ++r) {
+            for (int r = r0; r < r1; ++r) {
                 const int pos = L + (st ? st->row_depth[r] : r);
                 const float cs = a.rope_cos[(size_t)pos * half + (fl % half)];
                 const float sn = a.rope_sin[(size_t)pos * half + (fl % half)];
@@ -104,7 +86,7 @@ __device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, cons
         } else {
             if (a.qk_norm) epi_bar(bar_id);
             epi_bar(bar_id);
-            for (int r = 0; r < n_rows; ++r)
+            for (int r = r0; r < r1; ++r)
                 reinterpret_cast<T*>(a.vcache)[(((size_t)seq * a.Hkv + head) * a.cap + (L + r)) * h + fl] =
                     from_f32<T>(s_acc[r * ACC_LD + f]);
         }
@@ -120,7 +102,7 @@ __device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, cons
         const int S = n_rows <= 80 ? 80 : RT;                             // s_aux holds at least 3 * S words
         uint32_t* s_floor = reinterpret_cast<uint32_t*>(s_aux);          // [S] in, [S] out, [S] "this probe row has entries at or above its floor"
         uint32_t* s_need = s_floor + 2 * S;
-        for (int r = f; r < n_rows; r += 128) {
+        for (int r = r0 + f; r < r1; r += 128) {
             s_floor[r] = (r >= n_nodes && a.cand_floor) ? __ldcg(a.cand_floor + grow0 + r) : 0u;
             s_floor[S + r] = 0u;
         }
@@ -131,8 +113,8 @@ __device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, cons
         // probe rows per block nearly all rows of nearly all tiles end here, without one warp-wide reduction.
         const bool many_probes = n_rows - n_nodes >= 16;     // block-uniform; a handful of probe rows is cheaper warp by warp
         if (many_probes) {
-            const int r = n_nodes + f;
-            if (r < n_rows) {
+            const int r = (n_nodes > r0 ? n_nodes : r0) + f;
+            if (r < r1) {
                 const int n_valid = a.n_out - n0 < TILE_N ? a.n_out - n0 : TILE_N;
                 const float* row = s_acc + r * ACC_LD;
                 float tmax = -INFINITY;
@@ -149,7 +131,7 @@ __device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, cons
             }
         }
         epi_bar(bar_id);
-        for (int r = warp; r < n_rows; r += 4) {
+        for (int r = r0 + warp; r < r1; r += 4) {
             float v[4];
             int id[4];
 #pragma unroll
@@ -211,9 +193,17 @@ __device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, cons
             if (lane < kp) { out[lane].val = keep_v; out[lane].id = keep_i; }
         }
         epi_bar(bar_id);
-        for (int r = f; r < n_rows; r += 128)
+        for (int r = r0 + f; r < r1; r += 128)
             if (s_floor[S + r] > s_floor[r]) atomicMax(a.cand_floor + grow0 + r, s_floor[S + r]);
     }
+}
+
+// the whole block
+template <typename T, int EPI>
+__device__ void run_epilogue(float* s_acc, float* s_aux, int tile, int seq, const EpiArgs& a, int tid, int bar_id) {
+    const SeqState* st = a.st ? a.st + seq : nullptr;
+    const int n_rows = st ? st->n_rows : a.rows_fixed;
+    run_epilogue_rows<T, EPI>(s_acc, s_aux, tile, seq, a, tid, bar_id, st, n_rows, 0, n_rows);
 }
 
 }  // namespace esp

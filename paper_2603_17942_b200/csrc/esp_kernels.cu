@@ -209,98 +209,229 @@ __global__ void __launch_bounds__(256) k_swiglu_finish(const SeqState* states, i
 }
 
 // ------------------------------------------------------------------ CUDA-core GEMM
-// y[row][n] = sum_k x[row][k] * w[n][k], k ascending, one thread per output feature of a
-// 128-feature tile and all RT rows of one sequence.  Used for fp32 models and as the on-GPU
-// cross-check of the tcgen05 kernel.  Tile -> weight rows mapping is the same as there:
-// up to three stacked matrices (q|k|v), or gate/up halves interleaved per tile.
+// y[row][n] = sum_k x[row][k] * w[n][k], one running fp32 sum per output with k ascending, one thread per output
+// feature of a 128-feature tile.  Used for fp32 models and as the on-GPU cross-check of the tcgen05 kernel.
+// Tile -> weight rows mapping is the same as there: up to three stacked matrices (q|k|v), or gate/up halves
+// interleaved per tile.
+//
+// What bounds it: latency.  A small model's matrix is a few hundred KB and a block has a few dozen rows, so there is
+// little work per launch and what counts is how many SMs share a weight tile's trip from L2 and through shared memory.
+// A CTA takes 8 rows; where the epilogue works feature by feature (residual add, SiLU*up, plain store) also only 32
+// features (k_gemm_simt_narrow), elsewhere -- rotary pairs and head norms, per-tile selection -- the whole 128-feature
+// tile.  Weights and rows arrive by asynchronous copies several stages ahead, the weights of the first stages
+// requested before the wait for the preceding kernel.  Measured on the tiny fp32 decoder (d_model 256, 35 rows; device
+// time of a launch on its own): QKV 11, O and down 9, gate/up 7, LM head (vocabulary 4096) 13 us, where one CTA per
+// 128-feature tile with all rows took 140 to 240; its 64-token request 103 -> 9.9 ms.
 struct SimtGemmArgs {
     const void* w[3];   // stacked matrices (rows_w[i] rows each); SWIGLU: w[0]=gate, w[1]=up
     int32_t rows_w[3];
     const void* x;      // [batch*RT][K]
     int32_t K;
 };
-
-template <typename T, int EPI>
-__global__ void __launch_bounds__(128) k_gemm_simt(SimtGemmArgs g, EpiArgs a) {
-    extern __shared__ float smem[];
-    float* s_acc = smem;                       // RT * ACC_LD
-    float* s_aux = s_acc + RT * ACC_LD;        // RT * 4
-    float* s_x = s_aux + RT * 4;               // RT * 32
-    float* s_w = s_x + RT * 32;                // 128 * 33
-    pdl_wait();
-    const int tile = blockIdx.x, seq = blockIdx.y, f = threadIdx.x;
-    if (a.st && !a.st[seq].active) return;
-    const int n_rows = a.st ? a.st[seq].n_rows : a.rows_fixed;
-    const T* x = reinterpret_cast<const T*>(g.x) + (size_t)seq * RT * g.K;
-    // weight row of feature i of this tile (nullptr if outside)
-    auto wrow = [&](int i) -> const T* {
-        if (EPI == EPI_SWIGLU) {
-            int feat = tile * 64 + (i & 63);
-            if (feat >= g.rows_w[0]) return nullptr;
-            return reinterpret_cast<const T*>(g.w[i >> 6]) + (size_t)feat * g.K;
-        }
-        int feat = tile * TILE_N + i;
-        for (int m = 0; m < 3; ++m) {
-            if (feat < g.rows_w[m]) return reinterpret_cast<const T*>(g.w[m]) + (size_t)feat * g.K;
-            feat -= g.rows_w[m];
-        }
-        return nullptr;
-    };
-    float acc[RT];
-#pragma unroll
-    for (int r = 0; r < RT; ++r) acc[r] = 0.f;
-    for (int k0 = 0; k0 < g.K; k0 += 32) {
-        for (int i = f; i < RT * 32; i += 128) {
-            int r = i >> 5, c = i & 31;
-            s_x[i] = (r < n_rows && k0 + c < g.K) ? to_f32(x[(size_t)r * g.K + k0 + c]) : 0.f;
-        }
-        for (int i = 0; i < 32; ++i) {
-            int row = (f >> 5) + 4 * i, c = f & 31;
-            const T* wr = wrow(row);
-            s_w[row * 33 + c] = (wr && k0 + c < g.K) ? to_f32(wr[k0 + c]) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int c = 0; c < 32; ++c) {
-            float w = s_w[f * 33 + c];
-#pragma unroll
-            for (int r = 0; r < RT; ++r) acc[r] = fmaf(s_x[r * 32 + c], w, acc[r]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int r = 0; r < RT; ++r) s_acc[r * ACC_LD + f] = acc[r];
-    __syncthreads();
-    run_epilogue<T, EPI>(s_acc, s_aux, tile, seq, a, f, 1);
+constexpr int SIMT_ROWS = 8;
+constexpr int SIMT_KC = 32, SIMT_STAGES = 4;       // whole tile: two CTAs of 84 KB per SM
+constexpr int NARROW_F = 32, NARROW_KC = 64, NARROW_STAGES = 6;
+// elements between two rows of a stage: 16 bytes of padding put the eight rows of a quarter-warp's 16-byte loads on
+// different banks
+template <typename T> __host__ __device__ constexpr int simt_ld(int kc) { return kc + 16 / (int)sizeof(T); }
+template <typename T> constexpr size_t simt_smem_bytes() {
+    return sizeof(T) * SIMT_STAGES * (TILE_N + SIMT_ROWS) * simt_ld<T>(SIMT_KC) + sizeof(float) * (SIMT_ROWS * ACC_LD + RT * 4);
+}
+template <typename T> constexpr size_t narrow_smem_bytes() {
+    return sizeof(T) * NARROW_STAGES * (NARROW_F + SIMT_ROWS) * simt_ld<T>(NARROW_KC);
 }
 
-template <typename T>
-void launch_gemm_simt_t(int epi, int n_tiles, int batch, const SimtGemmArgs& g, const EpiArgs& a, cudaStream_t s, bool pdl) {
-    size_t smem = sizeof(float) * (RT * ACC_LD + RT * 4 + RT * 32 + 128 * 33);
-    dim3 grid(n_tiles, batch);
-#define ESP_SIMT_CASE(E)                                                                                  \
-    case E:                                                                                               \
-        cudaFuncSetAttribute(k_gemm_simt<T, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);  \
-        launch_k(k_gemm_simt<T, E>, grid, dim3(128), smem, s, pdl, g, a);                                 \
-        break;
+// 16 bytes to shared memory; `ok` false: zeros (the source is not read)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool ok) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// four consecutive elements of a stage row as floats
+__device__ __forceinline__ float4 load_f4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load_f4(const __nv_bfloat16* p) {
+    const uint2 raw = *reinterpret_cast<const uint2*>(p);
+    const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&raw.x), hi = *reinterpret_cast<const __nv_bfloat162*>(&raw.y);
+    return make_float4(__low2float(lo), __high2float(lo), __low2float(hi), __high2float(hi));
+}
+
+// Stage `dst` [n_rows][LD] <- rows 0..n_valid-1 of `src` (K elements apart), elements k0 .. k0+KC-1; zeros outside.
+// All 128 threads take part, 16 bytes each per pass.  VEC: src starts on 16 bytes (its rows then do too, K is a
+// multiple of 8): asynchronous copies.  Otherwise element by element (a caller's matrix needs no more than its
+// type's alignment).
+template <typename T, int KC, int N_ROWS, bool VEC>
+__device__ __forceinline__ void simt_load(T* dst, const T* src, int n_valid, int K, int k0) {
+    constexpr int LD = simt_ld<T>(KC), V = 16 / (int)sizeof(T), PER_ROW = KC / V, STEP = 128 / PER_ROW;
+    const int j = (threadIdx.x % PER_ROW) * V, first = threadIdx.x / PER_ROW;
+    const bool k_ok = k0 + j < K;
+    const T* p = src + (size_t)first * K + k0 + j;
+    T* d = dst + first * LD + j;
+#pragma unroll
+    for (int row = 0; row < N_ROWS; row += STEP, p += (size_t)STEP * K, d += STEP * LD) {
+        if (N_ROWS % STEP && first + row >= N_ROWS) break;
+        const bool ok = k_ok && first + row < n_valid;
+        if constexpr (VEC) cp_async16(d, ok ? p : src, ok);
+        else {
+#pragma unroll
+            for (int e = 0; e < V; ++e) d[e] = ok ? p[e] : from_f32<T>(0.f);
+        }
+    }
+}
+
+// acc[r] += x[r][k] * w[k] over one stage, k ascending
+template <int R, int KC, typename T>
+__device__ __forceinline__ void simt_mac(float (&acc)[R], const T* w, const T* x, int ld) {
+#pragma unroll 8
+    for (int k = 0; k < KC; k += 4) {
+        const float4 wv = load_f4(w + k);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4 xv = load_f4(x + r * ld + k);
+            acc[r] = fmaf(xv.w, wv.w, fmaf(xv.z, wv.z, fmaf(xv.y, wv.y, fmaf(xv.x, wv.x, acc[r]))));
+        }
+    }
+}
+
+// 8 rows x one 128-feature tile, one thread per feature.  EPI_QKV (the stacked matrices end on tile boundaries) and
+// EPI_LOGITS.
+template <typename T, int EPI, bool VEC>
+__global__ void __launch_bounds__(128) k_gemm_simt(SimtGemmArgs g, EpiArgs a) {
+    constexpr int LD = simt_ld<T>(SIMT_KC);
+    extern __shared__ __align__(16) unsigned char simt_smem[];
+    T* s_w = reinterpret_cast<T*>(simt_smem);                   // [STAGES][128][LD]
+    T* s_x = s_w + SIMT_STAGES * TILE_N * LD;                   // [STAGES][ROWS][LD]
+    float* s_acc = reinterpret_cast<float*>(s_x + SIMT_STAGES * SIMT_ROWS * LD);   // [ROWS][ACC_LD]
+    float* s_aux = s_acc + SIMT_ROWS * ACC_LD;                  // RT * 4
+    if (threadIdx.x == 0) pdl_launch_dependents();
+    const int tile = blockIdx.x, r0 = blockIdx.y * SIMT_ROWS, seq = blockIdx.z, f = threadIdx.x;
+    int m = 0, feat = tile * TILE_N;
+    while (m < 2 && feat >= g.rows_w[m]) feat -= g.rows_w[m++];
+    const T* w = reinterpret_cast<const T*>(g.w[m]) + (size_t)feat * g.K;
+    const int n_feat = g.rows_w[m] - feat < TILE_N ? g.rows_w[m] - feat : TILE_N;
+    const int n_chunks = (g.K + SIMT_KC - 1) / SIMT_KC;
+    auto load_w = [&](int c) { simt_load<T, SIMT_KC, TILE_N, VEC>(s_w + (c % SIMT_STAGES) * TILE_N * LD, w, n_feat, g.K, c * SIMT_KC); };
+    for (int c = 0; c < SIMT_STAGES - 1 && c < n_chunks; ++c) load_w(c);      // (they join the first group below)
+    pdl_wait();
+    const SeqState* st = a.st ? a.st + seq : nullptr;
+    const int n_rows = st ? (st->active ? st->n_rows : 0) : a.rows_fixed;
+    if (r0 >= n_rows) { cp_async_wait<0>(); return; }
+    const int r1 = r0 + SIMT_ROWS < n_rows ? r0 + SIMT_ROWS : n_rows;
+    const T* x = reinterpret_cast<const T*>(g.x) + (size_t)(seq * RT + r0) * g.K;
+    auto load_x = [&](int c) { simt_load<T, SIMT_KC, SIMT_ROWS, VEC>(s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD, x, r1 - r0, g.K, c * SIMT_KC); };
+    for (int c = 0; c < SIMT_STAGES - 1; ++c) {
+        if (c < n_chunks) load_x(c);
+        cp_async_commit();
+    }
+    float acc[SIMT_ROWS];
+#pragma unroll
+    for (int r = 0; r < SIMT_ROWS; ++r) acc[r] = 0.f;
+    for (int c = 0; c < n_chunks; ++c) {
+        cp_async_wait<SIMT_STAGES - 2>();
+        __syncthreads();                                // chunk c has landed, and chunk c - 1's buffer is free
+        if (c + SIMT_STAGES - 1 < n_chunks) { load_w(c + SIMT_STAGES - 1); load_x(c + SIMT_STAGES - 1); }
+        cp_async_commit();
+        simt_mac<SIMT_ROWS, SIMT_KC>(acc, s_w + ((c % SIMT_STAGES) * TILE_N + f) * LD, s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD, LD);
+    }
+#pragma unroll
+    for (int r = 0; r < SIMT_ROWS; ++r) s_acc[r * ACC_LD + f] = acc[r];
+    __syncthreads();
+    run_epilogue_rows<T, EPI>(s_acc, s_aux, tile, seq, a, f, 1, st, n_rows, r0, r1);
+}
+
+// 8 rows x 32 features (SWIGLU: 16 gate features and the matching 16 up features), a lane per feature, two rows per
+// warp.  EPI_STORE_F32, EPI_RESID, EPI_SWIGLU.
+template <typename T, int EPI, bool VEC>
+__global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArgs a) {
+    constexpr int LD = simt_ld<T>(NARROW_KC), HALF = NARROW_F / 2;
+    extern __shared__ __align__(16) unsigned char simt_smem[];
+    T* s_w = reinterpret_cast<T*>(simt_smem);                   // [STAGES][32][LD]
+    T* s_x = s_w + NARROW_STAGES * NARROW_F * LD;               // [STAGES][ROWS][LD]
+    if (threadIdx.x == 0) pdl_launch_dependents();
+    const int r0 = blockIdx.y * SIMT_ROWS, seq = blockIdx.z, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n0 = blockIdx.x * (EPI == EPI_SWIGLU ? HALF : NARROW_F);
+    const int n_feat = a.n_out - n0 < NARROW_F ? a.n_out - n0 : NARROW_F;      // (SWIGLU: of either half, cut below)
+    const T* w0 = reinterpret_cast<const T*>(g.w[0]) + (size_t)n0 * g.K;
+    const int n_chunks = (g.K + NARROW_KC - 1) / NARROW_KC;
+    auto load_w = [&](int c) {
+        T* dst = s_w + (c % NARROW_STAGES) * NARROW_F * LD;
+        if constexpr (EPI == EPI_SWIGLU) {
+            const int n = n_feat < HALF ? n_feat : HALF;
+            simt_load<T, NARROW_KC, HALF, VEC>(dst, w0, n, g.K, c * NARROW_KC);
+            simt_load<T, NARROW_KC, HALF, VEC>(dst + HALF * LD, reinterpret_cast<const T*>(g.w[1]) + (size_t)n0 * g.K, n, g.K, c * NARROW_KC);
+        } else {
+            simt_load<T, NARROW_KC, NARROW_F, VEC>(dst, w0, n_feat, g.K, c * NARROW_KC);
+        }
+    };
+    for (int c = 0; c < NARROW_STAGES - 1 && c < n_chunks; ++c) load_w(c);
+    pdl_wait();
+    const SeqState* st = a.st ? a.st + seq : nullptr;
+    const int n_rows = st ? (st->active ? st->n_rows : 0) : a.rows_fixed;
+    if (r0 >= n_rows) { cp_async_wait<0>(); return; }
+    const int r1 = r0 + SIMT_ROWS < n_rows ? r0 + SIMT_ROWS : n_rows;
+    const T* x = reinterpret_cast<const T*>(g.x) + (size_t)(seq * RT + r0) * g.K;
+    auto load_x = [&](int c) { simt_load<T, NARROW_KC, SIMT_ROWS, VEC>(s_x + (c % NARROW_STAGES) * SIMT_ROWS * LD, x, r1 - r0, g.K, c * NARROW_KC); };
+    for (int c = 0; c < NARROW_STAGES - 1; ++c) {
+        if (c < n_chunks) load_x(c);
+        cp_async_commit();
+    }
+    float acc[2] = {0.f, 0.f};
+    for (int c = 0; c < n_chunks; ++c) {
+        cp_async_wait<NARROW_STAGES - 2>();
+        __syncthreads();
+        if (c + NARROW_STAGES - 1 < n_chunks) { load_w(c + NARROW_STAGES - 1); load_x(c + NARROW_STAGES - 1); }
+        cp_async_commit();
+        simt_mac<2, NARROW_KC>(acc, s_w + ((c % NARROW_STAGES) * NARROW_F + lane) * LD, s_x + ((c % NARROW_STAGES) * SIMT_ROWS + warp * 2) * LD, LD);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int r = r0 + warp * 2 + i;
+        const size_t row = (size_t)(seq * RT + r) * a.n_out;
+        if constexpr (EPI == EPI_SWIGLU) {
+            const float up = __shfl_down_sync(0xffffffffu, acc[i], HALF), gate = acc[i];
+            if (lane < HALF && lane < n_feat && r < r1)
+                reinterpret_cast<T*>(a.act_out)[row + n0 + lane] = from_f32<T>((gate / (1.0f + expf(-gate))) * up);
+        } else if (lane < n_feat && r < r1) {
+            if constexpr (EPI == EPI_RESID) a.hres[row + n0 + lane] = a.hres[row + n0 + lane] + acc[i];
+            else a.y_f32[row + n0 + lane] = acc[i];
+        }
+    }
+}
+
+template <typename T, bool VEC>
+int launch_gemm_simt_t(int epi, int n_tiles, int batch, const SimtGemmArgs& g, const EpiArgs& a, int rows_cap, cudaStream_t s, bool pdl) {
+    const int groups = (rows_cap + SIMT_ROWS - 1) / SIMT_ROWS;
+#define ESP_SIMT_CASE(E, KERNEL, TILES, SMEM)                                                                       \
+    case E:                                                                                                         \
+        if (ensure_dynamic_smem(reinterpret_cast<const void*>(KERNEL<T, E, VEC>), (int)SMEM<T>())) return ESP_E_CUDA; \
+        return launch_k(KERNEL<T, E, VEC>, dim3(TILES, groups, batch), dim3(128), SMEM<T>(), s, pdl, g, a) == cudaSuccess ? ESP_OK : ESP_E_CUDA;
     switch (epi) {
-        ESP_SIMT_CASE(EPI_STORE_F32)
-        ESP_SIMT_CASE(EPI_QKV)
-        ESP_SIMT_CASE(EPI_RESID)
-        ESP_SIMT_CASE(EPI_SWIGLU)
-        ESP_SIMT_CASE(EPI_LOGITS)
+        ESP_SIMT_CASE(EPI_STORE_F32, k_gemm_simt_narrow, (a.n_out + NARROW_F - 1) / NARROW_F, narrow_smem_bytes)
+        ESP_SIMT_CASE(EPI_RESID, k_gemm_simt_narrow, (a.n_out + NARROW_F - 1) / NARROW_F, narrow_smem_bytes)
+        ESP_SIMT_CASE(EPI_SWIGLU, k_gemm_simt_narrow, (a.n_out + NARROW_F / 2 - 1) / (NARROW_F / 2), narrow_smem_bytes)
+        ESP_SIMT_CASE(EPI_QKV, k_gemm_simt, n_tiles, simt_smem_bytes)
+        ESP_SIMT_CASE(EPI_LOGITS, k_gemm_simt, n_tiles, simt_smem_bytes)
     }
 #undef ESP_SIMT_CASE
+    return ESP_E_ARG;
 }
 
-void launch_gemm_simt(int dtype, int epi, int n_tiles, int batch, const void* const w[3], const int32_t rows_w[3],
-                      const void* x, int K, const EpiArgs& a, cudaStream_t s, bool pdl) {
+// rows_cap: no block has more rows (sizes the grid)
+int launch_gemm_simt(int dtype, int epi, int n_tiles, int batch, const void* const w[3], const int32_t rows_w[3],
+                     const void* x, int K, const EpiArgs& a, int rows_cap, cudaStream_t s, bool pdl) {
     SimtGemmArgs g;
-    for (int i = 0; i < 3; ++i) { g.w[i] = w[i]; g.rows_w[i] = rows_w[i]; }
+    bool vec = reinterpret_cast<uintptr_t>(x) % 16 == 0;
+    for (int i = 0; i < 3; ++i) {
+        g.w[i] = w[i]; g.rows_w[i] = rows_w[i];
+        vec = vec && reinterpret_cast<uintptr_t>(w[i]) % 16 == 0;
+    }
     g.x = x;
     g.K = K;
-    if (dtype == 0) launch_gemm_simt_t<float>(epi, n_tiles, batch, g, a, s, pdl);
-    else launch_gemm_simt_t<__nv_bfloat16>(epi, n_tiles, batch, g, a, s, pdl);
+    if (dtype == 0) return vec ? launch_gemm_simt_t<float, true>(epi, n_tiles, batch, g, a, rows_cap, s, pdl)
+                               : launch_gemm_simt_t<float, false>(epi, n_tiles, batch, g, a, rows_cap, s, pdl);
+    return vec ? launch_gemm_simt_t<__nv_bfloat16, true>(epi, n_tiles, batch, g, a, rows_cap, s, pdl)
+               : launch_gemm_simt_t<__nv_bfloat16, false>(epi, n_tiles, batch, g, a, rows_cap, s, pdl);
 }
 
 // ------------------------------------------------------------------ attention (position-canonical)
@@ -344,9 +475,11 @@ __device__ __forceinline__ void attn_row_info(const AttnArgs& a, int seq, int r,
     }
 }
 
-// One chunk of up to 32 keys for one (row, head) handled by one warp: lane j owns key j.
-// Returns the chunk's own (max, sum, weighted values) relative to its own max, in the log2 domain.
-template <typename T, int HD>
+// One chunk of up to 32 keys for one (row, head) handled by one warp: lane j owns key j (its row gathered straight
+// from the cache).  Returns the chunk's own (max, sum, weighted values) relative to its own max, in the log2 domain.
+// Every load of a key row, and eight value rows at a time, are in flight together (lanes without a key hold slot 0,
+// whose value row is read and not used).  VEC: the cache starts on 16 bytes.
+template <typename T, int HD, bool VEC>
 __device__ __forceinline__ void warp_chunk(const float* s_q, const T* kbase, const T* vbase, int slot, bool valid,
                                            float scale_log2, float& cm, float& cl, float (&co)[HD / 32]) {
     const int lane = threadIdx.x & 31;
@@ -354,8 +487,16 @@ __device__ __forceinline__ void warp_chunk(const float* s_q, const T* kbase, con
     if (valid) {
         const T* kr = kbase + (size_t)slot * HD;
         float acc = 0.f;
-#pragma unroll 8
-        for (int d = 0; d < HD; ++d) acc = fmaf(s_q[d], to_f32(kr[d]), acc);
+        if constexpr (VEC) {
+#pragma unroll
+            for (int d = 0; d < HD; d += 4) {
+                const float4 kv = load_f4(kr + d), qv = load_f4(s_q + d);
+                acc = fmaf(qv.w, kv.w, fmaf(qv.z, kv.z, fmaf(qv.y, kv.y, fmaf(qv.x, kv.x, acc))));
+            }
+        } else {
+#pragma unroll 16
+            for (int d = 0; d < HD; ++d) acc = fmaf(s_q[d], to_f32(kr[d]), acc);
+        }
         s = acc * scale_log2;
     }
     cm = warp_max(s);
@@ -363,13 +504,22 @@ __device__ __forceinline__ void warp_chunk(const float* s_q, const T* kbase, con
     cl = warp_sum(p);
 #pragma unroll
     for (int i = 0; i < HD / 32; ++i) co[i] = 0.f;
-    for (int j = 0; j < 32; ++j) {
-        float pj = __shfl_sync(0xffffffffu, p, j);
-        int sj = __shfl_sync(0xffffffffu, slot, j);
-        if (pj != 0.f) {
-            const T* vr = vbase + (size_t)sj * HD;
+#pragma unroll 1
+    for (int j0 = 0; j0 < 32; j0 += 8) {
+        float v[8][HD / 32];
 #pragma unroll
-            for (int i = 0; i < HD / 32; ++i) co[i] = fmaf(pj, to_f32(vr[lane + 32 * i]), co[i]);
+        for (int j = 0; j < 8; ++j) {
+            const T* vr = vbase + (size_t)__shfl_sync(0xffffffffu, slot, j0 + j) * HD;
+#pragma unroll
+            for (int i = 0; i < HD / 32; ++i) v[j][i] = to_f32(vr[lane + 32 * i]);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float pj = __shfl_sync(0xffffffffu, p, j0 + j);
+            if (pj != 0.f) {
+#pragma unroll
+                for (int i = 0; i < HD / 32; ++i) co[i] = fmaf(pj, v[j][i], co[i]);
+            }
         }
     }
 }
@@ -384,47 +534,147 @@ __device__ __forceinline__ void merge_partial(float& m, float& l, float (&o)[N],
     m = mn;
 }
 
-// Bulk, CUDA-core version: one warp per (row, head, split).  grid = (ceil(RT/4), Hq, n_split*batch).
-template <typename T, int HD>
+// Bulk, CUDA-core version.  A CTA takes one cache split of one KV head for 4 * BS_PW (row, head) pairs of that head's
+// group, a warp BS_PW of them; keys and values pass through shared memory in chunks of 32 positions, the next chunk
+// loading (16-byte asynchronous copies) while the current one is used.  What bounds it is a warp's serial chain over
+// the split: with four pairs a warp shares every key and value read from shared memory between them and the CTA reads
+// the split from L2 for 16 pairs; with one pair the chain is a third as long, which is what counts while the four-pair
+// CTAs would leave SMs idle (launch_attn_simt_t).  Measured with the tail kernel behind it, 3 sequences x 35 rows x 4
+// fp32 heads of 64 over 777 positions: 184 us with a warp per (row, head) gathering its keys from L1, 33 us now; one
+// split of 100 positions on its own 13.4 us with four pairs per warp, 7.3 with one.
+// grid = (ceil(rows * group / (4 * BS_PW)), Hkv, n_split * batch).
+constexpr int BS_WARPS = 4;
+template <typename T, int HD> __host__ __device__ constexpr int bulk_simt_ld() { return HD + 16 / (int)sizeof(T); }
+template <typename T, int HD> constexpr size_t bulk_simt_smem(int pw) { return sizeof(T) * 4 * 32 * bulk_simt_ld<T, HD>() + sizeof(float) * BS_WARPS * pw * HD; }
+template <typename T, int HD, bool VEC, int BS_PW>
 __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_launch) {
-    __shared__ float s_qall[4][HD];
+    constexpr int LD = bulk_simt_ld<T, HD>(), V = 16 / (int)sizeof(T), PER_ROW = HD / V;
+    extern __shared__ __align__(16) unsigned char bulk_smem[];
+    T* s_k = reinterpret_cast<T*>(bulk_smem);            // [2][32][LD]
+    T* s_v = s_k + 2 * 32 * LD;                          // [2][32][LD]
+    float* s_qall = reinterpret_cast<float*>(s_v + 2 * 32 * LD);
+    if (threadIdx.x == 0) pdl_launch_dependents();
     pdl_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = blockIdx.x * 4 + warp, head = blockIdx.y;
+    const int kvh = blockIdx.y, group = a.Hq / a.Hkv;
     const int split = blockIdx.z % n_split_launch, seq = blockIdx.z / n_split_launch;
-    int n_rows, L, depth;
-    unsigned long long lo, hi;
-    attn_row_info(a, seq, r < RT ? r : 0, n_rows, L, depth, lo, hi);
-    if (r >= n_rows) return;
-    const int T0 = tail_start(L + depth, a.dcap);
-    const int beg = split * a.split_len, end = min(beg + a.split_len, T0);
-    if (beg >= end) return;
-    const int kvh = head / (a.Hq / a.Hkv);
-    const T* q = reinterpret_cast<const T*>(a.q) + ((size_t)(seq * RT + r) * a.Hq + head) * HD;
-    float* s_q = s_qall[warp];
-    for (int d = lane; d < HD; d += 32) s_q[d] = to_f32(q[d]);
-    __syncwarp();
+    const int beg = split * a.split_len;
+    int row[BS_PW], end[BS_PW], cta_end = 0;
+    const int pair0 = (blockIdx.x * BS_WARPS + warp) * BS_PW;
+    float* s_q = s_qall + warp * BS_PW * HD;
+#pragma unroll
+    for (int w = 0; w < BS_PW; ++w) {
+        row[w] = (pair0 + w) / group;
+        end[w] = 0;
+        int n_rows, L, depth;
+        unsigned long long lo, hi;
+        attn_row_info(a, seq, row[w] < RT ? row[w] : 0, n_rows, L, depth, lo, hi);
+        if (row[w] < n_rows) {
+            end[w] = min(beg + a.split_len, tail_start(L + depth, a.dcap));
+            const T* q = reinterpret_cast<const T*>(a.q) + ((size_t)(seq * RT + row[w]) * a.Hq + kvh * group + (pair0 + w) % group) * HD;
+            for (int d = lane; d < HD; d += 32) s_q[w * HD + d] = to_f32(q[d]);
+        }
+        cta_end = max(cta_end, end[w]);
+    }
+    __shared__ int s_end[BS_WARPS];
+    if (lane == 0) s_end[warp] = cta_end;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < BS_WARPS; ++w) cta_end = max(cta_end, s_end[w]);
+    if (beg >= cta_end) return;
     const T* kb = reinterpret_cast<const T*>(a.kc) + ((size_t)seq * a.Hkv + kvh) * a.cap * HD;
     const T* vb = reinterpret_cast<const T*>(a.vc) + ((size_t)seq * a.Hkv + kvh) * a.cap * HD;
-    float m = -INFINITY, l = 0.f, o[HD / 32];
+    auto load = [&](int p0, int buf) {
+        for (int i = threadIdx.x; i < 32 * PER_ROW; i += 128) {
+            const int pos = p0 + i / PER_ROW, e0 = (i % PER_ROW) * V;
+            const bool ok = pos < cta_end;
+            const size_t src = (size_t)(ok ? pos : beg) * HD + e0;
+            T* dk = s_k + (buf * 32 + i / PER_ROW) * LD + e0;
+            T* dv = s_v + (buf * 32 + i / PER_ROW) * LD + e0;
+            if constexpr (VEC) {
+                cp_async16(dk, kb + src, ok);
+                cp_async16(dv, vb + src, ok);
+            } else {
 #pragma unroll
-    for (int i = 0; i < HD / 32; ++i) o[i] = 0.f;
-    for (int p0 = beg; p0 < end; p0 += 32) {
-        float cm, cl, co[HD / 32];
-        int pos = p0 + lane;
-        warp_chunk<T, HD>(s_q, kb, vb, pos, pos < end, a.scale_log2, cm, cl, co);
-        merge_partial(m, l, o, cm, cl, co);
+                for (int e = 0; e < V; ++e) {
+                    dk[e] = ok ? kb[src + e] : from_f32<T>(0.f);
+                    dv[e] = ok ? vb[src + e] : from_f32<T>(0.f);
+                }
+            }
+        }
+        cp_async_commit();
+    };
+    float m[BS_PW], l[BS_PW], o[BS_PW][HD / 32];
+#pragma unroll
+    for (int w = 0; w < BS_PW; ++w) {
+        m[w] = -INFINITY;
+        l[w] = 0.f;
+#pragma unroll
+        for (int i = 0; i < HD / 32; ++i) o[w][i] = 0.f;
     }
-    size_t idx = ((size_t)(seq * RT + r) * a.Hq + head) * a.n_split_max + split;
-    if (lane == 0) a.part_ml[idx] = make_float2(m, l);
+    load(beg, 0);
+    for (int p0 = beg, buf = 0; p0 < cta_end; p0 += 32, buf ^= 1) {
+        if (p0 + 32 < cta_end) load(p0 + 32, buf ^ 1);
+        else cp_async_commit();
+        cp_async_wait<1>();
+        __syncthreads();
+        const T* kr = s_k + (buf * 32 + lane) * LD;
+        float acc[BS_PW], p[BS_PW], cm[BS_PW], cl[BS_PW], co[BS_PW][HD / 32];
 #pragma unroll
-    for (int i = 0; i < HD / 32; ++i) a.part_o[idx * HD + lane + 32 * i] = o[i];
+        for (int w = 0; w < BS_PW; ++w) acc[w] = 0.f;
+#pragma unroll 8
+        for (int d = 0; d < HD; d += 4) {
+            const float4 kv = load_f4(kr + d);
+#pragma unroll
+            for (int w = 0; w < BS_PW; ++w) {
+                const float4 qv = load_f4(s_q + w * HD + d);
+                acc[w] = fmaf(qv.w, kv.w, fmaf(qv.z, kv.z, fmaf(qv.y, kv.y, fmaf(qv.x, kv.x, acc[w]))));
+            }
+        }
+#pragma unroll
+        for (int w = 0; w < BS_PW; ++w) {
+            const bool valid = p0 + lane < end[w];
+            const float s = valid ? acc[w] * a.scale_log2 : -INFINITY;
+            cm[w] = warp_max(s);
+            p[w] = valid ? exp2f(s - cm[w]) : 0.f;
+            cl[w] = warp_sum(p[w]);
+#pragma unroll
+            for (int i = 0; i < HD / 32; ++i) co[w][i] = 0.f;
+        }
+        const T* vr = s_v + buf * 32 * LD + lane;
+#pragma unroll 8
+        for (int j = 0; j < 32; ++j) {
+            float v[HD / 32];
+#pragma unroll
+            for (int i = 0; i < HD / 32; ++i) v[i] = to_f32(vr[j * LD + 32 * i]);
+#pragma unroll
+            for (int w = 0; w < BS_PW; ++w) {
+                const float pj = __shfl_sync(0xffffffffu, p[w], j);
+                if (pj != 0.f) {
+#pragma unroll
+                    for (int i = 0; i < HD / 32; ++i) co[w][i] = fmaf(pj, v[i], co[w][i]);
+                }
+            }
+        }
+#pragma unroll
+        for (int w = 0; w < BS_PW; ++w)
+            if (p0 < end[w]) merge_partial(m[w], l[w], o[w], cm[w], cl[w], co[w]);
+        __syncthreads();       // this buffer is loaded again in the next round but one
+    }
+#pragma unroll
+    for (int w = 0; w < BS_PW; ++w) {
+        if (end[w] <= beg) continue;
+        const size_t idx = ((size_t)(seq * RT + row[w]) * a.Hq + kvh * group + (pair0 + w) % group) * a.n_split_max + split;
+        if (lane == 0) a.part_ml[idx] = make_float2(m[w], l[w]);
+#pragma unroll
+        for (int i = 0; i < HD / 32; ++i) a.part_o[idx * HD + lane + 32 * i] = o[w][i];
+    }
 }
 
-// Tail + merge: one warp per (row, head).  grid = (ceil(RT/4), Hq, batch).
-template <typename T, int HD>
+// Tail + merge: one warp per (row, head).  grid = (ceil(rows/4), Hq, batch).
+template <typename T, int HD, bool VEC>
 __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a) {
-    __shared__ float s_qall[4][HD];
+    __shared__ __align__(16) float s_qall[4][HD];
     // let the next kernel start its own preamble (for a GEMM: the first weight tiles) while this one runs; it still
     // waits for this kernel to complete before it touches anything this kernel or its predecessors write
     if (threadIdx.x == 0) pdl_launch_dependents();
@@ -473,7 +723,7 @@ __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a) {
             }
         }
         float cm, cl, co[HD / 32];
-        warp_chunk<T, HD>(s_q, kb, vb, slot, valid, a.scale_log2, cm, cl, co);
+        warp_chunk<T, HD, VEC>(s_q, kb, vb, slot, valid, a.scale_log2, cm, cl, co);
         merge_partial(m, l, o, cm, cl, co);
     }
     T* out = reinterpret_cast<T*>(a.out) + ((size_t)(seq * RT + r) * a.Hq + head) * HD;
@@ -493,16 +743,32 @@ __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a) {
     }
 }
 
-template <typename T, int HD>
-static void launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, bool bulk_too, cudaStream_t s, bool pdl) {
-    dim3 g1((RT + 3) / 4, a.Hq, n_split_launch * batch);
-    if (bulk_too && n_split_launch > 0) launch_k(k_attn_bulk_simt<T, HD>, g1, dim3(128), 0, s, pdl, a, n_split_launch);
-    dim3 g2((RT + 3) / 4, a.Hq, batch);
-    launch_k(k_attn_tail_merge<T, HD>, g2, dim3(128), 0, s, pdl, a);
+template <typename T, int HD, bool VEC>
+static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, bool bulk_too, cudaStream_t s, bool pdl) {
+    if (bulk_too && n_split_launch > 0) {
+        const int pairs = a.rows_cap * (a.Hq / a.Hkv);
+        const long long ctas4 = (long long)((pairs + 15) / 16) * a.Hkv * n_split_launch * batch;
+        // four-pair warps once their CTAs cover half of the SMs
+#define ESP_BULK_SIMT(PW)                                                                                              \
+        {                                                                                                              \
+            if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_attn_bulk_simt<T, HD, VEC, PW>), (int)bulk_simt_smem<T, HD>(PW))) return -1; \
+            launch_k(k_attn_bulk_simt<T, HD, VEC, PW>, dim3((pairs + 4 * PW - 1) / (4 * PW), a.Hkv, n_split_launch * batch), dim3(128),          \
+                     bulk_simt_smem<T, HD>(PW), s, pdl, a, n_split_launch);                                            \
+        }
+        if (ctas4 >= 74) ESP_BULK_SIMT(4) else ESP_BULK_SIMT(1)
+#undef ESP_BULK_SIMT
+    }
+    const dim3 g2((a.rows_cap + 3) / 4, a.Hq, batch);
+    launch_k(k_attn_tail_merge<T, HD, VEC>, g2, dim3(128), 0, s, pdl, a);
+    return 0;
 }
 
 int launch_attn_simt(int dtype, const AttnArgs& a, int batch, int n_split_launch, bool bulk_too, cudaStream_t s, bool pdl) {
-#define ESP_ATTN_CASE(TT, H) launch_attn_simt_t<TT, H>(a, batch, n_split_launch, bulk_too, s, pdl); return 0;
+    // 16-byte loads where the caches start on 16 bytes (their rows then do too)
+    const bool vec = (reinterpret_cast<uintptr_t>(a.kc) | reinterpret_cast<uintptr_t>(a.vc)) % 16 == 0;
+#define ESP_ATTN_CASE(TT, H)                                                              \
+    return vec ? launch_attn_simt_t<TT, H, true>(a, batch, n_split_launch, bulk_too, s, pdl) \
+               : launch_attn_simt_t<TT, H, false>(a, batch, n_split_launch, bulk_too, s, pdl);
     if (dtype == 0) {
         if (a.h == 32) { ESP_ATTN_CASE(float, 32) }
         if (a.h == 64) { ESP_ATTN_CASE(float, 64) }
@@ -1091,8 +1357,8 @@ void launch_assemble(int dtype, const SeqState* st, const void* embed, const flo
     else launch_k(k_assemble<__nv_bfloat16>, grid, dim3(128), 0, s, pdl, st, (const __nv_bfloat16*)embed, mvec, hres, d, mask_slots);
 }
 void launch_rmsnorm(int dtype, const SeqState* st, const float* x, const void* g, void* y, int d, float eps, int batch,
-                    float* copy_out, cudaStream_t s, bool pdl) {
-    dim3 grid(RT, batch);
+                    float* copy_out, cudaStream_t s, bool pdl, int rows_cap) {
+    dim3 grid(rows_cap, batch);
     if (dtype == 0) launch_k(k_rmsnorm<float>, grid, dim3(256), 0, s, pdl, st, x, (const float*)g, (float*)y, d, eps, copy_out);
     else launch_k(k_rmsnorm<__nv_bfloat16>, grid, dim3(256), 0, s, pdl, st, x, (const __nv_bfloat16*)g, (__nv_bfloat16*)y, d, eps, copy_out);
 }

@@ -46,7 +46,7 @@ void launch_mask_init(int dtype, const void* embed, const int32_t* prompt, int t
 void launch_assemble(int dtype, const SeqState* st, const void* embed, const float* mvec, float* hres, int d, int mask_slots,
                      int batch, cudaStream_t s, bool pdl, int rows_cap = RT);
 void launch_rmsnorm(int dtype, const SeqState* st, const float* x, const void* g, void* y, int d, float eps, int batch,
-                    float* copy_out, cudaStream_t s, bool pdl);
+                    float* copy_out, cudaStream_t s, bool pdl, int rows_cap = RT);
 // consumers of the split (EPI_PARTIAL) tensor-core GEMMs, bf16 models; nq = sequences the GEMM launch covered
 // y_lo / act_lo: optional low-order planes (the next GEMM then reads the activation as hi + lo)
 void launch_resid_norm(const SeqState* st, float* hres, const StreamK& sk, const void* g, void* y, void* y_lo, int d, float eps,
@@ -61,8 +61,9 @@ void launch_topk_merge(const SeqState* st, const Cand* cand, const float2* cand_
 void launch_tree_step(int dtype, const TreeArgs& A, cudaStream_t s, bool pdl);
 
 // CUDA-core GEMM (fp32 models; on-GPU cross-check for bf16)
-void launch_gemm_simt(int dtype, int epi, int n_tiles, int batch, const void* const w[3], const int32_t rows_w[3],
-                      const void* x, int K, const EpiArgs& a, cudaStream_t s, bool pdl);
+// (rows_cap: no block has more rows; sizes the grid)
+int launch_gemm_simt(int dtype, int epi, int n_tiles, int batch, const void* const w[3], const int32_t rows_w[3],
+                     const void* x, int K, const EpiArgs& a, int rows_cap, cudaStream_t s, bool pdl);
 
 // position-canonical attention: CUDA-core bulk (+ tail/merge), or tail/merge only when the
 // tensor-core bulk kernel already produced the split partials

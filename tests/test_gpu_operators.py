@@ -57,6 +57,21 @@ def test_gemm_rows_do_not_depend_on_their_neighbours():
     assert np.array_equal(full, again)       # run-to-run deterministic (no arrival-order dependence)
 
 
+@pytest.mark.parametrize("rows", [1, 7, 8, 9, 128])
+def test_cuda_core_gemm_by_elements_equals_16_byte_copies(rows):
+    """A matrix that does not start on 16 bytes goes through the element-wise loads of the CUDA-core kernel: the same
+    sums in the same order, so the same bits, for every remainder of the kernel's groups of 8 rows and 64 k."""
+    g = torch.Generator().manual_seed(rows)
+    n_out, k_in = 200, 136
+    x = torch.randn(rows, k_in, generator=g).bfloat16()
+    flat = torch.zeros(n_out * k_in + 8, dtype=torch.bfloat16, device="cuda")
+    w = (torch.randn(n_out, k_in, generator=g) * 0.05).bfloat16().cuda()
+    odd = flat[1:1 + n_out * k_in].view(n_out, k_in)
+    odd.copy_(w)
+    assert w.data_ptr() % 16 == 0 and odd.data_ptr() % 16 == 2
+    assert np.array_equal(_gemm(1, x, w, rows), _gemm(1, x, odd, rows))
+
+
 # ------------------------------------------------------------------ tree attention (the stand-alone operator workload)
 def _tree_block(n_nodes, n_probes, max_depth, seed):
     parents = synth.random_tree_parents(n_nodes, max_depth, seed)
@@ -189,6 +204,38 @@ def test_tree_attention_rows_equal_decoding_each_path_alone():
             anc1[0, i, i // 64] = np.uint64(1) << np.uint64(i % 64)
         alone = _run_attention(1, q1, kc1, vc1, anc1, np.zeros((1, R), np.int32), 1, L + d, Hq, Hkv, h)
         assert torch.equal(alone[0, 0], tree_out[0, r]), f"row {r} (depth {d})"
+
+
+@pytest.mark.parametrize("dt,h,group,n_rows,L", [("fp32", 64, 2, 35, 777), ("fp32", 128, 1, 17, 300), ("fp32", 32, 8, 3, 33),
+                                                 ("bf16", 64, 4, 9, 1025), ("bf16", 32, 3, 128, 64)])
+def test_cuda_core_attention_edges(dt, h, group, n_rows, L):
+    """The CUDA-core attention against its definition in fp64 at the edges of its 16-pair CTAs, 32-key chunks and
+    splits, with a cache that starts on 16 bytes and one that does not (same bits).  A chain of n_rows rows, so that
+    row r sees positions 0..L+r.  fp32: sums of at most L + n_rows terms; bf16: the result's own rounding."""
+    dtype = torch.float32 if dt == "fp32" else torch.bfloat16
+    Hkv, cap, b = 2, L + R, 2
+    Hq = Hkv * group
+    g = torch.Generator().manual_seed(h + L)
+    q = torch.randn(b, R, Hq, h, generator=g).to(dtype).cuda()
+    kc, vc = (torch.randn(b, Hkv, cap, h, generator=g).to(dtype).cuda() for _ in range(2))
+    vis = np.tril(np.ones((n_rows, n_rows), np.uint8))
+    anc = np.stack([_anc_words(vis)] * b)
+    depth = np.zeros((b, R), np.int32)
+    depth[:, :n_rows] = np.arange(n_rows)
+    dcap = (max(16, n_rows) + 15) // 16 * 16
+    out = _run_attention(int(dt == "bf16"), q, kc, vc, anc, depth, n_rows, L, Hq, Hkv, h, dcap)[:, :n_rows]
+    odd = []
+    for t in (kc, vc):
+        flat = torch.zeros(t.numel() + 8, dtype=dtype, device="cuda")
+        odd.append(flat[1:1 + t.numel()].view(t.shape))
+        odd[-1].copy_(t)
+    assert torch.equal(out, _run_attention(int(dt == "bf16"), q, odd[0], odd[1], anc, depth, n_rows, L, Hq, Hkv, h, dcap)[:, :n_rows])
+    s = torch.einsum("brhd,bhcd->bhrc", q[:, :n_rows].double(), kc.repeat_interleave(group, 1)[:, :, :L + n_rows].double()) / h ** 0.5
+    hide = torch.arange(L + n_rows)[None] > L + torch.arange(n_rows)[:, None]
+    s.masked_fill_(hide.cuda(), -float("inf"))
+    ref = torch.einsum("bhrc,bhcd->brhd", s.softmax(-1), vc.repeat_interleave(group, 1)[:, :, :L + n_rows].double())
+    tol = 2e-5 if dt == "fp32" else 2.0 ** -8 * float(ref.abs().max())
+    assert (out.double() - ref).abs().max() <= tol
 
 
 def test_tree_attention_one_item_and_persistent_kernels_agree_bitwise():
