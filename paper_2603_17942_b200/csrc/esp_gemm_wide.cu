@@ -1,0 +1,344 @@
+// bf16 GEMM over several blocks of rows at once -- the full blocks of a prompt, or the blocks of several sequences in a
+// decode step -- on the Blackwell tensor cores: y[row][n] = sum_k (x_hi[row][k] + x_lo[row][k]) * w[n][k], fp32
+// accumulation, both planes of the activations (see esp_gemm_tc.cu) into one accumulator.
+//
+// With hundreds of rows per weight stream the work is a matter of the tensor cores, and what has to be kept up is
+// their operand supply: shared memory delivers 128 bytes per clock, an MMA of N = 240 takes 98 of them for its
+// operands, and what a tile needs from L2 passes through the same port.  A 256-feature x 240-row tile needs 32 KB of
+// weights and 60 KB of activations per 64 k for 16 MMAs of N = 240 (48 bytes per clock); a 128-feature tile, as the
+// small-M kernel has it, would need 79.  The tile is the whole tensor memory (two accumulators of up to 240 of 256
+// columns), so there is one in flight per CTA.
+//
+// Work split: a row tile is BPT blocks of WB rows (one TMA box of BPT x WB rows per plane).  The CTAs form groups of
+// one CTA per row tile; a group owns a contiguous range of the (256-feature tile, k-block) units, stream-K style, and
+// its CTAs walk it in step, so that a weight unit is read from HBM once and from L2 by the other row tiles.  Every
+// piece is stored as an fp32 partial; the kernel that consumes the result sums a tile's pieces in group order, as it
+// does for the small-M kernel (StreamK with one row space for all row tiles).
+//
+// Ring: seven slots of 32 KB, filled in the order [two weight units | hi rows | lo rows] per k-block.  The hi slot is
+// released half a k-block before the other two.  Roles: warp 0 producer, warp 1 MMA issuer, warps 2-9 epilogue (four
+// per accumulator).  Every mbarrier wait is bounded, as in esp_gemm_tc.cu.
+#include <new>
+#include <string.h>
+
+#include "esp_gemm_tc.cuh"
+#include "esp_launch.h"
+
+namespace esp {
+
+namespace {
+
+using namespace tc;
+
+constexpr int SLOT_BYTES = 2 * A_BYTES;        // 32 KB: two weight units, or one plane of a row tile
+constexpr int SLOTS = 7;
+constexpr int WIDE_THREADS = 320;
+constexpr size_t WIDE_SMEM = 1024 + (size_t)SLOTS * SLOT_BYTES + 256;
+static_assert(WIDE_SMEM <= 232448, "shared memory");
+
+struct WideParams {
+    CUtensorMap map_b;          // activations [2 planes x x_blocks][RT][K], box 64 x WB x BPT
+    const unsigned char* w;     // packed weight units [n_tiles][KB][A_BYTES]
+    const SeqState* st;         // one state per block
+    float* partials;            // [group][slot][2 halves][n_rt * WR rows][128 features]
+    int* err;
+    int32_t n_tiles, n_ft, KB, n_groups, n_rt, slots, plane_blocks, n_blocks;
+};
+
+template <int WB, int BPT>
+__global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_constant__ WideParams p) {
+    constexpr int WR = WB * BPT;               // rows of a row tile = MMA N
+    constexpr int X_BYTES = WR * BK * 2;
+    static_assert(WR % 16 == 0 && WR <= 256 && X_BYTES <= SLOT_BYTES && WB % 8 == 0 && WB <= RT, "row tile");
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint64_t* full = reinterpret_cast<uint64_t*>(ring + SLOTS * SLOT_BYTES);
+    uint64_t* empty = full + SLOTS;
+    uint64_t* tfull = empty + SLOTS;
+    uint64_t* tempty = tfull + 1;
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(tempty + 1);
+    volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rt = blockIdx.x % p.n_rt, grp = blockIdx.x / p.n_rt;
+    const long long U = (long long)p.n_ft * p.KB;
+    const int u0 = (int)sk_begin(grp, U, p.n_groups), u1 = (int)sk_begin(grp + 1, U, p.n_groups);
+    const int n_units = u1 - u0;
+
+    if (threadIdx.x == 0) {
+        pdl_launch_dependents();
+        prefetch_tensormap(&p.map_b);
+        for (int i = 0; i < SLOTS; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+        mbar_init(tfull, 1);
+        mbar_init(tempty, 8);           // one arrival per epilogue warp
+        *s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = *s_tmem;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            const uint64_t pol_w = l2_policy_evict_first(), pol_x = l2_policy_evict_last();
+            // item i: unit u0 + i / 3; i % 3 = 0 weights, 1 hi rows, 2 lo rows
+            auto load = [&](int i, int slot) {
+                unsigned char* dst = ring + slot * SLOT_BYTES;
+                const int u = u0 + i / 3, kind = i % 3, ft = u / p.KB, kb = u % p.KB;
+                if (kind == 0) {
+                    mbar_expect_tx(&full[slot], SLOT_BYTES);
+                    const int t1 = 2 * ft + 1 < p.n_tiles ? 2 * ft + 1 : 2 * ft;      // (an odd last tile fills both halves)
+                    bulk_load(dst, p.w + ((size_t)(2 * ft) * p.KB + kb) * A_BYTES, A_BYTES, &full[slot], pol_w);
+                    bulk_load(dst + A_BYTES, p.w + ((size_t)t1 * p.KB + kb) * A_BYTES, A_BYTES, &full[slot], pol_w);
+                } else {
+                    mbar_expect_tx(&full[slot], X_BYTES);
+                    tma_load_3d_hint(dst, &p.map_b, kb * BK, 0, (kind - 1) * p.plane_blocks + rt * BPT, &full[slot], pol_x);
+                }
+            };
+            const int n_items = 3 * n_units, n_pre = n_items < SLOTS ? n_items : SLOTS;
+            // the weights do not depend on the kernel before this one, the activations do
+            for (int i = 0; i < n_pre; i += 3) load(i, i);
+            pdl_wait();
+            for (int i = 0; i < n_pre; ++i)
+                if (i % 3) load(i, i);
+            bool ok = true;
+            int slot = 0;
+            uint32_t phase = 0;          // parity of the slot's release that item i waits for
+            for (int i = n_pre; i < n_items; ++i) {
+                if (!mbar_wait(&empty[slot], phase, s_abort)) { ok = false; break; }
+                load(i, slot);
+                if (++slot == SLOTS) { slot = 0; phase ^= 1; }
+            }
+            if (!ok) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t IDESC = idesc_of(WR);
+            bool ok = true;
+            int slot = 0, piece = 0;
+            uint32_t phase = 0;
+            auto next = [&](int& s, uint32_t& ph) { if (++s == SLOTS) { s = 0; ph ^= 1; } };
+            for (int u = u0; u < u1 && ok; ++piece) {
+                const int end = (u / p.KB + 1) * p.KB < u1 ? (u / p.KB + 1) * p.KB : u1;
+                if (!mbar_wait(tempty, (piece & 1) ^ 1, s_abort)) { ok = false; break; }     // (a fresh barrier passes parity 1)
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                for (const int beg = u; u < end; ++u) {
+                    const int sw = slot;
+                    const uint32_t pw = phase;
+                    next(slot, phase);
+                    const int sh = slot;
+                    const uint32_t ph = phase;
+                    next(slot, phase);
+                    const int sl = slot;
+                    const uint32_t pl = phase;
+                    next(slot, phase);
+                    if (!mbar_wait(&full[sw], pw, s_abort) || !mbar_wait(&full[sh], ph, s_abort)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint64_t dw = smem_desc(smem_u32(ring + sw * SLOT_BYTES), 16);
+                    const uint64_t dh = smem_desc(smem_u32(ring + sh * SLOT_BYTES), 16);
+#pragma unroll
+                    for (int k = 0; k < BK / 16; ++k) {
+                        const uint32_t acc = (u > beg || k > 0) ? 1u : 0u;
+                        umma(tmem_base, dw + (uint64_t)(k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
+                        umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
+                    }
+                    umma_commit(&empty[sh]);
+                    if (!mbar_wait(&full[sl], pl, s_abort)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint64_t dl = smem_desc(smem_u32(ring + sl * SLOT_BYTES), 16);
+#pragma unroll
+                    for (int k = 0; k < BK / 16; ++k) {
+                        umma(tmem_base, dw + (uint64_t)(k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
+                        umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
+                    }
+                    umma_commit(&empty[sw]);
+                    umma_commit(&empty[sl]);
+                }
+                if (ok) umma_commit(tfull);
+            }
+            if (!ok) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
+        }
+    } else {
+        // ---------------- epilogue: tensor memory -> registers -> partial
+        pdl_wait();                              // the partials' last reader has finished
+        const int half = (warp - 2) >> 2, q = warp & 3, f = q * 32 + lane;
+        const uint32_t taddr = tmem_base + half * 256 + ((uint32_t)(q * 32) << 16);
+        const size_t rows = (size_t)p.n_rt * WR;
+        int nr[BPT];
+#pragma unroll
+        for (int b = 0; b < BPT; ++b)
+            nr[b] = rt * BPT + b < p.n_blocks && p.st[rt * BPT + b].active ? min(p.st[rt * BPT + b].n_rows, WB) : 0;
+        bool ok = true;
+        int piece = 0;
+        const int ft0 = u0 / p.KB;
+        for (int u = u0; u < u1 && ok; ++piece) {
+            const int ft = u / p.KB;
+            u = (ft + 1) * p.KB < u1 ? (ft + 1) * p.KB : u1;
+            // (a wait that fails takes the whole warp out: the tensor-memory loads below are warp-wide)
+            if (!__all_sync(0xffffffffu, mbar_wait(tfull, piece & 1, s_abort))) { ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const bool real = 2 * ft + half < p.n_tiles;
+            float* part = p.partials + (((size_t)(grp * p.slots + (ft - ft0)) * 2 + half) * rows + (size_t)rt * WR) * TILE_N + f;
+            // CH columns at a time: as many 16-column loads as fit, an 8-column load for the rest, one wait
+            constexpr int CH = WB % 24 == 0 ? 24 : (WB % 40 == 0 ? 40 : 32);
+            static_assert(WB % CH == 0 && (CH % 16 == 0 || CH % 16 == 8), "columns per wait");
+#pragma unroll
+            for (int b = 0; b < BPT; ++b) {
+                const int n = real ? nr[b] : 0;
+#pragma unroll
+                for (int c0 = 0; c0 < WB; c0 += CH) {
+                    uint32_t v[CH];
+#pragma unroll
+                    for (int c = 0; c + 16 <= CH; c += 16) tmem_ld16_issue(taddr + b * WB + c0 + c, *reinterpret_cast<uint32_t(*)[16]>(&v[c]));
+                    if constexpr (CH % 16 == 8)
+                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                                     : "=r"(v[CH - 8]), "=r"(v[CH - 7]), "=r"(v[CH - 6]), "=r"(v[CH - 5]), "=r"(v[CH - 4]), "=r"(v[CH - 3]),
+                                       "=r"(v[CH - 2]), "=r"(v[CH - 1])
+                                     : "r"(taddr + b * WB + c0 + CH - 8));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (b == BPT - 1 && c0 + CH >= WB) {        // the accumulator is in registers
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(tempty);
+                    }
+#pragma unroll
+                    for (int i = 0; i < CH; ++i)
+                        if (c0 + i < n) __stcg(part + (size_t)(b * WB + c0 + i) * TILE_N, __uint_as_float(v[i]));
+                }
+            }
+        }
+        if (!ok && lane == 0) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
+    }
+    // ---------------- teardown (every thread arrives here)
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (*s_abort) {
+        for (int i = 0; i < 64; ++i) __nanosleep(10000);   // let copies in flight land before shared memory goes away
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp == 1) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+    }
+}
+
+constexpr int WIDE_SM = 148;
+
+}  // namespace
+
+// Groups and partial slots of a GEMM of n_tiles 128-feature tiles and KB k-blocks over n_rt row tiles.
+void wide_geometry(int n_tiles, int KB, int n_rt, int* n_groups, int* slots) {
+    const int n_ft = (n_tiles + 1) / 2;
+    const long long U = (long long)n_ft * KB;
+    long long g = WIDE_SM / n_rt;
+    if (g > U) g = U;
+    // a consumer sums at most 15 pieces of a tile: no group smaller than a 13th of a tile
+    while (g > 1 && U / g * 13 < KB) --g;
+    int most = 1;
+    for (int c = 0; c < g; ++c) {
+        const int n = (int)((sk_begin(c + 1, U, g) - 1) / KB - sk_begin(c, U, g) / KB) + 1;
+        most = n > most ? n : most;
+    }
+    *n_groups = (int)g;
+    *slots = most;
+}
+
+size_t wide_partial_bytes(int n_tiles, int KB, int n_rt, int tile_rows) {
+    int g, slots;
+    wide_geometry(n_tiles, KB, n_rt, &g, &slots);
+    return (size_t)g * slots * 2 * n_rt * tile_rows * TILE_N * sizeof(float);
+}
+
+struct WideGemm {
+    WideParams p;
+    int n_rt_max, wb, bpt;      // row tiles at most; rows per block, blocks per row tile
+    int groups[WIDE_MAX_RT], slots[WIDE_MAX_RT];
+    TileSrc* tables;            // [n_rt_max][n_tiles]
+};
+
+int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int wb, int bpt, int n_rt_max, float* partials, size_t partial_bytes,
+                     TileSrc* tables_dev, int* err, cudaStream_t stream) {
+    if (!out || n_rt_max < 1 || n_rt_max > WIDE_MAX_RT || x_blocks < bpt || K % 8 || reinterpret_cast<uintptr_t>(x) % 16) return -1;
+    EncodeFn enc = get_encode();
+    if (!enc) return -1;
+    WideGemm* g = new (std::nothrow) WideGemm();
+    if (!g) return -1;
+    memset(&g->p, 0, sizeof(g->p));
+    WideParams& p = g->p;
+    p.n_tiles = n_tiles; p.n_ft = (n_tiles + 1) / 2; p.KB = (K + BK - 1) / BK;
+    p.partials = partials; p.err = err; p.plane_blocks = x_blocks;
+    g->n_rt_max = n_rt_max; g->wb = wb; g->bpt = bpt;
+    g->tables = tables_dev;
+    {
+        cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)RT, (cuuint64_t)2 * x_blocks};
+        cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)RT * K * 2};
+        cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)wb, (cuuint32_t)bpt};
+        cuuint32_t estr[3] = {1, 1, 1};
+        if (enc(&p.map_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) { delete g; return -1; }
+    }
+    TileSrc* tab = new (std::nothrow) TileSrc[(size_t)n_rt_max * n_tiles];
+    bool fits = tab != nullptr;
+    for (int r = 1; r <= n_rt_max && fits; ++r) {
+        wide_geometry(n_tiles, p.KB, r, &g->groups[r - 1], &g->slots[r - 1]);
+        fits = wide_partial_bytes(n_tiles, p.KB, r, wb * bpt) <= partial_bytes;
+        const long long U = (long long)p.n_ft * p.KB, G = g->groups[r - 1];
+        for (int t = 0; t < n_tiles && fits; ++t) {
+            TileSrc& e = tab[(size_t)(r - 1) * n_tiles + t];
+            memset(&e, 0, sizeof(e));
+            const int ft = t / 2;
+            const int c0 = sk_cta_of_unit((long long)ft * p.KB, U, G), c1 = sk_cta_of_unit((long long)ft * p.KB + p.KB - 1, U, G);
+            if (c1 - c0 + 1 > 15 || ((long long)c1 + 1) * g->slots[r - 1] * 2 > 65535) { fits = false; break; }
+            e.n = (uint16_t)(c1 - c0 + 1);
+            for (int c = c0; c <= c1; ++c)
+                e.idx[c - c0] = (uint16_t)((c * g->slots[r - 1] + (ft - (int)(sk_begin(c, U, G) / p.KB))) * 2 + (t & 1));
+        }
+    }
+    if (fits && cudaMemcpyAsync(tables_dev, tab, sizeof(TileSrc) * n_rt_max * n_tiles, cudaMemcpyHostToDevice, stream) != cudaSuccess) fits = false;
+    if (fits && cudaStreamSynchronize(stream) != cudaSuccess) fits = false;
+    delete[] tab;
+    if (!fits) { delete g; return -1; }
+    *out = g;
+    return 0;
+}
+
+void wide_gemm_destroy(WideGemm* g) { delete g; }
+
+int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, int n_blocks, cudaStream_t s, bool pdl) {
+    if (!g || n_blocks < 1) return ESP_E_ARG;
+    const int n_rt = (n_blocks + g->bpt - 1) / g->bpt;
+    if (n_rt > g->n_rt_max) return ESP_E_ARG;
+    WideParams p = g->p;
+    p.w = reinterpret_cast<const unsigned char*>(packed);
+    p.st = st;
+    p.n_rt = n_rt; p.n_blocks = n_blocks; p.n_groups = g->groups[n_rt - 1]; p.slots = g->slots[n_rt - 1];
+#define ESP_WIDE_CASE(WB, BPT)                                                                                          \
+    if (g->wb == WB && g->bpt == BPT) {                                                                                \
+        if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_gemm_wide<WB, BPT>), (int)WIDE_SMEM)) return ESP_E_CUDA; \
+        return launch_k(k_gemm_wide<WB, BPT>, dim3(p.n_groups * n_rt), dim3(WIDE_THREADS), WIDE_SMEM, s, pdl, p) == cudaSuccess ? ESP_OK : ESP_E_CUDA; \
+    }
+    ESP_WIDE_CASE(PREFILL_CHUNK, 2)
+    ESP_WIDE_CASE(80, 2)
+    ESP_WIDE_CASE(80, 3)
+    ESP_WIDE_CASE(RT, 2)
+#undef ESP_WIDE_CASE
+    return ESP_E_ARG;
+}
+
+// the row of block b, row r in the partials is b * wb + r
+StreamK wide_gemm_streamk(const WideGemm* g, int n_blocks) {
+    const int n_rt = (n_blocks + g->bpt - 1) / g->bpt;
+    StreamK k;
+    k.partials = g->p.partials;
+    k.table = g->tables + (size_t)(n_rt - 1) * g->p.n_tiles;
+    k.n_tiles = g->p.n_tiles; k.KB = g->p.KB; k.G = g->groups[n_rt - 1]; k.slots = g->slots[n_rt - 1];
+    k.rows = n_rt * g->bpt * g->wb;
+    k.seq_rows = g->wb;
+    return k;
+}
+
+}  // namespace esp
