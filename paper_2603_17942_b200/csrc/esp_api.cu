@@ -426,16 +426,17 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
         h->launches++;
         mark(h, KIND_MISC);
         const int n_tiles = (D.V + TILE_N - 1) / TILE_N;
-        // tensor-core path: the LM head and its selection run once per sequence (the candidate lists are shared)
-        const int n_lm = tc ? nb : 1, per = tc ? 1 : nb;
-        for (int q = 0; q < n_lm; ++q) {
-            const int sq = s0 + q;
+        // tensor-core path: the sequences of a pass share the LM head's weight stream too (128-row plans: one at a time;
+        // the candidate lists are shared)
+        const int lm_nq = tc ? tc_gemm_nq(wide ? h->p_lm_w : h->p_lm) : nb;
+        for (int q = 0; q < nb; q += lm_nq) {
+            const int sq = s0 + q, per = nb - q < lm_nq ? nb - q : lm_nq;
             EpiArgs a = base_epi(h, D.V, sq, per);
             a.cand = b.cand; a.cand_ms = b.cand_ms; a.cand_floor = b.cand_floor; a.n_tiles = n_tiles;
             a.logits_dump = h->dbg_logits ? h->dbg_logits + (size_t)sq * RT * D.V : nullptr;
             const void* w[3] = {h->lm_head, nullptr, nullptr};
             const int32_t rows[3] = {D.V, 0, 0};
-            int rc = run_gemm(h, wide ? h->p_lm_w : h->p_lm, EPI_LOGITS, n_tiles, w, rows, b.xn, D.d, a, tc, pdl, rc_rows, 1, q);
+            int rc = run_gemm(h, wide ? h->p_lm_w : h->p_lm, EPI_LOGITS, n_tiles, w, rows, b.xn, D.d, a, tc, pdl, rc_rows, per, q);
             if (rc) return rc;
             mark(h, KIND_LMHEAD);
             launch_topk_merge(b.states + sq, b.cand, b.cand_ms, n_tiles, D.KP, per, b.topk + (size_t)sq * RT * KP_MAX, b.lse + (size_t)sq * RT, s, pdl, rc_rows, b.cand_floor);
@@ -605,7 +606,7 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
         }
         const void* w5[3] = {h->lm_head, nullptr, nullptr};
         const int32_t r5[3] = {D.V, 0, 0};
-        ok = ok && !tc_gemm_create(&h->p_lm, EPI_LOGITS, false, w5, r5, D.d, h->b.xn, D.batch, nrs, 1, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, nullptr, 0, h->b.packed + h->b.pk_layer * D.n_layers, h->stream);
+        ok = ok && !tc_gemm_create(&h->p_lm, EPI_LOGITS, false, w5, r5, D.d, h->b.xn, D.batch, nrs, nrs == 80 ? nq_max : 1, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, nullptr, 0, h->b.packed + h->b.pk_layer * D.n_layers, h->stream);
         if (ok && nrs != RT) {
             // the prefill runs 120-row blocks: the same weights (already repacked) behind 128-row GEMM plans
             const size_t pbytes = tc_gemm_partial_bytes(148, 1, RT);

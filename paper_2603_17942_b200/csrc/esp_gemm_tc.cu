@@ -54,7 +54,7 @@ using namespace tc;
 // instead of 2^-9, for 10 KB more shared memory per stage and sequence.
 __host__ __device__ constexpr int stages_of(int epi, int nq, int nrs, int pl = 1) {
     return pl == 2 ? (nrs == 80 ? (nq == 2 ? 4 : 6) : 4)
-                   : (nrs == 80 ? (nq == 3 ? 4 : (nq == 2 ? 6 : (epi == EPI_PARTIAL ? 8 : 6)))
+                   : (nrs == 80 ? (nq == 3 ? 4 : (nq == 2 ? (epi == EPI_PARTIAL ? 6 : 5) : (epi == EPI_PARTIAL ? 8 : 6)))
                                 : (nq == 2 ? 4 : (epi == EPI_PARTIAL ? 7 : 4)));
 }
 __host__ __device__ constexpr int b_bytes_of(int nq, int nrs) { return nq * nrs * BK * 2; }   // 10240 per 80-row sequence and plane
@@ -92,7 +92,7 @@ __device__ __forceinline__ void tile_source(const TcParams& p, int tile, int hal
 
 template <int EPI, int NQ, int NRS, int PL>
 __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constant__ TcParams p) {
-    static_assert(NQ == 1 || EPI == EPI_PARTIAL, "several sequences per launch: partial-only output");
+    static_assert(NQ == 1 || EPI == EPI_PARTIAL || EPI == EPI_LOGITS, "several sequences per launch: partials or logits");
     static_assert(NQ * NRS <= 256 && (PL == 1 || NQ > 1 || 2 * NRS <= 256) && NRS % 16 == 0 && NRS <= RT, "MMA N");
     static_assert(PL == 1 || EPI == EPI_PARTIAL, "two activation planes: partial-only output");
     // One sequence with two planes: hi and lo rows sit back to back in the stage and form ONE B operand of 2 * NRS
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
         const int q = warp & 3;                 // TMEM lane quarter this warp may read
         const int f = q * 32 + lane;            // feature of the tile owned by this thread
         const int et = threadIdx.x - 64;        // 0..127 index among the epilogue threads
-        const int n_rows = p.a.st ? (p.a.st->active ? p.a.st->n_rows : 0) : p.a.rows_fixed;
+        auto rows_of = [&](int sq) { return p.a.st ? (p.a.st[sq].active ? p.a.st[sq].n_rows : 0) : p.a.rows_fixed; };
         StreamK sk;
         sk.partials = p.partials; sk.table = nullptr; sk.n_tiles = p.n_tiles; sk.KB = p.KB; sk.G = p.grid; sk.slots = p.slots;
         sk.rows = NQ * NRS; sk.seq_rows = NRS;
@@ -258,55 +258,46 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
             if (s_flag[0]) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t taddr = tmem_base + buf * ACC_COLS + ((uint32_t)(q * 32) << 16);
-            uint32_t v[NRS];
-            if constexpr (NQ > 1) {
-                // sequence by sequence: 80 accumulator columns -> that sequence's rows of the partial
-                float* part = p.partials + ((size_t)(blockIdx.x * p.slots + sg.slot) * (NQ * NRS)) * TILE_N + f;
+            const bool direct = EPI != EPI_PARTIAL && sg.whole;
+            float* part = p.partials + ((size_t)(blockIdx.x * p.slots + sg.slot) * (NQ * NRS)) * TILE_N + f;
+            // sequence by sequence: NRS accumulator columns -> that sequence's rows of the partial, or (a whole tile of a
+            // fused epilogue) shared memory and the epilogue
 #pragma unroll 1
-                for (int sq = 0; sq < NQ; ++sq) {
+            for (int sq = 0; sq < NQ; ++sq) {
+                uint32_t v[NRS];
 #pragma unroll
-                    for (int c = 0; c < NRS / 16; ++c)
-                        tmem_ld16_issue(taddr + sq * NRS + c * 16, *reinterpret_cast<uint32_t(*)[16]>(&v[c * 16]));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    const SeqState* sst = p.a.st + sq;
-                    const int nr = sst->active ? sst->n_rows : 0;
+                for (int c = 0; c < NRS / 16; ++c)
+                    tmem_ld16_issue(taddr + sq * NRS + c * 16, *reinterpret_cast<uint32_t(*)[16]>(&v[c * 16]));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if constexpr (JOINT) {      // + the product with the low-order plane
+#pragma unroll
+                    for (int c = 0; c < NRS / 16; ++c) {
+                        uint32_t lo16[16];
+                        tmem_ld16_issue(taddr + NRS + c * 16, lo16);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) v[c * 16 + j] = __float_as_uint(__fadd_rn(__uint_as_float(v[c * 16 + j]), __uint_as_float(lo16[j])));
+                    }
+                }
+                if (sq == NQ - 1) {         // the accumulator is in registers: hand the tensor-memory buffer back to the MMA warp
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    mbar_arrive(&tempty[buf]);
+                }
+                const int nr = rows_of(sq);
+                if (!direct) {
 #pragma unroll
                     for (int r = 0; r < NRS; ++r)
                         if (r < nr) __stcg(part + (size_t)(sq * NRS + r) * TILE_N, __uint_as_float(v[r]));
-                }
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                mbar_arrive(&tempty[buf]);
-                continue;
-            }
+                } else if constexpr (EPI != EPI_PARTIAL) {
 #pragma unroll
-            for (int c = 0; c < NRS / 16; ++c) tmem_ld16_issue(taddr + c * 16, *reinterpret_cast<uint32_t(*)[16]>(&v[c * 16]));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if constexpr (JOINT) {      // + the product with the low-order plane
-#pragma unroll
-                for (int c = 0; c < NRS / 16; ++c) {
-                    uint32_t lo16[16];
-                    tmem_ld16_issue(taddr + NRS + c * 16, lo16);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) v[c * 16 + j] = __float_as_uint(__fadd_rn(__uint_as_float(v[c * 16 + j]), __uint_as_float(lo16[j])));
+                    for (int r = 0; r < NRS; ++r) s_acc[r * ACC_LD + f] = __uint_as_float(v[r]);
+                    epi_bar(2);
+                    if (NQ == 1 || nr > 0) run_epilogue<__nv_bfloat16, EPI>(s_acc, s_aux, sg.tile, sq, p.a, f, 2);
+                    epi_bar(2);
                 }
             }
-            // the accumulator is in registers: hand the tensor-memory buffer back to the MMA warp
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            mbar_arrive(&tempty[buf]);
-            const bool direct = EPI != EPI_PARTIAL && sg.whole;
-            if (direct) {
-#pragma unroll
-                for (int r = 0; r < NRS; ++r) s_acc[r * ACC_LD + f] = __uint_as_float(v[r]);
-            } else {
-                float* part = p.partials + ((size_t)(blockIdx.x * p.slots + sg.slot) * NRS) * TILE_N + f;
-#pragma unroll
-                for (int r = 0; r < NRS; ++r)
-                    if (r < n_rows) __stcg(part + r * TILE_N, __uint_as_float(v[r]));
-            }
-            if (EPI == EPI_PARTIAL) continue;   // the consumer kernel sums the partials
-            bool finish = direct;
-            if (!direct) {
+            if constexpr (EPI != EPI_PARTIAL) {     // (EPI_PARTIAL: the consumer kernel sums the partials)
+                if (direct) continue;
                 int c_first, c_last;
                 sk_contributors(sk, sg.tile, c_first, c_last);
                 __threadfence();
@@ -316,56 +307,58 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
                     s_flag[1] = (old == c_last - c_first) ? 1 : 0;
                 }
                 epi_bar(2);
-                finish = s_flag[1] != 0;
-                if (finish) {
+                if (s_flag[1]) {
                     // last contributor of this tile: sum the partials in CTA order (fixed, whoever arrives last)
                     __threadfence();
-                    // thread et: features 4*(et%32)..+3, rows et/32 + 4*i; every load of a batch is issued before the sums
-                    const int f4 = (et & 31) * 4, rg = et >> 5;
-                    for (int i0 = 0; i0 < NRS / 4; i0 += 4) {
-                        if (rg + 4 * i0 >= n_rows) break;
-                        float4 acc[4];
+#pragma unroll 1
+                    for (int sq = 0; sq < NQ; ++sq) {
+                        const int nr = rows_of(sq);
+                        // thread et: features 4*(et%32)..+3, rows et/32 + 4*i; every load of a batch is issued before the sums
+                        const int f4 = (et & 31) * 4, rg = et >> 5;
+                        for (int i0 = 0; i0 < NRS / 4; i0 += 4) {
+                            if (rg + 4 * i0 >= nr) break;
+                            float4 acc[4];
 #pragma unroll
-                        for (int ii = 0; ii < 4; ++ii) acc[ii] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        for (int cb = c_first; cb <= c_last; cb += 4) {
-                            float4 t[4][4];
+                            for (int ii = 0; ii < 4; ++ii) acc[ii] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            for (int cb = c_first; cb <= c_last; cb += 4) {
+                                float4 t[4][4];
 #pragma unroll
-                            for (int cc = 0; cc < 4; ++cc) {
-                                const int c = cb + cc;
-                                const bool cv = c <= c_last;
-                                const float* src = sk_partial(sk, cv ? c : c_first, sg.tile, 0) + f4;
+                                for (int cc = 0; cc < 4; ++cc) {
+                                    const int c = cb + cc;
+                                    const bool cv = c <= c_last;
+                                    const float* src = sk_partial(sk, cv ? c : c_first, sg.tile, sq * NRS) + f4;
 #pragma unroll
-                                for (int ii = 0; ii < 4; ++ii) {
-                                    const int r = rg + 4 * (i0 + ii);
-                                    t[cc][ii] = (cv && r < n_rows) ? __ldcg(reinterpret_cast<const float4*>(src + (size_t)r * TILE_N))
+                                    for (int ii = 0; ii < 4; ++ii) {
+                                        const int r = rg + 4 * (i0 + ii);
+                                        t[cc][ii] = (cv && r < nr) ? __ldcg(reinterpret_cast<const float4*>(src + (size_t)r * TILE_N))
                                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+                                    }
                                 }
+#pragma unroll
+                                for (int cc = 0; cc < 4; ++cc)
+#pragma unroll
+                                    for (int ii = 0; ii < 4; ++ii) {
+                                        acc[ii].x += t[cc][ii].x; acc[ii].y += t[cc][ii].y;
+                                        acc[ii].z += t[cc][ii].z; acc[ii].w += t[cc][ii].w;
+                                    }
                             }
 #pragma unroll
-                            for (int cc = 0; cc < 4; ++cc)
-#pragma unroll
-                                for (int ii = 0; ii < 4; ++ii) {
-                                    acc[ii].x += t[cc][ii].x; acc[ii].y += t[cc][ii].y;
-                                    acc[ii].z += t[cc][ii].z; acc[ii].w += t[cc][ii].w;
+                            for (int ii = 0; ii < 4; ++ii) {
+                                const int r = rg + 4 * (i0 + ii);
+                                if (r < NRS) {
+                                    float* d = s_acc + r * ACC_LD + f4;
+                                    d[0] = acc[ii].x; d[1] = acc[ii].y; d[2] = acc[ii].z; d[3] = acc[ii].w;
                                 }
-                        }
-#pragma unroll
-                        for (int ii = 0; ii < 4; ++ii) {
-                            const int r = rg + 4 * (i0 + ii);
-                            if (r < NRS) {
-                                float* d = s_acc + r * ACC_LD + f4;
-                                d[0] = acc[ii].x; d[1] = acc[ii].y; d[2] = acc[ii].z; d[3] = acc[ii].w;
                             }
                         }
+                        epi_bar(2);
+                        if (NQ == 1 || nr > 0) run_epilogue<__nv_bfloat16, EPI>(s_acc, s_aux, sg.tile, sq, p.a, f, 2);
+                        epi_bar(2);
                     }
                     if (et == 0) p.counters[sg.tile] = 0;
                 }
-            }
-            if (finish) {
                 epi_bar(2);
-                run_epilogue<__nv_bfloat16, EPI>(s_acc, s_aux, sg.tile, 0, p.a, f, 2);
             }
-            epi_bar(2);
         }
         if (!ok && lane == 0) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
     }
@@ -463,6 +456,7 @@ size_t tc_gemm_packed_bytes(int epi, const int32_t rows_w[3], int K) {
     const long long n_tiles = epi == EPI_SWIGLU ? (rows_w[0] + 63) / 64 : (total + TILE_N - 1) / TILE_N;
     return (size_t)(n_tiles * ((K + BK - 1) / BK)) * A_BYTES;
 }
+int tc_gemm_nq(const TcGemm* g) { return g->nq_max; }
 int tc_gemm_tiles(const TcGemm* g) { return g ? g->p.n_tiles : 0; }
 void tc_gemm_geometry(const TcGemm* g, TcGemmGeom* out) {
     out->n_tiles = g->p.n_tiles; out->KB = g->p.KB; out->grid = g->p.grid; out->slots = g->p.slots;
@@ -477,7 +471,7 @@ int tc_gemm_create(TcGemm** out, int epi, bool defer, const void* const w[3], co
     if (!out || (nrs != 80 && nrs != RT) || (planes != 1 && planes != 2) || nq_max < 1 || nq_max > max_nq_of(nrs, planes) ||
         x_seqs < nq_max || K % 8 || n_sm < 1)
         return -1;
-    if ((nq_max > 1 || planes > 1) && !defer) return -1;
+    if (((nq_max > 1 && (epi != EPI_LOGITS || nq_max > 2 || nrs != 80)) || planes > 1) && !defer) return -1;
     if (reinterpret_cast<uintptr_t>(x) % 16) return -1;
     TcGemm* g = new (std::nothrow) TcGemm();
     if (!g) return -1;
@@ -590,7 +584,6 @@ StreamK tc_gemm_streamk(const TcGemm* g, int nq) {
 // nq sequences starting at sequence b_seq0 of the plan's activation buffer
 int tc_gemm_launch(const TcGemm* g, const EpiArgs& a, cudaStream_t s, bool pdl, int nq, int b_seq0) {
     if (!g || nq < 1 || nq > g->nq_max || b_seq0 < 0) return ESP_E_ARG;
-    if (nq > 1 && g->p.epi != EPI_PARTIAL) return ESP_E_ARG;
     TcParams p = g->p;
     p.a = a;
     p.map_b = g->map_b_nq[nq - 1];
@@ -611,7 +604,8 @@ int tc_gemm_launch(const TcGemm* g, const EpiArgs& a, cudaStream_t s, bool pdl, 
     }
     else if (p.epi == EPI_STORE_F32 && !wide) ESP_TC_CASE(EPI_STORE_F32, 1, 80, 1)
     else if (p.epi == EPI_STORE_F32) ESP_TC_CASE(EPI_STORE_F32, 1, RT, 1)
-    else if (p.epi == EPI_LOGITS && !wide) ESP_TC_CASE(EPI_LOGITS, 1, 80, 1)
+    else if (p.epi == EPI_LOGITS && !wide && nq == 1) ESP_TC_CASE(EPI_LOGITS, 1, 80, 1)
+    else if (p.epi == EPI_LOGITS && !wide && nq == 2) ESP_TC_CASE(EPI_LOGITS, 2, 80, 1)
     else if (p.epi == EPI_LOGITS) ESP_TC_CASE(EPI_LOGITS, 1, RT, 1)
     else if (p.epi == EPI_PARTIAL && !wide && nq == 1) ESP_TC_CASE(EPI_PARTIAL, 1, 80, 1)
     else if (p.epi == EPI_PARTIAL && !wide && nq == 2) ESP_TC_CASE(EPI_PARTIAL, 2, 80, 1)

@@ -121,6 +121,7 @@ int tc_gemm_launch(const TcGemm* g, const EpiArgs& a, cudaStream_t s, bool pdl, 
 StreamK tc_gemm_streamk(const TcGemm* g, int nq = 1);
 int tc_wait_selftest(int* err_dev, cudaStream_t s);
 int tc_gemm_tiles(const TcGemm* g);
+int tc_gemm_nq(const TcGemm* g);     // sequences one launch of the plan may cover
 size_t tc_gemm_partial_bytes(int n_sm, int nq = 1, int nrs = 80);
 int tc_gemm_max_nq(int nrs = 80, int planes = 1);
 int tc_gemm_counter_ints();
