@@ -46,6 +46,10 @@ struct Buffers {
     float *rope_cos, *rope_sin;
     void* gemm_partials;
     int* gemm_counters;
+    SeqState* pre_states;      // [pre_blocks]: the blocks of a wide prefill pass
+    float* wide_partials;
+    size_t wide_bytes;
+    TileSrc* wide_tables;      // [4][WIDE_MAX_RT][SK_TABLE_TILES]
     TileSrc* sk_tables;   // [4][SK_TABLE_TILES]: QKV, O, gate/up, down (every layer has the same partition)
     // weights repacked for streaming (bf16 models, one sequence): per layer [qkv | o | gate/up | down], then the LM head
     char* packed;
@@ -127,6 +131,10 @@ int check_cfg(const esp_model_cfg* m, const esp_spec_cfg* s, Dims* D) {
         D->F = m->d_ffn; D->V = m->vocab; D->qk_norm = m->qk_norm;
         D->cap = m->max_seq_len + RT;
         D->batch = m->max_batch;
+        // wide prefill passes: bf16 models on the tensor-core attention whose longest prompt has two full blocks before its last
+        const int full = m->dtype == 1 && attn_tc_supported(m->head_dim, m->n_q_heads, m->n_kv_heads) ? (m->max_seq_len - 1) / PREFILL_CHUNK : 0;
+        D->pre_blocks = full < 2 ? 0 : (full < WIDE_MAX_BLOCKS ? full : WIDE_MAX_BLOCKS);
+        D->blocks = D->batch > D->pre_blocks ? D->batch : D->pre_blocks;
         const int S = attn_split_len(m->max_seq_len, m->max_batch, m->n_kv_heads);
         D->split_len = S;
         D->n_split_max = (m->max_seq_len + RT + S - 1) / S + 1;   // a prefill block's own rows count as cache positions
@@ -149,27 +157,28 @@ size_t carve_all(const Dims& D, int dtype, int n_sm, char* base, Buffers* b) {
     c.base = base;
     const size_t es = dtype ? 2 : 4;
     const size_t Mtot = (size_t)D.batch * RT;
+    const size_t Atot = (size_t)D.blocks * RT;      // rows of the activation buffers
     const size_t kv = (size_t)D.n_layers * D.batch * D.Hkv * D.cap * D.h * es;
     const int n_tiles_v = (D.V + TILE_N - 1) / TILE_N;
     Buffers tmp;
     Buffers& o = b ? *b : tmp;
     o.kcache = c.take<char>(kv);
     o.vcache = c.take<char>(kv);
-    o.hres = c.take<float>(Mtot * D.d);
-    // activations that feed the tensor-core GEMMs are kept as bf16 pairs hi + lo (ACT_PLANES planes, Mtot rows apart)
+    o.hres = c.take<float>(Atot * D.d);
+    // activations that feed the tensor-core GEMMs are kept as bf16 pairs hi + lo (ACT_PLANES planes, Atot rows apart)
     const size_t pl = dtype ? ACT_PLANES : 1;
-    o.xn = c.take<char>(pl * Mtot * D.d * es);
-    o.qbuf = c.take<char>(Mtot * D.Hq * D.h * es);
-    o.attn_out = c.take<char>(pl * Mtot * D.Hq * D.h * es);
-    o.act = c.take<char>(pl * Mtot * D.F * es);
+    o.xn = c.take<char>(pl * Atot * D.d * es);
+    o.qbuf = c.take<char>(Atot * D.Hq * D.h * es);
+    o.attn_out = c.take<char>(pl * Atot * D.Hq * D.h * es);
+    o.act = c.take<char>(pl * Atot * D.F * es);
     o.xn_lo = o.attn_out_lo = o.act_lo = nullptr;
     if (base && pl == 2) {
-        o.xn_lo = reinterpret_cast<char*>(o.xn) + Mtot * D.d * es;
-        o.attn_out_lo = reinterpret_cast<char*>(o.attn_out) + Mtot * D.Hq * D.h * es;
-        o.act_lo = reinterpret_cast<char*>(o.act) + Mtot * D.F * es;
+        o.xn_lo = reinterpret_cast<char*>(o.xn) + Atot * D.d * es;
+        o.attn_out_lo = reinterpret_cast<char*>(o.attn_out) + Atot * D.Hq * D.h * es;
+        o.act_lo = reinterpret_cast<char*>(o.act) + Atot * D.F * es;
     }
-    o.part_o = c.take<float>(Mtot * D.Hq * D.n_split_max * D.h);
-    o.part_ml = c.take<float2>(Mtot * D.Hq * D.n_split_max);
+    o.part_o = c.take<float>(Atot * D.Hq * D.n_split_max * D.h);
+    o.part_ml = c.take<float2>(Atot * D.Hq * D.n_split_max);
     o.cand = c.take<Cand>((size_t)n_tiles_v * Mtot * D.KP);
     o.cand_ms = c.take<float2>((size_t)n_tiles_v * Mtot);
     o.cand_floor = c.take<uint32_t>(Mtot);
@@ -189,6 +198,19 @@ size_t carve_all(const Dims& D, int dtype, int n_sm, char* base, Buffers* b) {
         const size_t pre_b = tc_gemm_partial_bytes(n_sm, 1, RT);
         o.gemm_partials = c.take<char>(step_b > pre_b ? step_b : pre_b);
     }
+    o.pre_states = c.take<SeqState>(D.pre_blocks);
+    o.wide_bytes = 0;
+    if (D.pre_blocks) {
+        const int tiles[4] = {(D.Hq + 2 * D.Hkv) * D.h / TILE_N, (D.d + TILE_N - 1) / TILE_N, (D.F + 63) / 64, (D.d + TILE_N - 1) / TILE_N};
+        const int K[4] = {D.d, D.Hq * D.h, D.d, D.F};
+        for (int i = 0; i < 4; ++i)
+            for (int rt = 1; rt <= (D.pre_blocks + 1) / 2; ++rt) {
+                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, rt);
+                o.wide_bytes = n > o.wide_bytes ? n : o.wide_bytes;
+            }
+    }
+    o.wide_partials = c.take<float>(o.wide_bytes / sizeof(float));
+    o.wide_tables = c.take<TileSrc>(D.pre_blocks ? (size_t)4 * WIDE_MAX_RT * SK_TABLE_TILES : 0);
     o.gemm_counters = c.take<int>(tc_gemm_counter_ints());
     o.sk_tables = c.take<TileSrc>(4 * SK_TABLE_TILES);
     o.layer_ptrs = c.take<const void*>((size_t)4 * D.n_layers);
@@ -227,6 +249,8 @@ struct esp_handle {
     std::vector<TcGemm*> p_qkv_w, p_o_w, p_gu_w, p_down_w;
     TcGemm* p_lm_w = nullptr;
     int rows_cap_prefill = RT;
+    WideGemm* p_wide[4] = {nullptr, nullptr, nullptr, nullptr};   // QKV, O, gate/up, down over the blocks of a wide prefill pass
+    AttnTc* p_attn_pre = nullptr;  // ... and their query descriptor
     std::vector<AttnTc*> p_attn;   // per layer, bf16 models with head_dim 128
     TcGemm* p_lm = nullptr;
     LayersTc* p_layers = nullptr;  // all layers in one launch (one sequence per pass, blocks of at most 80 rows)
@@ -447,6 +471,65 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
     return cuda_ok(cudaGetLastError());
 }
 
+// A prefill pass over nb full blocks of one prompt (b.pre_states), tensor-core path: their keys and values enter
+// sequence seq's cache, nothing else of them is needed.  The layer GEMMs run over all blocks at once; the kernels that
+// consume them and the attention take the block as a grid dimension, as they take a batch's sequences in a step.  A
+// row's earlier rows, of its own block and of the blocks before it, are cache positions to it: every block's keys and
+// values are written before the attention starts.
+int forward_prefill_wide(esp_handle* h, int seq, int nb, int off) {
+    const Dims& D = h->D;
+    Buffers& b = h->b;
+    cudaStream_t s = h->stream;
+    const bool pdl = h->use_pdl;
+    const size_t kv_seq_off = (size_t)seq * D.Hkv * D.cap * D.h * 2;
+    const int rows = PREFILL_CHUNK, n_split_launch = (off + nb * rows + D.split_len - 1) / D.split_len;
+    StreamK pending;
+    memset(&pending, 0, sizeof(pending));
+    pending.KB = pending.G = 1; pending.slots = 2; pending.rows = pending.seq_rows = RT;
+    launch_setup_chains(b.pre_states, nb, b.prompt_dev, off, s);
+    launch_assemble(1, b.pre_states, h->embed, b.mvec + (size_t)seq * D.mask_slots * D.d, b.hres, D.d, D.mask_slots, nb, s, false, rows);
+    for (int l = 0; l < D.n_layers; ++l) {
+        const char* pk = b.packed + b.pk_layer * l;
+        EpiArgs e = base_epi(h, 0, 0, nb);
+        e.st = b.pre_states;
+        e.q_out = b.qbuf;
+        e.kcache = reinterpret_cast<char*>(layer_ptr(b.kcache, h->layer_kv_stride, l)) + kv_seq_off;
+        e.vcache = reinterpret_cast<char*>(layer_ptr(b.vcache, h->layer_kv_stride, l)) + kv_seq_off;
+        e.kv_shared = 1;
+        e.q_norm = D.qk_norm ? h->qn[l] : nullptr;
+        e.k_norm = D.qk_norm ? h->kn[l] : nullptr;
+        launch_resid_norm(b.pre_states, b.hres, pending, h->na[l], b.xn, b.xn_lo, D.d, D.rms_eps, nullptr, nb, s, pdl, rows);
+        int rc = wide_gemm_launch(h->p_wide[0], pk, b.pre_states, nb, s, pdl);
+        if (!rc && launch_qkv_finish(e, wide_gemm_streamk(h->p_wide[0], nb), nb, s, pdl, rows)) rc = ESP_E_BADCFG;
+        if (rc) return rc;
+        if (l == D.n_layers - 1) break;      // the last layer's keys and values were all that was missing
+        AttnArgs a;
+        memset(&a, 0, sizeof(a));
+        a.q = b.qbuf;
+        a.kc = e.kcache; a.vc = e.vcache; a.kv_shared = 1;
+        a.out = b.attn_out; a.out_lo = b.attn_out_lo;
+        a.part_o = b.part_o; a.part_ml = b.part_ml;
+        a.st = b.pre_states;
+        a.Hq = D.Hq; a.Hkv = D.Hkv; a.h = D.h; a.cap = D.cap; a.split_len = D.split_len; a.n_split_max = D.n_split_max;
+        a.dcap = DCAP_PREFILL;
+        a.rows_cap = rows;
+        a.cache_in_flight = 1;
+        a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)D.h));
+        a.err = b.err;
+        if (attn_tc_launch(h->p_attn[(size_t)l * D.batch + seq], a, nb, n_split_launch, s, pdl, h->p_attn_pre)) return ESP_E_BADCFG;
+        rc = wide_gemm_launch(h->p_wide[1], pk + b.pk_qkv, b.pre_states, nb, s, pdl);
+        if (rc) return rc;
+        launch_resid_norm(b.pre_states, b.hres, wide_gemm_streamk(h->p_wide[1], nb), h->nf[l], b.xn, b.xn_lo, D.d, D.rms_eps, nullptr, nb, s, pdl, rows);
+        rc = wide_gemm_launch(h->p_wide[2], pk + b.pk_qkv + b.pk_o, b.pre_states, nb, s, pdl);
+        if (rc) return rc;
+        launch_swiglu_finish(b.pre_states, wide_gemm_streamk(h->p_wide[2], nb), b.act, b.act_lo, D.F, nb, s, pdl, rows);
+        rc = wide_gemm_launch(h->p_wide[3], pk + b.pk_qkv + b.pk_o + b.pk_gu, b.pre_states, nb, s, pdl);
+        if (rc) return rc;
+        pending = wide_gemm_streamk(h->p_wide[3], nb);
+    }
+    return cuda_ok(cudaGetLastError());
+}
+
 // Forward over the sequences that take part: `only_seq` (prefill) or every prefilled sequence (a step).
 int forward(esp_handle* h, bool with_lm, int dcap, int only_seq) {
     const bool tc = h->dtype == 1 && h->gemm_impl == 0 && h->p_lm != nullptr;
@@ -503,6 +586,16 @@ int read_ring(esp_handle* h, int slot) {
     if (cudaMemcpyAsync(h->pinned + n, h->b.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess) return ESP_E_CUDA;
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return ESP_E_CUDA;
     return h->pinned[n] ? ESP_E_DEVICE : ESP_OK;
+}
+
+// A prefill that could not be enqueued: the other sequences keep their lengths; this one has to be prefilled again
+// before it can step.
+int prefill_failed(esp_handle* h, int seq, const std::vector<int>& saved, int rc) {
+    k_select<<<1, 32, 0, h->stream>>>(h->b.states, h->D.batch, -1);
+    h->L_host = saved;
+    h->L_host[seq] = 0;
+    h->ready[seq] = 0;
+    return rc;
 }
 
 }  // namespace
@@ -586,27 +679,27 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
             char* pk = h->b.packed + h->b.pk_layer * l;
             const void* w1[3] = {h->wq[l], h->wk[l], h->wv[l]};
             const int32_t r1[3] = {dq, dkv, dkv};
-            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w1, r1, D.d, h->b.xn, D.batch, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 0 * SK_TABLE_TILES, SK_TABLE_TILES, pk, h->stream, ACT_PLANES);
+            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w1, r1, D.d, h->b.xn, D.blocks, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 0 * SK_TABLE_TILES, SK_TABLE_TILES, pk, h->stream, ACT_PLANES);
             h->p_qkv.push_back(p);
             const void* w2[3] = {h->wo[l], nullptr, nullptr};
             const int32_t r2[3] = {D.d, 0, 0};
             p = nullptr;
-            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w2, r2, dq, h->b.attn_out, D.batch, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 1 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv, h->stream, ACT_PLANES);
+            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w2, r2, dq, h->b.attn_out, D.blocks, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 1 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv, h->stream, ACT_PLANES);
             h->p_o.push_back(p);
             const void* w3[3] = {h->wg[l], h->wu[l], nullptr};
             const int32_t r3[3] = {D.F, D.F, 0};
             p = nullptr;
-            ok = ok && !tc_gemm_create(&p, EPI_SWIGLU, true, w3, r3, D.d, h->b.xn, D.batch, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 2 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o, h->stream, ACT_PLANES);
+            ok = ok && !tc_gemm_create(&p, EPI_SWIGLU, true, w3, r3, D.d, h->b.xn, D.blocks, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 2 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o, h->stream, ACT_PLANES);
             h->p_gu.push_back(p);
             const void* w4[3] = {h->wd[l], nullptr, nullptr};
             const int32_t r4[3] = {D.d, 0, 0};
             p = nullptr;
-            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w4, r4, D.F, h->b.act, D.batch, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 3 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o + h->b.pk_gu, h->stream, ACT_PLANES);
+            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w4, r4, D.F, h->b.act, D.blocks, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 3 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o + h->b.pk_gu, h->stream, ACT_PLANES);
             h->p_down.push_back(p);
         }
         const void* w5[3] = {h->lm_head, nullptr, nullptr};
         const int32_t r5[3] = {D.V, 0, 0};
-        ok = ok && !tc_gemm_create(&h->p_lm, EPI_LOGITS, false, w5, r5, D.d, h->b.xn, D.batch, nrs, nrs == 80 ? nq_max : 1, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, nullptr, 0, h->b.packed + h->b.pk_layer * D.n_layers, h->stream);
+        ok = ok && !tc_gemm_create(&h->p_lm, EPI_LOGITS, false, w5, r5, D.d, h->b.xn, D.blocks, nrs, nrs == 80 ? nq_max : 1, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, nullptr, 0, h->b.packed + h->b.pk_layer * D.n_layers, h->stream);
         if (ok && nrs != RT) {
             // the prefill runs 120-row blocks: the same weights (already repacked) behind 128-row GEMM plans
             const size_t pbytes = tc_gemm_partial_bytes(148, 1, RT);
@@ -615,27 +708,37 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
                 char* pk = h->b.packed + h->b.pk_layer * l;
                 const void* w1[3] = {h->wq[l], h->wk[l], h->wv[l]};
                 const int32_t r1[3] = {dq, dkv, dkv};
-                ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w1, r1, D.d, h->b.xn, D.batch, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 0 * SK_TABLE_TILES, SK_TABLE_TILES, pk, h->stream, ACT_PLANES);
+                ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w1, r1, D.d, h->b.xn, D.blocks, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 0 * SK_TABLE_TILES, SK_TABLE_TILES, pk, h->stream, ACT_PLANES);
                 h->p_qkv_w.push_back(p);
                 const void* w2[3] = {h->wo[l], nullptr, nullptr};
                 const int32_t r2[3] = {D.d, 0, 0};
                 p = nullptr;
-                ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w2, r2, dq, h->b.attn_out, D.batch, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 1 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv, h->stream, ACT_PLANES);
+                ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w2, r2, dq, h->b.attn_out, D.blocks, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 1 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv, h->stream, ACT_PLANES);
                 h->p_o_w.push_back(p);
                 const void* w3[3] = {h->wg[l], h->wu[l], nullptr};
                 const int32_t r3[3] = {D.F, D.F, 0};
                 p = nullptr;
-                ok = ok && !tc_gemm_create(&p, EPI_SWIGLU, true, w3, r3, D.d, h->b.xn, D.batch, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 2 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o, h->stream, ACT_PLANES);
+                ok = ok && !tc_gemm_create(&p, EPI_SWIGLU, true, w3, r3, D.d, h->b.xn, D.blocks, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 2 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o, h->stream, ACT_PLANES);
                 h->p_gu_w.push_back(p);
                 const void* w4[3] = {h->wd[l], nullptr, nullptr};
                 const int32_t r4[3] = {D.d, 0, 0};
                 p = nullptr;
-                ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w4, r4, D.F, h->b.act, D.batch, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 3 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o + h->b.pk_gu, h->stream, ACT_PLANES);
+                ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w4, r4, D.F, h->b.act, D.blocks, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 3 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o + h->b.pk_gu, h->stream, ACT_PLANES);
                 h->p_down_w.push_back(p);
             }
-            ok = ok && !tc_gemm_create(&h->p_lm_w, EPI_LOGITS, false, w5, r5, D.d, h->b.xn, D.batch, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, nullptr, 0, h->b.packed + h->b.pk_layer * D.n_layers, h->stream);
+            ok = ok && !tc_gemm_create(&h->p_lm_w, EPI_LOGITS, false, w5, r5, D.d, h->b.xn, D.blocks, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, nullptr, 0, h->b.packed + h->b.pk_layer * D.n_layers, h->stream);
         }
         if (!ok) { esp_free(h); return ESP_E_CUDA; }
+        if (D.pre_blocks && n_sm >= 148) {
+            const TcGemm* narrow[4] = {h->p_qkv[0], h->p_o[0], h->p_gu[0], h->p_down[0]};
+            const void* x[4] = {h->b.xn, h->b.attn_out, h->b.xn, h->b.act};
+            const int K[4] = {D.d, dq, D.d, D.F};
+            bool have = attn_tc_create(&h->p_attn_pre, h->b.qbuf, h->b.kcache, h->b.vcache, D.pre_blocks, D.Hq, D.Hkv, D.cap) == 0;
+            for (int i = 0; i < 4 && have; ++i)
+                have = !wide_gemm_create(&h->p_wide[i], tc_gemm_tiles(narrow[i]), K[i], x[i], D.blocks, (D.pre_blocks + 1) / 2, h->b.wide_partials,
+                                         h->b.wide_bytes, h->b.wide_tables + (size_t)i * WIDE_MAX_RT * SK_TABLE_TILES, h->b.err, h->stream);
+            if (!have) { esp_free(h); return ESP_E_CUDA; }
+        }
         // the all-layers kernel: per-layer pointer tables and the plan
         if (nrs == 80 && D.batch == 1) {
             std::vector<const void*> tab((size_t)4 * D.n_layers, nullptr);
@@ -683,21 +786,24 @@ int esp_prefill(esp_handle* h, int32_t seq, const int32_t* prompt, int32_t n_pro
     k_select<<<1, 32, 0, s>>>(h->b.states, h->D.batch, seq);
     std::vector<int> saved = h->L_host;
     for (int i = 0; i < h->D.batch; ++i) h->L_host[i] = 0;
-    for (int off = 0; off < n_prompt; off += PREFILL_CHUNK) {
+    const bool wide = h->p_wide[3] && h->gemm_impl == 0;
+    for (int off = 0, step; off < n_prompt; off += step) {
+        step = PREFILL_CHUNK;
+        int full = (n_prompt - 1 - off) / PREFILL_CHUNK;      // full blocks before the last one
+        if (wide && full >= 2) {
+            if (full > h->D.pre_blocks) full = h->D.pre_blocks;
+            const int rc = forward_prefill_wide(h, seq, full, off);
+            if (rc) return prefill_failed(h, seq, saved, rc);
+            step = full * PREFILL_CHUNK;
+            continue;
+        }
         const int cn = n_prompt - off < PREFILL_CHUNK ? n_prompt - off : PREFILL_CHUNK;
         const int last = off + cn == n_prompt;
         launch_setup_chain(h->b.states, seq, h->b.prompt_dev, off, cn, last, h->D.k, s);
         h->L_host[seq] = off;
         int rc = forward(h, last, DCAP_PREFILL, seq);
         if (!rc) rc = tree_step(h, false);
-        if (rc) {
-            // the other sequences keep their lengths; this one has to be prefilled again before it can step
-            k_select<<<1, 32, 0, s>>>(h->b.states, h->D.batch, -1);
-            h->L_host = saved;
-            h->L_host[seq] = 0;
-            h->ready[seq] = 0;
-            return rc;
-        }
+        if (rc) return prefill_failed(h, seq, saved, rc);
     }
     k_mark_ready<<<1, 1, 0, s>>>(h->b.states, seq);
     k_select<<<1, 32, 0, s>>>(h->b.states, h->D.batch, -1);
@@ -988,6 +1094,8 @@ void esp_free(esp_handle* h) {
     for (auto* p : h->p_gu_w) tc_gemm_destroy(p);
     for (auto* p : h->p_down_w) tc_gemm_destroy(p);
     tc_gemm_destroy(h->p_lm_w);
+    for (auto* p : h->p_wide) wide_gemm_destroy(p);
+    attn_tc_destroy(h->p_attn_pre);
     layers_tc_destroy(h->p_layers);
     for (auto* t : h->p_attn) attn_tc_destroy(t);
     if (h->pinned) cudaFreeHost(h->pinned);

@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(ONCE_THREADS, 1) k_attn_bulk_tc_once(const __g
     it.beg = it.split * a.split_len;
     const int end = min(it.beg + a.split_len, T0max);
     it.n_chunks = (end - it.beg + CK - 1) / CK;
-    it.kv_row0 = (it.seq * a.Hkv + it.kvh) * a.cap;
+    it.kv_row0 = ((a.kv_shared ? 0 : it.seq) * a.Hkv + it.kvh) * a.cap;
 
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(TMEM_COLS) : "memory");
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
                 uint64_t* full = is_k ? k_full : v_full;
                 // a fresh barrier passes a wait on parity 1: the first use of a stage does not block
                 if (!mbar_wait(&empty[k.g & 1], ((k.g >> 1) & 1) ^ 1, s_abort)) return false;
-                const int row = (k.it.seq * a.Hkv + k.it.kvh) * a.cap + k.it.beg + k.c * CK;
+                const int row = ((a.kv_shared ? 0 : k.it.seq) * a.Hkv + k.it.kvh) * a.cap + k.it.beg + k.c * CK;
                 unsigned char* st = smem + OFF_KV + (k.g & 1) * KV_STAGE + (is_k ? 0 : K_BYTES);
                 const CUtensorMap* map = is_k ? &p.map_k : &p.map_v;
                 mbar_expect_tx(&full[k.g & 1], K_BYTES);
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(TM_WARPS * 32, 2) k_attn_tail_merge_many_tc(At
     w0 = __reduce_min_sync(0xffffffffu, w0);
     const int n_win = min(L + r_end - w0, window);
     {
-        const size_t row0 = ((size_t)seq * a.Hkv + kvh) * a.cap + w0;
+        const size_t row0 = ((size_t)(a.kv_shared ? 0 : seq) * a.Hkv + kvh) * a.cap + w0;
         const __nv_bfloat16* kb = reinterpret_cast<const __nv_bfloat16*>(a.kc) + row0 * HD;
         const __nv_bfloat16* vb = reinterpret_cast<const __nv_bfloat16*>(a.vc) + row0 * HD;
         for (int i = threadIdx.x; i < n_win * (HD / 8); i += TM_WARPS * 32) {
@@ -756,9 +756,10 @@ static int attn_tc_fill(AttnTc* t, const void* q, const void* kcache, const void
 void attn_tc_destroy(AttnTc* t) { delete t; }
 
 // Two launches: the bulk kernel (grid = splits x (KV heads x row tiles) x sequences), then tail + merge.
-int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_launch, cudaStream_t s, bool pdl) {
+int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_launch, cudaStream_t s, bool pdl, const AttnTc* q_of) {
     if (!t || n_split_launch + 1 > a.n_split_max || a.split_len % CK) return -1;
     BulkParams p = t->p;
+    if (q_of) p.map_q = q_of->p.map_q;
     p.a = a;
     const int rows_cap = a.rows_cap > 0 && a.rows_cap < RT ? a.rows_cap : RT;
     p.n_row_tiles = (rows_cap + p.rows_per_tile - 1) / p.rows_per_tile;   // row tiles that can hold rows

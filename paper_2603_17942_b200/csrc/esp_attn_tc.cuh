@@ -380,8 +380,9 @@ template <int KB8, int VB>
 __device__ __forceinline__ void tail_pair(TailAcc& t, const AttnArgs& a, const PairCtx& c, float* s_q, int lane) {
     const int kvh = c.head / (a.Hq / a.Hkv);
     const int P = c.L + c.depth, T0 = tail_start_tc(P, a.dcap);
-    const __nv_bfloat16* kbase = reinterpret_cast<const __nv_bfloat16*>(a.kc) + ((size_t)c.seq * a.Hkv + kvh) * a.cap * HD;
-    const __nv_bfloat16* vbase = reinterpret_cast<const __nv_bfloat16*>(a.vc) + ((size_t)c.seq * a.Hkv + kvh) * a.cap * HD;
+    const size_t kv0 = ((size_t)(a.kv_shared ? 0 : c.seq) * a.Hkv + kvh) * a.cap * HD;
+    const __nv_bfloat16* kbase = reinterpret_cast<const __nv_bfloat16*>(a.kc) + kv0;
+    const __nv_bfloat16* vbase = reinterpret_cast<const __nv_bfloat16*>(a.vc) + kv0;
     const __nv_bfloat16* q = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * HD;
     {
         const uint2 qq = __ldcg(reinterpret_cast<const uint2*>(q + lane * 4));

@@ -67,6 +67,8 @@ struct Dims {
     int32_t n_layers, d, Hq, Hkv, h, F, V, qk_norm;
     int32_t cap;        // KV positions allocated per sequence (max_seq_len + RT)
     int32_t batch;
+    int32_t pre_blocks; // full prefill blocks one pass of the wide GEMMs covers (0: one block per pass)
+    int32_t blocks;     // row blocks the activation buffers hold: max(batch, pre_blocks)
     int32_t split_len;  // attention split length in positions (multiple of 64)
     int32_t n_split_max;
     float rms_eps;
@@ -181,6 +183,7 @@ struct EpiArgs {
     const float* rope_cos;    // [cap][h/2]
     const float* rope_sin;
     int32_t Hq, Hkv, h, cap, qk_norm;
+    int32_t kv_shared;        // 1: every block of the launch writes the first sequence's cache (prefill blocks of one prompt)
     float rms_eps;
     // EPI_SWIGLU
     void* act_out;            // [batch*RT][F] T

@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(128) k_qkv_finish(EpiArgs a, StreamK sk) {
     if (work) qkv_prefetch<HD>(pf, qa, sk, hs, L + (st ? st->row_depth[r] : r), lane);
     pdl_wait();
     if (!work) return;
-    qkv_finish_task<HD>(pf, qa, sk, seq, seq * sk.seq_rows + r, seq * RT + r, L + r, hs, lane);
+    qkv_finish_task<HD>(pf, qa, sk, a.kv_shared ? 0 : seq, seq * sk.seq_rows + r, seq * RT + r, L + r, hs, lane);
 }
 
 // Consumer of the split gate/up GEMM: a tile holds 64 gate features (columns 0..63) and the matching 64 up
@@ -937,10 +937,8 @@ __device__ void write_probe_rows(SeqState* st, int N, int k, int first_anchor, i
     }
 }
 
-// Prefill chunk: rows are n consecutive prompt tokens (a chain); the last chunk appends k probes
-// behind the last prompt token (Figure 1 middle).
-__global__ void k_setup_chain(SeqState* states, int seq, const int32_t* prompt_dev, int off, int n, int last, int k) {
-    SeqState* st = states + seq;
+// rows = n consecutive prompt tokens (a chain)
+__device__ void write_chain_rows(SeqState* st, const int32_t* prompt_dev, int off, int n) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         st->row_token[i] = prompt_dev[off + i];
         st->row_parent[i] = i - 1;
@@ -951,6 +949,25 @@ __global__ void k_setup_chain(SeqState* states, int seq, const int32_t* prompt_d
         st->row_anc[i][1] = hi;
         st->row_logp[i] = 0.f;
     }
+}
+
+// Several full prefill blocks, a state each (block b of the grid: prompt tokens off + b * PREFILL_CHUNK ..).
+__global__ void k_setup_chains(SeqState* states, const int32_t* prompt_dev, int off) {
+    SeqState* st = states + blockIdx.x;
+    const int o = off + blockIdx.x * PREFILL_CHUNK;
+    write_chain_rows(st, prompt_dev, o, PREFILL_CHUNK);
+    if (threadIdx.x == 0) {
+        st->L = o;
+        st->n_nodes = st->n_rows = PREFILL_CHUNK;
+        st->mode = 1;
+        st->active = 1;
+    }
+}
+
+// Prefill chunk; the last chunk appends k probes behind the last prompt token (Figure 1 middle).
+__global__ void k_setup_chain(SeqState* states, int seq, const int32_t* prompt_dev, int off, int n, int last, int k) {
+    SeqState* st = states + seq;
+    write_chain_rows(st, prompt_dev, off, n);
     __syncthreads();
     if (last && k > 0) write_probe_rows(st, n, k, n - 1, 1);
     if (threadIdx.x == 0) {
@@ -958,7 +975,7 @@ __global__ void k_setup_chain(SeqState* states, int seq, const int32_t* prompt_d
         st->n_rows = n + (last ? k : 0);
         st->mode = last ? 2 : 1;
         st->active = 1;
-        if (off == 0) st->L = 0;
+        st->L = off;
     }
 }
 
@@ -1382,6 +1399,9 @@ int launch_qkv_finish(const EpiArgs& a, const StreamK& sk, int nq, cudaStream_t 
 }
 void launch_setup_chain(SeqState* st, int seq, const int32_t* prompt_dev, int off, int n, int last, int k, cudaStream_t s) {
     k_setup_chain<<<1, 128, 0, s>>>(st, seq, prompt_dev, off, n, last, k);
+}
+void launch_setup_chains(SeqState* st, int n, const int32_t* prompt_dev, int off, cudaStream_t s) {
+    k_setup_chains<<<n, 128, 0, s>>>(st, prompt_dev, off);
 }
 void launch_set_tree(SeqState* st, int seq, const int32_t* tokens, const int32_t* parents, int n, int k, int n_anchor,
                      int* err, cudaStream_t s) {

@@ -19,6 +19,7 @@ struct AttnArgs {
     int32_t rows_cap;               // no block of this launch has more rows than this (0: RT); sizes the grids
     int32_t cache_in_flight;        // 1: positions below T0 may have been written by the kernel before this one
                                     // (prefill blocks: a row's earlier rows sit in the cache already)
+    int32_t kv_shared;              // 1: every block of the launch belongs to the first sequence's cache (prefill blocks of one prompt)
     int32_t n_rows_fixed, L_fixed;
     int32_t Hq, Hkv, h, cap, split_len, n_split_max, dcap;
     float scale_log2;     // log2(e)/sqrt(h)
@@ -54,6 +55,8 @@ void launch_resid_norm(const SeqState* st, float* hres, const StreamK& sk, const
 int launch_qkv_finish(const EpiArgs& a, const StreamK& sk, int nq, cudaStream_t s, bool pdl, int rows_cap = RT);
 void launch_swiglu_finish(const SeqState* st, const StreamK& sk, void* act, void* act_lo, int F, int nq, cudaStream_t s, bool pdl, int rows_cap = RT);
 void launch_setup_chain(SeqState* st, int seq, const int32_t* prompt_dev, int off, int n, int last, int k, cudaStream_t s);
+// n blocks of PREFILL_CHUNK prompt tokens from position off on, one state each
+void launch_setup_chains(SeqState* st, int n, const int32_t* prompt_dev, int off, cudaStream_t s);
 void launch_set_tree(SeqState* st, int seq, const int32_t* tokens, const int32_t* parents, int n, int k, int n_anchor,
                      int* err, cudaStream_t s);
 void launch_topk_merge(const SeqState* st, const Cand* cand, const float2* cand_ms, int n_tiles, int KP, int batch,
@@ -99,7 +102,8 @@ inline int attn_split_len(int max_len, int batch, int Hkv) {
 }
 int attn_tc_create(AttnTc** out, const void* q, const void* kcache, const void* vcache, int batch, int Hq, int Hkv, int cap);
 void attn_tc_destroy(AttnTc* t);
-int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_launch, cudaStream_t s, bool pdl);
+// q_of: the plan whose query descriptor is used instead of t's own (launches over more blocks than t has sequences)
+int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_launch, cudaStream_t s, bool pdl, const AttnTc* q_of = nullptr);
 // the same for one call, descriptors built in the call's own frame (no allocation anywhere)
 int attn_tc_run(const void* q, const void* kcache, const void* vcache, int batch, int Hq, int Hkv, int cap, const AttnArgs& a,
                 int n_split_launch, cudaStream_t s);
@@ -126,6 +130,18 @@ size_t tc_gemm_partial_bytes(int n_sm, int nq = 1, int nrs = 80);
 int tc_gemm_max_nq(int nrs = 80, int planes = 1);
 int tc_gemm_counter_ints();
 
+
+// tcgen05 GEMM over several full prefill blocks at once (esp_gemm_wide.cu): activations [2 planes][x_blocks][RT][K], of
+// every block the first PREFILL_CHUNK rows; partials and contributor tables for the same consumers as above.
+struct WideGemm;
+constexpr int WIDE_MAX_BLOCKS = 8, WIDE_MAX_RT = WIDE_MAX_BLOCKS / 2;
+size_t wide_partial_bytes(int n_tiles, int KB, int n_rt);
+// tables_dev: device memory for n_rt_max * n_tiles entries
+int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int n_rt_max, float* partials, size_t partial_bytes,
+                     TileSrc* tables_dev, int* err, cudaStream_t stream);
+void wide_gemm_destroy(WideGemm* g);
+int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, int n_blocks, cudaStream_t s, bool pdl);
+StreamK wide_gemm_streamk(const WideGemm* g, int n_blocks);
 
 // All layers of a step in one persistent cooperative launch (esp_layers_tc.cu): bf16, head_dim 128, blocks of at
 // most 80 rows, one sequence per pass.  Same phases, same partition and same bits as the kernels above.
