@@ -395,6 +395,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
             int T0row = 0;
             if (pv) T0row = tail_start_tc(it.L + (a.st ? a.st[it.seq].row_depth[r] : a.depth[it.seq * RT + r]), a.dcap);
             const uint32_t o_addr = lane_addr + 256 + (n_it & 1) * 128;
+            if (!__any_sync(0xffffffffu, pv)) {      // no pair in this warp (nor in the one that shares its lanes)
+                for (int c = 0; c < it.n_chunks && ok; ++c) ok = softmax_chunk_idle(gc + c > 0, pv_done, (gc + c - 1) & 1, p_ready, s_abort);
+                gc += it.n_chunks;
+                ++n_it;
+                continue;
+            }
             float m_run = -INFINITY, l_run = 0.f;
             for (int c = 0; c < it.n_chunks && ok; ++c) {
                 const uint32_t g = gc + c;

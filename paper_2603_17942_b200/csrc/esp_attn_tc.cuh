@@ -142,6 +142,15 @@ __device__ __forceinline__ bool softmax_chunk(uint32_t s_addr, uint32_t o_addr, 
     return true;
 }
 
+// The same step for a softmax warp none of whose 32 lanes has a pair (the last row tile of a block is rarely full: 68
+// rows x 4 heads leave 16 pairs in the third tile): no scores, no exponentials -- its rows of P and O are never used,
+// whatever they hold --, only its arrival, behind the previous chunk's P V so that it cannot run a phase ahead.
+__device__ __forceinline__ bool softmax_chunk_idle(bool wait_pv, uint64_t* pv_done, uint32_t pv_parity, uint64_t* p_ready, volatile int* s_abort) {
+    if (wait_pv && !__all_sync(0xffffffffu, mbar_wait(pv_done, pv_parity, s_abort))) return false;
+    if ((threadIdx.x & 31) == 0) mbar_arrive(p_ready);
+    return true;
+}
+
 // ---- one item, start to finish, on freshly initialised barriers.
 struct BulkMaps {
     const CUtensorMap* q;   // [rows][Hq][128], box 64 x group x rows_per_tile
@@ -280,7 +289,12 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16) + hf * 64;   // this thread's 64 columns of S / O
         float m_run = -INFINITY, l_run = 0.f;
         bool ok = true;
+        const bool live = __any_sync(0xffffffffu, pv);      // the same for the two warps that share the lanes' pairs
         for (int c = 0; c < it.n_chunks && ok; ++c) {
+            if (!live) {
+                ok = softmax_chunk_idle(c > 0, sm.pv_done, (c - 1) & 1, sm.p_ready, s_abort);
+                continue;
+            }
             // (a wait that fails must take the whole warp out: the tensor-memory accesses below are warp-wide)
             if (!__all_sync(0xffffffffu, mbar_wait(&sm.s_full[c & 1], (c >> 1) & 1, s_abort))) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -290,14 +304,14 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
         }
         if (ok && !__all_sync(0xffffffffu, mbar_wait(sm.pv_done, (it.n_chunks - 1) & 1, s_abort))) ok = false;
         float* xl = sm.s_xchg + (it.n_chunks & 1) * 2 * MP;
-        if (ok) {
+        if (ok && live) {
             // the row sum = first half's share + second half's share
             xl[hf * MP + pair] = l_run;
             __syncwarp();
             if (lane == 0) mbar_arrive(sm.xchg + q4);
             if (!__all_sync(0xffffffffu, mbar_wait(sm.xchg + q4, it.n_chunks & 1, s_abort))) ok = false;
         }
-        if (ok) {
+        if (ok && live) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // O half-row -> shared memory (the K/V stages are free now) -> one 256-byte bulk copy per thread.  The
             // tensor-memory load is warp-wide: every lane takes part, lanes without a pair copy nothing.
@@ -316,7 +330,7 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
             }
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");        // copies complete: shared memory may be released
-        } else if (lane == 0) {
+        } else if (!ok && lane == 0) {
             set_error(a.err, DEV_E_WAIT_TIMEOUT);
             *s_abort = 1;
         }

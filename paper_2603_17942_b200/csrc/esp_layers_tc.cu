@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_layers_tc(const __grid_const
     bmp.q = &p.map_q; bmp.k = &p.map_k; bmp.v = &p.map_v; bmp.group = p.group; bmp.rows_per_tile = p.rows_per_tile;
     AttnArgs aa;
     aa.q = p.qbuf; aa.out = p.attn_out; aa.out_lo = p.attn_out_lo; aa.part_o = p.part_o; aa.part_ml = p.part_ml; aa.st = st; aa.anc = nullptr; aa.depth = nullptr;
-    aa.rows_cap = NRS; aa.cache_in_flight = 0; aa.n_rows_fixed = 0; aa.L_fixed = 0;
+    aa.rows_cap = NRS; aa.cache_in_flight = 0; aa.kv_shared = 0; aa.n_rows_fixed = 0; aa.L_fixed = 0;
     aa.Hq = p.Hq; aa.Hkv = p.Hkv; aa.h = attn::HD; aa.cap = p.cap; aa.split_len = p.split_len; aa.n_split_max = p.n_split_max; aa.dcap = p.dcap;
     aa.scale_log2 = p.scale_log2; aa.err = p.err;
     const int n_heads_qkv = p.Hq + 2 * p.Hkv;
