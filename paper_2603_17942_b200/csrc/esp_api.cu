@@ -181,7 +181,7 @@ size_t carve_all(const Dims& D, int dtype, int n_sm, char* base, Buffers* b) {
     o.part_ml = c.take<float2>(Atot * D.Hq * D.n_split_max);
     o.cand = c.take<Cand>((size_t)n_tiles_v * Mtot * D.KP);
     o.cand_ms = c.take<float2>((size_t)n_tiles_v * Mtot);
-    o.cand_floor = c.take<uint32_t>(Mtot);
+    o.cand_floor = c.take<uint32_t>(Mtot * KP_MAX);
     o.topk = c.take<Cand>(Mtot * KP_MAX);
     o.lse = c.take<float>(Mtot);
     o.mvec = c.take<float>((size_t)D.batch * D.mask_slots * D.d);

@@ -97,14 +97,33 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
         const int Mtot = a.batch * RT;
         uint32_t noise_pos = 0xffffffffu;   // rows come in breadth-first order: equal depths are neighbours and
         float noise[4] = {0.f, 0.f, 0.f, 0.f};   // share their noise, which is a function of (position, token)
-        // The rows' floors (see below) are fetched once per tile, all rows at a time, and the floors this tile
-        // establishes go back in one batch at the end: no L2 round trip or atomic inside the row loop.
-        const int S = n_rows <= 80 ? 80 : RT;                             // s_aux holds at least 3 * S words
-        uint32_t* s_floor = reinterpret_cast<uint32_t*>(s_aux);          // [S] in, [S] out, [S] "this probe row has entries at or above its floor"
-        uint32_t* s_need = s_floor + 2 * S;
+        // Floors.  What is already known of a probe row bounds its K'-th largest logit from below, and an entry strictly
+        // below the bound cannot be in the row's final list.  The vocabulary tiles fall into K' groups (tile mod K'); the
+        // largest logit of each group so far is kept as an order-preserving key (atomicMax, one per tile and row), and
+        // the smallest of the K' group maxima is the bound: K' different tokens reach it.  (The K'-th best of a single
+        // tile, the bound used before, is an ordinary value, the best 9 % of the tile: hardly any tile stayed below it.)
+        // The bounds are fetched once per tile, all rows at a time.  Measured, 90 probe rows of 120, vocabulary 128256,
+        // K' = 11: LM head 368 -> 240 us; 36 of 48 rows: 192 -> 178 us.
+        const int S = n_rows <= 80 ? 80 : RT;                             // s_aux holds at least 2 * S words
+        uint32_t* s_floor = reinterpret_cast<uint32_t*>(s_aux);          // [S] bounds, [S] "this probe row has entries at or above its bound"
+        uint32_t* s_need = s_floor + S;
+        uint32_t* group_max = a.cand_floor ? a.cand_floor + (size_t)grow0 * KP_MAX + tile % a.KP : nullptr;
         for (int r = r0 + f; r < r1; r += 128) {
-            s_floor[r] = (r >= n_nodes && a.cand_floor) ? __ldcg(a.cand_floor + grow0 + r) : 0u;
-            s_floor[S + r] = 0u;
+            uint32_t bound = 0u;
+            if (r >= n_nodes && a.cand_floor) {
+                const uint4* g = reinterpret_cast<const uint4*>(a.cand_floor + (size_t)(grow0 + r) * KP_MAX);
+                bound = 0xffffffffu;
+#pragma unroll
+                for (int j = 0; j < KP_MAX; j += 4) {
+                    if (j >= a.KP) break;
+                    const uint4 w = __ldcg(g + j / 4);
+                    bound = min(bound, w.x);
+                    if (j + 1 < a.KP) bound = min(bound, w.y);
+                    if (j + 2 < a.KP) bound = min(bound, w.z);
+                    if (j + 3 < a.KP) bound = min(bound, w.w);
+                }
+            }
+            s_floor[r] = bound;
         }
         epi_bar(bar_id);
         // Probe rows, one thread per row (the padded row stride keeps the threads on different banks): the tile's
@@ -122,6 +141,7 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
                 float sum = 0.f;
                 for (int i = 0; i < n_valid; ++i) sum += expf(row[i] - tmax);
                 a.cand_ms[(size_t)tile * Mtot + grow0 + r] = make_float2(tmax, sum);
+                if (group_max) atomicMax(group_max + (size_t)r * KP_MAX, float_order_key(tmax));
                 const bool need = float_order_key(tmax) >= s_floor[r];
                 s_need[r] = need ? 1u : 0u;
                 if (!need) {
@@ -162,10 +182,11 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
 #pragma unroll
                 for (int i = 0; i < 4; ++i) s += id[i] < a.n_out ? expf(v[i] - tmax) : 0.f;
                 s = warp_sum(s);
-                if (lane == 0) a.cand_ms[(size_t)tile * Mtot + grow0 + r] = make_float2(tmax, s);
+                if (lane == 0) {
+                    a.cand_ms[(size_t)tile * Mtot + grow0 + r] = make_float2(tmax, s);
+                    if (group_max) atomicMax(group_max + (size_t)r * KP_MAX, float_order_key(tmax));
+                }
             }
-            // what other tiles have already established about this row's K'-th largest logit: a tile's own K'-th
-            // best is a lower bound of it, so an entry strictly below the bound cannot make the final list
             const uint32_t floor_key = s_floor[r];
             unsigned used = 0;
             float keep_v = -INFINITY;          // lane j keeps the j-th entry (K' <= 32); one coalesced store per row
@@ -187,14 +208,9 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
                 if (wi == bi && bslot >= 0) used |= 1u << bslot;
                 if (probe && wi != 0x7fffffff && wkey < floor_key) break;   // warp-uniform: this and all later entries are out
                 if (lane == j) { keep_v = wv; keep_i = wi == 0x7fffffff ? -1 : wi; }
-                if (probe && a.cand_floor && j == kp - 1 && wi != 0x7fffffff && lane == 0)
-                    s_floor[S + r] = wkey;                                    // this tile holds kp entries >= wv
             }
             if (lane < kp) { out[lane].val = keep_v; out[lane].id = keep_i; }
         }
-        epi_bar(bar_id);
-        for (int r = r0 + f; r < r1; r += 128)
-            if (s_floor[S + r] > s_floor[r]) atomicMax(a.cand_floor + grow0 + r, s_floor[S + r]);
     }
 }
 

@@ -889,7 +889,7 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_topk_merge(const SeqState* sta
             __syncthreads();
         }
         if (tid == 0) lse[grow] = s_v[0] + logf(s_s[0]);
-        if (tid == 0 && cand_floor) cand_floor[grow] = 0;     // nothing is known about the next forward's logits
+        if (tid < KP_MAX && cand_floor) cand_floor[(size_t)grow * KP_MAX + tid] = 0;     // nothing is known about the next forward's logits
     }
 }
 
