@@ -1,0 +1,94 @@
+"""The passes that cover several blocks of rows at once (the full blocks of a prompt; the sequences of a decode step) and
+the attention kernels large launches take, against the paths small ones take (need a B200)."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+import paper_2603_17942_b200 as P
+from tests.test_gpu_operators import R, _anc_words, _run_attention, _tree_block
+from tests.test_gpu_parity import BF16_SMALL, TOL_BF16
+
+pytestmark = pytest.mark.gpu
+
+
+def _handle(w, max_seq, spec, batch=1):
+    h = P.Handle(BF16_SMALL, spec, w, max_seq_len=max_seq, max_batch=batch)
+    logits = torch.zeros(batch, R, BF16_SMALL.vocab, dtype=torch.float32, device="cuda")
+    P.esp_debug_capture(h.h, logits)
+    return h, logits
+
+
+@pytest.fixture(scope="module")
+def weights():
+    return synth.make_weights(BF16_SMALL, seed=3, device="cuda", gain_jitter=True, std=0.05)
+
+
+@pytest.mark.parametrize("n_prompt", [120, 121, 240, 241, 361, 1081, 1200])
+def test_wide_prefill_against_cuda_core_path(weights, n_prompt):
+    """Prompts whose full blocks make no wide pass, one of 2, of 3 (a ragged row tile), of 8, and one of 8 with a single
+    block left over: the last prompt row's and the probe rows' logits against the CUDA-core GEMMs, which never take it.
+    Both round the same activations to bf16 once or twice, so they agree to the bar bf16 logits are held to anywhere."""
+    spec = P.spec_cfg(n_probes=3, topk=5, max_nodes=16, expand_width=0, n_anchor=1)
+    prompt = synth.make_prompt(BF16_SMALL.vocab, n_prompt, 7)
+    rows = slice((n_prompt - 1) % P.ESP_PREFILL_CHUNK, (n_prompt - 1) % P.ESP_PREFILL_CHUNK + 4)
+    got = []
+    for impl in (0, 1):
+        h, logits = _handle(weights, 1300, spec)
+        P.esp_debug_set_gemm(h.h, impl)
+        h.prefill(prompt)
+        got.append(logits[0, rows].clone())
+        assert h.stats().device_error == 0 and h.state()["L"] == n_prompt
+        h.close()
+    span = float(got[1].max() - got[1].min())
+    assert (got[0] - got[1]).abs().max() <= TOL_BF16 * span
+
+
+@pytest.mark.parametrize("n_seq,nodes,n_anchor", [(2, 16, 1), (4, 16, 1), (5, 16, 1), (7, 16, 1), (13, 16, 1), (3, 25, 0)])
+def test_batch_steps_against_each_sequence_alone(weights, n_seq, nodes, n_anchor):
+    """One step of a handle with several sequences (row tiles of two or three blocks, ragged ones, more sequences than a
+    pass covers, blocks of 100 rows) against the step each sequence takes in a handle of its own: the same trees (the
+    prefill does not depend on the batch), logits equal to the bar bf16 logits are held to; one sequence stays idle."""
+    spec = P.spec_cfg(n_probes=3, topk=5, max_nodes=nodes, expand_width=0 if n_anchor else 1, n_anchor=n_anchor)
+    idle = n_seq // 2
+    h, logits = _handle(weights, 400, spec, n_seq)
+    prompts = [synth.make_prompt(BF16_SMALL.vocab, 17 + 40 * (i % 5), 10 + i) for i in range(n_seq)]
+    for i in range(n_seq):
+        if i != idle:
+            h.prefill(prompts[i], i)
+    rows = {i: h.state(i)["n_rows"] for i in range(n_seq) if i != idle}
+    P.esp_step(h.h, h.tokens_out, h.n_out)
+    assert h.stats().device_error == 0 and h.n_out[idle] == 0
+    for i in (0, n_seq - 1):
+        if i == idle:
+            continue
+        one, alone = _handle(weights, 400, spec)
+        one.prefill(prompts[i])
+        assert one.state()["n_rows"] == rows[i]
+        one.step()
+        span = float(alone[0, :rows[i]].max() - alone[0, :rows[i]].min())
+        assert (logits[i, :rows[i]] - alone[0, :rows[i]]).abs().max() <= TOL_BF16 * span, f"sequence {i}"
+        one.close()
+    h.close()
+
+
+@pytest.mark.parametrize("group,n_rows,batch,L", [(4, 68, 3, 500), (2, 128, 5, 130), (1, 41, 24, 64), (8, 9, 70, 250), (4, 120, 8, 15)])
+def test_attention_tail_of_large_launches_bitwise(group, n_rows, batch, L):
+    """(Lengths for which the split grid does not follow the batch.)  The tail kernel of launches with many (row, head)
+    pairs adds in the order of the one that takes a warp per pair: every sequence of a batch has the bits it has in a
+    launch of its own, for every group size and ragged row counts."""
+    Hkv = 8 if group > 1 else 16
+    Hq, h, cap = Hkv * group, 128, L + R
+    n_probes = min(4, n_rows - 1)
+    _, depth1, vis = _tree_block(n_rows - n_probes, n_probes, 5, n_rows)
+    g = torch.Generator(device="cuda").manual_seed(group)
+    q = torch.randn(batch, R, Hq, h, generator=g, device="cuda").bfloat16()
+    kc, vc = (torch.randn(batch, Hkv, cap, h, generator=g, device="cuda").bfloat16() for _ in range(2))
+    anc = np.stack([_anc_words(vis)] * batch)
+    depth = np.zeros((batch, R), np.int32)
+    depth[:, :n_rows] = depth1
+    out = _run_attention(1, q, kc, vc, anc, depth, n_rows, L, Hq, Hkv, h)
+    for s in (0, batch - 1):
+        alone = _run_attention(1, q[s:s + 1].contiguous(), kc[s:s + 1].contiguous(), vc[s:s + 1].contiguous(), anc[:1], depth[:1],
+                               n_rows, L, Hq, Hkv, h)
+        assert torch.equal(out[s, :n_rows], alone[0, :n_rows]), f"sequence {s}"
