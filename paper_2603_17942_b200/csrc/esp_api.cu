@@ -49,7 +49,7 @@ struct Buffers {
     SeqState* pre_states;      // [pre_blocks]: the blocks of a wide prefill pass
     float* wide_partials;
     size_t wide_bytes;
-    TileSrc* wide_tables;      // [4][WIDE_MAX_RT][SK_TABLE_TILES]
+    TileSrc* wide_tables;      // [prefill passes, decode passes of a batch][4][WIDE_MAX_RT][SK_TABLE_TILES], those that exist
     TileSrc* sk_tables;   // [4][SK_TABLE_TILES]: QKV, O, gate/up, down (every layer has the same partition)
     // weights repacked for streaming (bf16 models, one sequence): per layer [qkv | o | gate/up | down], then the LM head
     char* packed;
@@ -67,6 +67,22 @@ constexpr int SK_TABLE_TILES = 2048;
 // queries and probabilities stay single bf16 numbers (the cache is bf16).
 constexpr int ACT_PLANES = 2;
 
+
+// Decode steps of several sequences: how many blocks a row tile of the wide GEMMs holds.  Blocks of up to 80 rows: two or
+// three, whichever is the cheaper for the batch -- per weight unit and tile the kernel takes 856 (two) or 1089 cycles
+// (three) of shared-memory time, operands and fill --; larger blocks: two.
+int batch_bpt(const Dims& D) {
+    if (D.gemm_rows != 80) return 2;
+    return (D.batch + 1) / 2 * 856 <= (D.batch + 2) / 3 * 1089 ? 2 : 3;
+}
+// sequences that share the LM head's weight stream
+int lm_nq(const Dims& D) { return D.gemm_rows == 80 && D.batch > 1 ? 2 : 1; }
+// sequences one pass of a decode step covers
+int batch_pass(const Dims& D) {
+    if (D.batch == 1) return 1;
+    const int most = WIDE_MAX_RT * batch_bpt(D);
+    return D.batch < most ? D.batch : most;
+}
 
 // tree nodes including the root: max_nodes, or 1 + the fixed widths of a static tree
 int spec_nodes(const esp_spec_cfg& s) {
@@ -193,24 +209,30 @@ size_t carve_all(const Dims& D, int dtype, int n_sm, char* base, Buffers* b) {
     o.rope_cos = c.take<float>((size_t)D.cap * (D.h / 2));
     o.rope_sin = c.take<float>((size_t)D.cap * (D.h / 2));
     {
-        // the decode steps' passes (several sequences of gemm_rows rows) or one 128-row prefill block, whichever is larger
-        const size_t step_b = tc_gemm_partial_bytes(n_sm, D.batch < tc_gemm_max_nq(D.gemm_rows, ACT_PLANES) ? D.batch : tc_gemm_max_nq(D.gemm_rows, ACT_PLANES), D.gemm_rows);
+        // a decode step's block of gemm_rows rows (two sequences' in the LM head) or one 128-row prefill block, whichever is larger
+        const size_t step_b = tc_gemm_partial_bytes(n_sm, lm_nq(D), D.gemm_rows);
         const size_t pre_b = tc_gemm_partial_bytes(n_sm, 1, RT);
         o.gemm_partials = c.take<char>(step_b > pre_b ? step_b : pre_b);
     }
     o.pre_states = c.take<SeqState>(D.pre_blocks);
     o.wide_bytes = 0;
-    if (D.pre_blocks) {
+    const bool batched = dtype == 1 && D.batch > 1;
+    if (D.pre_blocks || batched) {
         const int tiles[4] = {(D.Hq + 2 * D.Hkv) * D.h / TILE_N, (D.d + TILE_N - 1) / TILE_N, (D.F + 63) / 64, (D.d + TILE_N - 1) / TILE_N};
         const int K[4] = {D.d, D.Hq * D.h, D.d, D.F};
         for (int i = 0; i < 4; ++i)
             for (int rt = 1; rt <= (D.pre_blocks + 1) / 2; ++rt) {
-                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, rt);
+                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, rt, 2 * PREFILL_CHUNK);
+                o.wide_bytes = n > o.wide_bytes ? n : o.wide_bytes;
+            }
+        for (int i = 0; i < 4 && batched; ++i)
+            for (int rt = 1; rt <= (batch_pass(D) + batch_bpt(D) - 1) / batch_bpt(D); ++rt) {
+                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, rt, batch_bpt(D) * D.gemm_rows);
                 o.wide_bytes = n > o.wide_bytes ? n : o.wide_bytes;
             }
     }
     o.wide_partials = c.take<float>(o.wide_bytes / sizeof(float));
-    o.wide_tables = c.take<TileSrc>(D.pre_blocks ? (size_t)4 * WIDE_MAX_RT * SK_TABLE_TILES : 0);
+    o.wide_tables = c.take<TileSrc>((size_t)4 * WIDE_MAX_RT * SK_TABLE_TILES * ((D.pre_blocks ? 1 : 0) + (batched ? 1 : 0)));
     o.gemm_counters = c.take<int>(tc_gemm_counter_ints());
     o.sk_tables = c.take<TileSrc>(4 * SK_TABLE_TILES);
     o.layer_ptrs = c.take<const void*>((size_t)4 * D.n_layers);
@@ -251,6 +273,7 @@ struct esp_handle {
     int rows_cap_prefill = RT;
     WideGemm* p_wide[4] = {nullptr, nullptr, nullptr, nullptr};   // QKV, O, gate/up, down over the blocks of a wide prefill pass
     AttnTc* p_attn_pre = nullptr;  // ... and their query descriptor
+    WideGemm* p_batch[4] = {nullptr, nullptr, nullptr, nullptr};  // the same GEMMs over the sequences of a decode step (max_batch > 1)
     std::vector<AttnTc*> p_attn;   // per layer, bf16 models with head_dim 128
     TcGemm* p_lm = nullptr;
     LayersTc* p_layers = nullptr;  // all layers in one launch (one sequence per pass, blocks of at most 80 rows)
@@ -318,10 +341,10 @@ int run_gemm(esp_handle* h, TcGemm* plan, int epi, int n_tiles, const void* cons
 }
 
 // One decoder forward over the block every active sequence of [s0, s0 + nb) has in its row table.
-// Tensor-core path (bf16, nb <= 3 sequences whose activation blocks sit RT rows apart): the layer GEMMs stream
-// their weights once for all nb sequences and store stream-K partials that the next kernel sums (k_qkv_finish;
-// k_resid_norm = residual add + RMSNorm; k_swiglu_finish); the LM head runs once per sequence and finishes
-// in-kernel.  CUDA-core path (fp32 models): the same layer with every epilogue fused in the GEMM.
+// Tensor-core path (bf16; the sequences' activation blocks sit RT rows apart): the layer GEMMs stream their weights once
+// for all nb sequences (one: k_gemm_tc, several: k_gemm_wide) and store stream-K partials that the next kernel sums
+// (k_qkv_finish; k_resid_norm = residual add + RMSNorm; k_swiglu_finish); the LM head runs once per two sequences and
+// finishes in-kernel.  CUDA-core path (fp32 models): the same layer with every epilogue fused in the GEMM.
 int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc, bool prefill) {
     const Dims& D = h->D;
     Buffers& b = h->b;
@@ -342,6 +365,16 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
     const int rc_rows = prefill ? h->rows_cap_prefill : h->rows_cap;   // no block has more rows: sizes the row dimension of the grids
     const bool wide = prefill && !h->p_qkv_w.empty();                  // 128-row GEMM plans for the prefill blocks
     auto plan = [&](std::vector<TcGemm*>& narrow, std::vector<TcGemm*>& w128, int l) -> TcGemm* { return wide ? w128[l] : narrow[l]; };
+    // several sequences in a step: one GEMM over all their blocks (kind 0..3 = QKV, O, gate/up, down)
+    const bool multi = tc && !prefill && h->p_batch[3];
+    auto gemm = [&](int kind, TcGemm* one, int l, int epi, int n_tiles, const void* const w[3], const int32_t rows[3], const void* x, int K,
+                    const EpiArgs& a) -> int {
+        if (!multi) return run_gemm(h, one, epi, n_tiles, w, rows, x, K, a, tc, pdl, rc_rows);
+        const size_t off[4] = {0, b.pk_qkv, b.pk_qkv + b.pk_o, b.pk_qkv + b.pk_o + b.pk_gu};
+        h->launches++;
+        return wide_gemm_launch(h->p_batch[kind], b.packed + b.pk_layer * l + off[kind], st0, nb, s, pdl);
+    };
+    auto pieces = [&](int kind, const TcGemm* one) -> StreamK { return multi ? wide_gemm_streamk(h->p_batch[kind], nb) : tc_gemm_streamk(one); };
     launch_assemble(h->dtype, st0, h->embed, mvec0, b.hres, D.d, D.mask_slots, nb, s, false, rc_rows);
     h->launches++;
     // One sequence, a block of at most 80 rows, bf16: every layer in one persistent launch (same bits as the
@@ -371,11 +404,11 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.k_norm = D.qk_norm ? h->kn[l] : nullptr;
             const void* w[3] = {h->wq[l], h->wk[l], h->wv[l]};
             const int32_t rows[3] = {dq, dkv, dkv};
-            int rc = run_gemm(h, tc ? plan(h->p_qkv, h->p_qkv_w, l) : nullptr, EPI_QKV, (dq + 2 * dkv) / TILE_N, w, rows, b.xn, D.d, a, tc, pdl, rc_rows, tc ? nb : 1);
+            int rc = gemm(0, tc ? plan(h->p_qkv, h->p_qkv_w, l) : nullptr, l, EPI_QKV, (dq + 2 * dkv) / TILE_N, w, rows, b.xn, D.d, a);
             if (rc) return rc;
             mark(h, KIND_QKV);
             if (tc) {
-                if (launch_qkv_finish(a, tc_gemm_streamk(plan(h->p_qkv, h->p_qkv_w, l), nb), nb, s, pdl, rc_rows)) return ESP_E_BADCFG;
+                if (launch_qkv_finish(a, pieces(0, plan(h->p_qkv, h->p_qkv_w, l)), nb, s, pdl, rc_rows)) return ESP_E_BADCFG;
                 h->launches++;
                 mark(h, KIND_MISC);
             }
@@ -410,11 +443,11 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.hres = b.hres;
             const void* w[3] = {h->wo[l], nullptr, nullptr};
             const int32_t rows[3] = {D.d, 0, 0};
-            int rc = run_gemm(h, tc ? plan(h->p_o, h->p_o_w, l) : nullptr, EPI_RESID, (D.d + TILE_N - 1) / TILE_N, w, rows, b.attn_out, dq, a, tc, pdl, rc_rows, tc ? nb : 1);
+            int rc = gemm(1, tc ? plan(h->p_o, h->p_o_w, l) : nullptr, l, EPI_RESID, (D.d + TILE_N - 1) / TILE_N, w, rows, b.attn_out, dq, a);
             if (rc) return rc;
             mark(h, KIND_O);
         }
-        if (tc) launch_resid_norm(st0, b.hres, tc_gemm_streamk(plan(h->p_o, h->p_o_w, l), nb), h->nf[l], b.xn, b.xn_lo, D.d, D.rms_eps, nullptr, nb, s, pdl, rc_rows);
+        if (tc) launch_resid_norm(st0, b.hres, pieces(1, plan(h->p_o, h->p_o_w, l)), h->nf[l], b.xn, b.xn_lo, D.d, D.rms_eps, nullptr, nb, s, pdl, rc_rows);
         else launch_rmsnorm(h->dtype, st0, b.hres, h->nf[l], b.xn, D.d, D.rms_eps, nb, nullptr, s, pdl, rc_rows);
         h->launches++;
         mark(h, KIND_MISC);
@@ -423,11 +456,11 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.act_out = b.act;
             const void* w[3] = {h->wg[l], h->wu[l], nullptr};
             const int32_t rows[3] = {D.F, D.F, 0};
-            int rc = run_gemm(h, tc ? plan(h->p_gu, h->p_gu_w, l) : nullptr, EPI_SWIGLU, (D.F + 63) / 64, w, rows, b.xn, D.d, a, tc, pdl, rc_rows, tc ? nb : 1);
+            int rc = gemm(2, tc ? plan(h->p_gu, h->p_gu_w, l) : nullptr, l, EPI_SWIGLU, (D.F + 63) / 64, w, rows, b.xn, D.d, a);
             if (rc) return rc;
             mark(h, KIND_GATEUP);
             if (tc) {
-                launch_swiglu_finish(st0, tc_gemm_streamk(plan(h->p_gu, h->p_gu_w, l), nb), b.act, b.act_lo, D.F, nb, s, pdl, rc_rows);
+                launch_swiglu_finish(st0, pieces(2, plan(h->p_gu, h->p_gu_w, l)), b.act, b.act_lo, D.F, nb, s, pdl, rc_rows);
                 h->launches++;
                 mark(h, KIND_MISC);
             }
@@ -437,9 +470,9 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.hres = b.hres;
             const void* w[3] = {h->wd[l], nullptr, nullptr};
             const int32_t rows[3] = {D.d, 0, 0};
-            int rc = run_gemm(h, tc ? plan(h->p_down, h->p_down_w, l) : nullptr, EPI_RESID, (D.d + TILE_N - 1) / TILE_N, w, rows, b.act, D.F, a, tc, pdl, rc_rows, tc ? nb : 1);
+            int rc = gemm(3, tc ? plan(h->p_down, h->p_down_w, l) : nullptr, l, EPI_RESID, (D.d + TILE_N - 1) / TILE_N, w, rows, b.act, D.F, a);
             if (rc) return rc;
-            if (tc) pending = tc_gemm_streamk(plan(h->p_down, h->p_down_w, l), nb);
+            if (tc) pending = pieces(3, plan(h->p_down, h->p_down_w, l));
             mark(h, KIND_DOWN);
         }
     }
@@ -452,9 +485,9 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
         const int n_tiles = (D.V + TILE_N - 1) / TILE_N;
         // tensor-core path: the sequences of a pass share the LM head's weight stream too (128-row plans: one at a time;
         // the candidate lists are shared)
-        const int lm_nq = tc ? tc_gemm_nq(wide ? h->p_lm_w : h->p_lm) : nb;
-        for (int q = 0; q < nb; q += lm_nq) {
-            const int sq = s0 + q, per = nb - q < lm_nq ? nb - q : lm_nq;
+        const int share = tc ? tc_gemm_nq(wide ? h->p_lm_w : h->p_lm) : nb;
+        for (int q = 0; q < nb; q += share) {
+            const int sq = s0 + q, per = nb - q < share ? nb - q : share;
             EpiArgs a = base_epi(h, D.V, sq, per);
             a.cand = b.cand; a.cand_ms = b.cand_ms; a.cand_floor = b.cand_floor; a.n_tiles = n_tiles;
             a.logits_dump = h->dbg_logits ? h->dbg_logits + (size_t)sq * RT * D.V : nullptr;
@@ -537,7 +570,7 @@ int forward(esp_handle* h, bool with_lm, int dcap, int only_seq) {
     if (!tc) return forward_pass(h, with_lm, dcap, 0, h->D.batch, false, prefill);
     if (only_seq >= 0) return forward_pass(h, with_lm, dcap, only_seq, 1, true, true);
     // consecutive sequences share a pass (and a weight stream); sequences that are not ready are inactive in it
-    const int per_pass = tc_gemm_max_nq(h->D.gemm_rows, ACT_PLANES);
+    const int per_pass = h->p_batch[3] ? batch_pass(h->D) : 1;
     for (int s0 = 0; s0 < h->D.batch; s0 += per_pass) {
         const int nb = h->D.batch - s0 < per_pass ? h->D.batch - s0 : per_pass;
         bool any = false;
@@ -672,34 +705,33 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
     if (model->dtype == 1) {
         const int dq = D.Hq * D.h, dkv = D.Hkv * D.h;
         const int nrs = D.gemm_rows;
-        const int nq_max = D.batch < tc_gemm_max_nq(nrs, ACT_PLANES) ? D.batch : tc_gemm_max_nq(nrs, ACT_PLANES);   // sequences sharing a weight stream
         bool ok = true;
         for (int l = 0; l < D.n_layers && ok; ++l) {
             TcGemm* p = nullptr;
             char* pk = h->b.packed + h->b.pk_layer * l;
             const void* w1[3] = {h->wq[l], h->wk[l], h->wv[l]};
             const int32_t r1[3] = {dq, dkv, dkv};
-            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w1, r1, D.d, h->b.xn, D.blocks, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 0 * SK_TABLE_TILES, SK_TABLE_TILES, pk, h->stream, ACT_PLANES);
+            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w1, r1, D.d, h->b.xn, D.blocks, nrs, 1, h->b.gemm_partials, tc_gemm_partial_bytes(148, 1, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 0 * SK_TABLE_TILES, SK_TABLE_TILES, pk, h->stream, ACT_PLANES);
             h->p_qkv.push_back(p);
             const void* w2[3] = {h->wo[l], nullptr, nullptr};
             const int32_t r2[3] = {D.d, 0, 0};
             p = nullptr;
-            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w2, r2, dq, h->b.attn_out, D.blocks, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 1 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv, h->stream, ACT_PLANES);
+            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w2, r2, dq, h->b.attn_out, D.blocks, nrs, 1, h->b.gemm_partials, tc_gemm_partial_bytes(148, 1, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 1 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv, h->stream, ACT_PLANES);
             h->p_o.push_back(p);
             const void* w3[3] = {h->wg[l], h->wu[l], nullptr};
             const int32_t r3[3] = {D.F, D.F, 0};
             p = nullptr;
-            ok = ok && !tc_gemm_create(&p, EPI_SWIGLU, true, w3, r3, D.d, h->b.xn, D.blocks, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 2 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o, h->stream, ACT_PLANES);
+            ok = ok && !tc_gemm_create(&p, EPI_SWIGLU, true, w3, r3, D.d, h->b.xn, D.blocks, nrs, 1, h->b.gemm_partials, tc_gemm_partial_bytes(148, 1, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 2 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o, h->stream, ACT_PLANES);
             h->p_gu.push_back(p);
             const void* w4[3] = {h->wd[l], nullptr, nullptr};
             const int32_t r4[3] = {D.d, 0, 0};
             p = nullptr;
-            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w4, r4, D.F, h->b.act, D.blocks, nrs, nq_max, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 3 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o + h->b.pk_gu, h->stream, ACT_PLANES);
+            ok = ok && !tc_gemm_create(&p, EPI_PARTIAL, true, w4, r4, D.F, h->b.act, D.blocks, nrs, 1, h->b.gemm_partials, tc_gemm_partial_bytes(148, 1, nrs), h->b.gemm_counters, n_sm, h->b.err, h->b.sk_tables + 3 * SK_TABLE_TILES, SK_TABLE_TILES, pk + h->b.pk_qkv + h->b.pk_o + h->b.pk_gu, h->stream, ACT_PLANES);
             h->p_down.push_back(p);
         }
         const void* w5[3] = {h->lm_head, nullptr, nullptr};
         const int32_t r5[3] = {D.V, 0, 0};
-        ok = ok && !tc_gemm_create(&h->p_lm, EPI_LOGITS, false, w5, r5, D.d, h->b.xn, D.blocks, nrs, nrs == 80 ? nq_max : 1, h->b.gemm_partials, tc_gemm_partial_bytes(148, nq_max, nrs), h->b.gemm_counters, n_sm, h->b.err, nullptr, 0, h->b.packed + h->b.pk_layer * D.n_layers, h->stream);
+        ok = ok && !tc_gemm_create(&h->p_lm, EPI_LOGITS, false, w5, r5, D.d, h->b.xn, D.blocks, nrs, lm_nq(D), h->b.gemm_partials, tc_gemm_partial_bytes(148, lm_nq(D), nrs), h->b.gemm_counters, n_sm, h->b.err, nullptr, 0, h->b.packed + h->b.pk_layer * D.n_layers, h->stream);
         if (ok && nrs != RT) {
             // the prefill runs 120-row blocks: the same weights (already repacked) behind 128-row GEMM plans
             const size_t pbytes = tc_gemm_partial_bytes(148, 1, RT);
@@ -729,13 +761,23 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
             ok = ok && !tc_gemm_create(&h->p_lm_w, EPI_LOGITS, false, w5, r5, D.d, h->b.xn, D.blocks, RT, 1, h->b.gemm_partials, pbytes, h->b.gemm_counters, n_sm, h->b.err, nullptr, 0, h->b.packed + h->b.pk_layer * D.n_layers, h->stream);
         }
         if (!ok) { esp_free(h); return ESP_E_CUDA; }
+        const TcGemm* narrow[4] = {h->p_qkv[0], h->p_o[0], h->p_gu[0], h->p_down[0]};
+        const void* x[4] = {h->b.xn, h->b.attn_out, h->b.xn, h->b.act};
+        const int K[4] = {D.d, dq, D.d, D.F};
+        if (D.batch > 1 && n_sm >= 148) {
+            TileSrc* tables = h->b.wide_tables + (D.pre_blocks ? (size_t)4 * WIDE_MAX_RT * SK_TABLE_TILES : 0);
+            const int bpt = batch_bpt(D);
+            for (int i = 0; i < 4; ++i)
+                if (wide_gemm_create(&h->p_batch[i], tc_gemm_tiles(narrow[i]), K[i], x[i], D.blocks, nrs, bpt, (batch_pass(D) + bpt - 1) / bpt,
+                                     h->b.wide_partials, h->b.wide_bytes, tables + (size_t)i * WIDE_MAX_RT * SK_TABLE_TILES, h->b.err, h->stream)) {
+                    esp_free(h);
+                    return ESP_E_CUDA;
+                }
+        }
         if (D.pre_blocks && n_sm >= 148) {
-            const TcGemm* narrow[4] = {h->p_qkv[0], h->p_o[0], h->p_gu[0], h->p_down[0]};
-            const void* x[4] = {h->b.xn, h->b.attn_out, h->b.xn, h->b.act};
-            const int K[4] = {D.d, dq, D.d, D.F};
             bool have = attn_tc_create(&h->p_attn_pre, h->b.qbuf, h->b.kcache, h->b.vcache, D.pre_blocks, D.Hq, D.Hkv, D.cap) == 0;
             for (int i = 0; i < 4 && have; ++i)
-                have = !wide_gemm_create(&h->p_wide[i], tc_gemm_tiles(narrow[i]), K[i], x[i], D.blocks, (D.pre_blocks + 1) / 2, h->b.wide_partials,
+                have = !wide_gemm_create(&h->p_wide[i], tc_gemm_tiles(narrow[i]), K[i], x[i], D.blocks, PREFILL_CHUNK, 2, (D.pre_blocks + 1) / 2, h->b.wide_partials,
                                          h->b.wide_bytes, h->b.wide_tables + (size_t)i * WIDE_MAX_RT * SK_TABLE_TILES, h->b.err, h->stream);
             if (!have) { esp_free(h); return ESP_E_CUDA; }
         }
@@ -1095,6 +1137,7 @@ void esp_free(esp_handle* h) {
     for (auto* p : h->p_down_w) tc_gemm_destroy(p);
     tc_gemm_destroy(h->p_lm_w);
     for (auto* p : h->p_wide) wide_gemm_destroy(p);
+    for (auto* p : h->p_batch) wide_gemm_destroy(p);
     attn_tc_destroy(h->p_attn_pre);
     layers_tc_destroy(h->p_layers);
     for (auto* t : h->p_attn) attn_tc_destroy(t);

@@ -40,30 +40,26 @@ namespace {
 
 using namespace tc;
 
-// NRS = rows of a sequence's block that take part (80, or 128 for blocks of more than 80 rows); NQ = sequences
-// one launch covers: the first NRS rows of their activation blocks ([RT][K] each, consecutive) are gathered by
-// one 3-D TMA box into one B operand of NQ*NRS <= 256 rows, so the weights are streamed once for all of them
-// (partial-only output only).
+// NRS = rows of a block that take part (80, or 128 for blocks of more than 80 rows); NQ = sequences one launch covers
+// (the LM head takes two): the first NRS rows of their activation blocks ([RT][K] each, consecutive) are gathered by one
+// 3-D TMA box into one B operand of NQ*NRS <= 256 rows, so the weights are streamed once for both.  (The layer GEMMs of
+// several sequences: esp_gemm_wide.cu.)
 //
 // Ring depth.  The bytes in flight per SM (depth x 16 KB of weights) over the load round trip bound the stream rate,
-// and the ring is also what is requested before the preceding kernel has finished: deeper is better.  The
-// partial-only kernel keeps no accumulator copy in shared memory and spends that room on the ring.
+// and the ring is also what is requested before the preceding kernel has finished: deeper is better.
 // Planes (PL).  The activations reach the tensor cores as bf16.  A plan with two planes reads them as a pair
-// x = hi + lo (hi = bf16(x), lo = bf16(x - hi), stored PL * n_seq blocks apart in the same buffer) and issues every
-// MMA twice into the same accumulator, first with hi, then with lo: the product then sees the activation to 2^-17
-// instead of 2^-9, for 10 KB more shared memory per stage and sequence.
+// x = hi + lo (hi = bf16(x), lo = bf16(x - hi), stored n_seq blocks apart in the same buffer) and takes every product
+// with both: it then sees the activation to 2^-17 instead of 2^-9, for 10 KB more shared memory per stage.
 __host__ __device__ constexpr int stages_of(int epi, int nq, int nrs, int pl = 1) {
-    return pl == 2 ? (nrs == 80 ? (nq == 2 ? 4 : 6) : 4)
-                   : (nrs == 80 ? (nq == 3 ? 4 : (nq == 2 ? (epi == EPI_PARTIAL ? 6 : 5) : (epi == EPI_PARTIAL ? 8 : 6)))
-                                : (nq == 2 ? 4 : (epi == EPI_PARTIAL ? 7 : 4)));
+    return pl == 2 ? (nrs == 80 ? 6 : 4) : (nrs == 80 ? (nq == 2 ? 5 : 6) : 4);
 }
 __host__ __device__ constexpr int b_bytes_of(int nq, int nrs) { return nq * nrs * BK * 2; }   // 10240 per 80-row sequence and plane
 __host__ __device__ constexpr int stage_bytes_of(int nq, int nrs, int pl = 1) { return A_BYTES + pl * b_bytes_of(nq, nrs); }
 // two accumulator buffers in tensor memory: 128 columns each for up to 128 rows, 256 each beyond
 __host__ __device__ constexpr int acc_cols_of(int nr) { return nr <= 128 ? 128 : 256; }
 constexpr int NUM_THREADS = 192;
-constexpr int MAX_NQ = 3;
-__host__ __device__ constexpr int max_nq_of(int nrs, int pl = 1) { return pl == 2 ? (nrs == 80 ? 2 : 1) : (nrs == 80 ? 3 : 2); }
+constexpr int MAX_NQ = 2;
+__host__ __device__ constexpr int max_nq_of(int nrs, int pl) { return pl == 1 && nrs == 80 ? 2 : 1; }
 
 struct TcParams {
     CUtensorMap map_a[3];
@@ -92,14 +88,14 @@ __device__ __forceinline__ void tile_source(const TcParams& p, int tile, int hal
 
 template <int EPI, int NQ, int NRS, int PL>
 __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constant__ TcParams p) {
-    static_assert(NQ == 1 || EPI == EPI_PARTIAL || EPI == EPI_LOGITS, "several sequences per launch: partials or logits");
-    static_assert(NQ * NRS <= 256 && (PL == 1 || NQ > 1 || 2 * NRS <= 256) && NRS % 16 == 0 && NRS <= RT, "MMA N");
-    static_assert(PL == 1 || EPI == EPI_PARTIAL, "two activation planes: partial-only output");
-    // One sequence with two planes: hi and lo rows sit back to back in the stage and form ONE B operand of 2 * NRS
+    static_assert(NQ == 1 || EPI == EPI_LOGITS, "several sequences per launch: logits");
+    static_assert(PL * NQ * NRS <= 256 && NRS % 16 == 0 && NRS <= RT, "MMA N");
+    static_assert((PL == 2) == (EPI == EPI_PARTIAL), "partials: two activation planes; fused epilogues: one");
+    // Two planes: hi and lo rows sit back to back in the stage and form ONE B operand of 2 * NRS
     // rows; the accumulator gets W x_hi in columns [0, NRS) and W x_lo in [NRS, 2 NRS), added by the epilogue.
     // (One MMA per k-step reads the weight slice once from shared memory; two MMAs would read it twice.)
-    constexpr bool JOINT = PL == 2 && NQ == 1;
-    constexpr int N_MMA = JOINT ? 2 * NRS : NQ * NRS;
+    constexpr bool JOINT = PL == 2;
+    constexpr int N_MMA = PL * NQ * NRS;
     constexpr int STAGE_BYTES = stage_bytes_of(NQ, NRS, PL), ACC_COLS = acc_cols_of(N_MMA), TMEM_COLS = 2 * ACC_COLS;
     constexpr int B_PLANE = b_bytes_of(NQ, NRS);
     constexpr uint32_t IDESC = idesc_of(N_MMA);
@@ -226,8 +222,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
                         umma(tmem_d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), IDESC, (kb > sg.kb0 || k > 0) ? 1u : 0u);
-                        if constexpr (PL == 2 && !JOINT)      // several sequences: the same step with their low-order planes
-                            umma(tmem_d, da + (uint64_t)(k * 2), db + (uint64_t)((B_PLANE >> 4) + k * 2), IDESC, 1u);
                     }
                     umma_commit(&empty[stage]);
                     if (++stage == STAGES) { stage = 0; phase ^= 1; }
@@ -449,7 +443,6 @@ struct TcGemm {
 
 constexpr int MAX_SLOTS = 4;
 size_t tc_gemm_partial_bytes(int n_sm, int nq, int nrs) { return (size_t)n_sm * MAX_SLOTS * nq * nrs * TILE_N * sizeof(float); }
-int tc_gemm_max_nq(int nrs, int planes) { return max_nq_of(nrs, planes); }
 int tc_gemm_counter_ints() { return 4096; }
 size_t tc_gemm_packed_bytes(int epi, const int32_t rows_w[3], int K) {
     const long long total = (long long)rows_w[0] + rows_w[1] + rows_w[2];
@@ -471,7 +464,7 @@ int tc_gemm_create(TcGemm** out, int epi, bool defer, const void* const w[3], co
     if (!out || (nrs != 80 && nrs != RT) || (planes != 1 && planes != 2) || nq_max < 1 || nq_max > max_nq_of(nrs, planes) ||
         x_seqs < nq_max || K % 8 || n_sm < 1)
         return -1;
-    if (((nq_max > 1 && (epi != EPI_LOGITS || nq_max > 2 || nrs != 80)) || planes > 1) && !defer) return -1;
+    if ((planes > 1) != defer || (nq_max > 1 && epi != EPI_LOGITS)) return -1;
     if (reinterpret_cast<uintptr_t>(x) % 16) return -1;
     TcGemm* g = new (std::nothrow) TcGemm();
     if (!g) return -1;
@@ -598,7 +591,6 @@ int tc_gemm_launch(const TcGemm* g, const EpiArgs& a, cudaStream_t s, bool pdl, 
     if (g->planes == 2) {
         if (p.epi != EPI_PARTIAL) return ESP_E_ARG;
         if (!wide && nq == 1) ESP_TC_CASE(EPI_PARTIAL, 1, 80, 2)
-        else if (!wide && nq == 2) ESP_TC_CASE(EPI_PARTIAL, 2, 80, 2)
         else if (wide && nq == 1) ESP_TC_CASE(EPI_PARTIAL, 1, RT, 2)
         else return ESP_E_ARG;
     }
@@ -607,11 +599,6 @@ int tc_gemm_launch(const TcGemm* g, const EpiArgs& a, cudaStream_t s, bool pdl, 
     else if (p.epi == EPI_LOGITS && !wide && nq == 1) ESP_TC_CASE(EPI_LOGITS, 1, 80, 1)
     else if (p.epi == EPI_LOGITS && !wide && nq == 2) ESP_TC_CASE(EPI_LOGITS, 2, 80, 1)
     else if (p.epi == EPI_LOGITS) ESP_TC_CASE(EPI_LOGITS, 1, RT, 1)
-    else if (p.epi == EPI_PARTIAL && !wide && nq == 1) ESP_TC_CASE(EPI_PARTIAL, 1, 80, 1)
-    else if (p.epi == EPI_PARTIAL && !wide && nq == 2) ESP_TC_CASE(EPI_PARTIAL, 2, 80, 1)
-    else if (p.epi == EPI_PARTIAL && !wide && nq == 3) ESP_TC_CASE(EPI_PARTIAL, 3, 80, 1)
-    else if (p.epi == EPI_PARTIAL && wide && nq == 1) ESP_TC_CASE(EPI_PARTIAL, 1, RT, 1)
-    else if (p.epi == EPI_PARTIAL && wide && nq == 2) ESP_TC_CASE(EPI_PARTIAL, 2, RT, 1)
     else return ESP_E_ARG;
 #undef ESP_TC_CASE
     return e == cudaSuccess ? ESP_OK : ESP_E_CUDA;

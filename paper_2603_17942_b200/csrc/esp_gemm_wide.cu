@@ -1,13 +1,15 @@
-// bf16 GEMM over several blocks of rows at once (the prefill's passes over many prompt blocks), on the Blackwell
-// tensor cores: y[row][n] = sum_k (x_hi[row][k] + x_lo[row][k]) * w[n][k], fp32 accumulation, both planes of the
-// activations (see esp_gemm_tc.cu) into one accumulator.
+// bf16 GEMM over several blocks of rows at once -- the full blocks of a prompt, or the blocks of several sequences in a
+// decode step -- on the Blackwell tensor cores: y[row][n] = sum_k (x_hi[row][k] + x_lo[row][k]) * w[n][k], fp32
+// accumulation, both planes of the activations (see esp_gemm_tc.cu) into one accumulator.
 //
 // With hundreds of rows per weight stream the work is a matter of the tensor cores, and what has to be kept up is
-// their operand supply: a 256-feature x 240-row tile needs 32 KB of weights and 60 KB of activations per 64 k for
-// 16 MMAs of N = 240, about 48 bytes per clock and SM from L2 (a 128-feature tile would need 79).  The tile is the
-// whole tensor memory (two accumulators of 240 of 256 columns), so there is one in flight per CTA.
+// their operand supply: shared memory delivers 128 bytes per clock, an MMA of N = 240 takes 98 of them for its
+// operands, and what a tile needs from L2 passes through the same port.  A 256-feature x 240-row tile needs 32 KB of
+// weights and 60 KB of activations per 64 k for 16 MMAs of N = 240 (48 bytes per clock); a 128-feature tile, as the
+// small-M kernel has it, would need 79.  The tile is the whole tensor memory (two accumulators of up to 240 of 256
+// columns), so there is one in flight per CTA.
 //
-// Work split: a row tile is two blocks of 120 rows (one TMA box of 2 x 120 rows per plane).  The CTAs form groups of
+// Work split: a row tile is BPT blocks of WB rows (one TMA box of BPT x WB rows per plane).  The CTAs form groups of
 // one CTA per row tile; a group owns a contiguous range of the (256-feature tile, k-block) units, stream-K style, and
 // its CTAs walk it in step, so that a weight unit is read from HBM once and from L2 by the other row tiles.  Every
 // piece is stored as an fp32 partial; the kernel that consumes the result sums a tile's pieces in group order, as it
@@ -19,7 +21,9 @@
 //
 // Measured, 960 rows (eight prefill blocks) of an 8B layer, on their own: QKV 71, O 52, gate/up 280, down 145 us = 1.24 to
 // 1.61 PFLOP/s of two-plane products, 0.75 to 0.98 of the measured cuBLAS rate; eight passes of the small-M kernel took
-// 8 x 108 us.
+// 8 x 108 us.  Four sequences of 80 rows: 229 us per layer against 2 x 129 for two passes of the small-M kernel over two
+// sequences (56 KB of shared-memory fill and 74 KB of operand reads per 16 KB weight unit were its bound); eight: 424
+// against 4 x 128.
 #include <new>
 #include <string.h>
 
@@ -32,18 +36,14 @@ namespace {
 
 using namespace tc;
 
-constexpr int WB = PREFILL_CHUNK;              // rows of a block
-constexpr int WR = 2 * WB;                     // rows of a row tile = MMA N
-constexpr int SLOT_BYTES = 2 * A_BYTES;        // 32 KB: two weight units, or one plane of a row tile (30 KB)
-constexpr int X_BYTES = WR * BK * 2;
+constexpr int SLOT_BYTES = 2 * A_BYTES;        // 32 KB: two weight units, or one plane of a row tile
 constexpr int SLOTS = 7;
 constexpr int WIDE_THREADS = 320;
 constexpr size_t WIDE_SMEM = 1024 + (size_t)SLOTS * SLOT_BYTES + 256;
-static_assert(WR % 16 == 0 && WR <= 256 && X_BYTES <= SLOT_BYTES && X_BYTES % 1024 == 0, "row tile");
 static_assert(WIDE_SMEM <= 232448, "shared memory");
 
 struct WideParams {
-    CUtensorMap map_b;          // activations [2 planes x x_blocks][RT][K], box 64 x WB x 2
+    CUtensorMap map_b;          // activations [2 planes x x_blocks][RT][K], box 64 x WB x BPT
     const unsigned char* w;     // packed weight units [n_tiles][KB][A_BYTES]
     const SeqState* st;         // one state per block
     float* partials;            // [group][slot][2 halves][n_rt * WR rows][128 features]
@@ -51,7 +51,11 @@ struct WideParams {
     int32_t n_tiles, n_ft, KB, n_groups, n_rt, slots, plane_blocks, n_blocks;
 };
 
+template <int WB, int BPT>
 __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_constant__ WideParams p) {
+    constexpr int WR = WB * BPT;               // rows of a row tile = MMA N
+    constexpr int X_BYTES = WR * BK * 2;
+    static_assert(WR % 16 == 0 && WR <= 256 && X_BYTES <= SLOT_BYTES && WB % 8 == 0 && WB <= RT, "row tile");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t* full = reinterpret_cast<uint64_t*>(ring + SLOTS * SLOT_BYTES);
@@ -98,7 +102,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
                     bulk_load(dst + A_BYTES, p.w + ((size_t)t1 * p.KB + kb) * A_BYTES, A_BYTES, &full[slot], pol_w);
                 } else {
                     mbar_expect_tx(&full[slot], X_BYTES);
-                    tma_load_3d_hint(dst, &p.map_b, kb * BK, 0, (kind - 1) * p.plane_blocks + rt * 2, &full[slot], pol_x);
+                    tma_load_3d_hint(dst, &p.map_b, kb * BK, 0, (kind - 1) * p.plane_blocks + rt * BPT, &full[slot], pol_x);
                 }
             };
             const int n_items = 3 * n_units, n_pre = n_items < SLOTS ? n_items : SLOTS;
@@ -170,9 +174,10 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
         const int half = (warp - 2) >> 2, q = warp & 3, f = q * 32 + lane;
         const uint32_t taddr = tmem_base + half * 256 + ((uint32_t)(q * 32) << 16);
         const size_t rows = (size_t)p.n_rt * WR;
-        int nr[2];
+        int nr[BPT];
 #pragma unroll
-        for (int b = 0; b < 2; ++b) nr[b] = rt * 2 + b < p.n_blocks && p.st[rt * 2 + b].active ? min(p.st[rt * 2 + b].n_rows, WB) : 0;
+        for (int b = 0; b < BPT; ++b)
+            nr[b] = rt * BPT + b < p.n_blocks && p.st[rt * BPT + b].active ? min(p.st[rt * BPT + b].n_rows, WB) : 0;
         bool ok = true;
         int piece = 0;
         const int ft0 = u0 / p.KB;
@@ -184,27 +189,30 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const bool real = 2 * ft + half < p.n_tiles;
             float* part = p.partials + (((size_t)(grp * p.slots + (ft - ft0)) * 2 + half) * rows + (size_t)rt * WR) * TILE_N + f;
+            // CH columns at a time: as many 16-column loads as fit, an 8-column load for the rest, one wait
+            constexpr int CH = WB % 24 == 0 ? 24 : (WB % 40 == 0 ? 40 : 32);
+            static_assert(WB % CH == 0 && (CH % 16 == 0 || CH % 16 == 8), "columns per wait");
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
+            for (int b = 0; b < BPT; ++b) {
                 const int n = real ? nr[b] : 0;
 #pragma unroll
-                for (int c0 = 0; c0 < WB; c0 += 24) {           // 120 = 5 x 24 columns: an x16 and an x8 load
-                    uint32_t v[24];
-                    uint32_t v16[16];
-                    tmem_ld16_issue(taddr + b * WB + c0, v16);
-                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                                 : "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23])
-                                 : "r"(taddr + b * WB + c0 + 16));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                for (int c0 = 0; c0 < WB; c0 += CH) {
+                    uint32_t v[CH];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = v16[i];
-                    if (b == 1 && c0 + 24 >= WB) {              // the accumulator is in registers
+                    for (int c = 0; c + 16 <= CH; c += 16) tmem_ld16_issue(taddr + b * WB + c0 + c, *reinterpret_cast<uint32_t(*)[16]>(&v[c]));
+                    if constexpr (CH % 16 == 8)
+                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                                     : "=r"(v[CH - 8]), "=r"(v[CH - 7]), "=r"(v[CH - 6]), "=r"(v[CH - 5]), "=r"(v[CH - 4]), "=r"(v[CH - 3]),
+                                       "=r"(v[CH - 2]), "=r"(v[CH - 1])
+                                     : "r"(taddr + b * WB + c0 + CH - 8));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (b == BPT - 1 && c0 + CH >= WB) {        // the accumulator is in registers
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         __syncwarp();
                         if (lane == 0) mbar_arrive(tempty);
                     }
 #pragma unroll
-                    for (int i = 0; i < 24; ++i)
+                    for (int i = 0; i < CH; ++i)
                         if (c0 + i < n) __stcg(part + (size_t)(b * WB + c0 + i) * TILE_N, __uint_as_float(v[i]));
                 }
             }
@@ -244,22 +252,22 @@ void wide_geometry(int n_tiles, int KB, int n_rt, int* n_groups, int* slots) {
     *slots = most;
 }
 
-size_t wide_partial_bytes(int n_tiles, int KB, int n_rt) {
+size_t wide_partial_bytes(int n_tiles, int KB, int n_rt, int tile_rows) {
     int g, slots;
     wide_geometry(n_tiles, KB, n_rt, &g, &slots);
-    return (size_t)g * slots * 2 * n_rt * WR * TILE_N * sizeof(float);
+    return (size_t)g * slots * 2 * n_rt * tile_rows * TILE_N * sizeof(float);
 }
 
 struct WideGemm {
     WideParams p;
-    int n_rt_max;
+    int n_rt_max, wb, bpt;      // row tiles at most; rows per block, blocks per row tile
     int groups[WIDE_MAX_RT], slots[WIDE_MAX_RT];
     TileSrc* tables;            // [n_rt_max][n_tiles]
 };
 
-int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int n_rt_max, float* partials, size_t partial_bytes,
+int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int wb, int bpt, int n_rt_max, float* partials, size_t partial_bytes,
                      TileSrc* tables_dev, int* err, cudaStream_t stream) {
-    if (!out || n_rt_max < 1 || n_rt_max > WIDE_MAX_RT || x_blocks < 2 || K % 8 || reinterpret_cast<uintptr_t>(x) % 16) return -1;
+    if (!out || n_rt_max < 1 || n_rt_max > WIDE_MAX_RT || x_blocks < bpt || K % 8 || reinterpret_cast<uintptr_t>(x) % 16) return -1;
     EncodeFn enc = get_encode();
     if (!enc) return -1;
     WideGemm* g = new (std::nothrow) WideGemm();
@@ -268,12 +276,12 @@ int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_bl
     WideParams& p = g->p;
     p.n_tiles = n_tiles; p.n_ft = (n_tiles + 1) / 2; p.KB = (K + BK - 1) / BK;
     p.partials = partials; p.err = err; p.plane_blocks = x_blocks;
-    g->n_rt_max = n_rt_max;
+    g->n_rt_max = n_rt_max; g->wb = wb; g->bpt = bpt;
     g->tables = tables_dev;
     {
         cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)RT, (cuuint64_t)2 * x_blocks};
         cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)RT * K * 2};
-        cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)WB, 2};
+        cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)wb, (cuuint32_t)bpt};
         cuuint32_t estr[3] = {1, 1, 1};
         if (enc(&p.map_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -283,7 +291,7 @@ int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_bl
     bool fits = tab != nullptr;
     for (int r = 1; r <= n_rt_max && fits; ++r) {
         wide_geometry(n_tiles, p.KB, r, &g->groups[r - 1], &g->slots[r - 1]);
-        fits = wide_partial_bytes(n_tiles, p.KB, r) <= partial_bytes;
+        fits = wide_partial_bytes(n_tiles, p.KB, r, wb * bpt) <= partial_bytes;
         const long long U = (long long)p.n_ft * p.KB, G = g->groups[r - 1];
         for (int t = 0; t < n_tiles && fits; ++t) {
             TileSrc& e = tab[(size_t)(r - 1) * n_tiles + t];
@@ -307,25 +315,35 @@ int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_bl
 void wide_gemm_destroy(WideGemm* g) { delete g; }
 
 int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, int n_blocks, cudaStream_t s, bool pdl) {
-    const int n_rt = (n_blocks + 1) / 2;
-    if (!g || n_blocks < 1 || n_rt > g->n_rt_max) return ESP_E_ARG;
+    if (!g || n_blocks < 1) return ESP_E_ARG;
+    const int n_rt = (n_blocks + g->bpt - 1) / g->bpt;
+    if (n_rt > g->n_rt_max) return ESP_E_ARG;
     WideParams p = g->p;
     p.w = reinterpret_cast<const unsigned char*>(packed);
     p.st = st;
     p.n_rt = n_rt; p.n_blocks = n_blocks; p.n_groups = g->groups[n_rt - 1]; p.slots = g->slots[n_rt - 1];
-    if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_gemm_wide), (int)WIDE_SMEM)) return ESP_E_CUDA;
-    return launch_k(k_gemm_wide, dim3(p.n_groups * n_rt), dim3(WIDE_THREADS), WIDE_SMEM, s, pdl, p) == cudaSuccess ? ESP_OK : ESP_E_CUDA;
+#define ESP_WIDE_CASE(WB, BPT)                                                                                          \
+    if (g->wb == WB && g->bpt == BPT) {                                                                                \
+        if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_gemm_wide<WB, BPT>), (int)WIDE_SMEM)) return ESP_E_CUDA; \
+        return launch_k(k_gemm_wide<WB, BPT>, dim3(p.n_groups * n_rt), dim3(WIDE_THREADS), WIDE_SMEM, s, pdl, p) == cudaSuccess ? ESP_OK : ESP_E_CUDA; \
+    }
+    ESP_WIDE_CASE(PREFILL_CHUNK, 2)
+    ESP_WIDE_CASE(80, 2)
+    ESP_WIDE_CASE(80, 3)
+    ESP_WIDE_CASE(RT, 2)
+#undef ESP_WIDE_CASE
+    return ESP_E_ARG;
 }
 
-// the row of block b, row r in the partials is b * WB + r
+// the row of block b, row r in the partials is b * wb + r
 StreamK wide_gemm_streamk(const WideGemm* g, int n_blocks) {
-    const int n_rt = (n_blocks + 1) / 2;
+    const int n_rt = (n_blocks + g->bpt - 1) / g->bpt;
     StreamK k;
     k.partials = g->p.partials;
     k.table = g->tables + (size_t)(n_rt - 1) * g->p.n_tiles;
     k.n_tiles = g->p.n_tiles; k.KB = g->p.KB; k.G = g->groups[n_rt - 1]; k.slots = g->slots[n_rt - 1];
-    k.rows = n_rt * WR;
-    k.seq_rows = WB;
+    k.rows = n_rt * g->bpt * g->wb;
+    k.seq_rows = g->wb;
     return k;
 }
 

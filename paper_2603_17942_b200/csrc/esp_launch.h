@@ -112,9 +112,9 @@ int attn_tc_run(const void* q, const void* kcache, const void* vcache, int batch
 struct TcGemm;
 // epi selects the tile -> weight-row mapping and the fused epilogue; with defer the kernel only stores partials
 // (EPI_PARTIAL) and the caller runs the matching consumer kernel.  x: activations [x_seqs][RT][K]; nrs = rows of a
-// block that take part (80, or RT for blocks of more than 80 rows); a deferred plan may cover up to nq_max
-// sequences per launch, so that the weights are streamed once for all of them.  planes = 2 (deferred plans only):
-// x holds the activations as hi + lo bf16 pairs, [2][x_seqs][RT][K], and every product is taken with both
+// block that take part (80, or RT for blocks of more than 80 rows); an 80-row EPI_LOGITS plan may cover nq_max = 2
+// sequences per launch, so that the weights are streamed once for both.  Deferred plans have planes = 2: x holds the
+// activations as hi + lo bf16 pairs, [2][x_seqs][RT][K], and every product is taken with both
 int tc_gemm_create(TcGemm** out, int epi, bool defer, const void* const w[3], const int32_t rows_w[3], int K, const void* x,
                    int x_seqs, int nrs, int nq_max, void* partials, size_t partial_bytes, int* counters, int n_sm, int* err, TileSrc* table_dev,
                    int table_entries, void* packed, cudaStream_t stream, int planes = 1);
@@ -127,18 +127,19 @@ int tc_wait_selftest(int* err_dev, cudaStream_t s);
 int tc_gemm_tiles(const TcGemm* g);
 int tc_gemm_nq(const TcGemm* g);     // sequences one launch of the plan may cover
 size_t tc_gemm_partial_bytes(int n_sm, int nq = 1, int nrs = 80);
-int tc_gemm_max_nq(int nrs = 80, int planes = 1);
 int tc_gemm_counter_ints();
 
 
-// tcgen05 GEMM over several full prefill blocks at once (esp_gemm_wide.cu): activations [2 planes][x_blocks][RT][K], of
-// every block the first PREFILL_CHUNK rows; partials and contributor tables for the same consumers as above.
+// tcgen05 GEMM over several blocks at once (esp_gemm_wide.cu): activations [2 planes][x_blocks][RT][K], of every block
+// the first wb rows, bpt blocks to a row tile ((PREFILL_CHUNK, 2), (80, 2), (80, 3) or (RT, 2)); partials and contributor
+// tables for the same consumers as above.
 struct WideGemm;
-constexpr int WIDE_MAX_BLOCKS = 8, WIDE_MAX_RT = WIDE_MAX_BLOCKS / 2;
-size_t wide_partial_bytes(int n_tiles, int KB, int n_rt);
+constexpr int WIDE_MAX_RT = 4;                       // row tiles of one launch
+constexpr int WIDE_MAX_BLOCKS = 2 * WIDE_MAX_RT;     // full prefill blocks of one pass
+size_t wide_partial_bytes(int n_tiles, int KB, int n_rt, int tile_rows);
 // tables_dev: device memory for n_rt_max * n_tiles entries
-int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int n_rt_max, float* partials, size_t partial_bytes,
-                     TileSrc* tables_dev, int* err, cudaStream_t stream);
+int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int wb, int bpt, int n_rt_max, float* partials,
+                     size_t partial_bytes, TileSrc* tables_dev, int* err, cudaStream_t stream);
 void wide_gemm_destroy(WideGemm* g);
 int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, int n_blocks, cudaStream_t s, bool pdl);
 StreamK wide_gemm_streamk(const WideGemm* g, int n_blocks);
