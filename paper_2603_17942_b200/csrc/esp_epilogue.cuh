@@ -91,10 +91,20 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
                     from_f32<T>(s_acc[r * ACC_LD + f]);
         }
     } else if constexpr (EPI == EPI_LOGITS) {
-        // warp w takes rows w, w+4, ...; a lane holds features lane, lane+32, lane+64, lane+96 of the row
+        // (the row loop at the end) warp w takes every fourth row; a lane holds features lane, lane+32, lane+64, lane+96 of the row
         const int warp = f >> 5, lane = f & 31;
         const int n_nodes = st ? st->n_nodes : a.rows_fixed;
         const int Mtot = a.batch * RT;
+        // Everything the row loop needs of `a` and `st`, once: behind the loop's stores the compiler has to fetch a member
+        // again at every use.
+        const int n_out = a.n_out, KP = a.KP;
+        Cand* const cand = a.cand;
+        float2* const cand_ms = a.cand_ms;
+        uint32_t* const cand_floor = a.cand_floor;
+        float* const logits_dump = a.logits_dump;
+        const float inv_temp = st ? a.samp_inv_temp : 0.f;
+        const uint32_t key0 = a.samp_key0, key1 = a.samp_key1;
+        const int L = st ? st->L : 0;
         uint32_t noise_pos = 0xffffffffu;   // rows come in breadth-first order: equal depths are neighbours and
         float noise[4] = {0.f, 0.f, 0.f, 0.f};   // share their noise, which is a function of (position, token)
         // Floors.  What is already known of a probe row bounds its K'-th largest logit from below, and an entry strictly
@@ -107,20 +117,20 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
         const int S = n_rows <= 80 ? 80 : RT;                             // s_aux holds at least 2 * S words
         uint32_t* s_floor = reinterpret_cast<uint32_t*>(s_aux);          // [S] bounds, [S] "this probe row has entries at or above its bound"
         uint32_t* s_need = s_floor + S;
-        uint32_t* group_max = a.cand_floor ? a.cand_floor + (size_t)grow0 * KP_MAX + tile % a.KP : nullptr;
+        uint32_t* group_max = cand_floor ? cand_floor + (size_t)grow0 * KP_MAX + tile % KP : nullptr;
         for (int r = r0 + f; r < r1; r += 128) {
             uint32_t bound = 0u;
-            if (r >= n_nodes && a.cand_floor) {
-                const uint4* g = reinterpret_cast<const uint4*>(a.cand_floor + (size_t)(grow0 + r) * KP_MAX);
+            if (r >= n_nodes && cand_floor) {
+                const uint4* g = reinterpret_cast<const uint4*>(cand_floor + (size_t)(grow0 + r) * KP_MAX);
                 bound = 0xffffffffu;
 #pragma unroll
                 for (int j = 0; j < KP_MAX; j += 4) {
-                    if (j >= a.KP) break;
+                    if (j >= KP) break;
                     const uint4 w = __ldcg(g + j / 4);
                     bound = min(bound, w.x);
-                    if (j + 1 < a.KP) bound = min(bound, w.y);
-                    if (j + 2 < a.KP) bound = min(bound, w.z);
-                    if (j + 3 < a.KP) bound = min(bound, w.w);
+                    if (j + 1 < KP) bound = min(bound, w.y);
+                    if (j + 2 < KP) bound = min(bound, w.z);
+                    if (j + 3 < KP) bound = min(bound, w.w);
                 }
             }
             s_floor[r] = bound;
@@ -134,56 +144,88 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
         if (many_probes) {
             const int r = (n_nodes > r0 ? n_nodes : r0) + f;
             if (r < r1) {
-                const int n_valid = a.n_out - n0 < TILE_N ? a.n_out - n0 : TILE_N;
+                const int n_valid = n_out - n0 < TILE_N ? n_out - n0 : TILE_N;
                 const float* row = s_acc + r * ACC_LD;
                 float tmax = -INFINITY;
                 for (int i = 0; i < n_valid; ++i) tmax = fmaxf(tmax, row[i]);
                 float sum = 0.f;
                 for (int i = 0; i < n_valid; ++i) sum += expf(row[i] - tmax);
-                a.cand_ms[(size_t)tile * Mtot + grow0 + r] = make_float2(tmax, sum);
+                cand_ms[(size_t)tile * Mtot + grow0 + r] = make_float2(tmax, sum);
                 if (group_max) atomicMax(group_max + (size_t)r * KP_MAX, float_order_key(tmax));
                 const bool need = float_order_key(tmax) >= s_floor[r];
                 s_need[r] = need ? 1u : 0u;
                 if (!need) {
-                    Cand* out = a.cand + ((size_t)tile * Mtot + grow0 + r) * a.KP;
-                    for (int j = 0; j < a.KP; ++j) { out[j].val = -INFINITY; out[j].id = -1; }
+                    Cand* out = cand + ((size_t)tile * Mtot + grow0 + r) * KP;
+                    for (int j = 0; j < KP; ++j) { out[j].val = -INFINITY; out[j].id = -1; }
                 }
             }
         }
+        // Tree rows under greedy matching: one thread per row too, four runs of 32 features side by side, merged in order
+        // (largest value, smallest id among equals).  A warp per row spent 1750 cycles on each -- its chain of shared-memory
+        // loads, comparisons and two warp-wide reductions, one row after the other --, 19 us per tile of a 64-node tree.
+        // Measured, vocabulary 128256: LM head of one sequence of 68 rows 176 -> 163 us, of two 247 -> 185, 30 tree rows and
+        // 90 probe rows 237 -> 220.
+        const int n_arg = inv_temp > 0.f ? 0 : (n_nodes < r1 ? n_nodes : r1) - r0;     // rows r0 .. r0 + n_arg - 1
+        if (f < n_arg) {
+            const int r = r0 + f;
+            const float* row = s_acc + r * ACC_LD;
+            float bv[4];
+            int bi[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) { bv[c] = -INFINITY; bi[c] = 0x7fffffff; }
+#pragma unroll 8
+            for (int i = 0; i < 32; ++i)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int id = n0 + 32 * c + i;
+                    const float v = row[32 * c + i];
+                    if (id < n_out && cand_before(v, id, bv[c], bi[c])) { bv[c] = v; bi[c] = id; }
+                }
+#pragma unroll
+            for (int c = 1; c < 4; ++c)
+                if (cand_before(bv[c], bi[c], bv[0], bi[0])) { bv[0] = bv[c]; bi[0] = bi[c]; }
+            Cand* out = cand + ((size_t)tile * Mtot + grow0 + r) * KP;
+            out->val = bv[0];
+            out->id = bi[0] == 0x7fffffff ? -1 : bi[0];
+        }
+        if (logits_dump)
+            for (int r = r0 + warp; r < r1; r += 4)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (n0 + lane + 32 * i < n_out) logits_dump[(size_t)(grow0 + r) * n_out + n0 + lane + 32 * i] = s_acc[r * ACC_LD + lane + 32 * i];
         epi_bar(bar_id);
-        for (int r = r0 + warp; r < r1; r += 4) {
+        for (int r = r0 + (n_arg > 0 ? n_arg : 0) + warp; r < r1; r += 4) {
             float v[4];
             int id[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 id[i] = n0 + lane + 32 * i;
-                v[i] = id[i] < a.n_out ? s_acc[r * ACC_LD + lane + 32 * i] : -INFINITY;
-                if (a.logits_dump && id[i] < a.n_out) a.logits_dump[(size_t)(grow0 + r) * a.n_out + id[i]] = v[i];
+                v[i] = id[i] < n_out ? s_acc[r * ACC_LD + lane + 32 * i] : -INFINITY;
             }
             if (many_probes && r >= n_nodes && !s_need[r]) continue;       // warp-uniform
             const bool probe = r >= n_nodes;
-            const int kp = probe ? a.KP : 1;
-            Cand* out = a.cand + ((size_t)tile * Mtot + grow0 + r) * a.KP;
-            if (!probe && st && a.samp_inv_temp > 0.f) {
+            const int kp = probe ? KP : 1;
+            Cand* out = cand + ((size_t)tile * Mtot + grow0 + r) * KP;
+            if (!probe && inv_temp > 0.f) {
                 // sample matching: this row's token for position L + depth + 1 is the arg-max of the noisy scores
-                const uint32_t pos = (uint32_t)(st->L + st->row_depth[r] + 1);
+                const uint32_t pos = (uint32_t)(L + st->row_depth[r] + 1);
                 if (pos != noise_pos) {
                     noise_pos = pos;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) noise[i] = gumbel_noise(a.samp_key0, a.samp_key1, pos, (uint32_t)id[i]);
+                    for (int i = 0; i < 4; ++i) noise[i] = gumbel_noise(key0, key1, pos, (uint32_t)id[i]);
                 }
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if (id[i] < a.n_out) v[i] = sample_score(v[i], a.samp_inv_temp, noise[i]);
+                    if (id[i] < n_out) v[i] = sample_score(v[i], inv_temp, noise[i]);
             }
             if (probe && !many_probes) {
                 float tmax = warp_max(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])));
                 float s = 0.f;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) s += id[i] < a.n_out ? expf(v[i] - tmax) : 0.f;
+                for (int i = 0; i < 4; ++i) s += id[i] < n_out ? expf(v[i] - tmax) : 0.f;
                 s = warp_sum(s);
                 if (lane == 0) {
-                    a.cand_ms[(size_t)tile * Mtot + grow0 + r] = make_float2(tmax, s);
+                    cand_ms[(size_t)tile * Mtot + grow0 + r] = make_float2(tmax, s);
                     if (group_max) atomicMax(group_max + (size_t)r * KP_MAX, float_order_key(tmax));
                 }
             }
@@ -197,7 +239,7 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
                 int bi = 0x7fffffff, bslot = -1;
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if (!(used >> i & 1) && id[i] < a.n_out && cand_before(v[i], id[i], bv, bi)) { bv = v[i]; bi = id[i]; bslot = i; }
+                    if (!(used >> i & 1) && id[i] < n_out && cand_before(v[i], id[i], bv, bi)) { bv = v[i]; bi = id[i]; bslot = i; }
                 // two warp-wide integer reductions: the largest value (as an order-preserving key), then the smallest
                 // token id among the lanes that hold it
                 const uint32_t key = bslot >= 0 ? float_order_key(bv) : 0u;
