@@ -515,7 +515,12 @@ int forward_prefill_wide(esp_handle* h, int seq, int nb, int off) {
     cudaStream_t s = h->stream;
     const bool pdl = h->use_pdl;
     const size_t kv_seq_off = (size_t)seq * D.Hkv * D.cap * D.h * 2;
-    const int rows = PREFILL_CHUNK, n_split_launch = (off + nb * rows + D.split_len - 1) / D.split_len;
+    const int rows = PREFILL_CHUNK;
+    // Cache splits: the pass has its own grid, a function of its last position.  Its blocks alone fill the SMs, and short
+    // splits would only add partials (each split writes 16 MB of them for 8 blocks, and the merge reads them back).
+    int split_len = attn_split_len(off + nb * rows, nb, D.Hkv);
+    if (split_len < D.split_len) split_len = D.split_len;
+    const int n_split_launch = (off + nb * rows + split_len - 1) / split_len;
     StreamK pending;
     memset(&pending, 0, sizeof(pending));
     pending.KB = pending.G = 1; pending.slots = 2; pending.rows = pending.seq_rows = RT;
@@ -543,7 +548,7 @@ int forward_prefill_wide(esp_handle* h, int seq, int nb, int off) {
         a.out = b.attn_out; a.out_lo = b.attn_out_lo;
         a.part_o = b.part_o; a.part_ml = b.part_ml;
         a.st = b.pre_states;
-        a.Hq = D.Hq; a.Hkv = D.Hkv; a.h = D.h; a.cap = D.cap; a.split_len = D.split_len; a.n_split_max = D.n_split_max;
+        a.Hq = D.Hq; a.Hkv = D.Hkv; a.h = D.h; a.cap = D.cap; a.split_len = split_len; a.n_split_max = D.n_split_max;
         a.dcap = DCAP_PREFILL;
         a.rows_cap = rows;
         a.cache_in_flight = 1;

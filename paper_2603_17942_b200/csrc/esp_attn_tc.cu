@@ -688,12 +688,46 @@ __global__ void __launch_bounds__(TM_WARPS * 32, 2) k_attn_tail_merge_many_tc(At
         // (the warp-per-pair kernel merges its one chunk into an empty running sum: the same values)
         if (!waited) { pdl_wait(); waited = true; }      // the bulk partials
         __syncwarp();
-        constexpr int PB = 2;
-        FirstPartials<PB> fp[GH];
+        // Merge: bulk partials in split order, the tail last.  The next split's values of all GH heads are requested
+        // before the current one's are used: a round trip per split, not per split and head.
+        const int n_sp = (T0 + a.split_len - 1) / a.split_len;
+        const size_t base = ((size_t)(seq * RT + c.r) * a.Hq + head0) * a.n_split_max;
+        float m[GH], l[GH], o[GH][4];
+        float2 ml[GH];
+        float4 c4[GH];
+        auto request = [&](int sp) {
 #pragma unroll
-        for (int h = 0; h < GH; ++h) { c.head = head0 + h; request_partials<PB>(fp[h], a, c, lane); }
+            for (int h = 0; h < GH; ++h) {
+                const size_t i = base + (size_t)h * a.n_split_max + sp;
+                ml[h] = __ldcg(a.part_ml + i);
+                c4[h] = __ldcg(reinterpret_cast<const float4*>(a.part_o + i * HD + lane * 4));
+            }
+        };
+        if (n_sp > 0) request(0);
 #pragma unroll
-        for (int h = 0; h < GH; ++h) { c.head = head0 + h; merge_pair<PB>(fp[h], t[h], a, c, lane); }
+        for (int h = 0; h < GH; ++h) {
+            m[h] = -INFINITY; l[h] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) o[h][i] = 0.f;
+        }
+        for (int sp = 0; sp < n_sp; ++sp) {
+            float2 ml0[GH];
+            float4 c40[GH];
+#pragma unroll
+            for (int h = 0; h < GH; ++h) { ml0[h] = ml[h]; c40[h] = c4[h]; }
+            if (sp + 1 < n_sp) request(sp + 1);
+#pragma unroll
+            for (int h = 0; h < GH; ++h) {
+                const float co[4] = {c40[h].x, c40[h].y, c40[h].z, c40[h].w};
+                merge_ml(m[h], l[h], o[h], ml0[h].x, ml0[h].y, co);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < GH; ++h) {
+            c.head = head0 + h;
+            merge_ml(m[h], l[h], o[h], t[h].m, t[h].l, t[h].o);
+            store_pair(l[h], o[h], a, c, lane);
+        }
     }
     if (!waited) pdl_wait();
 }

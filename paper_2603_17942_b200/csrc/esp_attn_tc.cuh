@@ -478,6 +478,23 @@ __device__ __forceinline__ void tail_pair(TailAcc& t, const AttnArgs& a, const P
     __syncwarp();     // s_q may be rewritten by the warp's next pair
 }
 
+// The output of a pair, o / l, as bf16 and (a.out_lo) its low-order plane; a lane owns 4 of the 128 output dims.
+__device__ __forceinline__ void store_pair(float l, const float (&o)[4], const AttnArgs& a, const PairCtx& c, int lane) {
+    const float inv = 1.0f / l;
+    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out) + ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * HD + lane * 4;
+    __nv_bfloat16 oh[4], ol[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float v = __fmul_rn(o[i], inv);
+        oh[i] = __float2bfloat16_rn(v);
+        ol[i] = __float2bfloat16_rn(__fsub_rn(v, __bfloat162float(oh[i])));
+    }
+    *reinterpret_cast<uint2*>(out) = *reinterpret_cast<const uint2*>(oh);
+    if (a.out_lo)      // low-order plane for an O projection that reads the output as hi + lo
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out_lo) + ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * HD + lane * 4) =
+            *reinterpret_cast<const uint2*>(ol);
+}
+
 // The merge: bulk partials in split order, the tail last; a lane owns 4 of the 128 output dims.
 template <int PB>
 __device__ __forceinline__ void merge_pair(const FirstPartials<PB>& fp, const TailAcc& t, const AttnArgs& a, const PairCtx& c, int lane) {
@@ -510,19 +527,7 @@ __device__ __forceinline__ void merge_pair(const FirstPartials<PB>& fp, const Ta
         }
     }
     merge_ml(m, l, o, t.m, t.l, t.o);
-    const float inv = 1.0f / l;
-    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out) + ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * HD + lane * 4;
-    __nv_bfloat16 oh[4], ol[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float v = __fmul_rn(o[i], inv);
-        oh[i] = __float2bfloat16_rn(v);
-        ol[i] = __float2bfloat16_rn(__fsub_rn(v, __bfloat162float(oh[i])));
-    }
-    *reinterpret_cast<uint2*>(out) = *reinterpret_cast<const uint2*>(oh);
-    if (a.out_lo)      // low-order plane for an O projection that reads the output as hi + lo
-        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out_lo) + ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * HD + lane * 4) =
-            *reinterpret_cast<const uint2*>(ol);
+    store_pair(l, o, a, c, lane);
 }
 
 }  // namespace attn
