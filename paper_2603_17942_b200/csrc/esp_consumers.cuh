@@ -104,6 +104,73 @@ __device__ __forceinline__ void resid_norm_row(float* xr, const StreamK& sk, int
     }
 }
 
+// The same for launches of many rows (d <= 128 * NW * 4): NW warps per row, four groups per warp in registers, the pieces
+// of the four groups requested together.  Sums, products and their order are resid_norm_row's, so are the bits.
+constexpr int NORM_MANY_WARPS = 8, NORM_MANY_D = TILE_N * NORM_MANY_WARPS * 4;
+template <typename T, typename Bar>
+__device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk, int sk_row, const T* g, T* yr, T* yr_lo, int d, float eps,
+                                                    float* copy_row, float* red, int warp, int lane, Bar bar) {
+    const int ng = (d + TILE_N - 1) / TILE_N;
+    float4 x[4], acc[4];
+    int n[4], idx0[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int gi = warp + NORM_MANY_WARPS * u, j = gi * TILE_N + lane * 4;
+        x[u] = acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        n[u] = 0;
+        idx0[u] = gi;
+        if (gi < ng && j < d) {
+            x[u] = __ldcg(reinterpret_cast<const float4*>(xr + j));
+            if (sk.partials) n[u] = __ldg(&sk.table[gi].n);
+        }
+    }
+    int most = n[0] > n[1] ? n[0] : n[1];
+    most = max(most, max(n[2], n[3]));
+    const float* base = sk.partials + (size_t)sk_row * TILE_N + lane * 4;
+    const size_t piece = (size_t)sk.rows * TILE_N;
+#pragma unroll 2
+    for (int c = 0; c < most; ++c) {          // pieces in ascending order, as sk_sum4 adds them
+        float4 t[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            t[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c < n[u]) t[u] = __ldcg(reinterpret_cast<const float4*>(base + (size_t)__ldg(&sk.table[idx0[u]].idx[c]) * piece));
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { acc[u].x += t[u].x; acc[u].y += t[u].y; acc[u].z += t[u].z; acc[u].w += t[u].w; }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int gi = warp + NORM_MANY_WARPS * u, j = gi * TILE_N + lane * 4;
+        if (gi >= ng) break;
+        if (sk.partials && j < d) {
+            x[u].x = __fadd_rn(x[u].x, acc[u].x); x[u].y = __fadd_rn(x[u].y, acc[u].y);
+            x[u].z = __fadd_rn(x[u].z, acc[u].z); x[u].w = __fadd_rn(x[u].w, acc[u].w);
+            __stcg(reinterpret_cast<float4*>(xr + j), x[u]);
+        }
+        float ss = __fmaf_rn(x[u].w, x[u].w, __fmaf_rn(x[u].z, x[u].z, __fmaf_rn(x[u].y, x[u].y, __fmul_rn(x[u].x, x[u].x))));
+        ss = warp_sum(ss);
+        if (lane == 0) red[gi] = ss;
+    }
+    bar();
+    float tot = 0.f;
+    for (int gi = 0; gi < ng; ++gi) tot = __fadd_rn(tot, red[gi]);
+    const float rinv = 1.0f / sqrtf(__fadd_rn(tot / (float)d, eps));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int j = (warp + NORM_MANY_WARPS * u) * TILE_N + lane * 4;
+        if (j >= d) break;
+        const float xv[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+        T gg[4], o[4], ol[4];
+        load4(gg, g + j);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) split_bf16(__fmul_rn(__fmul_rn(xv[i], rinv), to_f32(gg[i])), o[i], ol[i]);
+        *reinterpret_cast<uint2*>(yr + j) = *reinterpret_cast<const uint2*>(o);
+        if (yr_lo) *reinterpret_cast<uint2*>(yr_lo + j) = *reinterpret_cast<const uint2*>(ol);
+        if (copy_row) *reinterpret_cast<float4*>(copy_row + j) = x[u];
+    }
+}
+
 // ------------------------------------------------------------------ QKV: (row, head) tasks, one warp each
 struct QkvArgs {
     void* q_out;              // [seq*RT + row][Hq*h] bf16
