@@ -113,28 +113,26 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
         // the smallest of the K' group maxima is the bound: K' different tokens reach it.  (The K'-th best of a single
         // tile, the bound used before, is an ordinary value, the best 9 % of the tile: hardly any tile stayed below it.)
         // The bounds are fetched once per tile, all rows at a time.  Measured, 90 probe rows of 120, vocabulary 128256,
-        // K' = 11: LM head 368 -> 240 us; 36 of 48 rows: 192 -> 178 us.
+        // K' = 11: LM head 368 -> 240 us; 36 of 48 rows: 192 -> 178 us.  The second look of a CTA's first tile: 220 -> 206 us.
         const int S = n_rows <= 80 ? 80 : RT;                             // s_aux holds at least 2 * S words
         uint32_t* s_floor = reinterpret_cast<uint32_t*>(s_aux);          // [S] bounds, [S] "this probe row has entries at or above its bound"
         uint32_t* s_need = s_floor + S;
         uint32_t* group_max = cand_floor ? cand_floor + (size_t)grow0 * KP_MAX + tile % KP : nullptr;
-        for (int r = r0 + f; r < r1; r += 128) {
-            uint32_t bound = 0u;
-            if (r >= n_nodes && cand_floor) {
-                const uint4* g = reinterpret_cast<const uint4*>(cand_floor + (size_t)(grow0 + r) * KP_MAX);
-                bound = 0xffffffffu;
+        auto fetch_bound = [&](int r) -> uint32_t {
+            const uint4* g = reinterpret_cast<const uint4*>(cand_floor + (size_t)(grow0 + r) * KP_MAX);
+            uint32_t bound = 0xffffffffu;
 #pragma unroll
-                for (int j = 0; j < KP_MAX; j += 4) {
-                    if (j >= KP) break;
-                    const uint4 w = __ldcg(g + j / 4);
-                    bound = min(bound, w.x);
-                    if (j + 1 < KP) bound = min(bound, w.y);
-                    if (j + 2 < KP) bound = min(bound, w.z);
-                    if (j + 3 < KP) bound = min(bound, w.w);
-                }
+            for (int j = 0; j < KP_MAX; j += 4) {
+                if (j >= KP) break;
+                const uint4 w = __ldcg(g + j / 4);
+                bound = min(bound, w.x);
+                if (j + 1 < KP) bound = min(bound, w.y);
+                if (j + 2 < KP) bound = min(bound, w.z);
+                if (j + 3 < KP) bound = min(bound, w.w);
             }
-            s_floor[r] = bound;
-        }
+            return bound;
+        };
+        for (int r = r0 + f; r < r1; r += 128) s_floor[r] = r >= n_nodes && cand_floor ? fetch_bound(r) : 0u;
         epi_bar(bar_id);
         // Probe rows, one thread per row (the padded row stride keeps the threads on different banks): the tile's
         // (max, sum-exp) for the row's log-sum-exp, and whether anything of the tile can still reach the row's final
@@ -148,10 +146,12 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
                 const float* row = s_acc + r * ACC_LD;
                 float tmax = -INFINITY;
                 for (int i = 0; i < n_valid; ++i) tmax = fmaxf(tmax, row[i]);
+                if (group_max) atomicMax(group_max + (size_t)r * KP_MAX, float_order_key(tmax));
                 float sum = 0.f;
                 for (int i = 0; i < n_valid; ++i) sum += expf(row[i] - tmax);
                 cand_ms[(size_t)tile * Mtot + grow0 + r] = make_float2(tmax, sum);
-                if (group_max) atomicMax(group_max + (size_t)r * KP_MAX, float_order_key(tmax));
+                // nothing was known when the tile began (every CTA's first): by now most CTAs have reported this tile's maxima
+                if (cand_floor && s_floor[r] == 0u) s_floor[r] = fetch_bound(r);
                 const bool need = float_order_key(tmax) >= s_floor[r];
                 s_need[r] = need ? 1u : 0u;
                 if (!need) {
