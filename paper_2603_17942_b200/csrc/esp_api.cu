@@ -40,7 +40,6 @@ struct Buffers {
     float* mvec;
     SeqState* states;
     int* err;
-    int32_t* out_ring;
     int32_t* prompt_dev;
     int32_t* tree_dev;
     float *rope_cos, *rope_sin;
@@ -203,7 +202,6 @@ size_t carve_all(const Dims& D, int dtype, int n_sm, char* base, Buffers* b) {
     o.mvec = c.take<float>((size_t)D.batch * D.mask_slots * D.d);
     o.states = c.take<SeqState>(D.batch);
     o.err = c.take<int>(4);
-    o.out_ring = c.take<int32_t>((size_t)(NREC + 1) * D.batch * RING);
     o.prompt_dev = c.take<int32_t>(D.cap);
     o.tree_dev = c.take<int32_t>(2 * RT);
     o.rope_cos = c.take<float>((size_t)D.cap * (D.h / 2));
@@ -282,7 +280,8 @@ struct esp_handle {
     std::vector<int> L_host, ready;
     unsigned long long issued = 0;      // decode steps enqueued on this handle
     unsigned long long consumed = 0;    // ... whose records esp_read has returned
-    int32_t* pinned = nullptr;  // [batch][RING] + 4 ints (error words)
+    int32_t* records = nullptr;      // [NREC + 1][batch][RING], host memory the tree kernel writes its records to
+    int32_t* records_dev = nullptr;  // the same as the device sees it
     float *dbg_logits = nullptr, *dbg_hidden = nullptr;
     int launches = 0, kernels_per_step = 0;
     size_t layer_kv_stride = 0;  // bytes
@@ -599,7 +598,7 @@ int tree_step(esp_handle* h, bool is_step) {
     A.kcache = h->b.kcache;
     A.vcache = h->b.vcache;
     A.err = h->b.err;
-    A.out_ring = h->b.out_ring;
+    A.out_ring = h->records_dev;
     launch_tree_step(h->dtype, A, h->stream, h->use_pdl && !h->prof);
     h->launches++;
     mark(h, KIND_SELECT);
@@ -617,13 +616,15 @@ __global__ void k_select(SeqState* st, int batch, int seq_only) {
 }
 __global__ void k_mark_ready(SeqState* st, int seq) { st[seq].ready = 1; }
 
-// Copies the records of slot `slot` (all sequences) and the error word to pinned memory; synchronises.
-int read_ring(esp_handle* h, int slot) {
-    const int n = h->D.batch * RING;
-    if (cudaMemcpyAsync(h->pinned, h->b.out_ring + (size_t)slot * n, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess) return ESP_E_CUDA;
-    if (cudaMemcpyAsync(h->pinned + n, h->b.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess) return ESP_E_CUDA;
+// Waits for everything enqueued and points at the records of slot `slot` (all sequences).  The tree kernel writes its
+// records, the device error word among them, straight to host memory: a step ends with its kernels, not with two copies
+// behind them.
+int wait_records(esp_handle* h, int slot, const int32_t** rec) {
+    *rec = h->records + (size_t)slot * h->D.batch * RING;
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return ESP_E_CUDA;
-    return h->pinned[n] ? ESP_E_DEVICE : ESP_OK;
+    for (int i = 0; i < h->D.batch; ++i)
+        if ((*rec)[i * RING + RING - 1]) return ESP_E_DEVICE;
+    return ESP_OK;
 }
 
 // A prefill that could not be enqueued: the other sequences keep their lengths; this one has to be prefilled again
@@ -690,10 +691,14 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
     h->ready.assign(D.batch, 0);
     h->layer_kv_stride = (size_t)D.batch * D.Hkv * D.cap * D.h * (model->dtype ? 2 : 4);
     if (cudaMemsetAsync(workspace, 0, need, h->stream) != cudaSuccess) { delete h; return ESP_E_CUDA; }
-    if (cudaHostAlloc(reinterpret_cast<void**>(&h->pinned), sizeof(int32_t) * (D.batch * RING + 4), cudaHostAllocDefault) != cudaSuccess) {
+    const size_t rec_bytes = sizeof(int32_t) * (NREC + 1) * (size_t)D.batch * RING;
+    if (cudaHostAlloc(reinterpret_cast<void**>(&h->records), rec_bytes, cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->records_dev), h->records, 0) != cudaSuccess) {
+        if (h->records) cudaFreeHost(h->records);
         delete h;
         return ESP_E_CUDA;
     }
+    memset(h->records, 0, rec_bytes);
     launch_rope_table(h->b.rope_cos, h->b.rope_sin, D.cap, D.h, model->rope_base, h->stream);
     if (model->dtype == 1 && attn_tc_supported(D.h, D.Hq, D.Hkv)) {
         const size_t seq_bytes = (size_t)D.Hkv * D.cap * D.h * 2;
@@ -854,12 +859,13 @@ int esp_prefill(esp_handle* h, int32_t seq, const int32_t* prompt, int32_t n_pro
     }
     k_mark_ready<<<1, 1, 0, s>>>(h->b.states, seq);
     k_select<<<1, 32, 0, s>>>(h->b.states, h->D.batch, -1);
-    int rc = read_ring(h, NREC);
+    const int32_t* rec = nullptr;
+    int rc = wait_records(h, NREC, &rec);
     h->L_host = saved;
     h->L_host[seq] = n_prompt;
     h->ready[seq] = 1;
     if (rc) return rc;
-    if (first_token_out) *first_token_out = h->pinned[seq * RING + 2];
+    if (first_token_out) *first_token_out = rec[seq * RING + 2];
     return ESP_OK;
 }
 
@@ -943,11 +949,12 @@ int esp_read(esp_handle* h, int32_t* tokens_out, int32_t* n_out) {
         if (cudaMemcpy(&e, h->b.err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return ESP_E_CUDA;
         return e ? ESP_E_DEVICE : ESP_OK;
     }
-    int rc = read_ring(h, (int)(h->consumed % NREC));
+    const int32_t* rec = nullptr;
+    int rc = wait_records(h, (int)(h->consumed % NREC), &rec);
     ++h->consumed;
     const int unread = (int)(h->issued - h->consumed);
     for (int i = 0; i < h->D.batch; ++i) {
-        const int32_t* r = h->pinned + i * RING;
+        const int32_t* r = rec + i * RING;
         if (!h->ready[i] || r[0] <= 0) { if (n_out) n_out[i] = 0; continue; }   // took no part in that step
         h->L_host[i] = r[1] + unread * (h->D.k + 1);     // steps still unread can each add at most k + 1 positions
         if (n_out) n_out[i] = r[0];
@@ -1146,7 +1153,7 @@ void esp_free(esp_handle* h) {
     attn_tc_destroy(h->p_attn_pre);
     layers_tc_destroy(h->p_layers);
     for (auto* t : h->p_attn) attn_tc_destroy(t);
-    if (h->pinned) cudaFreeHost(h->pinned);
+    if (h->records) cudaFreeHost(h->records);
     drop_graphs(h);
     for (auto e : h->ev) cudaEventDestroy(e);
     delete h;

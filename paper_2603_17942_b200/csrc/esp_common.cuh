@@ -19,7 +19,7 @@ constexpr int MAX_CAND = 4096;          // nodes Algorithm 1 may create in one s
 constexpr int PREFILL_CHUNK = ESP_PREFILL_CHUNK;   // prompt rows per prefill block
 constexpr int DCAP_STEP = 16;           // tail cap of decode steps (>= 2k)
 constexpr int DCAP_PREFILL = 16;        // tail cap of prefill blocks: their earlier rows are cache positions already
-constexpr int RING = ESP_MAX_PROBES + 4; // per-sequence result record: n_out, L, tokens
+constexpr int RING = ESP_MAX_PROBES + 4; // per-sequence result record: n_out, L, tokens, ..., device error word
 // Result records: a decode step writes every sequence's record into slot (steps so far) % NREC, so that steps
 // enqueued without a read in between keep their results; the prefill uses slot NREC.  [NREC + 1][batch][RING].
 constexpr int NREC = ESP_MAX_UNREAD_STEPS;

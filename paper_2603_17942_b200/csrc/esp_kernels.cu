@@ -1085,7 +1085,7 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
     __syncthreads();      // every thread has read the counter
     if (A.is_step && tid == 0) st->rec = rec_no + 1;
     if (!st->active) {
-        if (tid == 0) rec[0] = 0;
+        if (tid == 0) { rec[0] = 0; rec[RING - 1] = __ldcg(A.err); }
         return;
     }
     const int mode = st->mode;
@@ -1385,6 +1385,7 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
         st->mode = 0;
         st->forced = 0;
         if (Lnew + RT > D.cap) set_error(A.err, DEV_E_CAPACITY);
+        rec[RING - 1] = atomicAdd(A.err, 0);       // the error word as this step leaves it
     }
 }
 

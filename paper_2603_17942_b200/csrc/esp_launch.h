@@ -36,7 +36,7 @@ struct TreeArgs {
     void* kcache;       // [n_layers][batch][Hkv][cap][h]
     void* vcache;
     int* err;
-    int32_t* out_ring;  // [NREC + 1][batch][RING]: n_out, new L, tokens  (copied to the host by esp_read)
+    int32_t* out_ring;  // [NREC + 1][batch][RING]: n_out, new L, tokens; last word: device error.  Mapped host memory (esp_read)
     int32_t is_step;    // 1: a decode step (record slot = steps so far % NREC), 0: a prefill block (slot NREC)
 };
 
