@@ -137,10 +137,11 @@ __global__ void __launch_bounds__(256) k_rmsnorm(const SeqState* states, const f
     // let the next kernel start its own preamble (for a GEMM: the first weight tiles) while this one runs; it still
     // waits for this kernel to complete before it touches anything this kernel or its predecessors write
     if (threadIdx.x == 0) pdl_launch_dependents();
-    pdl_wait();
     int seq = blockIdx.y, r = blockIdx.x;
     const SeqState* st = states + seq;
-    if (!st->active || r >= st->n_rows) return;
+    const bool idle = !st->active || r >= st->n_rows;     // the row table was written by an earlier step
+    pdl_wait();
+    if (idle) return;
     const float* xr = x + (size_t)(seq * RT + r) * d;
     __shared__ float red[8];
     float ss = 0.f;
@@ -354,9 +355,10 @@ __global__ void __launch_bounds__(128) k_gemm_simt(SimtGemmArgs g, EpiArgs a) {
     const int n_chunks = (g.K + SIMT_KC - 1) / SIMT_KC;
     auto load_w = [&](int c) { simt_load<T, SIMT_KC, TILE_N, VEC>(s_w + (c % SIMT_STAGES) * TILE_N * LD, w, n_feat, g.K, c * SIMT_KC); };
     for (int c = 0; c < SIMT_STAGES - 1 && c < n_chunks; ++c) load_w(c);      // (they join the first group below)
-    pdl_wait();
+    // (the row table was written by an earlier step: read before the wait, like the weights)
     const SeqState* st = a.st ? a.st + seq : nullptr;
     const int n_rows = st ? (st->active ? st->n_rows : 0) : a.rows_fixed;
+    pdl_wait();
     if (r0 >= n_rows) { cp_async_wait<0>(); return; }
     const int r1 = r0 + SIMT_ROWS < n_rows ? r0 + SIMT_ROWS : n_rows;
     const T* x = reinterpret_cast<const T*>(g.x) + (size_t)(seq * RT + r0) * g.K;
@@ -406,9 +408,10 @@ __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArg
         }
     };
     for (int c = 0; c < NARROW_STAGES - 1 && c < n_chunks; ++c) load_w(c);
-    pdl_wait();
+    // (the row table was written by an earlier step: read before the wait, like the weights)
     const SeqState* st = a.st ? a.st + seq : nullptr;
     const int n_rows = st ? (st->active ? st->n_rows : 0) : a.rows_fixed;
+    pdl_wait();
     if (r0 >= n_rows) { cp_async_wait<0>(); return; }
     const int r1 = r0 + SIMT_ROWS < n_rows ? r0 + SIMT_ROWS : n_rows;
     const T* x = reinterpret_cast<const T*>(g.x) + (size_t)(seq * RT + r0) * g.K;
@@ -416,6 +419,14 @@ __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArg
     for (int c = 0; c < NARROW_STAGES - 1; ++c) {
         if (c < n_chunks) load_x(c);
         cp_async_commit();
+    }
+    float old[2] = {0.f, 0.f};        // EPI_RESID: the residual stream, on its way while the product is taken
+    if constexpr (EPI == EPI_RESID) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = r0 + warp * 2 + i;
+            if (lane < n_feat && r < r1) old[i] = a.hres[(size_t)(seq * RT + r) * a.n_out + n0 + lane];
+        }
     }
     float acc[2] = {0.f, 0.f};
     for (int c = 0; c < n_chunks; ++c) {
@@ -434,7 +445,7 @@ __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArg
             if (lane < HALF && lane < n_feat && r < r1)
                 reinterpret_cast<T*>(a.act_out)[row + n0 + lane] = from_f32<T>((gate / (1.0f + expf(-gate))) * up);
         } else if (lane < n_feat && r < r1) {
-            if constexpr (EPI == EPI_RESID) a.hres[row + n0 + lane] = a.hres[row + n0 + lane] + acc[i];
+            if constexpr (EPI == EPI_RESID) a.hres[row + n0 + lane] = old[i] + acc[i];
             else a.y_f32[row + n0 + lane] = acc[i];
         }
     }
@@ -595,7 +606,6 @@ __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_
     T* s_v = s_k + 2 * 32 * LD;                          // [2][32][LD]
     float* s_qall = reinterpret_cast<float*>(s_v + 2 * 32 * LD);
     if (threadIdx.x == 0) pdl_launch_dependents();
-    pdl_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int kvh = blockIdx.y, group = a.Hq / a.Hkv;
     const int split = blockIdx.z % n_split_launch, seq = blockIdx.z / n_split_launch;
@@ -610,13 +620,16 @@ __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_
         int n_rows, L, depth;
         unsigned long long lo, hi;
         attn_row_info(a, seq, row[w] < RT ? row[w] : 0, n_rows, L, depth, lo, hi);
-        if (row[w] < n_rows) {
-            end[w] = min(beg + a.split_len, tail_start(L + depth, a.dcap));
+        if (row[w] < n_rows) end[w] = min(beg + a.split_len, tail_start(L + depth, a.dcap));
+        cta_end = max(cta_end, end[w]);
+    }
+    pdl_wait();             // (the row table above was written by an earlier step)
+#pragma unroll
+    for (int w = 0; w < BS_PW; ++w)
+        if (end[w] > 0) {
             const T* q = reinterpret_cast<const T*>(a.q) + ((size_t)(seq * RT + row[w]) * a.Hq + kvh * group + (pair0 + w) % group) * HD;
             for (int d = lane; d < HD; d += 32) s_q[w * HD + d] = to_f32(q[d]);
         }
-        cta_end = max(cta_end, end[w]);
-    }
     __shared__ int s_end[BS_WARPS];
     if (lane == 0) s_end[warp] = cta_end;
     __syncthreads();
@@ -719,12 +732,12 @@ __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a) {
     // let the next kernel start its own preamble (for a GEMM: the first weight tiles) while this one runs; it still
     // waits for this kernel to complete before it touches anything this kernel or its predecessors write
     if (threadIdx.x == 0) pdl_launch_dependents();
-    pdl_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r = blockIdx.x * 4 + warp, head = blockIdx.y, seq = blockIdx.z;
     int n_rows, L, depth;
     unsigned long long lo, hi;
-    attn_row_info(a, seq, r < RT ? r : 0, n_rows, L, depth, lo, hi);
+    attn_row_info(a, seq, r < RT ? r : 0, n_rows, L, depth, lo, hi);      // (written by an earlier step)
+    pdl_wait();
     if (r >= n_rows) return;
     const int P = L + depth;
     const int T0 = tail_start(P, a.dcap);
@@ -837,12 +850,12 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_topk_merge(const SeqState* sta
     __shared__ float s_v[TOPK_THREADS];
     __shared__ int s_i[TOPK_THREADS];
     if (threadIdx.x == 0) pdl_launch_dependents();
-    pdl_wait();
     const int seq = blockIdx.y, r = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const SeqState* st = states + seq;
-    if (!st->active || r >= st->n_rows) return;
+    const bool idle = !st->active || r >= st->n_rows, probe = r >= st->n_nodes;     // written by an earlier step
+    pdl_wait();
+    if (idle) return;
     const int Mtot = batch * RT, grow = seq * RT + r;
-    const bool probe = r >= st->n_nodes;
     const int kp = probe ? KP : 1;
     if (stage) {
         for (int i = tid; i < n_tiles * kp; i += TOPK_THREADS) {
@@ -1075,33 +1088,34 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
     unsigned long long* c_key = reinterpret_cast<unsigned long long*>(c_rank + MAX_CAND);   // total-order keys
     unsigned long long* c_sort = c_key + MAX_CAND;                                           // scratch of the sorts
 
-    pdl_wait();
+    // Before the wait: the sequence's state and row table, which only this kernel and the set-up of a prefill block (plain
+    // launches) write.
     const Dims& D = A.D;
     const int seq = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
     SeqState* st = A.states + seq;
     // where this launch's record goes; every sequence, active or not, counts the handle's decode steps
     const unsigned long long rec_no = st->rec;
     int32_t* rec = A.out_ring + ((size_t)(A.is_step ? (int)(rec_no % NREC) : NREC) * D.batch + seq) * RING;
+    const int active = st->active, mode = st->mode, N0 = st->n_nodes, L0 = st->L;
+    for (int r = tid; r < N0 && r < RT; r += nt) {
+        s_rtok[r] = st->row_token[r];
+        s_rpar[r] = st->row_parent[r];
+        s_rdep[r] = st->row_depth[r];
+    }
+    pdl_wait();
     __syncthreads();      // every thread has read the counter
     if (A.is_step && tid == 0) st->rec = rec_no + 1;
-    if (!st->active) {
+    if (!active) {
         if (tid == 0) { rec[0] = 0; rec[RING - 1] = __ldcg(A.err); }
         return;
     }
-    const int mode = st->mode;
-    const int N0 = st->n_nodes, L0 = st->L;
     const int grow0 = seq * RT;
 
     if (mode == 1) {  // prefill chunk: every row is a prompt token and is already in place
         if (tid == 0) st->L = L0 + N0;
         return;
     }
-    for (int r = tid; r < N0; r += nt) {
-        s_rtok[r] = st->row_token[r];
-        s_rpar[r] = st->row_parent[r];
-        s_rdep[r] = st->row_depth[r];
-        s_arg[r] = A.topk[(size_t)(grow0 + r) * KP_MAX].id;
-    }
+    for (int r = tid; r < N0; r += nt) s_arg[r] = A.topk[(size_t)(grow0 + r) * KP_MAX].id;
     __syncthreads();
 
     // ---- verification (Section 2): follow the model's own next token through the tree
