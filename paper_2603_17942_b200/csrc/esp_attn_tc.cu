@@ -540,10 +540,9 @@ __global__ void __launch_bounds__(128, TAIL_FIRST ? 5 : 4) k_attn_tail_merge_tc(
 // works on GH query heads of one row together, so that every key and value it reads serves GH pairs.  What bounded
 // the warp-per-pair kernel in such launches was its key gather (32 lanes, 32 cache lines per load: 512 L1 tag cycles
 // per pair); this one is bound by its instruction count.  Measured on their own: 16 sequences x 68 rows x 32 heads 93 -> 46
-// us, 2 x 68 x 32 20.7 -> 11.6 us; one block's 68 x 32 pairs stay with the warp-per-pair kernel, which starts beside the
-// bulk kernel's CTAs, as this one's shared memory does not.
+// us, 2 x 68 x 32 20.7 -> 11.6 us; one block's 68 x 32 pairs stay with the warp-per-pair kernel (see the launch rule).
 constexpr int TM_WARPS = 8, TM_LD = HD + 8;               // slot stride in elements: 272 bytes, gathers without bank conflicts
-constexpr long long TM_MIN_PAIRS = 2 * 68 * 32 - 1;
+constexpr long long TM_MIN_PAIRS = 3000;
 constexpr int TM_DCAP = 16, TM_WINDOW = TM_DCAP + 15 + RT; // slots a CTA's rows can name, at most
 __host__ __device__ constexpr size_t tail_many_smem(int window, int gh) {
     return (size_t)2 * window * TM_LD * 2 + sizeof(float) * TM_WARPS * (gh * HD + 32 * gh);
@@ -832,8 +831,9 @@ int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_la
     // their own wait, so its start-up, and its tail where it fits beside them, overlaps them
     const bool behind_bulk = n_split_launch > 0, tail_pdl = pdl || behind_bulk;
     const int group = a.Hq / a.Hkv;
-    // More than two blocks' worth of pairs: the kernel that shares keys and values between the rows and heads of a CTA
-    // (dcap 16: a row's tail is one chunk of at most 32 keys and the window fits shared memory).
+    // From 3000 pairs on the kernel that shares keys and values between the rows and heads of a CTA (dcap 16: a row's tail is
+    // one chunk of at most 32 keys and the window fits shared memory).  Measured in a step of 120 rows x 32 heads: 1.66 ->
+    // 1.61 ms at 8 layers; at 68 x 32 the warp-per-pair kernel, part of which starts beside the bulk CTAs, is as fast.
     const long long pairs = (long long)rows_cap * a.Hq * batch;
     if (a.dcap == TM_DCAP && pairs > TM_MIN_PAIRS) {
         const int gh = group % 4 == 0 ? 4 : (group % 2 == 0 ? 2 : 1);
