@@ -75,7 +75,7 @@ int batch_bpt(const Dims& D) {
     return (D.batch + 1) / 2 * 856 <= (D.batch + 2) / 3 * 1089 ? 2 : 3;
 }
 // sequences that share the LM head's weight stream
-int lm_nq(const Dims& D) { return D.gemm_rows == 80 && D.batch > 1 ? 2 : 1; }
+int lm_nq(const Dims& D) { return D.gemm_rows != 80 ? 1 : (D.batch < 3 ? D.batch : 3); }
 // sequences one pass of a decode step covers
 int batch_pass(const Dims& D) {
     if (D.batch == 1) return 1;
@@ -207,7 +207,7 @@ size_t carve_all(const Dims& D, int dtype, int n_sm, char* base, Buffers* b) {
     o.rope_cos = c.take<float>((size_t)D.cap * (D.h / 2));
     o.rope_sin = c.take<float>((size_t)D.cap * (D.h / 2));
     {
-        // a decode step's block of gemm_rows rows (two sequences' in the LM head) or one 128-row prefill block, whichever is larger
+        // a decode step's block of gemm_rows rows (of up to three sequences in the LM head) or one 128-row prefill block, whichever is larger
         const size_t step_b = tc_gemm_partial_bytes(n_sm, lm_nq(D), D.gemm_rows);
         const size_t pre_b = tc_gemm_partial_bytes(n_sm, 1, RT);
         o.gemm_partials = c.take<char>(step_b > pre_b ? step_b : pre_b);
@@ -342,7 +342,7 @@ int run_gemm(esp_handle* h, TcGemm* plan, int epi, int n_tiles, const void* cons
 // One decoder forward over the block every active sequence of [s0, s0 + nb) has in its row table.
 // Tensor-core path (bf16; the sequences' activation blocks sit RT rows apart): the layer GEMMs stream their weights once
 // for all nb sequences (one: k_gemm_tc, several: k_gemm_wide) and store stream-K partials that the next kernel sums
-// (k_qkv_finish; k_resid_norm = residual add + RMSNorm; k_swiglu_finish); the LM head runs once per two sequences and
+// (k_qkv_finish; k_resid_norm = residual add + RMSNorm; k_swiglu_finish); the LM head runs once per up to three sequences and
 // finishes in-kernel.  CUDA-core path (fp32 models): the same layer with every epilogue fused in the GEMM.
 int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc, bool prefill) {
     const Dims& D = h->D;
@@ -484,7 +484,8 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
         const int n_tiles = (D.V + TILE_N - 1) / TILE_N;
         // tensor-core path: the sequences of a pass share the LM head's weight stream too (128-row plans: one at a time;
         // the candidate lists are shared)
-        const int share = tc ? tc_gemm_nq(wide ? h->p_lm_w : h->p_lm) : nb;
+        int share = tc ? tc_gemm_nq(wide ? h->p_lm_w : h->p_lm) : nb;
+        share = (nb + (nb + share - 1) / share - 1) / ((nb + share - 1) / share);      // as few launches, evenly filled
         for (int q = 0; q < nb; q += share) {
             const int sq = s0 + q, per = nb - q < share ? nb - q : share;
             EpiArgs a = base_epi(h, D.V, sq, per);

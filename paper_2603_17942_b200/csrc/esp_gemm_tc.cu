@@ -41,8 +41,8 @@ namespace {
 using namespace tc;
 
 // NRS = rows of a block that take part (80, or 128 for blocks of more than 80 rows); NQ = sequences one launch covers
-// (the LM head takes two): the first NRS rows of their activation blocks ([RT][K] each, consecutive) are gathered by one
-// 3-D TMA box into one B operand of NQ*NRS <= 256 rows, so the weights are streamed once for both.  (The layer GEMMs of
+// (the LM head takes up to three): the first NRS rows of their activation blocks ([RT][K] each, consecutive) are gathered by one
+// 3-D TMA box into one B operand of NQ*NRS <= 256 rows, so the weights are streamed once for all.  (The layer GEMMs of
 // several sequences: esp_gemm_wide.cu.)
 //
 // Ring depth.  The bytes in flight per SM (depth x 16 KB of weights) over the load round trip bound the stream rate,
@@ -51,15 +51,15 @@ using namespace tc;
 // x = hi + lo (hi = bf16(x), lo = bf16(x - hi), stored n_seq blocks apart in the same buffer) and takes every product
 // with both: it then sees the activation to 2^-17 instead of 2^-9, for 10 KB more shared memory per stage.
 __host__ __device__ constexpr int stages_of(int epi, int nq, int nrs, int pl = 1) {
-    return pl == 2 ? (nrs == 80 ? 6 : 4) : (nrs == 80 ? (nq == 2 ? 5 : 6) : 4);
+    return pl == 2 ? (nrs == 80 ? 6 : 4) : (nrs == 80 ? (nq == 3 ? 4 : (nq == 2 ? 5 : 6)) : 4);
 }
 __host__ __device__ constexpr int b_bytes_of(int nq, int nrs) { return nq * nrs * BK * 2; }   // 10240 per 80-row sequence and plane
 __host__ __device__ constexpr int stage_bytes_of(int nq, int nrs, int pl = 1) { return A_BYTES + pl * b_bytes_of(nq, nrs); }
 // two accumulator buffers in tensor memory: 128 columns each for up to 128 rows, 256 each beyond
 __host__ __device__ constexpr int acc_cols_of(int nr) { return nr <= 128 ? 128 : 256; }
 constexpr int NUM_THREADS = 192;
-constexpr int MAX_NQ = 2;
-__host__ __device__ constexpr int max_nq_of(int nrs, int pl) { return pl == 1 && nrs == 80 ? 2 : 1; }
+constexpr int MAX_NQ = 3;
+__host__ __device__ constexpr int max_nq_of(int nrs, int pl) { return pl == 1 && nrs == 80 ? MAX_NQ : 1; }
 
 struct TcParams {
     CUtensorMap map_a[3];
@@ -598,6 +598,7 @@ int tc_gemm_launch(const TcGemm* g, const EpiArgs& a, cudaStream_t s, bool pdl, 
     else if (p.epi == EPI_STORE_F32) ESP_TC_CASE(EPI_STORE_F32, 1, RT, 1)
     else if (p.epi == EPI_LOGITS && !wide && nq == 1) ESP_TC_CASE(EPI_LOGITS, 1, 80, 1)
     else if (p.epi == EPI_LOGITS && !wide && nq == 2) ESP_TC_CASE(EPI_LOGITS, 2, 80, 1)
+    else if (p.epi == EPI_LOGITS && !wide && nq == 3) ESP_TC_CASE(EPI_LOGITS, 3, 80, 1)
     else if (p.epi == EPI_LOGITS) ESP_TC_CASE(EPI_LOGITS, 1, RT, 1)
     else return ESP_E_ARG;
 #undef ESP_TC_CASE

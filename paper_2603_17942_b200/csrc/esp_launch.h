@@ -112,8 +112,8 @@ int attn_tc_run(const void* q, const void* kcache, const void* vcache, int batch
 struct TcGemm;
 // epi selects the tile -> weight-row mapping and the fused epilogue; with defer the kernel only stores partials
 // (EPI_PARTIAL) and the caller runs the matching consumer kernel.  x: activations [x_seqs][RT][K]; nrs = rows of a
-// block that take part (80, or RT for blocks of more than 80 rows); an 80-row EPI_LOGITS plan may cover nq_max = 2
-// sequences per launch, so that the weights are streamed once for both.  Deferred plans have planes = 2: x holds the
+// block that take part (80, or RT for blocks of more than 80 rows); an 80-row EPI_LOGITS plan may cover nq_max <= 3
+// sequences per launch, so that the weights are streamed once for them.  Deferred plans have planes = 2: x holds the
 // activations as hi + lo bf16 pairs, [2][x_seqs][RT][K], and every product is taken with both
 int tc_gemm_create(TcGemm** out, int epi, bool defer, const void* const w[3], const int32_t rows_w[3], int K, const void* x,
                    int x_seqs, int nrs, int nq_max, void* partials, size_t partial_bytes, int* counters, int n_sm, int* err, TileSrc* table_dev,
