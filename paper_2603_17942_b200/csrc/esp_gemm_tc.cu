@@ -493,6 +493,9 @@ int tc_gemm_create(TcGemm** out, int epi, bool defer, const void* const w[3], co
     p.KB = (K + BK - 1) / BK;
     const long long U = (long long)p.n_tiles * p.KB;
     p.grid = (int)(U < n_sm ? U : n_sm);
+    // A fused epilogue over a short k-range: a CTA per tile rather than tiles in pieces.  Up to 16 k-blocks pass faster than
+    // a tile's pieces meet through memory (stores, a counter, loads by the last one).
+    if (!defer && p.n_tiles <= n_sm && p.KB <= 16) p.grid = p.n_tiles;
     if (p.n_tiles > tc_gemm_counter_ints() || tc_gemm_partial_bytes(p.grid, nq_max, nrs) > partial_bytes) { delete g; return -1; }
     // fused epilogues store only the head and tail pieces of a range (2 slots); partial-only output stores every
     // piece, one slot per tile the range touches

@@ -1118,48 +1118,55 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
     for (int r = tid; r < N0; r += nt) s_arg[r] = A.topk[(size_t)(grow0 + r) * KP_MAX].id;
     __syncthreads();
 
-    // ---- verification (Section 2): follow the model's own next token through the tree
-    if (tid == 0) {
+    // ---- verification (Section 2): follow the model's own next token through the tree.  One warp walks; its lanes look for
+    // the child (one thread looking through the rows took 5000 cycles for a 32-node tree).
+    if (tid < 32) {
         int a = 0, cur, n_emit = 0;
-        s_abort = 0;
         if (mode == 2) {
             cur = N0 - 1;  // last prompt token; nothing to verify, its argmax is the first generated token
-            s_path[0] = cur;
-            s_out[n_emit++] = s_arg[cur];
-            s_ustar = cur;
-            s_delta = 0;
+            if (tid == 0) { s_path[0] = cur; s_out[0] = s_arg[cur]; s_ustar = cur; s_delta = 0; }
+            n_emit = 1;
         } else {
             cur = 0;
-            s_path[0] = 0;
+            if (tid == 0) s_path[0] = 0;
             for (;;) {
-                int y = s_arg[cur];
-                s_out[n_emit++] = y;
-                int nxt = -1;
-                for (int c = cur + 1; c < N0; ++c)
-                    if (s_rpar[c] == cur && s_rtok[c] == y) { nxt = c; break; }
-                if (nxt < 0 || n_emit > PROBES_MAX) break;
-                cur = nxt;
-                s_path[++a] = cur;
+                const int y = s_arg[cur];
+                if (tid == 0) s_out[n_emit] = y;
+                ++n_emit;
+                unsigned nxt = 0xffffffffu;               // the first row below cur with parent cur and token y
+                for (int c = cur + 1 + tid; c < N0; c += 32)
+                    if (s_rpar[c] == cur && s_rtok[c] == y) { nxt = (unsigned)c; break; }
+                nxt = __reduce_min_sync(0xffffffffu, nxt);
+                if (nxt == 0xffffffffu || n_emit > PROBES_MAX) break;
+                cur = (int)nxt;
+                ++a;
+                if (tid == 0) s_path[a] = cur;
             }
-            // deepest anchored node on the accepted path
-            int nA = D.k > 0 ? (D.n_anchor == 0 ? N0 : min(D.n_anchor, N0)) : 0;
-            int us = 0;
-            for (int j = 0; j <= a; ++j) if (s_path[j] < nA) us = s_path[j];
-            s_ustar = us;
-            s_delta = a - s_rdep[us];
         }
-        s_na = a;
-        st->n_out = n_emit;
-        for (int j = 0; j < n_emit; ++j) st->out_tokens[j] = s_out[j];
-        rec[0] = n_emit;
-        rec[1] = mode == 2 ? L0 + N0 : L0 + a + 1;
-        for (int j = 0; j < n_emit; ++j) rec[2 + j] = s_out[j];
-        if (mode == 0) {
-            const int rows = st->n_rows;
-            st->rows_hist[rows <= 16 ? 0 : (rows <= 32 ? 1 : (rows <= 64 ? 2 : 3))] += 1;
-            st->steps += 1;
-            st->emitted += n_emit;
-            st->accept_hist[a < PROBES_MAX ? a : PROBES_MAX] += 1;
+        __syncwarp();
+        if (tid == 0) {
+            s_abort = 0;
+            if (mode != 2) {
+                // deepest anchored node on the accepted path
+                int nA = D.k > 0 ? (D.n_anchor == 0 ? N0 : min(D.n_anchor, N0)) : 0;
+                int us = 0;
+                for (int q = 0; q <= a; ++q) if (s_path[q] < nA) us = s_path[q];
+                s_ustar = us;
+                s_delta = a - s_rdep[us];
+            }
+            s_na = a;
+            st->n_out = n_emit;
+            for (int q = 0; q < n_emit; ++q) st->out_tokens[q] = s_out[q];
+            rec[0] = n_emit;
+            rec[1] = mode == 2 ? L0 + N0 : L0 + a + 1;
+            for (int q = 0; q < n_emit; ++q) rec[2 + q] = s_out[q];
+            if (mode == 0) {
+                const int rows = st->n_rows;
+                st->rows_hist[rows <= 16 ? 0 : (rows <= 32 ? 1 : (rows <= 64 ? 2 : 3))] += 1;
+                st->steps += 1;
+                st->emitted += n_emit;
+                st->accept_hist[a < PROBES_MAX ? a : PROBES_MAX] += 1;
+            }
         }
     }
     __syncthreads();
