@@ -16,9 +16,9 @@
 //   S = Q K^T   tcgen05.mma, Q (128 pairs x 128 dims) and the K chunk both
 //               K-major in shared memory, S (128 x 128 fp32) in tensor memory;
 //   softmax     256 threads, two per pair (= tensor-memory lane): mask by the
-//               row's T0, running max / sum in the log2 domain, P as bf16 into
-//               shared memory in the A-operand layout;
-//   O += P V    tcgen05.mma with V as the MN-major B operand (the cache keeps
+//               row's T0, running max / sum in the log2 domain, P as bf16 back
+//               into tensor memory, over the scores;
+//   O += P V    tcgen05.mma with P as the tensor-memory A operand and V as the MN-major B operand (the cache keeps
 //               values as [key][dim]); O (128 x 128 fp32) stays in tensor
 //               memory; the softmax reference follows the running max lazily
 //               (it moves, and O is rescaled, only after a growth of 2^8).
@@ -41,7 +41,7 @@ using namespace tc;
 using namespace attn;
 
 constexpr int STG_BYTES = 4 * 32 * 128;     // output staging: 32 rows x 128 bytes for each of the 4 output warps
-constexpr int OFF_STG = OFF_P + P_BYTES, OFF_BAR = OFF_STG + STG_BYTES;
+constexpr int OFF_STG = ITEM_BYTES, OFF_BAR = OFF_STG + STG_BYTES;
 constexpr size_t SMEM_BYTES = 1024 + OFF_BAR + 256;
 constexpr int MAX_T0_ENTRIES = 256;       // sequences x row tiles one launch may cover
 constexpr int NUM_THREADS = 448;           // producer warp, MMA warp, 8 softmax warps, 4 output warps
@@ -224,7 +224,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *s_tmem;
     unsigned char* sQ = smem + OFF_Q;
-    unsigned char* sP = smem + OFF_P;
 
     // Items are dealt round-robin; every role walks the same list and skips the same empty items, so the
     // per-chunk and per-item counters below advance identically in all of them.
@@ -328,7 +327,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
         if (lane == 0) {
             bool ok = true;
             uint32_t gc = 0, n_it = 0;
-            const uint32_t q_addr = smem_u32(sQ), p_addr = smem_u32(sP);
+            const uint32_t q_addr = smem_u32(sQ);
             for (int idx = blockIdx.x; idx < n_items && ok; idx += gridDim.x) {
                 Item it;
                 if (!get_item(idx, it)) continue;
@@ -363,10 +362,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
                     const uint32_t v_addr = smem_u32(smem + OFF_KV + (g & 1) * KV_STAGE + K_BYTES);
 #pragma unroll
                     for (int kk = 0; kk < CK / 16; ++kk) {
-                        const uint32_t p_off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;     // P: K-major over keys
                         const uint32_t v_off = kk * 16 * 128;                              // V: 16 key rows of 128 bytes further
-                        umma(tmem_o, smem_desc(p_addr + p_off, 16), smem_desc(v_addr + v_off, HALF_BYTES), IDESC_PV,
-                             (c > 0 || kk > 0) ? 1u : 0u);
+                        umma_ta(tmem_o, tmem_base + (g & 1) * 128 + kk * 8, smem_desc(v_addr + v_off, HALF_BYTES), IDESC_PV,
+                                (c > 0 || kk > 0) ? 1u : 0u);
                     }
                     umma_commit(pv_done);
                     umma_commit(&v_empty[g & 1]);
@@ -409,7 +407,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 ok = softmax_chunk(lane_addr + (g & 1) * 128, o_addr, it.beg + c * CK + hf * 64, T0row, a.scale_log2, m_run, l_run,
                                    &s_xchg[xc & 1][0], xchg + q4, xc & 1, g > 0, pv_done, (g - 1) & 1, c > 0,
-                                   sP + hf * HALF_BYTES + pair * 128, pair, hf, p_ready, s_abort);
+                                   pair, hf, p_ready, s_abort);
                 ++xc;
             }
             if (!ok) break;

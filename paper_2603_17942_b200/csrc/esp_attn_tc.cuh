@@ -16,11 +16,11 @@ constexpr int HD = 128;
 constexpr int CK = 128;                   // keys per chunk
 constexpr int MP = 128;                   // (row, head) pairs per CTA
 constexpr int HALF_BYTES = 128 * 128;     // one 128-row x 64-element (128-byte) swizzled tile
-constexpr int Q_BYTES = 2 * HALF_BYTES, K_BYTES = 2 * HALF_BYTES, V_BYTES = 2 * HALF_BYTES, P_BYTES = 2 * HALF_BYTES;
+constexpr int Q_BYTES = 2 * HALF_BYTES, K_BYTES = 2 * HALF_BYTES, V_BYTES = 2 * HALF_BYTES;
 constexpr int KV_STAGE = K_BYTES + V_BYTES;
-constexpr int OFF_Q = 0, OFF_KV = Q_BYTES, OFF_P = OFF_KV + 2 * KV_STAGE;
-constexpr int ITEM_BYTES = OFF_P + P_BYTES;   // shared memory one item needs: Q, two K/V stages, P
-constexpr int TMEM_COLS = 512;            // S0 at 0, S1 at 128, O0 at 256, O1 at 384
+constexpr int OFF_Q = 0, OFF_KV = Q_BYTES;
+constexpr int ITEM_BYTES = OFF_KV + 2 * KV_STAGE;   // shared memory one item needs: Q, two K/V stages
+constexpr int TMEM_COLS = 512;            // S0 at 0, S1 at 128, O0 at 256, O1 at 384; P of a chunk in the first 64 columns of its S
 
 __device__ __forceinline__ int tail_start_tc(int P, int dcap) {
     int t = P - dcap;
@@ -54,13 +54,15 @@ __device__ __forceinline__ float ex2_approx(float x) {
 
 // ---- one 128-key chunk of the online softmax, for one thread = one half (64 keys) of one pair's row.
 // S (raw scores) is read from tensor memory; keys at or beyond T0row are masked; the two threads of a pair
-// exchange their maxima through `xch` ([2 * MP] floats); P goes to shared memory as bf16 in the A-operand
-// layout; O is rescaled in tensor memory when the running maximum moved.  Scores enter the exponent as
+// exchange their maxima through `xch` ([2 * MP] floats); P goes back to tensor memory as bf16 pairs, over the scores it
+// came from (the A operand of P V; S of this chunk is in both threads' registers before the exchange ends), 32 columns
+// per half (P through shared memory took a proxy fence and 16 KB of stores per tile and chunk: operator at 16 x 4k 203 us
+// against 189 now, batch 1 38.9 against 36.6); O is rescaled in tensor memory when the running maximum moved.  Scores enter the exponent as
 // fma(s, scale, -m): one rounding, spelled out so that every kernel that inlines this rounds alike.
 // All 32 lanes of a warp call this together (the tensor-memory accesses are warp-wide); false = a wait ran out.
 __device__ __forceinline__ bool softmax_chunk(uint32_t s_addr, uint32_t o_addr, int cbase, int T0row, float scale_log2, float& m_run,
                                               float& l_run, float* xch, uint64_t* xchg, uint32_t xchg_parity, bool wait_pv,
-                                              uint64_t* pv_done, uint32_t pv_parity, bool rescale, unsigned char* prow, int pair,
+                                              uint64_t* pv_done, uint32_t pv_parity, bool rescale, int pair,
                                               int hf, uint64_t* p_ready, volatile int* s_abort) {
     uint32_t sv[64];
     tmem_ld64(s_addr, sv);
@@ -95,8 +97,7 @@ __device__ __forceinline__ bool softmax_chunk(uint32_t s_addr, uint32_t o_addr, 
     const float m_new = (m_run == -INFINITY || __fsub_rn(m_max, m_run) > 8.f) ? m_max : m_run;
     const float m_use = m_new == -INFINITY ? 0.f : m_new;
     const float alpha = exp2f(__fsub_rn(m_run, m_use));
-    // probabilities and their sum (key order), packed as bf16 pairs in registers: the P V of the previous chunk may
-    // still be reading P from shared memory, and this is the long part of the chunk
+    // probabilities and their sum (key order), packed as bf16 pairs
     float csum = 0.f;
     const float neg_m = -m_use;
     uint32_t pk[32];
@@ -112,14 +113,10 @@ __device__ __forceinline__ bool softmax_chunk(uint32_t s_addr, uint32_t o_addr, 
     // (the values are pinned here: without it the compiler is free to sink the arithmetic behind the wait)
 #pragma unroll
     for (int i = 0; i < 32; ++i) asm volatile("" : "+r"(pk[i]));
-    // P of the previous chunk must have been consumed before it is overwritten, and O must be final
-    // before it is rescaled
+    // O must be final before it is rescaled (and no warp may signal this chunk's P before the previous chunk's was taken)
     if (wait_pv && !__all_sync(0xffffffffu, mbar_wait(pv_done, pv_parity, s_abort))) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // P as bf16 in the A-operand layout (this half = one swizzled tile)
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        *reinterpret_cast<uint4*>(prow + ((j ^ (pair & 7)) << 4)) = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+    tmem_st32(s_addr - hf * 32, pk);      // s_addr: column 64 * hf of S
     if (rescale) {
         // O <- alpha * O (in tensor memory), this thread's 64 of the 128 columns
         if (__any_sync(0xffffffffu, alpha != 1.0f)) {   // warp-uniform: skip when no lane's maximum moved
@@ -130,12 +127,11 @@ __device__ __forceinline__ bool softmax_chunk(uint32_t s_addr, uint32_t o_addr, 
                 for (int i = 0; i < 32; ++i) sv[blk * 32 + i] = __float_as_uint(__fmul_rn(__uint_as_float(sv[blk * 32 + i]), alpha));
                 tmem_st32(o_addr + blk * 32, *reinterpret_cast<const uint32_t(*)[32]>(&sv[blk * 32]));
             }
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         }
     }
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     l_run = __fmaf_rn(l_run, alpha, csum);     // this half's share of the row sum
     m_run = m_new;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // P: generic-proxy writes -> tensor-core reads
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(p_ready);      // one arrival per softmax warp
@@ -191,7 +187,6 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
                                                 uint32_t tmem_base, int warp, int lane) {
     unsigned char* smem = sm.buf;
     unsigned char* sQ = smem + OFF_Q;
-    unsigned char* sP = smem + OFF_P;
     volatile int* s_abort = sm.s_abort;
     if (warp == 0) {
         // ---------------- TMA producer
@@ -233,7 +228,7 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
         // ---------------- MMA issuer
         if (lane == 0) {
             bool ok = true;
-            const uint32_t q_addr = smem_u32(sQ), p_addr = smem_u32(sP);
+            const uint32_t q_addr = smem_u32(sQ);
             auto issue_qk = [&](int c) {
                 const uint32_t k_addr = smem_u32(smem + OFF_KV + (c & 1) * KV_STAGE);
                 const uint32_t tmem_s = tmem_base + (c & 1) * 128;
@@ -261,10 +256,9 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
                 const uint32_t v_addr = smem_u32(smem + OFF_KV + (c & 1) * KV_STAGE + K_BYTES);
 #pragma unroll
                 for (int kk = 0; kk < CK / 16; ++kk) {
-                    const uint32_t p_off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;     // P: K-major over keys
                     const uint32_t v_off = kk * 16 * 128;                              // V: 16 key rows of 128 bytes further
-                    umma(tmem_base + 256, smem_desc(p_addr + p_off, 16), smem_desc(v_addr + v_off, HALF_BYTES), IDESC_PV,
-                         (c > 0 || kk > 0) ? 1u : 0u);
+                    umma_ta(tmem_base + 256, tmem_base + (c & 1) * 128 + kk * 8, smem_desc(v_addr + v_off, HALF_BYTES), IDESC_PV,
+                            (c > 0 || kk > 0) ? 1u : 0u);
                 }
                 umma_commit(sm.pv_done);
                 umma_commit(&sm.v_empty[c & 1]);
@@ -300,7 +294,7 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             ok = softmax_chunk(lane_addr + (c & 1) * 128, lane_addr + 256, it.beg + c * CK + hf * 64, T0row, a.scale_log2, m_run, l_run,
                                sm.s_xchg + (c & 1) * 2 * MP, sm.xchg + q4, c & 1, c > 0, sm.pv_done, (c - 1) & 1, c > 0,
-                               sP + hf * HALF_BYTES + pair * 128, pair, hf, sm.p_ready, s_abort);
+                               pair, hf, sm.p_ready, s_abort);
         }
         if (ok && !__all_sync(0xffffffffu, mbar_wait(sm.pv_done, (it.n_chunks - 1) & 1, s_abort))) ok = false;
         float* xl = sm.s_xchg + (it.n_chunks & 1) * 2 * MP;
