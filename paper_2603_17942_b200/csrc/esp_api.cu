@@ -67,19 +67,27 @@ constexpr int SK_TABLE_TILES = 2048;
 constexpr int ACT_PLANES = 2;
 
 
-// Decode steps of several sequences: how many blocks a row tile of the wide GEMMs holds.  Blocks of up to 80 rows: two or
-// three, whichever is the cheaper for the batch -- per weight unit and tile the kernel takes 856 (two) or 1089 cycles
-// (three) of shared-memory time, operands and fill --; larger blocks: two.
-int batch_bpt(const Dims& D) {
-    if (D.gemm_rows != 80) return 2;
-    return (D.batch + 1) / 2 * 856 <= (D.batch + 2) / 3 * 1089 ? 2 : 3;
+// Decode steps of several sequences: how many blocks a row tile of the wide GEMMs holds, two or three, whichever is the
+// cheaper for the batch at 80 rows a block -- per weight unit and tile the kernel takes 856 (two) or 1089 cycles (three) of
+// shared-memory time, operands and fill.  The split of k follows from this and not from the rows of a block, so that a
+// row of a handle has the bits it has in any other handle of its max_batch, the greedy one for instance.  A block is
+// carried as 32, 64 or 80 rows, as many as its trees need; more than 80 rows leave room for two blocks per tile.
+// Measured against blocks of 80 rows for every smaller tree (8B shapes, four layers and the LM head, L 300, us per step; 2 /
+// 3 / 8 sequences): one row 724 / 881 / 2200 -> 653 / 696 / 1689, 20 rows 849 / 1083 / 2513 -> 773 / 844 / 2045, 52 rows 888 /
+// 1171 / 2953 -> 879 / 1099 / 2694.  Trees of 100 rows pay for the common split with a second turn where three blocks would
+// share a tile: 3 / 5 / 8 sequences 2246 / 3488 / 5046 -> 2502 / 3870 / 5673 (one pass of the small-M kernel each: 2633 /
+// 4419 / 6972).
+void choose_batch_tile(Dims* D, int rows) {
+    D->batch_split_bpt = (D->batch + 1) / 2 * 856 <= (D->batch + 2) / 3 * 1089 ? 2 : 3;
+    D->batch_rows = rows <= 32 ? 32 : (rows <= 64 ? 64 : (rows <= 80 ? 80 : RT));
+    D->batch_bpt = rows <= 80 ? D->batch_split_bpt : 2;
 }
 // sequences that share the LM head's weight stream
 int lm_nq(const Dims& D) { return D.gemm_rows != 80 ? 1 : (D.batch < 3 ? D.batch : 3); }
 // sequences one pass of a decode step covers
 int batch_pass(const Dims& D) {
     if (D.batch == 1) return 1;
-    const int most = WIDE_MAX_RT * batch_bpt(D);
+    const int most = WIDE_MAX_RT * D.batch_split_bpt;
     return D.batch < most ? D.batch : most;
 }
 
@@ -149,7 +157,6 @@ int check_cfg(const esp_model_cfg* m, const esp_spec_cfg* s, Dims* D) {
         // wide prefill passes: bf16 models on the tensor-core attention whose longest prompt has two full blocks before its last
         const int full = m->dtype == 1 && attn_tc_supported(m->head_dim, m->n_q_heads, m->n_kv_heads) ? (m->max_seq_len - 1) / PREFILL_CHUNK : 0;
         D->pre_blocks = full < 2 ? 0 : (full < WIDE_MAX_BLOCKS ? full : WIDE_MAX_BLOCKS);
-        D->blocks = D->batch > D->pre_blocks ? D->batch : D->pre_blocks;
         const int S = attn_split_len(m->max_seq_len, m->max_batch, m->n_kv_heads);
         D->split_len = S;
         D->n_split_max = (m->max_seq_len + RT + S - 1) / S + 1;   // a prefill block's own rows count as cache positions
@@ -161,6 +168,9 @@ int check_cfg(const esp_model_cfg* m, const esp_spec_cfg* s, Dims* D) {
         D->ema_per_token = s->ema_per_token; D->lambda = s->lambda;
         // rows of a block the tensor-core GEMMs carry: 80 covers every tree of at most 80 rows and the prefill blocks
         D->gemm_rows = spec_rows(*s) <= 80 ? 80 : RT;
+        choose_batch_tile(D, spec_rows(*s));
+        D->blocks = D->batch > D->pre_blocks ? D->batch : D->pre_blocks;
+        if (D->batch > 1 && D->blocks < D->batch_bpt) D->blocks = D->batch_bpt;
         D->inv_temp = s->temperature > 0.f ? 1.0f / s->temperature : 0.f;
         D->seed_lo = s->seed_lo; D->seed_hi = s->seed_hi;
     }
@@ -219,13 +229,13 @@ size_t carve_all(const Dims& D, int dtype, int n_sm, char* base, Buffers* b) {
         const int tiles[4] = {(D.Hq + 2 * D.Hkv) * D.h / TILE_N, (D.d + TILE_N - 1) / TILE_N, (D.F + 63) / 64, (D.d + TILE_N - 1) / TILE_N};
         const int K[4] = {D.d, D.Hq * D.h, D.d, D.F};
         for (int i = 0; i < 4; ++i)
-            for (int rt = 1; rt <= (D.pre_blocks + 1) / 2; ++rt) {
-                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, rt, 2 * PREFILL_CHUNK);
+            for (int nb = 2; nb <= D.pre_blocks; ++nb) {
+                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, nb, PREFILL_CHUNK, 2, 2);
                 o.wide_bytes = n > o.wide_bytes ? n : o.wide_bytes;
             }
         for (int i = 0; i < 4 && batched; ++i)
-            for (int rt = 1; rt <= (batch_pass(D) + batch_bpt(D) - 1) / batch_bpt(D); ++rt) {
-                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, rt, batch_bpt(D) * D.gemm_rows);
+            for (int nb = 1; nb <= batch_pass(D); ++nb) {
+                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, nb, D.batch_rows, D.batch_bpt, D.batch_split_bpt);
                 o.wide_bytes = n > o.wide_bytes ? n : o.wide_bytes;
             }
     }
@@ -777,9 +787,8 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
         const int K[4] = {D.d, dq, D.d, D.F};
         if (D.batch > 1 && n_sm >= 148) {
             TileSrc* tables = h->b.wide_tables + (D.pre_blocks ? (size_t)4 * WIDE_MAX_RT * SK_TABLE_TILES : 0);
-            const int bpt = batch_bpt(D);
             for (int i = 0; i < 4; ++i)
-                if (wide_gemm_create(&h->p_batch[i], tc_gemm_tiles(narrow[i]), K[i], x[i], D.blocks, nrs, bpt, (batch_pass(D) + bpt - 1) / bpt,
+                if (wide_gemm_create(&h->p_batch[i], tc_gemm_tiles(narrow[i]), K[i], x[i], D.blocks, D.batch_rows, D.batch_bpt, D.batch_split_bpt, batch_pass(D),
                                      h->b.wide_partials, h->b.wide_bytes, tables + (size_t)i * WIDE_MAX_RT * SK_TABLE_TILES, h->b.err, h->stream)) {
                     esp_free(h);
                     return ESP_E_CUDA;
@@ -788,7 +797,7 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
         if (D.pre_blocks && n_sm >= 148) {
             bool have = attn_tc_create(&h->p_attn_pre, h->b.qbuf, h->b.kcache, h->b.vcache, D.pre_blocks, D.Hq, D.Hkv, D.cap) == 0;
             for (int i = 0; i < 4 && have; ++i)
-                have = !wide_gemm_create(&h->p_wide[i], tc_gemm_tiles(narrow[i]), K[i], x[i], D.blocks, PREFILL_CHUNK, 2, (D.pre_blocks + 1) / 2, h->b.wide_partials,
+                have = !wide_gemm_create(&h->p_wide[i], tc_gemm_tiles(narrow[i]), K[i], x[i], D.blocks, PREFILL_CHUNK, 2, 2, D.pre_blocks, h->b.wide_partials,
                                          h->b.wide_bytes, h->b.wide_tables + (size_t)i * WIDE_MAX_RT * SK_TABLE_TILES, h->b.err, h->stream);
             if (!have) { esp_free(h); return ESP_E_CUDA; }
         }

@@ -68,7 +68,7 @@ struct Dims {
     int32_t cap;        // KV positions allocated per sequence (max_seq_len + RT)
     int32_t batch;
     int32_t pre_blocks; // full prefill blocks one pass of the wide GEMMs covers (0: one block per pass)
-    int32_t blocks;     // row blocks the activation buffers hold: max(batch, pre_blocks)
+    int32_t blocks;     // row blocks the activation buffers hold: max(batch, pre_blocks), a row tile at least
     int32_t split_len;  // attention split length in positions (multiple of 64)
     int32_t n_split_max;
     float rms_eps;
@@ -78,6 +78,9 @@ struct Dims {
     int32_t mask_slots;             // mask vectors per sequence: max(k, 1)
     float lambda;
     int32_t gemm_rows;              // rows of a block the tensor-core GEMMs carry: 80, or RT for larger blocks
+    // steps of several sequences: rows of a block the wide GEMMs carry, blocks per row tile, blocks per row tile of the split
+    // of k (a function of max_batch alone)
+    int32_t batch_rows, batch_bpt, batch_split_bpt;
     float inv_temp;                 // 1 / temperature, 0 = greedy matching
     uint32_t seed_lo, seed_hi;      // key of the sampling noise
 };

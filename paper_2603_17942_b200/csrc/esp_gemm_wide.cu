@@ -9,11 +9,14 @@
 // small-M kernel has it, would need 79.  The tile is the whole tensor memory (two accumulators of up to 240 of 256
 // columns), so there is one in flight per CTA.
 //
-// Work split: a row tile is BPT blocks of WB rows (one TMA box of BPT x WB rows per plane).  The CTAs form groups of
-// one CTA per row tile; a group owns a contiguous range of the (256-feature tile, k-block) units, stream-K style, and
-// its CTAs walk it in step, so that a weight unit is read from HBM once and from L2 by the other row tiles.  Every
-// piece is stored as an fp32 partial; the kernel that consumes the result sums a tile's pieces in group order, as it
-// does for the small-M kernel (StreamK with one row space for all row tiles).
+// Work split: a row tile is BPT blocks of WB rows (one TMA box of BPT x WB rows per plane).  The (256-feature tile,
+// k-block) units are cut into contiguous ranges, stream-K style; an item is a range x a row tile, the items of a range lie
+// next to each other in the grid, and their CTAs walk it in step, so that a weight unit is read from HBM once and from L2
+// by the other row tiles.  Every piece is stored as an fp32 partial; the kernel that consumes the result sums a tile's
+// pieces in range order, as it does for the small-M kernel (StreamK with one row space for all row tiles).
+// The number of ranges (WIDE_SM over row tiles of split_bpt blocks) depends on the number of blocks and not on the rows of
+// a block: a row's sums have the same order in a step of 128-row trees and in a greedy step.  With BPT = split_bpt every
+// CTA has one item; 128-row blocks of which two make a row tile where smaller ones would be three take two turns.
 //
 // Ring: seven slots of 32 KB, filled in the order [two weight units | hi rows | lo rows] per k-block.  The hi slot is
 // released half a k-block before the other two.  Roles: warp 0 producer, warp 1 MMA issuer, warps 2-9 epilogue (four
@@ -46,7 +49,7 @@ struct WideParams {
     CUtensorMap map_b;          // activations [2 planes x x_blocks][RT][K], box 64 x WB x BPT
     const unsigned char* w;     // packed weight units [n_tiles][KB][A_BYTES]
     const SeqState* st;         // one state per block
-    float* partials;            // [group][slot][2 halves][n_rt * WR rows][128 features]
+    float* partials;            // [range][slot][2 halves][n_rt * WR rows][128 features]
     int* err;
     int32_t n_tiles, n_ft, KB, n_groups, n_rt, slots, plane_blocks, n_blocks;
 };
@@ -55,6 +58,7 @@ template <int WB, int BPT>
 __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_constant__ WideParams p) {
     constexpr int WR = WB * BPT;               // rows of a row tile = MMA N
     constexpr int X_BYTES = WR * BK * 2;
+    constexpr bool TURNS = WB == RT;           // may have more items than CTAs
     static_assert(WR % 16 == 0 && WR <= 256 && X_BYTES <= SLOT_BYTES && WB % 8 == 0 && WB <= RT, "row tile");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -65,10 +69,18 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(tempty + 1);
     volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rt = blockIdx.x % p.n_rt, grp = blockIdx.x / p.n_rt;
     const long long U = (long long)p.n_ft * p.KB;
-    const int u0 = (int)sk_begin(grp, U, p.n_groups), u1 = (int)sk_begin(grp + 1, U, p.n_groups);
-    const int n_units = u1 - u0;
+    const int n_work = p.n_groups * p.n_rt;        // items: range w / n_rt, row tile w % n_rt
+    int rt = blockIdx.x % p.n_rt, grp = blockIdx.x / p.n_rt;
+    int u0 = (int)sk_begin(grp, U, p.n_groups), u1 = (int)sk_begin(grp + 1, U, p.n_groups);
+    // the CTA's next item, if it has one
+    auto next_item = [&](int& w) {
+        w += gridDim.x;
+        if (!TURNS || w >= n_work) return false;
+        rt = w % p.n_rt; grp = w / p.n_rt;
+        u0 = (int)sk_begin(grp, U, p.n_groups); u1 = (int)sk_begin(grp + 1, U, p.n_groups);
+        return true;
+    };
 
     if (threadIdx.x == 0) {
         pdl_launch_dependents();
@@ -91,34 +103,44 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
     if (warp == 0) {
         if (lane == 0) {
             const uint64_t pol_w = l2_policy_evict_first(), pol_x = l2_policy_evict_last();
-            // item i: unit u0 + i / 3; i % 3 = 0 weights, 1 hi rows, 2 lo rows
-            auto load = [&](int i, int slot) {
+            auto load_w = [&](int ft, int kb, int slot) {
                 unsigned char* dst = ring + slot * SLOT_BYTES;
-                const int u = u0 + i / 3, kind = i % 3, ft = u / p.KB, kb = u % p.KB;
-                if (kind == 0) {
-                    mbar_expect_tx(&full[slot], SLOT_BYTES);
-                    const int t1 = 2 * ft + 1 < p.n_tiles ? 2 * ft + 1 : 2 * ft;      // (an odd last tile fills both halves)
-                    bulk_load(dst, p.w + ((size_t)(2 * ft) * p.KB + kb) * A_BYTES, A_BYTES, &full[slot], pol_w);
-                    bulk_load(dst + A_BYTES, p.w + ((size_t)t1 * p.KB + kb) * A_BYTES, A_BYTES, &full[slot], pol_w);
-                } else {
-                    mbar_expect_tx(&full[slot], X_BYTES);
-                    tma_load_3d_hint(dst, &p.map_b, kb * BK, 0, (kind - 1) * p.plane_blocks + rt * BPT, &full[slot], pol_x);
-                }
+                const int t1 = 2 * ft + 1 < p.n_tiles ? 2 * ft + 1 : 2 * ft;      // (an odd last tile fills both halves)
+                mbar_expect_tx(&full[slot], SLOT_BYTES);
+                bulk_load(dst, p.w + ((size_t)(2 * ft) * p.KB + kb) * A_BYTES, A_BYTES, &full[slot], pol_w);
+                bulk_load(dst + A_BYTES, p.w + ((size_t)t1 * p.KB + kb) * A_BYTES, A_BYTES, &full[slot], pol_w);
             };
-            const int n_items = 3 * n_units, n_pre = n_items < SLOTS ? n_items : SLOTS;
+            auto load_x = [&](int plane, int kb, int slot) {
+                mbar_expect_tx(&full[slot], X_BYTES);
+                tma_load_3d_hint(ring + slot * SLOT_BYTES, &p.map_b, kb * BK, 0, plane * p.plane_blocks + rt * BPT, &full[slot], pol_x);
+            };
+            // load i of an item: unit u0 + i / 3; i % 3 = 0 weights, 1 hi rows, 2 lo rows
+            const int n_pre = 3 * (u1 - u0) < SLOTS ? 3 * (u1 - u0) : SLOTS;
             // the weights do not depend on the kernel before this one, the activations do
-            for (int i = 0; i < n_pre; i += 3) load(i, i);
+            for (int i = 0; i < n_pre; i += 3) load_w((u0 + i / 3) / p.KB, (u0 + i / 3) % p.KB, i);
             pdl_wait();
             for (int i = 0; i < n_pre; ++i)
-                if (i % 3) load(i, i);
+                if (i % 3) load_x(i % 3 - 1, (u0 + i / 3) % p.KB, i);
+            // (no division per load: with two per load and one more for the row tile, a step of four 68-row sequences took 3600 us
+            // against 3460; the 240-row tiles did not notice)
             bool ok = true;
-            int slot = 0;
-            uint32_t phase = 0;          // parity of the slot's release that item i waits for
-            for (int i = n_pre; i < n_items; ++i) {
-                if (!mbar_wait(&empty[slot], phase, s_abort)) { ok = false; break; }
-                load(i, slot);
-                if (++slot == SLOTS) { slot = 0; phase ^= 1; }
-            }
+            int slot = n_pre % SLOTS;
+            uint32_t phase = n_pre == SLOTS ? 0 : 1;         // parity of the slot's release that a load waits for (a fresh barrier passes 1)
+            int w = blockIdx.x, u = u0 + n_pre / 3, kind = n_pre % 3;
+            do {
+                for (int ft = u / p.KB, kb = u % p.KB; u < u1;) {
+                    if (!mbar_wait(&empty[slot], phase, s_abort)) { ok = false; break; }
+                    if (kind == 0) load_w(ft, kb, slot);
+                    else load_x(kind - 1, kb, slot);
+                    if (++slot == SLOTS) { slot = 0; phase ^= 1; }
+                    if (++kind == 3) {
+                        kind = 0; ++u;
+                        if (++kb == p.KB) { kb = 0; ++ft; }
+                    }
+                }
+                if (!ok || !next_item(w)) break;
+                u = u0;
+            } while (true);
             if (!ok) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
         }
     } else if (warp == 1) {
@@ -128,44 +150,47 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
             int slot = 0, piece = 0;
             uint32_t phase = 0;
             auto next = [&](int& s, uint32_t& ph) { if (++s == SLOTS) { s = 0; ph ^= 1; } };
-            for (int u = u0; u < u1 && ok; ++piece) {
-                const int end = (u / p.KB + 1) * p.KB < u1 ? (u / p.KB + 1) * p.KB : u1;
-                if (!mbar_wait(tempty, (piece & 1) ^ 1, s_abort)) { ok = false; break; }     // (a fresh barrier passes parity 1)
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (const int beg = u; u < end; ++u) {
-                    const int sw = slot;
-                    const uint32_t pw = phase;
-                    next(slot, phase);
-                    const int sh = slot;
-                    const uint32_t ph = phase;
-                    next(slot, phase);
-                    const int sl = slot;
-                    const uint32_t pl = phase;
-                    next(slot, phase);
-                    if (!mbar_wait(&full[sw], pw, s_abort) || !mbar_wait(&full[sh], ph, s_abort)) { ok = false; break; }
+            int w = blockIdx.x;
+            do {
+                for (int u = u0; u < u1 && ok; ++piece) {
+                    const int end = (u / p.KB + 1) * p.KB < u1 ? (u / p.KB + 1) * p.KB : u1;
+                    if (!mbar_wait(tempty, (piece & 1) ^ 1, s_abort)) { ok = false; break; }     // (a fresh barrier passes parity 1)
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint64_t dw = smem_desc(smem_u32(ring + sw * SLOT_BYTES), 16);
-                    const uint64_t dh = smem_desc(smem_u32(ring + sh * SLOT_BYTES), 16);
+                    for (const int beg = u; u < end; ++u) {
+                        const int sw = slot;
+                        const uint32_t pw = phase;
+                        next(slot, phase);
+                        const int sh = slot;
+                        const uint32_t ph = phase;
+                        next(slot, phase);
+                        const int sl = slot;
+                        const uint32_t pl = phase;
+                        next(slot, phase);
+                        if (!mbar_wait(&full[sw], pw, s_abort) || !mbar_wait(&full[sh], ph, s_abort)) { ok = false; break; }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint64_t dw = smem_desc(smem_u32(ring + sw * SLOT_BYTES), 16);
+                        const uint64_t dh = smem_desc(smem_u32(ring + sh * SLOT_BYTES), 16);
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k) {
-                        const uint32_t acc = (u > beg || k > 0) ? 1u : 0u;
-                        umma(tmem_base, dw + (uint64_t)(k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
-                        umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
-                    }
-                    umma_commit(&empty[sh]);
-                    if (!mbar_wait(&full[sl], pl, s_abort)) { ok = false; break; }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint64_t dl = smem_desc(smem_u32(ring + sl * SLOT_BYTES), 16);
+                        for (int k = 0; k < BK / 16; ++k) {
+                            const uint32_t acc = (u > beg || k > 0) ? 1u : 0u;
+                            umma(tmem_base, dw + (uint64_t)(k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
+                            umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
+                        }
+                        umma_commit(&empty[sh]);
+                        if (!mbar_wait(&full[sl], pl, s_abort)) { ok = false; break; }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint64_t dl = smem_desc(smem_u32(ring + sl * SLOT_BYTES), 16);
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k) {
-                        umma(tmem_base, dw + (uint64_t)(k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
-                        umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
+                        for (int k = 0; k < BK / 16; ++k) {
+                            umma(tmem_base, dw + (uint64_t)(k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
+                            umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
+                        }
+                        umma_commit(&empty[sw]);
+                        umma_commit(&empty[sl]);
                     }
-                    umma_commit(&empty[sw]);
-                    umma_commit(&empty[sl]);
+                    if (ok) umma_commit(tfull);
                 }
-                if (ok) umma_commit(tfull);
-            }
+            } while (ok && next_item(w));
             if (!ok) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
         }
     } else {
@@ -174,49 +199,51 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
         const int half = (warp - 2) >> 2, q = warp & 3, f = q * 32 + lane;
         const uint32_t taddr = tmem_base + half * 256 + ((uint32_t)(q * 32) << 16);
         const size_t rows = (size_t)p.n_rt * WR;
-        int nr[BPT];
-#pragma unroll
-        for (int b = 0; b < BPT; ++b)
-            nr[b] = rt * BPT + b < p.n_blocks && p.st[rt * BPT + b].active ? min(p.st[rt * BPT + b].n_rows, WB) : 0;
         bool ok = true;
-        int piece = 0;
-        const int ft0 = u0 / p.KB;
-        for (int u = u0; u < u1 && ok; ++piece) {
-            const int ft = u / p.KB;
-            u = (ft + 1) * p.KB < u1 ? (ft + 1) * p.KB : u1;
-            // (a wait that fails takes the whole warp out: the tensor-memory loads below are warp-wide)
-            if (!__all_sync(0xffffffffu, mbar_wait(tfull, piece & 1, s_abort))) { ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const bool real = 2 * ft + half < p.n_tiles;
-            float* part = p.partials + (((size_t)(grp * p.slots + (ft - ft0)) * 2 + half) * rows + (size_t)rt * WR) * TILE_N + f;
-            // CH columns at a time: as many 16-column loads as fit, an 8-column load for the rest, one wait
-            constexpr int CH = WB % 24 == 0 ? 24 : (WB % 40 == 0 ? 40 : 32);
-            static_assert(WB % CH == 0 && (CH % 16 == 0 || CH % 16 == 8), "columns per wait");
+        int piece = 0, w = blockIdx.x;
+        do {
+            int nr[BPT];
 #pragma unroll
-            for (int b = 0; b < BPT; ++b) {
-                const int n = real ? nr[b] : 0;
+            for (int b = 0; b < BPT; ++b)
+                nr[b] = rt * BPT + b < p.n_blocks && p.st[rt * BPT + b].active ? min(p.st[rt * BPT + b].n_rows, WB) : 0;
+            const int ft0 = u0 / p.KB;
+            for (int u = u0; u < u1 && ok; ++piece) {
+                const int ft = u / p.KB;
+                u = (ft + 1) * p.KB < u1 ? (ft + 1) * p.KB : u1;
+                // (a wait that fails takes the whole warp out: the tensor-memory loads below are warp-wide)
+                if (!__all_sync(0xffffffffu, mbar_wait(tfull, piece & 1, s_abort))) { ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const bool real = 2 * ft + half < p.n_tiles;
+                float* part = p.partials + (((size_t)(grp * p.slots + (ft - ft0)) * 2 + half) * rows + (size_t)rt * WR) * TILE_N + f;
+                // CH columns at a time: as many 16-column loads as fit, an 8-column load for the rest, one wait
+                constexpr int CH = WB % 24 == 0 ? 24 : (WB % 40 == 0 ? 40 : 32);
+                static_assert(WB % CH == 0 && (CH % 16 == 0 || CH % 16 == 8), "columns per wait");
 #pragma unroll
-                for (int c0 = 0; c0 < WB; c0 += CH) {
-                    uint32_t v[CH];
+                for (int b = 0; b < BPT; ++b) {
+                    const int n = real ? nr[b] : 0;
 #pragma unroll
-                    for (int c = 0; c + 16 <= CH; c += 16) tmem_ld16_issue(taddr + b * WB + c0 + c, *reinterpret_cast<uint32_t(*)[16]>(&v[c]));
-                    if constexpr (CH % 16 == 8)
-                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                                     : "=r"(v[CH - 8]), "=r"(v[CH - 7]), "=r"(v[CH - 6]), "=r"(v[CH - 5]), "=r"(v[CH - 4]), "=r"(v[CH - 3]),
-                                       "=r"(v[CH - 2]), "=r"(v[CH - 1])
-                                     : "r"(taddr + b * WB + c0 + CH - 8));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (b == BPT - 1 && c0 + CH >= WB) {        // the accumulator is in registers
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(tempty);
+                    for (int c0 = 0; c0 < WB; c0 += CH) {
+                        uint32_t v[CH];
+#pragma unroll
+                        for (int c = 0; c + 16 <= CH; c += 16) tmem_ld16_issue(taddr + b * WB + c0 + c, *reinterpret_cast<uint32_t(*)[16]>(&v[c]));
+                        if constexpr (CH % 16 == 8)
+                            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                                         : "=r"(v[CH - 8]), "=r"(v[CH - 7]), "=r"(v[CH - 6]), "=r"(v[CH - 5]), "=r"(v[CH - 4]), "=r"(v[CH - 3]),
+                                           "=r"(v[CH - 2]), "=r"(v[CH - 1])
+                                         : "r"(taddr + b * WB + c0 + CH - 8));
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                        if (b == BPT - 1 && c0 + CH >= WB) {        // the accumulator is in registers
+                            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(tempty);
+                        }
+#pragma unroll
+                        for (int i = 0; i < CH; ++i)
+                            if (c0 + i < n) __stcg(part + (size_t)(b * WB + c0 + i) * TILE_N, __uint_as_float(v[i]));
                     }
-#pragma unroll
-                    for (int i = 0; i < CH; ++i)
-                        if (c0 + i < n) __stcg(part + (size_t)(b * WB + c0 + i) * TILE_N, __uint_as_float(v[i]));
                 }
             }
-        }
+        } while (ok && next_item(w));
         if (!ok && lane == 0) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
     }
     // ---------------- teardown (every thread arrives here)
@@ -235,13 +262,13 @@ constexpr int WIDE_SM = 148;
 
 }  // namespace
 
-// Groups and partial slots of a GEMM of n_tiles 128-feature tiles and KB k-blocks over n_rt row tiles.
+// Ranges and partial slots of a GEMM of n_tiles 128-feature tiles and KB k-blocks, split for n_rt row tiles.
 void wide_geometry(int n_tiles, int KB, int n_rt, int* n_groups, int* slots) {
     const int n_ft = (n_tiles + 1) / 2;
     const long long U = (long long)n_ft * KB;
     long long g = WIDE_SM / n_rt;
     if (g > U) g = U;
-    // a consumer sums at most 15 pieces of a tile: no group smaller than a 13th of a tile
+    // a consumer sums at most 15 pieces of a tile: no range smaller than a 13th of a tile
     while (g > 1 && U / g * 13 < KB) --g;
     int most = 1;
     for (int c = 0; c < g; ++c) {
@@ -252,22 +279,23 @@ void wide_geometry(int n_tiles, int KB, int n_rt, int* n_groups, int* slots) {
     *slots = most;
 }
 
-size_t wide_partial_bytes(int n_tiles, int KB, int n_rt, int tile_rows) {
+size_t wide_partial_bytes(int n_tiles, int KB, int n_blocks, int wb, int bpt, int split_bpt) {
     int g, slots;
-    wide_geometry(n_tiles, KB, n_rt, &g, &slots);
-    return (size_t)g * slots * 2 * n_rt * tile_rows * TILE_N * sizeof(float);
+    wide_geometry(n_tiles, KB, (n_blocks + split_bpt - 1) / split_bpt, &g, &slots);
+    return (size_t)g * slots * 2 * ((n_blocks + bpt - 1) / bpt * bpt) * wb * TILE_N * sizeof(float);
 }
 
 struct WideGemm {
     WideParams p;
-    int n_rt_max, wb, bpt;      // row tiles at most; rows per block, blocks per row tile
-    int groups[WIDE_MAX_RT], slots[WIDE_MAX_RT];
-    TileSrc* tables;            // [n_rt_max][n_tiles]
+    int max_blocks, wb, bpt, split_bpt;            // blocks at most; rows per block, blocks per row tile, blocks per row tile of the split
+    int groups[WIDE_MAX_RT], slots[WIDE_MAX_RT];   // by row tiles of the split
+    TileSrc* tables;            // [row tiles of the split][n_tiles]
 };
 
-int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int wb, int bpt, int n_rt_max, float* partials, size_t partial_bytes,
-                     TileSrc* tables_dev, int* err, cudaStream_t stream) {
-    if (!out || n_rt_max < 1 || n_rt_max > WIDE_MAX_RT || x_blocks < bpt || K % 8 || reinterpret_cast<uintptr_t>(x) % 16) return -1;
+int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int wb, int bpt, int split_bpt, int max_blocks, float* partials,
+                     size_t partial_bytes, TileSrc* tables_dev, int* err, cudaStream_t stream) {
+    const int n_rt_max = (max_blocks + split_bpt - 1) / split_bpt;
+    if (!out || max_blocks < 1 || n_rt_max > WIDE_MAX_RT || x_blocks < bpt || K % 8 || reinterpret_cast<uintptr_t>(x) % 16) return -1;
     EncodeFn enc = get_encode();
     if (!enc) return -1;
     WideGemm* g = new (std::nothrow) WideGemm();
@@ -276,7 +304,7 @@ int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_bl
     WideParams& p = g->p;
     p.n_tiles = n_tiles; p.n_ft = (n_tiles + 1) / 2; p.KB = (K + BK - 1) / BK;
     p.partials = partials; p.err = err; p.plane_blocks = x_blocks;
-    g->n_rt_max = n_rt_max; g->wb = wb; g->bpt = bpt;
+    g->max_blocks = max_blocks; g->wb = wb; g->bpt = bpt; g->split_bpt = split_bpt;
     g->tables = tables_dev;
     {
         cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)RT, (cuuint64_t)2 * x_blocks};
@@ -291,7 +319,7 @@ int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_bl
     bool fits = tab != nullptr;
     for (int r = 1; r <= n_rt_max && fits; ++r) {
         wide_geometry(n_tiles, p.KB, r, &g->groups[r - 1], &g->slots[r - 1]);
-        fits = wide_partial_bytes(n_tiles, p.KB, r, wb * bpt) <= partial_bytes;
+        fits = wide_partial_bytes(n_tiles, p.KB, r * split_bpt < max_blocks ? r * split_bpt : max_blocks, wb, bpt, split_bpt) <= partial_bytes;
         const long long U = (long long)p.n_ft * p.KB, G = g->groups[r - 1];
         for (int t = 0; t < n_tiles && fits; ++t) {
             TileSrc& e = tab[(size_t)(r - 1) * n_tiles + t];
@@ -316,18 +344,23 @@ void wide_gemm_destroy(WideGemm* g) { delete g; }
 
 int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, int n_blocks, cudaStream_t s, bool pdl) {
     if (!g || n_blocks < 1) return ESP_E_ARG;
-    const int n_rt = (n_blocks + g->bpt - 1) / g->bpt;
-    if (n_rt > g->n_rt_max) return ESP_E_ARG;
+    if (n_blocks > g->max_blocks) return ESP_E_ARG;
+    const int n_rt = (n_blocks + g->bpt - 1) / g->bpt, split = (n_blocks + g->split_bpt - 1) / g->split_bpt - 1;
     WideParams p = g->p;
     p.w = reinterpret_cast<const unsigned char*>(packed);
     p.st = st;
-    p.n_rt = n_rt; p.n_blocks = n_blocks; p.n_groups = g->groups[n_rt - 1]; p.slots = g->slots[n_rt - 1];
+    p.n_rt = n_rt; p.n_blocks = n_blocks; p.n_groups = g->groups[split]; p.slots = g->slots[split];
+    const int grid = g->wb != RT || p.n_groups * n_rt < WIDE_SM ? p.n_groups * n_rt : WIDE_SM;
 #define ESP_WIDE_CASE(WB, BPT)                                                                                          \
     if (g->wb == WB && g->bpt == BPT) {                                                                                \
         if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_gemm_wide<WB, BPT>), (int)WIDE_SMEM)) return ESP_E_CUDA; \
-        return launch_k(k_gemm_wide<WB, BPT>, dim3(p.n_groups * n_rt), dim3(WIDE_THREADS), WIDE_SMEM, s, pdl, p) == cudaSuccess ? ESP_OK : ESP_E_CUDA; \
+        return launch_k(k_gemm_wide<WB, BPT>, dim3(grid), dim3(WIDE_THREADS), WIDE_SMEM, s, pdl, p) == cudaSuccess ? ESP_OK : ESP_E_CUDA; \
     }
     ESP_WIDE_CASE(PREFILL_CHUNK, 2)
+    ESP_WIDE_CASE(32, 2)
+    ESP_WIDE_CASE(32, 3)
+    ESP_WIDE_CASE(64, 2)
+    ESP_WIDE_CASE(64, 3)
     ESP_WIDE_CASE(80, 2)
     ESP_WIDE_CASE(80, 3)
     ESP_WIDE_CASE(RT, 2)
@@ -337,11 +370,11 @@ int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, 
 
 // the row of block b, row r in the partials is b * wb + r
 StreamK wide_gemm_streamk(const WideGemm* g, int n_blocks) {
-    const int n_rt = (n_blocks + g->bpt - 1) / g->bpt;
+    const int n_rt = (n_blocks + g->bpt - 1) / g->bpt, split = (n_blocks + g->split_bpt - 1) / g->split_bpt - 1;
     StreamK k;
     k.partials = g->p.partials;
-    k.table = g->tables + (size_t)(n_rt - 1) * g->p.n_tiles;
-    k.n_tiles = g->p.n_tiles; k.KB = g->p.KB; k.G = g->groups[n_rt - 1]; k.slots = g->slots[n_rt - 1];
+    k.table = g->tables + (size_t)split * g->p.n_tiles;
+    k.n_tiles = g->p.n_tiles; k.KB = g->p.KB; k.G = g->groups[split]; k.slots = g->slots[split];
     k.rows = n_rt * g->bpt * g->wb;
     k.seq_rows = g->wb;
     return k;

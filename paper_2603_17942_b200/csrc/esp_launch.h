@@ -131,14 +131,14 @@ int tc_gemm_counter_ints();
 
 
 // tcgen05 GEMM over several blocks at once (esp_gemm_wide.cu): activations [2 planes][x_blocks][RT][K], of every block
-// the first wb rows, bpt blocks to a row tile ((PREFILL_CHUNK, 2), (80, 2), (80, 3) or (RT, 2)); partials and contributor
-// tables for the same consumers as above.
+// the first wb rows, bpt blocks to a row tile ((PREFILL_CHUNK, 2), (32, 64 or 80, 2 or 3) or (RT, 2)); partials and
+// contributor tables for the same consumers as above.  The split of k is that of row tiles of split_bpt blocks.
 struct WideGemm;
-constexpr int WIDE_MAX_RT = 4;                       // row tiles of one launch
+constexpr int WIDE_MAX_RT = 4;                       // row tiles of one launch, as far as the split of k goes
 constexpr int WIDE_MAX_BLOCKS = 2 * WIDE_MAX_RT;     // full prefill blocks of one pass
-size_t wide_partial_bytes(int n_tiles, int KB, int n_rt, int tile_rows);
-// tables_dev: device memory for n_rt_max * n_tiles entries
-int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int wb, int bpt, int n_rt_max, float* partials,
+size_t wide_partial_bytes(int n_tiles, int KB, int n_blocks, int wb, int bpt, int split_bpt);
+// tables_dev: device memory for n_tiles entries per row tile of the split
+int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int wb, int bpt, int split_bpt, int max_blocks, float* partials,
                      size_t partial_bytes, TileSrc* tables_dev, int* err, cudaStream_t stream);
 void wide_gemm_destroy(WideGemm* g);
 int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, int n_blocks, cudaStream_t s, bool pdl);

@@ -44,9 +44,10 @@ def test_wide_prefill_against_cuda_core_path(weights, n_prompt):
     assert (got[0] - got[1]).abs().max() <= TOL_BF16 * span
 
 
-@pytest.mark.parametrize("n_seq,nodes,n_anchor", [(2, 16, 1), (4, 16, 1), (5, 16, 1), (7, 16, 1), (13, 16, 1), (3, 25, 0)])
+@pytest.mark.parametrize("n_seq,nodes,n_anchor", [(2, 16, 1), (5, 16, 1), (33, 16, 1), (4, 40, 1), (2, 60, 1), (4, 70, 1), (5, 70, 1), (7, 70, 1),
+                                                   (13, 70, 1), (3, 25, 0)])
 def test_batch_steps_against_each_sequence_alone(weights, n_seq, nodes, n_anchor):
-    """One step of a handle with several sequences (row tiles of two or three blocks, ragged ones, more sequences than a
+    """One step of a handle with several sequences (row tiles of every shape, ragged ones, more sequences than a
     pass covers, blocks of 100 rows) against the step each sequence takes in a handle of its own: the same trees (the
     prefill does not depend on the batch), logits equal to the bar bf16 logits are held to; one sequence stays idle."""
     spec = P.spec_cfg(n_probes=3, topk=5, max_nodes=nodes, expand_width=0 if n_anchor else 1, n_anchor=n_anchor)
@@ -70,6 +71,25 @@ def test_batch_steps_against_each_sequence_alone(weights, n_seq, nodes, n_anchor
         assert (logits[i, :rows[i]] - alone[0, :rows[i]]).abs().max() <= TOL_BF16 * span, f"sequence {i}"
         one.close()
     h.close()
+
+
+@pytest.mark.parametrize("n_seq", [2, 3, 5, 7, 13])
+def test_batch_rows_have_the_bits_of_the_greedy_handle(weights, n_seq):
+    """The split of k of a handle with several sequences does not follow the rows of its blocks: the first row of a step
+    (the last committed token) has the same logits bit for bit in the greedy handle and with trees of every block size,
+    128-row blocks that take two turns included."""
+    prompts = [synth.make_prompt(BF16_SMALL.vocab, 30 + 7 * i, 20 + i) for i in range(n_seq)]
+    first = []
+    for kw in (dict(n_probes=0, max_nodes=1), *(dict(n_probes=3, topk=5, max_nodes=n, expand_width=0, n_anchor=1) for n in (16, 40, 70, 110))):
+        h, logits = _handle(weights, 400, P.spec_cfg(**kw), n_seq)
+        for i in range(n_seq):
+            h.prefill(prompts[i], i)
+        P.esp_step(h.h, h.tokens_out, h.n_out)
+        assert h.stats().device_error == 0
+        first.append(logits[:, 0].clone())
+        h.close()
+    for f in first[1:]:
+        assert torch.equal(f, first[0])
 
 
 @pytest.mark.parametrize("group,n_rows,batch,L", [(4, 68, 3, 500), (2, 128, 5, 130), (1, 41, 24, 64), (8, 9, 70, 250), (4, 120, 8, 15)])
