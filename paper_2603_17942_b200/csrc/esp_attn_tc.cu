@@ -534,8 +534,9 @@ __global__ void __launch_bounds__(128, TAIL_FIRST ? 5 : 4) k_attn_tail_merge_tc(
 
 // ---- tail + merge for launches with many (row, head) pairs: same sums in the same order, so the same bits.
 // A CTA takes some rows of one (sequence, KV head).  The keys and values any tail of the CTA can name -- a contiguous
-// run of cache slots, from the first row's T0 to the last row's own slot -- come to shared memory once, and a warp
-// works on GH query heads of one row together, so that every key and value it reads serves GH pairs.  What bounded
+// run of cache slots, from the smallest T0 of its rows to the last slot one of their ancestor masks names -- come to
+// shared memory once, and a warp works on GH query heads of one row together, so that every key and value it reads
+// serves GH pairs.  What bounded
 // the warp-per-pair kernel in such launches was its key gather (32 lanes, 32 cache lines per load: 512 L1 tag cycles
 // per pair); this one is bound by its instruction count.  Measured on their own: 16 sequences x 68 rows x 32 heads 93 -> 46
 // us, 2 x 68 x 32 20.7 -> 11.6 us; one block's 68 x 32 pairs stay with the warp-per-pair kernel (see the launch rule).
@@ -573,12 +574,16 @@ __global__ void __launch_bounds__(TM_WARPS * 32, 2) k_attn_tail_merge_many_tc(At
     }
     if (r_beg >= n_rows) { pdl_wait(); return; }
     const int r_end = min(r_beg + rows_per_cta, n_rows);
-    // first slot of the window: the smallest T0 of the CTA's rows (every thread looks at every row: at most 128)
-    int w0 = 0x7fffffff;
-    for (int r = r_beg + lane; r < r_end; r += 32)
+    // The window: from the smallest T0 of the CTA's rows (every warp looks at every row: at most 128) to the last block row
+    // they name.  In a step a row's ancestors stand before it; the rows of the operator come in any order.
+    int w0 = 0x7fffffff, last = r_end - 1;
+    for (int r = r_beg + lane; r < r_end; r += 32) {
         w0 = min(w0, tail_start_tc(L + (a.st ? a.st[seq].row_depth[r] : a.depth[seq * RT + r]), a.dcap));
+        if (!a.st) last = max(last, last_set_bit128(a.anc[(size_t)(seq * RT + r) * 2], a.anc[(size_t)(seq * RT + r) * 2 + 1]));
+    }
     w0 = __reduce_min_sync(0xffffffffu, w0);
-    const int n_win = min(L + r_end - w0, window);
+    last = __reduce_max_sync(0xffffffffu, last);
+    const int n_win = min(L + last + 1 - w0, window);
     {
         const size_t row0 = ((size_t)(a.kv_shared ? 0 : seq) * a.Hkv + kvh) * a.cap + w0;
         const __nv_bfloat16* kb = reinterpret_cast<const __nv_bfloat16*>(a.kc) + row0 * HD;
@@ -840,7 +845,7 @@ int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_la
         if (groups > (rows_cap + TM_WARPS - 1) / TM_WARPS) groups = (rows_cap + TM_WARPS - 1) / TM_WARPS;
         if (groups < 1) groups = 1;
         const int rpc = (rows_cap + groups - 1) / groups;
-        const int window = TM_DCAP + 15 + rows_cap;
+        const int window = a.st ? TM_DCAP + 15 + rows_cap : TM_WINDOW;
         const dim3 grid((rows_cap + rpc - 1) / rpc, a.Hkv, batch);
 #define ESP_TAIL_MANY(GH)                                                                                              \
         {                                                                                                              \

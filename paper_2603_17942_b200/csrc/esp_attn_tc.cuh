@@ -340,6 +340,10 @@ __device__ __forceinline__ int nth_set_bit128(unsigned long long lo, unsigned lo
     for (int i = 0; i < n; ++i) m &= m - 1;
     return m ? base + __ffsll((long long)m) - 1 : -1;
 }
+// highest set bit of a 128-bit mask, -1 if there is none
+__device__ __forceinline__ int last_set_bit128(unsigned long long lo, unsigned long long hi) {
+    return hi ? 127 - __clzll((long long)hi) : 63 - __clzll((long long)lo);
+}
 __device__ __forceinline__ void merge_ml(float& m, float& l, float (&o)[4], float cm, float cl, const float (&co)[4]) {
     // products and sums are rounded one by one, so that every instance of the kernel rounds alike
     const float mn = fmaxf(m, cm);

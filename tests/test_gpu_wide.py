@@ -112,3 +112,25 @@ def test_attention_tail_of_large_launches_bitwise(group, n_rows, batch, L):
         alone = _run_attention(1, q[s:s + 1].contiguous(), kc[s:s + 1].contiguous(), vc[s:s + 1].contiguous(), anc[:1], depth[:1],
                                n_rows, L, Hq, Hkv, h)
         assert torch.equal(out[s, :n_rows], alone[0, :n_rows]), f"sequence {s}"
+
+
+@pytest.mark.parametrize("group,n_rows,batch", [(4, 68, 16), (1, 128, 5), (8, 41, 12)])
+def test_attention_tail_of_large_launches_rows_in_any_order(group, n_rows, batch):
+    """The rows of the operator come in any order, so a row may stand before its ancestors, and its CTA has to fetch keys
+    of rows that other CTAs work on (with the rows reversed the root is the last one): the bits and the clean status of a
+    launch of its own, whose kernel takes every key from the cache."""
+    Hkv, h, L = 8, 128, 250          # (one cache split, whatever the batch)
+    Hq, cap = Hkv * group, L + R
+    _, depth1, vis = _tree_block(n_rows - 3, 3, 5, n_rows)
+    depth1, vis = depth1[::-1], vis[::-1, ::-1]
+    g = torch.Generator(device="cuda").manual_seed(group)
+    q = torch.randn(batch, R, Hq, h, generator=g, device="cuda").bfloat16()
+    kc, vc = (torch.randn(batch, Hkv, cap, h, generator=g, device="cuda").bfloat16() for _ in range(2))
+    anc = np.stack([_anc_words(vis)] * batch)
+    depth = np.zeros((batch, R), np.int32)
+    depth[:, :n_rows] = depth1
+    out = _run_attention(1, q, kc, vc, anc, depth, n_rows, L, Hq, Hkv, h)
+    for s in (0, batch - 1):
+        alone = _run_attention(1, q[s:s + 1].contiguous(), kc[s:s + 1].contiguous(), vc[s:s + 1].contiguous(), anc[:1], depth[:1],
+                               n_rows, L, Hq, Hkv, h)
+        assert torch.equal(out[s, :n_rows], alone[0, :n_rows]), f"sequence {s}"
