@@ -621,9 +621,13 @@ void drop_graphs(esp_handle* h) {
     h->graphs.clear();
 }
 
+// `active` of every sequence: only seq_only during its prefill, every prefilled one otherwise (seq_only < 0)
 __global__ void k_select(SeqState* st, int batch, int seq_only) {
-    int i = threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < batch) st[i].active = seq_only < 0 ? st[i].ready : (i == seq_only);
+}
+void select_sequences(esp_handle* h, int seq_only) {
+    k_select<<<(h->D.batch + 127) / 128, 128, 0, h->stream>>>(h->b.states, h->D.batch, seq_only);
 }
 __global__ void k_mark_ready(SeqState* st, int seq) { st[seq].ready = 1; }
 
@@ -641,7 +645,7 @@ int wait_records(esp_handle* h, int slot, const int32_t** rec) {
 // A prefill that could not be enqueued: the other sequences keep their lengths; this one has to be prefilled again
 // before it can step.
 int prefill_failed(esp_handle* h, int seq, const std::vector<int>& saved, int rc) {
-    k_select<<<1, 32, 0, h->stream>>>(h->b.states, h->D.batch, -1);
+    select_sequences(h, -1);
     h->L_host = saved;
     h->L_host[seq] = 0;
     h->ready[seq] = 0;
@@ -845,7 +849,7 @@ int esp_prefill(esp_handle* h, int32_t seq, const int32_t* prompt, int32_t n_pro
     if (h->sc.mask_init != 2)   // 2: the caller's vectors (esp_set_mask) stay
         launch_mask_init(h->dtype, h->embed, h->b.prompt_dev, n_prompt, h->D.d, h->b.mvec + (size_t)seq * h->D.mask_slots * h->D.d,
                          h->D.mask_slots, h->sc.mask_init, s);
-    k_select<<<1, 32, 0, s>>>(h->b.states, h->D.batch, seq);
+    select_sequences(h, seq);
     std::vector<int> saved = h->L_host;
     for (int i = 0; i < h->D.batch; ++i) h->L_host[i] = 0;
     const bool wide = h->p_wide[3] && h->gemm_impl == 0;
@@ -868,7 +872,7 @@ int esp_prefill(esp_handle* h, int32_t seq, const int32_t* prompt, int32_t n_pro
         if (rc) return prefill_failed(h, seq, saved, rc);
     }
     k_mark_ready<<<1, 1, 0, s>>>(h->b.states, seq);
-    k_select<<<1, 32, 0, s>>>(h->b.states, h->D.batch, -1);
+    select_sequences(h, -1);
     const int32_t* rec = nullptr;
     int rc = wait_records(h, NREC, &rec);
     h->L_host = saved;

@@ -134,3 +134,26 @@ def test_attention_tail_of_large_launches_rows_in_any_order(group, n_rows, batch
         alone = _run_attention(1, q[s:s + 1].contiguous(), kc[s:s + 1].contiguous(), vc[s:s + 1].contiguous(), anc[:1], depth[:1],
                                n_rows, L, Hq, Hkv, h)
         assert torch.equal(out[s, :n_rows], alone[0, :n_rows]), f"sequence {s}"
+
+
+@pytest.mark.parametrize("n_seq,early", [(34, 33), (34, 32), (130, 129)])
+def test_prefill_leaves_every_other_sequence_alone(weights, n_seq, early):
+    """Prefilling one sequence changes nothing of another that is waiting, whatever their places in a large handle: length,
+    draft tree, mask vectors and Top-K' lists stay, and its next step is that of a handle in which it was prefilled last."""
+    spec = P.spec_cfg(n_probes=3, topk=5, max_nodes=16, expand_width=0, n_anchor=1)
+    prompts = {early: synth.make_prompt(BF16_SMALL.vocab, 45, 1), 0: synth.make_prompt(BF16_SMALL.vocab, 130, 2)}
+    seen = []
+    for order in ((early, 0), (0, early)):
+        h, logits = _handle(weights, 200, spec, n_seq)
+        for i in order:
+            h.prefill(prompts[i], i)
+            if i == early:
+                before = h.state(early)
+        after = h.state(early)
+        for key in before:
+            assert np.array_equal(before[key], after[key]), key
+        h.step(early)
+        assert h.stats().device_error == 0
+        seen.append((h.n_out.copy(), h.tokens_out[early].copy(), logits[early, :after["n_rows"]].clone()))
+        h.close()
+    assert np.array_equal(seen[0][0], seen[1][0]) and np.array_equal(seen[0][1], seen[1][1]) and torch.equal(seen[0][2], seen[1][2])
