@@ -1115,7 +1115,11 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
         if (tid == 0) st->L = L0 + N0;
         return;
     }
-    for (int r = tid; r < N0; r += nt) s_arg[r] = A.topk[(size_t)(grow0 + r) * KP_MAX].id;
+    for (int r = tid; r < N0; r += nt) {
+        const int t = A.topk[(size_t)(grow0 + r) * KP_MAX].id;
+        s_arg[r] = t >= 0 ? t : 0;                       // a row of NaN has no arg-max: its token would index the embeddings
+        if (t < 0) set_error(A.err, DEV_E_INDEX);
+    }
     __syncthreads();
 
     // ---- verification (Section 2): follow the model's own next token through the tree.  One warp walks; its lanes look for
@@ -1275,10 +1279,10 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
                 ++seen;
             }
             const int c = base + w;
-            if (q < D.KP && list[q].id >= 0) {
+            if (ptok >= 0 && q < D.KP && list[q].id >= 0) {
                 c_tok[c] = list[q].id;
                 c_lp[c] = __fadd_rn(c_lp[p], __fsub_rn(list[q].val, lse_i));
-            } else {  // list exhausted (cannot happen when K' = K + pruner flags): never selectable
+            } else {  // list exhausted (logits of NaN; K' = K + pruner flags otherwise): neither it nor its children selectable
                 c_tok[c] = -1;
                 c_lp[c] = -INFINITY;
             }
@@ -1332,7 +1336,7 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
             const unsigned long long key = c_key[c];
             int rank = 0;
             for (int o = 0; o < n_surv; ++o) rank += c_key[surv[o]] < key ? 1 : 0;
-            if (rank < width && c_tok[c] >= 0) s_exp[rank] = c;
+            if (rank < width) s_exp[rank] = c;
             // a node with B-1 or more nodes of its own depth before it cannot be among the B-1 best overall
             if (rank < n_kept) s_keep[keep0 + rank] = c;
         }

@@ -510,3 +510,28 @@ def test_async_steps_then_reads_equal_synchronous_steps(pu):
     hb.step_async()                                          # one record is free again
     assert len(first) == 1
     ha.close(); hs.close(); hb.close()
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_logits_that_are_not_numbers_are_a_device_error(pu, dtype):
+    """Nothing indexes memory with the token of a row that has none.  An LM head of NaN: the prefill reports
+    ESP_E_DEVICE and the context stays usable.  One that is finite for five tokens: the probes' lists (K' = 6) run out, the
+    tree has fewer nodes, and the stream is the greedy one."""
+    import paper_2603_17942_b200 as P
+    shape = BF16_SMALL if dtype == "bf16" else synth.TINY.replace(tied=False)
+    w = synth.make_weights(shape, seed=5, std=0.1)
+    wd = pu.to_device(w)
+    prompt = synth.make_prompt(shape.vocab, 30, 3)
+    spec = O.SpecCfg(n_probes=3, topk=5, max_nodes=20, expand_width=0, n_anchor=1)
+    wd["lm_head"][5:] = float("nan")
+    h = P.Handle(shape, pu.c_spec(spec), wd, max_seq_len=100)
+    out = h.generate(prompt, 12)
+    assert h.stats().device_error == 0 and max(out) < 5
+    g, _ = pu.gpu_generate(shape, wd, pu.GREEDY, prompt, 12, max_seq_len=100)
+    assert out == g
+    wd["lm_head"][:] = float("nan")
+    bad = P.Handle(shape, pu.c_spec(spec), wd, max_seq_len=100)
+    with pytest.raises(P.EspError) as e:
+        bad.prefill(prompt)
+    assert e.value.code == -5 and bad.stats().device_error == 2        # ESP_E_DEVICE, an index outside its range
+    bad.close(); h.close()
