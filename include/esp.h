@@ -237,7 +237,8 @@ int esp_debug_wait_selftest(void* scratch, void* cuda_stream, int32_t* device_st
 int esp_debug_gumbel(uint32_t seed_lo, uint32_t seed_hi, uint32_t position, int32_t n_tokens, float* noise_out,
                      void* cuda_stream);
 
-/* Releases host-side bookkeeping only. */
+/* Releases host-side bookkeeping only (the device buffers are the caller's).  Waits for the handle's stream if steps
+ * are still unread: they write their records to host memory that belongs to the handle. */
 void esp_free(esp_handle* h);
 
 /* ---- stand-alone operators (the same kernels the step uses), for operator-level parity and timing ---- */

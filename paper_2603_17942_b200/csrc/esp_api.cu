@@ -649,6 +649,7 @@ int prefill_failed(esp_handle* h, int seq, const std::vector<int>& saved, int rc
     h->L_host = saved;
     h->L_host[seq] = 0;
     h->ready[seq] = 0;
+    cudaStreamSynchronize(h->stream);      // what was enqueued of it writes records: esp_free may follow
     return rc;
 }
 
@@ -1152,6 +1153,8 @@ int esp_debug_gumbel(uint32_t seed_lo, uint32_t seed_hi, uint32_t position, int3
 
 void esp_free(esp_handle* h) {
     if (!h) return;
+    // the steps that nobody has read yet still write their records to host memory that is freed below
+    if (h->issued != h->consumed) cudaStreamSynchronize(h->stream);
     for (auto* p : h->p_qkv) tc_gemm_destroy(p);
     for (auto* p : h->p_o) tc_gemm_destroy(p);
     for (auto* p : h->p_gu) tc_gemm_destroy(p);

@@ -535,3 +535,18 @@ def test_logits_that_are_not_numbers_are_a_device_error(pu, dtype):
         bad.prefill(prompt)
     assert e.value.code == -5 and bad.stats().device_error == 2        # ESP_E_DEVICE, an index outside its range
     bad.close(); h.close()
+
+
+def test_a_handle_freed_with_unread_steps_waits_for_them(pu):
+    """The records of enqueued steps are written to the handle's host memory: esp_free returns when nothing is in flight."""
+    import paper_2603_17942_b200 as P
+    w = pu.to_device(synth.make_weights(BF16_SMALL, seed=7, std=0.05))
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    h = P.Handle(BF16_SMALL, pu.c_spec(pu.GREEDY), w, max_seq_len=700, stream=stream)
+    h.prefill(synth.make_prompt(BF16_SMALL.vocab, 20, 1))
+    for _ in range(400):
+        h.step_async()
+    assert not stream.query()          # 400 steps of some 0.1 ms, enqueued in a few ms
+    h.close()
+    assert stream.query()
