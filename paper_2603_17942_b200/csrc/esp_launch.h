@@ -96,7 +96,7 @@ inline int attn_split_len(int max_len, int batch, int Hkv) {
         const double waves = (double)(long long)((items + 147) / 148);
         const double t = waves * ((c / 128) * 1.45 + 2.6) + items * 0.02;
         if (c == S || t < best_t) { best = c; best_t = t; }
-        if (splits == 1) break;
+        if (splits <= 1) break;      // (0: a capacity without cached positions)
     }
     return best;
 }

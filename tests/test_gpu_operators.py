@@ -312,3 +312,22 @@ def test_bounded_wait_gives_up_and_leaves_the_context_usable():
     got = _gemm(0, x, w, 4)
     ref = O.linear(x.float().numpy(), w.cpu())
     assert np.abs(got - ref).max() <= 2e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("dt,h", [("fp32", 64), ("bf16", 128)])
+def test_tree_attention_with_room_for_the_block_only(dt, h):
+    """cap = ESP_MAX_ROWS, L = 0: no cached position and no room for one, with several sequences."""
+    dtype = torch.float32 if dt == "fp32" else torch.bfloat16
+    b, Hq, Hkv, n_rows = 2, 4, 2, 9
+    g = torch.Generator().manual_seed(3)
+    q = torch.randn(b, R, Hq, h, generator=g).to(dtype).cuda()
+    kc, vc = (torch.randn(b, Hkv, R, h, generator=g).to(dtype).cuda() for _ in range(2))
+    _, depth1, vis = _tree_block(n_rows, 0, 4, 8)
+    depth = np.zeros((b, R), np.int32)
+    depth[:, :n_rows] = depth1
+    out = _run_attention(int(dt == "bf16"), q, kc, vc, np.stack([_anc_words(vis)] * b), depth, n_rows, 0, Hq, Hkv, h)[:, :n_rows]
+    s = torch.einsum("brhd,bhcd->bhrc", q[:, :n_rows].double(), kc.repeat_interleave(2, 1)[:, :, :n_rows].double()) / h ** 0.5
+    s.masked_fill_(torch.from_numpy(vis == 0).cuda(), -float("inf"))
+    ref = torch.einsum("bhrc,bhcd->brhd", s.softmax(-1), vc.repeat_interleave(2, 1)[:, :, :n_rows].double())
+    tol = 2e-5 if dt == "fp32" else 2.0 ** -8 * float(ref.abs().max())      # sums of a few terms; the result's own rounding
+    assert (out.double() - ref).abs().max() <= tol
