@@ -551,7 +551,7 @@ __device__ __forceinline__ void tm_copy16(void* dst, const void* src) {
 }
 
 template <int GH>
-__global__ void __launch_bounds__(TM_WARPS * 32, 2) k_attn_tail_merge_many_tc(AttnArgs a, int rows_per_cta, int window) {
+__global__ void __launch_bounds__(TM_WARPS * 32, 2) k_attn_tail_merge_many_tc(AttnArgs a, int rows_per_cta, int window, bool behind_bulk) {
     extern __shared__ __align__(16) unsigned char tm_smem[];
     __nv_bfloat16* s_k = reinterpret_cast<__nv_bfloat16*>(tm_smem);            // [window][TM_LD]
     __nv_bfloat16* s_v = s_k + (size_t)window * TM_LD;
@@ -561,8 +561,11 @@ __global__ void __launch_bounds__(TM_WARPS * 32, 2) k_attn_tail_merge_many_tc(At
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int kvh = blockIdx.y, seq = blockIdx.z, r_beg = blockIdx.x * rows_per_cta;
     const int group = a.Hq / a.Hkv;
-    // the sequence state was written by an earlier step, the queries and the block's keys and values by the kernel
-    // before the bulk kernel, which releases this one only after its own wait (see k_attn_tail_merge_tc)
+    // The sequence state was written by an earlier step.  The queries and the block's keys and values were written by the
+    // kernel before the bulk kernel, which releases this one only after its own wait (see k_attn_tail_merge_tc); without a
+    // bulk kernel in between (no cached position), by the kernel this one has to wait for.
+    bool waited = !behind_bulk;
+    if (waited) pdl_wait();
     int n_rows, L;
     if (a.st) {
         const SeqState* st = a.st + seq;
@@ -597,7 +600,6 @@ __global__ void __launch_bounds__(TM_WARPS * 32, 2) k_attn_tail_merge_many_tc(At
         asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
-    bool waited = false;
     float* s_q = s_qall + warp * GH * HD;
     float* s_p = s_pall + warp * 32 * GH;
     const int sets = group / GH;                     // GH heads of one row = one task of a warp
@@ -850,7 +852,7 @@ int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_la
 #define ESP_TAIL_MANY(GH)                                                                                              \
         {                                                                                                              \
             if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_attn_tail_merge_many_tc<GH>), (int)tail_many_smem(TM_WINDOW, GH))) return -1; \
-            return launch_k(k_attn_tail_merge_many_tc<GH>, grid, dim3(TM_WARPS * 32), tail_many_smem(window, GH), s, tail_pdl, a, rpc, window) == cudaSuccess ? 0 : -1; \
+            return launch_k(k_attn_tail_merge_many_tc<GH>, grid, dim3(TM_WARPS * 32), tail_many_smem(window, GH), s, tail_pdl, a, rpc, window, behind_bulk) == cudaSuccess ? 0 : -1; \
         }
         if (gh == 4) ESP_TAIL_MANY(4)
         if (gh == 2) ESP_TAIL_MANY(2)

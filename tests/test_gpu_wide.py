@@ -114,6 +114,26 @@ def test_attention_tail_of_large_launches_bitwise(group, n_rows, batch, L):
         assert torch.equal(out[s, :n_rows], alone[0, :n_rows]), f"sequence {s}"
 
 
+@pytest.mark.parametrize("group,n_rows,batch", [(4, 68, 3), (1, 120, 9)])
+def test_attention_tail_of_large_launches_without_a_cache(group, n_rows, batch):
+    """No cached position, so no bulk kernel in front of the tail kernel: it waits before it reads (the queries and keys come
+    from the kernel in front of it), and every sequence has the bits of a launch of its own."""
+    Hkv, h, L = 8, 128, 0
+    Hq, cap = Hkv * group, R
+    _, depth1, vis = _tree_block(n_rows, 0, 5, n_rows)
+    g = torch.Generator(device="cuda").manual_seed(group)
+    q = torch.randn(batch, R, Hq, h, generator=g, device="cuda").bfloat16()
+    kc, vc = (torch.randn(batch, Hkv, cap, h, generator=g, device="cuda").bfloat16() for _ in range(2))
+    anc = np.stack([_anc_words(vis)] * batch)
+    depth = np.zeros((batch, R), np.int32)
+    depth[:, :n_rows] = depth1
+    out = _run_attention(1, q, kc, vc, anc, depth, n_rows, L, Hq, Hkv, h)
+    for s in range(batch):
+        alone = _run_attention(1, q[s:s + 1].contiguous(), kc[s:s + 1].contiguous(), vc[s:s + 1].contiguous(), anc[:1], depth[:1],
+                               n_rows, L, Hq, Hkv, h)
+        assert torch.equal(out[s, :n_rows], alone[0, :n_rows]), f"sequence {s}"
+
+
 @pytest.mark.parametrize("group,n_rows,batch", [(4, 68, 16), (1, 128, 5), (8, 41, 12)])
 def test_attention_tail_of_large_launches_rows_in_any_order(group, n_rows, batch):
     """The rows of the operator come in any order, so a row may stand before its ancestors, and its CTA has to fetch keys
