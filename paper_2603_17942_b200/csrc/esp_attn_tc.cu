@@ -494,13 +494,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
     }
 }
 // ---- tail + merge: one warp per (row, head) pair (tail_pair, merge_pair).
-// TAIL_FIRST: launched behind a bulk kernel with programmatic dependent launch (see below).  Both instances add in
-// the same order and give the same bits.
-template <bool TAIL_FIRST>
-__global__ void __launch_bounds__(128, TAIL_FIRST ? 5 : 4) k_attn_tail_merge_tc(AttnArgs a) {
-    constexpr int KB8 = HD / 8;                 // 16-byte pieces of a key row loaded before they are used
-    constexpr int VB = 16;                      // value rows loaded before they are used
-    constexpr int PB = 8;                       // split partials loaded before they are merged
+// TAIL_FIRST: launched behind a bulk kernel with programmatic dependent launch (see below).  LEAN: smaller load batches
+// and 64 registers, eight CTAs per SM, for launches of their own with many waves of CTAs, where occupancy counts for more
+// than one warp's latency (see the launch rule).  All instances add in the same order and give the same bits.
+template <bool TAIL_FIRST, bool LEAN>
+__global__ void __launch_bounds__(128, LEAN ? 8 : (TAIL_FIRST ? 5 : 4)) k_attn_tail_merge_tc(AttnArgs a) {
+    constexpr int KB8 = LEAN ? 8 : HD / 8;      // 16-byte pieces of a key row loaded before they are used
+    constexpr int VB = LEAN ? 8 : 16;           // value rows loaded before they are used
+    constexpr int PB = LEAN ? 4 : 8;            // split partials loaded before they are merged
     __shared__ float s_qall[4][HD];
     if (threadIdx.x == 0) pdl_launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -860,8 +861,14 @@ int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_la
 #undef ESP_TAIL_MANY
     }
     const dim3 tgrid((rows_cap + 3) / 4, a.Hq, batch);
-    const cudaError_t e = behind_bulk ? launch_k(k_attn_tail_merge_tc<true>, tgrid, dim3(128), 0, s, tail_pdl, a)
-                                      : launch_k(k_attn_tail_merge_tc<false>, tgrid, dim3(128), 0, s, tail_pdl, a);
+    // Deeper trees (dcap > 16) of as many pairs, launched on their own: the lean instance.  Operator at KV 4096, us without ->
+    // with it: dcap 32, 1 x 68 rows x 32 heads 43.4 -> 50.9, 1 x 120 58.9 -> 55.8, 2 x 68 56.3 -> 55.7, 4 x 68 97.8 -> 91.1,
+    // 16 x 68 330 -> 301, 16 x 120 496 -> 442; dcap 48, 1 x 120 62.0 -> 60.6, 2 x 68 59.5 -> 59.6, 16 x 120 549 -> 496.
+    // (Inside a step, where the tail overlaps the bulk kernel, dcap is 16 and each CTA's own latency counts.)
+    const bool lean = behind_bulk && !pdl && pairs > TM_MIN_PAIRS;
+    const cudaError_t e = lean          ? launch_k(k_attn_tail_merge_tc<true, true>, tgrid, dim3(128), 0, s, tail_pdl, a)
+                          : behind_bulk ? launch_k(k_attn_tail_merge_tc<true, false>, tgrid, dim3(128), 0, s, tail_pdl, a)
+                                        : launch_k(k_attn_tail_merge_tc<false, false>, tgrid, dim3(128), 0, s, tail_pdl, a);
     if (e != cudaSuccess) return -1;
     return 0;
 }

@@ -114,6 +114,37 @@ def test_attention_tail_of_large_launches_bitwise(group, n_rows, batch, L):
         assert torch.equal(out[s, :n_rows], alone[0, :n_rows]), f"sequence {s}"
 
 
+@pytest.mark.parametrize("group,n_rows,batch,dcap", [(4, 68, 3, 32), (4, 128, 2, 128), (8, 41, 12, 48)])
+def test_attention_tail_of_large_launches_with_deep_trees_bitwise(group, n_rows, batch, dcap):
+    """More than 16 positions behind the root: tails of up to several 32-key chunks, in the instance that large launches take
+    for them.  Every sequence has the bits of a launch of its own (one cache split, whatever the batch)."""
+    Hkv, h, L = 8, 128, 250
+    Hq, cap = Hkv * group, L + R
+    vis = np.tril(np.ones((n_rows, n_rows), np.uint8)) if dcap == 128 else None
+    if vis is None:
+        _, depth1, vis = _tree_block(n_rows, 0, dcap, n_rows)
+    else:
+        depth1 = np.arange(n_rows)
+    g = torch.Generator(device="cuda").manual_seed(dcap)
+    q = torch.randn(batch, R, Hq, h, generator=g, device="cuda").bfloat16()
+    kc, vc = (torch.randn(batch, Hkv, cap, h, generator=g, device="cuda").bfloat16() for _ in range(2))
+    anc = np.stack([_anc_words(vis)] * batch)
+    depth = np.zeros((batch, R), np.int32)
+    depth[:, :n_rows] = depth1
+    out = _run_attention(1, q, kc, vc, anc, depth, n_rows, L, Hq, Hkv, h, dcap)
+    for s in (0, batch - 1):
+        alone = _run_attention(1, q[s:s + 1].contiguous(), kc[s:s + 1].contiguous(), vc[s:s + 1].contiguous(), anc[:1], depth[:1],
+                               n_rows, L, Hq, Hkv, h, dcap)
+        # (a launch of 128 rows x 32 heads takes the same instance: checked against fp64 as well)
+        assert torch.equal(out[s, :n_rows], alone[0, :n_rows]), f"sequence {s}"
+    sc = torch.einsum("rhd,hcd->hrc", q[0, :n_rows].double(), kc[0].repeat_interleave(group, 0)[:, :L + n_rows].double()) / h ** 0.5
+    hide = torch.zeros(n_rows, L + n_rows, dtype=torch.bool)
+    hide[:, L:] = torch.from_numpy(vis == 0)
+    ref = torch.einsum("hrc,hcd->rhd", sc.masked_fill_(hide.cuda(), -float("inf")).softmax(-1), vc[0].repeat_interleave(group, 0)[:, :L + n_rows].double())
+    # bf16 probabilities of the chunks below the tail (2^-9 each, sums of at most their number) and the result's own rounding
+    assert (out[0, :n_rows].double() - ref).abs().max() <= 2e-2
+
+
 @pytest.mark.parametrize("group,n_rows,batch", [(4, 68, 3), (1, 120, 9)])
 def test_attention_tail_of_large_launches_without_a_cache(group, n_rows, batch):
     """No cached position, so no bulk kernel in front of the tail kernel: it waits before it reads (the queries and keys come
