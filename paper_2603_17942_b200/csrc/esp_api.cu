@@ -91,6 +91,14 @@ int batch_pass(const Dims& D) {
     return D.batch < most ? D.batch : most;
 }
 
+// Cache splits of a wide prefill pass: it has its own grid, a function of its blocks and last position.  Its blocks alone
+// fill the SMs, and short splits would only add partials (each split writes 16 MB of them for 8 blocks, and the merge
+// reads them back).
+int pre_split_len(const Dims& D, int nb, int end) {
+    const int n = attn_split_len(end, nb, D.Hkv);
+    return n < D.split_len ? D.split_len : n;
+}
+
 // tree nodes including the root: max_nodes, or 1 + the fixed widths of a static tree
 int spec_nodes(const esp_spec_cfg& s) {
     if (s.n_probes > 0 && s.static_widths[0] > 0) {
@@ -160,6 +168,13 @@ int check_cfg(const esp_model_cfg* m, const esp_spec_cfg* s, Dims* D) {
         const int S = attn_split_len(m->max_seq_len, m->max_batch, m->n_kv_heads);
         D->split_len = S;
         D->n_split_max = (m->max_seq_len + RT + S - 1) / S + 1;   // a prefill block's own rows count as cache positions
+        // the most splits of any wide pass, and one (attn_split_len gives at most 16; a few ms at four million positions)
+        D->pre_split_max = D->pre_blocks && m->max_seq_len > (4 << 20) ? 17 : 0;
+        for (int nb = 2; nb <= D->pre_blocks; ++nb)
+            for (int end = nb * PREFILL_CHUNK; end < m->max_seq_len && D->pre_split_max < 17; end += PREFILL_CHUNK) {
+                const int len = pre_split_len(*D, nb, end), n = (end + len - 1) / len + 1;
+                D->pre_split_max = n > D->pre_split_max ? n : D->pre_split_max;
+            }
         D->rms_eps = m->rms_eps;
         D->k = s->n_probes; D->K = topk; D->KP = s->n_probes > 0 ? KP : 1; D->B = n_nodes; D->W = is_static ? 1 : s->expand_width;
         D->mask_slots = s->n_probes > 0 ? s->n_probes : 1;
@@ -202,8 +217,11 @@ size_t carve_all(const Dims& D, int dtype, int n_sm, char* base, Buffers* b) {
         o.attn_out_lo = reinterpret_cast<char*>(o.attn_out) + Atot * D.Hq * D.h * es;
         o.act_lo = reinterpret_cast<char*>(o.act) + Atot * D.F * es;
     }
-    o.part_o = c.take<float>(Atot * D.Hq * D.n_split_max * D.h);
-    o.part_ml = c.take<float2>(Atot * D.Hq * D.n_split_max);
+    // split partials: of the sequences of a step, or of the blocks of a wide prefill pass, which has few splits
+    const size_t step_parts = (size_t)D.batch * D.n_split_max, pre_parts = (size_t)D.pre_blocks * D.pre_split_max;
+    const size_t parts = (step_parts > pre_parts ? step_parts : pre_parts) * RT * D.Hq;
+    o.part_o = c.take<float>(parts * D.h);
+    o.part_ml = c.take<float2>(parts);
     o.cand = c.take<Cand>((size_t)n_tiles_v * Mtot * D.KP);
     o.cand_ms = c.take<float2>((size_t)n_tiles_v * Mtot);
     o.cand_floor = c.take<uint32_t>(Mtot * KP_MAX);
@@ -526,10 +544,7 @@ int forward_prefill_wide(esp_handle* h, int seq, int nb, int off) {
     const bool pdl = h->use_pdl;
     const size_t kv_seq_off = (size_t)seq * D.Hkv * D.cap * D.h * 2;
     const int rows = PREFILL_CHUNK;
-    // Cache splits: the pass has its own grid, a function of its last position.  Its blocks alone fill the SMs, and short
-    // splits would only add partials (each split writes 16 MB of them for 8 blocks, and the merge reads them back).
-    int split_len = attn_split_len(off + nb * rows, nb, D.Hkv);
-    if (split_len < D.split_len) split_len = D.split_len;
+    const int split_len = pre_split_len(D, nb, off + nb * rows);
     const int n_split_launch = (off + nb * rows + split_len - 1) / split_len;
     StreamK pending;
     memset(&pending, 0, sizeof(pending));
@@ -558,7 +573,7 @@ int forward_prefill_wide(esp_handle* h, int seq, int nb, int off) {
         a.out = b.attn_out; a.out_lo = b.attn_out_lo;
         a.part_o = b.part_o; a.part_ml = b.part_ml;
         a.st = b.pre_states;
-        a.Hq = D.Hq; a.Hkv = D.Hkv; a.h = D.h; a.cap = D.cap; a.split_len = split_len; a.n_split_max = D.n_split_max;
+        a.Hq = D.Hq; a.Hkv = D.Hkv; a.h = D.h; a.cap = D.cap; a.split_len = split_len; a.n_split_max = D.pre_split_max;
         a.dcap = DCAP_PREFILL;
         a.rows_cap = rows;
         a.cache_in_flight = 1;

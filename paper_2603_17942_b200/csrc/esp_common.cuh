@@ -71,6 +71,7 @@ struct Dims {
     int32_t blocks;     // row blocks the activation buffers hold: max(batch, pre_blocks), a row tile at least
     int32_t split_len;  // attention split length in positions (multiple of 64)
     int32_t n_split_max;
+    int32_t pre_split_max;          // the same for the wide prefill passes (their split length: pre_split_len)
     float rms_eps;
     // speculation
     int32_t k, K, KP, B, W, n_anchor, prune_parent, prune_root, ema_per_token;

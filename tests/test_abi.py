@@ -89,6 +89,18 @@ def test_workspace_bytes_and_config_checks(lib):
         P.esp_workspace_bytes(P.model_cfg(synth.LLAMA3_8B.replace(head_dim=96), 128), s)
 
 
+def test_split_partials_of_wide_prefill_passes_are_sized_by_their_own_splits(lib):
+    """A wide prefill pass covers eight blocks but few cache splits: a longer capacity adds to the workspace the cache, the
+    rotary table and the partials of the splits a pass or a step really has, 2 MB per block and split of the 8B shape
+    (eight blocks at a step's finest split would add 190 MB between these two)."""
+    s = P.spec_cfg(n_probes=4, topk=10, max_nodes=64, expand_width=0, n_anchor=1)
+
+    def extra(positions):
+        return P.esp_workspace_bytes(P.model_cfg(synth.LLAMA3_8B, positions), s) - 2 * 32 * 8 * (positions + P.ESP_MAX_ROWS) * 128 * 2
+    assert extra(8192) - extra(1300) < 100e6
+    assert extra(1 << 24) > extra(1 << 20)         # (no search over the positions of a very long capacity)
+
+
 def test_missing_library_fails_loudly(tmp_path):
     with pytest.raises(OSError):
         P.load_library(str(tmp_path / "nope.so"))
