@@ -49,6 +49,7 @@ struct Buffers {
     float* wide_partials;
     size_t wide_bytes;
     TileSrc* wide_tables;      // [prefill passes, decode passes of a batch][4][WIDE_MAX_RT][SK_TABLE_TILES], those that exist
+    char* some_tables[4];      // decode passes of a batch: items of the GEMMs when some of the sequences are idle
     TileSrc* sk_tables;   // [4][SK_TABLE_TILES]: QKV, O, gate/up, down (every layer has the same partition)
     // weights repacked for streaming (bf16 models, one sequence): per layer [qkv | o | gate/up | down], then the LM head
     char* packed;
@@ -243,22 +244,22 @@ size_t carve_all(const Dims& D, int dtype, int n_sm, char* base, Buffers* b) {
     o.pre_states = c.take<SeqState>(D.pre_blocks);
     o.wide_bytes = 0;
     const bool batched = dtype == 1 && D.batch > 1;
-    if (D.pre_blocks || batched) {
-        const int tiles[4] = {(D.Hq + 2 * D.Hkv) * D.h / TILE_N, (D.d + TILE_N - 1) / TILE_N, (D.F + 63) / 64, (D.d + TILE_N - 1) / TILE_N};
-        const int K[4] = {D.d, D.Hq * D.h, D.d, D.F};
-        for (int i = 0; i < 4; ++i)
-            for (int nb = 2; nb <= D.pre_blocks; ++nb) {
-                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, nb, PREFILL_CHUNK, 2, 2);
-                o.wide_bytes = n > o.wide_bytes ? n : o.wide_bytes;
-            }
-        for (int i = 0; i < 4 && batched; ++i)
-            for (int nb = 1; nb <= batch_pass(D); ++nb) {
-                const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, nb, D.batch_rows, D.batch_bpt, D.batch_split_bpt);
-                o.wide_bytes = n > o.wide_bytes ? n : o.wide_bytes;
-            }
-    }
+    const int tiles[4] = {(D.Hq + 2 * D.Hkv) * D.h / TILE_N, (D.d + TILE_N - 1) / TILE_N, (D.F + 63) / 64, (D.d + TILE_N - 1) / TILE_N};
+    const int K[4] = {D.d, D.Hq * D.h, D.d, D.F};
+    for (int i = 0; i < 4; ++i)
+        for (int nb = 2; nb <= D.pre_blocks; ++nb) {
+            const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, nb, PREFILL_CHUNK, 2, 2);
+            o.wide_bytes = n > o.wide_bytes ? n : o.wide_bytes;
+        }
+    for (int i = 0; i < 4 && batched; ++i)
+        for (int nb = 1; nb <= batch_pass(D); ++nb) {
+            const size_t n = wide_partial_bytes(tiles[i], (K[i] + 63) / 64, nb, D.batch_rows, D.batch_bpt, D.batch_split_bpt);
+            o.wide_bytes = n > o.wide_bytes ? n : o.wide_bytes;
+        }
     o.wide_partials = c.take<float>(o.wide_bytes / sizeof(float));
     o.wide_tables = c.take<TileSrc>((size_t)4 * WIDE_MAX_RT * SK_TABLE_TILES * ((D.pre_blocks ? 1 : 0) + (batched ? 1 : 0)));
+    for (int i = 0; i < 4 && batched; ++i)
+        o.some_tables[i] = c.take<char>(wide_some_bytes(tiles[i], (K[i] + 63) / 64, D.batch_rows, D.batch_split_bpt, batch_pass(D), D.batch));
     o.gemm_counters = c.take<int>(tc_gemm_counter_ints());
     o.sk_tables = c.take<TileSrc>(4 * SK_TABLE_TILES);
     o.layer_ptrs = c.take<const void*>((size_t)4 * D.n_layers);
@@ -369,10 +370,11 @@ int run_gemm(esp_handle* h, TcGemm* plan, int epi, int n_tiles, const void* cons
 
 // One decoder forward over the block every active sequence of [s0, s0 + nb) has in its row table.
 // Tensor-core path (bf16; the sequences' activation blocks sit RT rows apart): the layer GEMMs stream their weights once
-// for all nb sequences (one: k_gemm_tc, several: k_gemm_wide) and store stream-K partials that the next kernel sums
+// for all nb sequences (one: k_gemm_tc; of a batch: k_gemm_wide, with idle ones k_gemm_wide_some) and store stream-K partials that the next kernel sums
 // (k_qkv_finish; k_resid_norm = residual add + RMSNorm; k_swiglu_finish); the LM head runs once per up to three sequences and
 // finishes in-kernel.  CUDA-core path (fp32 models): the same layer with every epilogue fused in the GEMM.
-int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc, bool prefill) {
+// pass: sequences of the pass these are part of (steps of several sequences; see wide_gemm_launch).
+int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc, bool prefill, int pass = 0) {
     const Dims& D = h->D;
     Buffers& b = h->b;
     cudaStream_t s = h->stream;
@@ -394,14 +396,16 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
     auto plan = [&](std::vector<TcGemm*>& narrow, std::vector<TcGemm*>& w128, int l) -> TcGemm* { return wide ? w128[l] : narrow[l]; };
     // several sequences in a step: one GEMM over all their blocks (kind 0..3 = QKV, O, gate/up, down)
     const bool multi = tc && !prefill && h->p_batch[3];
+    uint32_t live = 0;                                                 // ... of which these take part
+    for (int i = 0; multi && i < nb; ++i) live |= (uint32_t)(h->ready[s0 + i] ? 1 : 0) << i;
     auto gemm = [&](int kind, TcGemm* one, int l, int epi, int n_tiles, const void* const w[3], const int32_t rows[3], const void* x, int K,
                     const EpiArgs& a) -> int {
         if (!multi) return run_gemm(h, one, epi, n_tiles, w, rows, x, K, a, tc, pdl, rc_rows);
         const size_t off[4] = {0, b.pk_qkv, b.pk_qkv + b.pk_o, b.pk_qkv + b.pk_o + b.pk_gu};
         h->launches++;
-        return wide_gemm_launch(h->p_batch[kind], b.packed + b.pk_layer * l + off[kind], st0, nb, s, pdl);
+        return wide_gemm_launch(h->p_batch[kind], b.packed + b.pk_layer * l + off[kind], st0, nb, s, pdl, pass, live);
     };
-    auto pieces = [&](int kind, const TcGemm* one) -> StreamK { return multi ? wide_gemm_streamk(h->p_batch[kind], nb) : tc_gemm_streamk(one); };
+    auto pieces = [&](int kind, const TcGemm* one) -> StreamK { return multi ? wide_gemm_streamk(h->p_batch[kind], nb, pass, live) : tc_gemm_streamk(one); };
     launch_assemble(h->dtype, st0, h->embed, mvec0, b.hres, D.d, D.mask_slots, nb, s, false, rc_rows);
     h->launches++;
     // One sequence, a block of at most 80 rows, bf16: every layer in one persistent launch (same bits as the
@@ -510,12 +514,15 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
         h->launches++;
         mark(h, KIND_MISC);
         const int n_tiles = (D.V + TILE_N - 1) / TILE_N;
-        // tensor-core path: the sequences of a pass share the LM head's weight stream too (128-row plans: one at a time;
-        // the candidate lists are shared)
+        // tensor-core path: the sequences of a pass share the LM head's weight stream too (128-row plans: one at a time; the
+        // candidate lists are shared); a launch starts and ends with a sequence that takes part
         int share = tc ? tc_gemm_nq(wide ? h->p_lm_w : h->p_lm) : nb;
         share = (nb + (nb + share - 1) / share - 1) / ((nb + share - 1) / share);      // as few launches, evenly filled
         for (int q = 0; q < nb; q += share) {
-            const int sq = s0 + q, per = nb - q < share ? nb - q : share;
+            if (multi && !(live >> q & 1)) { q -= share - 1; continue; }
+            int per = nb - q < share ? nb - q : share;
+            while (multi && !(live >> (q + per - 1) & 1)) --per;
+            const int sq = s0 + q;
             EpiArgs a = base_epi(h, D.V, sq, per);
             a.cand = b.cand; a.cand_ms = b.cand_ms; a.cand_floor = b.cand_floor; a.n_tiles = n_tiles;
             a.logits_dump = h->dbg_logits ? h->dbg_logits + (size_t)sq * RT * D.V : nullptr;
@@ -603,10 +610,11 @@ int forward(esp_handle* h, bool with_lm, int dcap, int only_seq) {
     const int per_pass = h->p_batch[3] ? batch_pass(h->D) : 1;
     for (int s0 = 0; s0 < h->D.batch; s0 += per_pass) {
         const int nb = h->D.batch - s0 < per_pass ? h->D.batch - s0 : per_pass;
-        bool any = false;
-        for (int i = s0; i < s0 + nb; ++i) any = any || h->ready[i];
-        if (!any) continue;
-        const int rc = forward_pass(h, with_lm, dcap, s0, nb, true, false);
+        int a = s0, e = s0 + nb;           // from the first sequence that takes part to the last one
+        while (a < e && !h->ready[a]) ++a;
+        while (e > a && !h->ready[e - 1]) --e;
+        if (a == e) continue;
+        const int rc = forward_pass(h, with_lm, dcap, a, e - a, true, false, nb);
         if (rc) return rc;
     }
     return ESP_OK;
@@ -809,7 +817,8 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
             TileSrc* tables = h->b.wide_tables + (D.pre_blocks ? (size_t)4 * WIDE_MAX_RT * SK_TABLE_TILES : 0);
             for (int i = 0; i < 4; ++i)
                 if (wide_gemm_create(&h->p_batch[i], tc_gemm_tiles(narrow[i]), K[i], x[i], D.blocks, D.batch_rows, D.batch_bpt, D.batch_split_bpt, batch_pass(D),
-                                     h->b.wide_partials, h->b.wide_bytes, tables + (size_t)i * WIDE_MAX_RT * SK_TABLE_TILES, h->b.err, h->stream)) {
+                                     h->b.wide_partials, h->b.wide_bytes, tables + (size_t)i * WIDE_MAX_RT * SK_TABLE_TILES, h->b.err, h->stream) ||
+                    wide_gemm_plan_some(h->p_batch[i], D.batch, h->b.some_tables[i], h->stream)) {
                     esp_free(h);
                     return ESP_E_CUDA;
                 }

@@ -136,13 +136,19 @@ int tc_gemm_counter_ints();
 struct WideGemm;
 constexpr int WIDE_MAX_RT = 4;                       // row tiles of one launch, as far as the split of k goes
 constexpr int WIDE_MAX_BLOCKS = 2 * WIDE_MAX_RT;     // full prefill blocks of one pass
+constexpr int WIDE_MAX_PASS = 3 * WIDE_MAX_RT;       // sequences of one pass of a step
 size_t wide_partial_bytes(int n_tiles, int KB, int n_blocks, int wb, int bpt, int split_bpt);
 // tables_dev: device memory for n_tiles entries per row tile of the split
 int wide_gemm_create(WideGemm** out, int n_tiles, int K, const void* x, int x_blocks, int wb, int bpt, int split_bpt, int max_blocks, float* partials,
                      size_t partial_bytes, TileSrc* tables_dev, int* err, cudaStream_t stream);
 void wide_gemm_destroy(WideGemm* g);
-int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, int n_blocks, cudaStream_t s, bool pdl);
-StreamK wide_gemm_streamk(const WideGemm* g, int n_blocks);
+// Blocks [0, n_blocks) of the plan's activation buffer.  Steps of several sequences: pass_blocks = blocks of the pass these are
+// part of (they fix the split of k), live = those that take part (bit per block; 0: all of them).
+int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, int n_blocks, cudaStream_t s, bool pdl, int pass_blocks = 0, uint32_t live = 0);
+StreamK wide_gemm_streamk(const WideGemm* g, int n_blocks, int pass_blocks = 0, uint32_t live = 0);
+// tables for passes with idle sequences: their size, and filling them (mem: device memory, 256-byte aligned)
+size_t wide_some_bytes(int n_tiles, int KB, int wb, int split_bpt, int max_blocks, int batch);
+int wide_gemm_plan_some(WideGemm* g, int batch, void* mem, cudaStream_t stream);
 
 // All layers of a step in one persistent cooperative launch (esp_layers_tc.cu): bf16, head_dim 128, blocks of at
 // most 80 rows, one sequence per pass.  Same phases, same partition and same bits as the kernels above.

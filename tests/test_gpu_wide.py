@@ -208,3 +208,56 @@ def test_prefill_leaves_every_other_sequence_alone(weights, n_seq, early):
         seen.append((h.n_out.copy(), h.tokens_out[early].copy(), logits[early, :after["n_rows"]].clone()))
         h.close()
     assert np.array_equal(seen[0][0], seen[1][0]) and np.array_equal(seen[0][1], seen[1][1]) and torch.equal(seen[0][2], seen[1][2])
+
+
+@pytest.mark.parametrize("n_seq,nodes,n_anchor", [(2, 16, 1), (3, 16, 1), (12, 16, 1), (5, 40, 1), (8, 60, 1), (4, 70, 1), (8, 70, 1), (13, 70, 1), (14, 70, 1),
+                                                   (3, 110, 1), (5, 110, 1), (13, 25, 0)])
+def test_rows_do_not_depend_on_who_else_takes_part(weights, n_seq, nodes, n_anchor):
+    """A step in which some sequences of the handle are idle packs the others into row tiles of their own: every row has the
+    bits it has when all take part, whoever is idle (the first, the last, all but one, every second), for every block size."""
+    spec = P.spec_cfg(n_probes=3, topk=5, max_nodes=nodes, expand_width=0 if n_anchor else 1, n_anchor=n_anchor)
+    prompts = [synth.make_prompt(BF16_SMALL.vocab, 17 + 40 * (i % 4), 30 + i) for i in range(n_seq)]
+    everyone = list(range(n_seq))
+    full = None
+    for who in (everyone, [0], [n_seq - 1], [n_seq // 2], everyone[:-1], everyone[1:], everyone[::2], [0, n_seq - 1], everyone[1::2], everyone[1:3]):
+        h, logits = _handle(weights, 300, spec, n_seq)
+        for i in who:
+            h.prefill(prompts[i], i)
+        rows = {i: h.state(i)["n_rows"] for i in who}
+        logits.zero_()
+        P.esp_step(h.h, h.tokens_out, h.n_out)
+        assert h.stats().device_error == 0 and [i for i in everyone if h.n_out[i]] == who
+        if full is None:
+            full = logits.clone()
+        for i in who:
+            assert torch.equal(logits[i, :rows[i]], full[i, :rows[i]]), f"{who}: sequence {i}"
+        h.close()
+
+
+def test_steps_of_a_partly_filled_handle_cost_what_takes_part():
+    """One sequence of eight: the layer GEMMs and the LM head run over its block alone.  (Layers of 0.44 GB; the step took
+    0.73 of the full one's time when a pass carried all of its blocks, 0.32 with the one that takes part.)"""
+    shape = synth.LLAMA3_8B.replace(n_layers=2, vocab=8192)
+    w = synth.make_weights(shape, 1, device="cuda")
+    spec = P.spec_cfg(n_probes=4, topk=10, max_nodes=64, expand_width=0, n_anchor=1)
+    us = []
+    for who in (range(8), [3]):
+        stream = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        h = P.Handle(shape, spec, w, 700, 8, stream)
+        for i in who:
+            h.prefill(synth.make_prompt(shape.vocab, 100, i), i)
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            h.step()
+            a.record(stream)
+            for _ in range(10):
+                h.step_async()
+            b.record(stream)
+            for _ in range(10):
+                h.read()
+            best = min(best, a.elapsed_time(b))
+        us.append(best)
+        h.close()
+    assert us[1] < 0.55 * us[0]
