@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(128, LEAN ? 8 : (TAIL_FIRST ? 5 : 4)) k_attn_t
 // serves GH pairs.  What bounded
 // the warp-per-pair kernel in such launches was its key gather (32 lanes, 32 cache lines per load: 512 L1 tag cycles
 // per pair); this one is bound by its instruction count.  Measured on their own: 16 sequences x 68 rows x 32 heads 93 -> 46
-// us, 2 x 68 x 32 20.7 -> 11.6 us; one block's 68 x 32 pairs stay with the warp-per-pair kernel (see the launch rule).
+// us, 2 x 68 x 32 20.7 -> 11.6 us; small launches stay with the warp-per-pair kernel (see the launch rule).
 constexpr int TM_WARPS = 8, TM_LD = HD + 8;               // slot stride in elements: 272 bytes, gathers without bank conflicts
 constexpr long long TM_MIN_PAIRS = 3000;
 constexpr int TM_DCAP = 16, TM_WINDOW = TM_DCAP + 15 + RT; // slots a CTA's rows can name, at most
@@ -838,8 +838,13 @@ int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_la
     const bool behind_bulk = n_split_launch > 0, tail_pdl = pdl || behind_bulk;
     const int group = a.Hq / a.Hkv;
     // From 3000 pairs on the kernel that shares keys and values between the rows and heads of a CTA (dcap 16: a row's tail is
-    // one chunk of at most 32 keys and the window fits shared memory).  Measured in a step of 120 rows x 32 heads: 1.66 ->
-    // 1.61 ms at 8 layers; at 68 x 32 the warp-per-pair kernel, part of which starts beside the bulk CTAs, is as fast.
+    // one chunk of at most 32 keys and the window fits shared memory).  Below, the warp-per-pair kernel's CTAs fit beside the
+    // bulk CTAs and run their tails there; with more of them most start when the bulk CTAs leave, and what counts is the
+    // work.  Where the two meet depends on the bulk kernel as well: its wave is shorter at 1024 positions than at 4096.
+    // Measured, us, warp per pair / shared.  Operator, KV 4096, 32 heads: 34 rows 29.7 / 33.1, 68 35.2 / 39.8, 94 (3008 pairs)
+    // 37.9 / 41.0, 108 45.1 / 45.1, 2 x 47 45.1 / 39.0, 2 x 68 48.6 / 40.7, 4 x 34 53.8 / 47.4; KV 1024: 34 rows 16.0 / 16.7, 68 21.5 /
+    // 19.3, 120 26.7 / 24.6, 2 x 47 24.9 / 18.5.  Step at 1024 positions, eight 8B layers, four runs: 32 rows 1061 / 1070, 68 1178 to
+    // 1243 / 1187 to 1224, 94 1356 to 1397 / 1359 to 1363, 128 1523 to 1620 / 1489 to 1528, 2 x 47 1520 to 1583 / 1466 to 1512.
     const long long pairs = (long long)rows_cap * a.Hq * batch;
     if (a.dcap == TM_DCAP && pairs > TM_MIN_PAIRS) {
         const int gh = group % 4 == 0 ? 4 : (group % 2 == 0 ? 2 : 1);

@@ -494,7 +494,11 @@ int tc_gemm_create(TcGemm** out, int epi, bool defer, const void* const w[3], co
     const long long U = (long long)p.n_tiles * p.KB;
     p.grid = (int)(U < n_sm ? U : n_sm);
     // A fused epilogue over a short k-range: a CTA per tile rather than tiles in pieces.  Up to 16 k-blocks pass faster than
-    // a tile's pieces meet through memory (stores, a counter, loads by the last one).
+    // a tile's pieces meet through memory (stores, a counter, loads by the last one), whatever the tiles and rows; beyond, a
+    // block of one row is faster in pieces.  Measured, us at 1 / 68 / 128 rows, pieces -> a CTA per tile: 8 tiles, 8 k-blocks 8.4 /
+    // 21.3 / 31.7 -> 6.5 / 7.7 / 9.0, 16 10.9 / 32.8 / 50.2 -> 8.7 / 10.0 / 11.3, 32 12.6 / 40.5 / 63.4 -> 13.2 / 14.5 / 15.9; 64 tiles, 8
+    // 9.8 / 16.9 / 23.0 -> 6.7 / 8.0 / 9.4, 16 11.0 / 18.8 / 25.3 -> 9.2 / 10.4 / 11.8, 32 13.3 / 21.3 / 27.8 -> 14.1 / 15.4 / 17.1, 64
+    // 17.9 / 25.9 / 32.5 -> 23.9 / 25.2 / 27.4.
     if (!defer && p.n_tiles <= n_sm && p.KB <= 16) p.grid = p.n_tiles;
     if (p.n_tiles > tc_gemm_counter_ints() || tc_gemm_partial_bytes(p.grid, nq_max, nrs) > partial_bytes) { delete g; return -1; }
     // fused epilogues store only the head and tail pieces of a range (2 slots); partial-only output stores every

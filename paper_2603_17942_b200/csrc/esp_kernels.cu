@@ -802,7 +802,9 @@ static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, 
     if (bulk_too && n_split_launch > 0) {
         const int pairs = a.rows_cap * (a.Hq / a.Hkv);
         const long long ctas4 = (long long)((pairs + 15) / 16) * a.Hkv * n_split_launch * batch;
-        // four-pair warps once their CTAs cover half of the SMs
+        // Four-pair warps once their CTAs cover half of the SMs.  Operator with the tail kernel, us, one pair / four pairs per warp:
+        // fp32, heads of 128: 36 CTAs 31 / 41, 72 39 / 43, 80 45 / 43, 128 47 / 45 and 66 / 43, 144 69 / 42, 480 147 / 88; heads of 64, whose
+        // chain is half as long, meet later: fp32 40 28 / 35, 80 31 / 35, 120 33 / 35, 240 50 / 41, bf16 128 31 / 35, 216 38 / 40, 480 66 / 53.
 #define ESP_BULK_SIMT(PW)                                                                                              \
         {                                                                                                              \
             if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_attn_bulk_simt<T, HD, VEC, PW>), (int)bulk_simt_smem<T, HD>(PW))) return -1; \

@@ -81,8 +81,9 @@ bool attn_tc_supported(int h, int Hq, int Hkv);
 // choice trades items for partial traffic.  One sequence keeps the finest split (the items are what fills the
 // SMs).  With several sequences the groups alone fill them, and the length is the one a small cost model prefers:
 // waves of items over the SMs x (1.45 us per 128-key chunk + 2.6 us per item) + the items' partial traffic.
-// It depends on nothing but the handle's capacity, batch and head count, so every row of a handle sees one
-// split grid, whatever the block it arrives in.
+// A handle's steps, and the prefill blocks that run on their own, take it from capacity, batch and head count and nothing
+// else, so their rows see one split grid whatever the block they arrive in.  (A wide prefill pass has a grid of its own, from
+// its blocks and its last position: pre_split_len.)
 inline int attn_split_len(int max_len, int batch, int Hkv) {
     int S = 256;
     while ((max_len + S - 1) / S > 16) S *= 2;
