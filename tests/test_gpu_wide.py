@@ -44,25 +44,24 @@ def test_wide_prefill_against_cuda_core_path(weights, n_prompt):
     assert (got[0] - got[1]).abs().max() <= TOL_BF16 * span
 
 
-@pytest.mark.parametrize("n_seq,nodes,n_anchor", [(2, 16, 1), (5, 16, 1), (33, 16, 1), (4, 40, 1), (2, 60, 1), (4, 70, 1), (5, 70, 1), (7, 70, 1),
-                                                   (13, 70, 1), (3, 25, 0)])
-def test_batch_steps_against_each_sequence_alone(weights, n_seq, nodes, n_anchor):
+@pytest.mark.parametrize("n_seq,nodes,n_anchor,idle", [(2, 16, 1, None), (2, 16, 1, 1), (5, 16, 1, 2), (33, 16, 1, 16), (4, 40, 1, 0), (2, 60, 1, 0), (4, 70, 1, None),
+                                                        (4, 70, 1, 2), (5, 70, 1, 3), (7, 70, 1, 2), (8, 70, 1, None), (13, 70, 1, 12), (3, 25, 0, None), (3, 25, 0, 1)])
+def test_batch_steps_against_each_sequence_alone(weights, n_seq, nodes, n_anchor, idle):
     """One step of a handle with several sequences (row tiles of every shape, ragged ones, more sequences than a
     pass covers, blocks of 100 rows) against the step each sequence takes in a handle of its own: the same trees (the
-    prefill does not depend on the batch), logits equal to the bar bf16 logits are held to; one sequence stays idle."""
+    prefill does not depend on the batch), logits equal to the bar bf16 logits are held to, for every sequence of every row
+    tile, LM-head group and pass.  All of them take part, or all but one: the first or the last of a row tile, of a pass, of
+    the handle."""
     spec = P.spec_cfg(n_probes=3, topk=5, max_nodes=nodes, expand_width=0 if n_anchor else 1, n_anchor=n_anchor)
-    idle = n_seq // 2
     h, logits = _handle(weights, 400, spec, n_seq)
     prompts = [synth.make_prompt(BF16_SMALL.vocab, 17 + 40 * (i % 5), 10 + i) for i in range(n_seq)]
-    for i in range(n_seq):
-        if i != idle:
-            h.prefill(prompts[i], i)
-    rows = {i: h.state(i)["n_rows"] for i in range(n_seq) if i != idle}
+    who = [i for i in range(n_seq) if i != idle]
+    for i in who:
+        h.prefill(prompts[i], i)
+    rows = {i: h.state(i)["n_rows"] for i in who}
     P.esp_step(h.h, h.tokens_out, h.n_out)
-    assert h.stats().device_error == 0 and h.n_out[idle] == 0
-    for i in (0, n_seq - 1):
-        if i == idle:
-            continue
+    assert h.stats().device_error == 0 and [i for i in range(n_seq) if h.n_out[i]] == who
+    for i in who:
         one, alone = _handle(weights, 400, spec)
         one.prefill(prompts[i])
         assert one.state()["n_rows"] == rows[i]
