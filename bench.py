@@ -506,8 +506,9 @@ def run_ours(args, shape, plen, k, K, B):
             "gpu_launches": launches,
             "stream_equals_greedy_tokens": stream_checked,
             "prefill": {"ms": prefill_ms, "prompt_tokens": plen * nbatch, "tokens_per_s": plen * nbatch / (prefill_ms * 1e-3),
-                        "note": "esp_prefill of every sequence from host memory, blocks of %d prompt rows" % P.ESP_PREFILL_CHUNK},
-            "roofline": {"bound": "hbm", "kernel": "k_gemm_tc<EPI_PARTIAL>, gate/up projection (235 MB of weights per launch)",
+                        "note": "esp_prefill of every sequence from host memory: full blocks of %d prompt rows, up to eight to "
+                                "a pass, then the last block on its own" % P.ESP_PREFILL_CHUNK},
+            "roofline": {"bound": "hbm", "kernel": "%s, gate/up projection (235 MB of weights per launch)" % ("k_gemm_tc<EPI_PARTIAL>" if nbatch == 1 else "k_gemm_wide"),
                          "achieved": gu_ach, "peak": peak, "unit": "GB/s", "frac": gu_ach / peak if gu_ach else None,
                          "traffic": GATEUP_DRAM_TRAFFIC.get(args.config) if nbatch == 1 and not args.per_node_probes else None,
                          "peak_source": peak_src, "bytes_per_launch": gu_bytes,

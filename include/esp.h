@@ -141,7 +141,11 @@ int esp_init(const esp_model_cfg* model, const esp_spec_cfg* spec, const esp_wei
  * embedding (Eq. mask_init_mean), runs the prompt in causal blocks with the
  * k mask rows appended to the last one, caches the prompt rows, emits the
  * first token (written to *first_token_out [host], may be NULL), applies the
- * mask update and builds the first draft tree (Algorithm 1).  Synchronises. */
+ * mask update and builds the first draft tree (Algorithm 1).  Synchronises.
+ * bf16: the full blocks before the last one run up to eight at a time, and how the sums of a block are cut follows from
+ * how many run with it.  The keys and values cached for one and the same prefix therefore agree to rounding, not bit for
+ * bit, between prompts of different length and between handles of different max_seq_len; two prefills of the same prompt
+ * in handles of the same max_seq_len and max_batch cache the same bits, whatever the spec. */
 int esp_prefill(esp_handle* h, int32_t seq, const int32_t* prompt, int32_t n_prompt, int32_t* first_token_out);
 
 /* One decode-and-verify step for every prefilled sequence (Figure 1 right):
@@ -150,6 +154,8 @@ int esp_prefill(esp_handle* h, int32_t seq, const int32_t* prompt, int32_t n_pro
  * log-sum-exp, lossless verification (Section 2),
  * KV compaction of the accepted path, mask update (Eq. mask_update_mean) and
  * the next tree (Algorithm 1 + pruner).  esp_step = esp_step_async + esp_read.
+ * A row's bits depend on its own sequence and on the handle's model, max_seq_len and max_batch, not on the spec (a tree's row
+ * has the bits of the greedy step) and not on which other sequences take part; handles of another max_batch agree to rounding.
  * tokens_out [host] [max_batch][ESP_MAX_PROBES+1], n_out [host] [max_batch].
  * esp_step_async only enqueues the step; nothing of it depends on the host, so several may be enqueued back to
  * back.  Every step leaves its result in a record of its own and esp_read returns the OLDEST unread step (0 tokens
