@@ -585,14 +585,19 @@ int wide_gemm_plan_some(WideGemm* g, int batch, void* mem, cudaStream_t stream) 
     return 0;
 }
 
-// The plan of k_gemm_wide_some for n_live of the pass's blocks, or null where k_gemm_wide is the faster: clocks of the shared-memory
+// The plan of k_gemm_wide_some for n_live of n_blocks blocks of a pass, or null where k_gemm_wide is the faster: clocks of the shared-memory
 // port per weight unit (fill + operands), times the units of the longest CTA; not less than the weights take from HBM (a unit
 // per SM and 710 clocks).
-static const WideGemm::Some* use_some(const WideGemm* g, int pass_blocks, int n_live) {
+// Measured, us per step of four 8B layers and a small LM head, k_gemm_wide / k_gemm_wide_some at 1, 2, .. sequences ready (in a row:
+// the pass ends with the last one): 68 rows, 4 sequences 963 1026 1115 / 653 718 1176; 8 sequences 1534 1608 1707 1814 1878 1929 2274 /
+// 767 803 1232 1357 1753 1883 2495; 12 sequences, 8 to 11 ready, 2679 2791 3059 3251 / 2453 2979 3129 3544; 52 rows, 8 sequences, 5 to 7 ready,
+// 1620 1711 1867 / 1560 1725 2215; 120 rows, 8 sequences, 3 to 7 ready (k_gemm_wide needs a second turn from 7 on), 2014 2216 2498 2830
+// 4238 / 1691 2344 2876 3479 4060.
+static const WideGemm::Some* use_some(const WideGemm* g, int n_blocks, int pass_blocks, int n_live) {
     for (const WideGemm::Some& s : g->some) {
         if (s.blocks != pass_blocks || n_live >= pass_blocks) continue;
-        const int n_rt = (pass_blocks + g->bpt - 1) / g->bpt, groups = g->groups[(pass_blocks + g->split_bpt - 1) / g->split_bpt - 1];
-        const double units = (double)g->p.n_ft * g->p.KB, turns = (groups * n_rt + WIDE_SM - 1) / WIDE_SM;
+        const int n_rt = (n_blocks + g->bpt - 1) / g->bpt, groups = g->groups[(pass_blocks + g->split_bpt - 1) / g->split_bpt - 1];
+        const double units = (double)g->p.n_ft * g->p.KB, turns = (groups * n_rt + WIDE_SM - 1) / WIDE_SM;      // (128-row blocks may take two)
         const double dense = turns * units / groups * (768 + 6 * g->wb * g->bpt);
         const int t = some_tiles(n_live, g->wb), rows = (n_live + t - 1) / t * g->wb;
         const double some = std::max(0.5 * s.load[t - 1] * (384 + 4 * rows), 2 * units * 710 / WIDE_SM);
@@ -661,7 +666,7 @@ int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, 
     if (pass_blocks < n_blocks) pass_blocks = n_blocks;
     const int split = (pass_blocks + g->split_bpt - 1) / g->split_bpt - 1;
     const int n_live = live ? __builtin_popcount(live) : n_blocks;
-    if (const WideGemm::Some* some = use_some(g, pass_blocks, n_live)) {
+    if (const WideGemm::Some* some = use_some(g, n_blocks, pass_blocks, n_live)) {
         SomeParams p;
         memset(&p, 0, sizeof(p));
         const int tiles = some_tiles(n_live, g->wb), most = (n_live + tiles - 1) / tiles;
@@ -718,7 +723,7 @@ int wide_gemm_launch(const WideGemm* g, const void* packed, const SeqState* st, 
 StreamK wide_gemm_streamk(const WideGemm* g, int n_blocks, int pass_blocks, uint32_t live) {
     if (pass_blocks < n_blocks) pass_blocks = n_blocks;
     const int split = (pass_blocks + g->split_bpt - 1) / g->split_bpt - 1;
-    const bool some = use_some(g, pass_blocks, live ? __builtin_popcount(live) : n_blocks) != nullptr;
+    const bool some = use_some(g, n_blocks, pass_blocks, live ? __builtin_popcount(live) : n_blocks) != nullptr;
     StreamK k;
     k.partials = g->p.partials;
     k.table = g->tables + (size_t)split * g->p.n_tiles;
