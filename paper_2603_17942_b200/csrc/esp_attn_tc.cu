@@ -493,20 +493,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
     }
 }
-// ---- tail + merge: one warp per (row, head) pair (tail_pair, merge_pair).
-// TAIL_FIRST: launched behind a bulk kernel with programmatic dependent launch (see below).  LEAN: smaller load batches
-// and 64 registers, eight CTAs per SM, for launches of their own with many waves of CTAs, where occupancy counts for more
-// than one warp's latency (see the launch rule).  All instances add in the same order and give the same bits.
-template <bool TAIL_FIRST, bool LEAN>
-__global__ void __launch_bounds__(128, LEAN ? 8 : (TAIL_FIRST ? 5 : 4)) k_attn_tail_merge_tc(AttnArgs a) {
-    constexpr int KB8 = LEAN ? 8 : HD / 8;      // 16-byte pieces of a key row loaded before they are used
-    constexpr int VB = LEAN ? 8 : 16;           // value rows loaded before they are used
-    constexpr int PB = LEAN ? 4 : 8;            // split partials loaded before they are merged
-    __shared__ float s_qall[4][HD];
+// ---- tail + merge: one warp per task of up to four heads of one row (tail_task, merge_task), four rows per CTA.
+// After a bulk launch this kernel starts once every bulk CTA's wait has returned: the kernel that wrote this step's
+// queries, keys and values has completed by then, and the tail is computed while the bulk CTAs run (one CTA of 128
+// threads fits beside a one-item bulk CTA).  Otherwise (no cached position) it waits before it reads.
+// Operator with its bulk kernel, a warp per (row, head) or keys and values of a CTA's rows in shared memory -> this, us: 1 x 68 rows
+// x 32 heads at 4096 positions 36.0 -> 34.8, 16 x 68 190.7 -> 182.1; the kernel on its own 14.6 -> 13.0 and 43 -> 32.  Step of the
+// 8B decoder at 1k positions 4.49 -> 4.35 ms.
+constexpr int TAIL_ROWS = 4;
+__global__ void __launch_bounds__(TAIL_ROWS * 32, 3) k_attn_tail_merge_tc(AttnArgs a, int gh, bool behind_bulk) {
     if (threadIdx.x == 0) pdl_launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    PairCtx c;
-    c.r = blockIdx.x * 4 + warp; c.head = blockIdx.y; c.seq = blockIdx.z;
+    TailTask c;
+    c.r = blockIdx.x * TAIL_ROWS + warp; c.head0 = blockIdx.y * gh; c.gh = gh; c.seq = blockIdx.z;
     c.depth = 0; c.lo = 0; c.hi = 0;
     // the sequence state was written by an earlier step; everything else is read after the wait
     int n_rows;
@@ -520,221 +519,12 @@ __global__ void __launch_bounds__(128, LEAN ? 8 : (TAIL_FIRST ? 5 : 4)) k_attn_t
         c.L = a.L_fixed;
         if (c.r < n_rows) { c.depth = a.depth[c.seq * RT + c.r]; c.lo = a.anc[(size_t)(c.seq * RT + c.r) * 2]; c.hi = a.anc[(size_t)(c.seq * RT + c.r) * 2 + 1]; }
     }
-    // After a bulk launch this kernel starts once every bulk CTA's wait has returned: the kernel that wrote this
-    // step's queries, keys and values has completed by then, and the tail may be computed while the bulk CTAs run.
-    // The tail reads those buffers with L2 loads only, so no stale line of an SM's L1 can be seen.
-    if (!TAIL_FIRST) pdl_wait();
+    if (!behind_bulk) pdl_wait();
     if (c.r >= n_rows) { pdl_wait(); return; }
-    FirstPartials<PB> fp;
-    if (!TAIL_FIRST) request_partials<PB>(fp, a, c, lane);      // in flight while the tail is computed
     TailAcc t;
-    tail_pair<KB8, VB>(t, a, c, s_qall[warp], lane);
-    if (TAIL_FIRST) { pdl_wait(); request_partials<PB>(fp, a, c, lane); }
-    merge_pair<PB>(fp, t, a, c, lane);
-}
-
-// ---- tail + merge for launches with many (row, head) pairs: same sums in the same order, so the same bits.
-// A CTA takes some rows of one (sequence, KV head).  The keys and values any tail of the CTA can name -- a contiguous
-// run of cache slots, from the smallest T0 of its rows to the last slot one of their ancestor masks names -- come to
-// shared memory once, and a warp works on GH query heads of one row together, so that every key and value it reads
-// serves GH pairs.  What bounded
-// the warp-per-pair kernel in such launches was its key gather (32 lanes, 32 cache lines per load: 512 L1 tag cycles
-// per pair); this one is bound by its instruction count.  Measured on their own: 16 sequences x 68 rows x 32 heads 93 -> 46
-// us, 2 x 68 x 32 20.7 -> 11.6 us; small launches stay with the warp-per-pair kernel (see the launch rule).
-constexpr int TM_WARPS = 8, TM_LD = HD + 8;               // slot stride in elements: 272 bytes, gathers without bank conflicts
-constexpr long long TM_MIN_PAIRS = 3000;
-constexpr int TM_DCAP = 16, TM_WINDOW = TM_DCAP + 15 + RT; // slots a CTA's rows can name, at most
-__host__ __device__ constexpr size_t tail_many_smem(int window, int gh) {
-    return (size_t)2 * window * TM_LD * 2 + sizeof(float) * TM_WARPS * (gh * HD + 32 * gh);
-}
-__device__ __forceinline__ void tm_copy16(void* dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-
-template <int GH>
-__global__ void __launch_bounds__(TM_WARPS * 32, 2) k_attn_tail_merge_many_tc(AttnArgs a, int rows_per_cta, int window, bool behind_bulk) {
-    extern __shared__ __align__(16) unsigned char tm_smem[];
-    __nv_bfloat16* s_k = reinterpret_cast<__nv_bfloat16*>(tm_smem);            // [window][TM_LD]
-    __nv_bfloat16* s_v = s_k + (size_t)window * TM_LD;
-    float* s_qall = reinterpret_cast<float*>(s_v + (size_t)window * TM_LD);    // [warp][GH][HD]
-    float* s_pall = s_qall + TM_WARPS * GH * HD;                               // [warp][32][GH]
-    if (threadIdx.x == 0) pdl_launch_dependents();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int kvh = blockIdx.y, seq = blockIdx.z, r_beg = blockIdx.x * rows_per_cta;
-    const int group = a.Hq / a.Hkv;
-    // The sequence state was written by an earlier step.  The queries and the block's keys and values were written by the
-    // kernel before the bulk kernel, which releases this one only after its own wait (see k_attn_tail_merge_tc); without a
-    // bulk kernel in between (no cached position), by the kernel this one has to wait for.
-    bool waited = !behind_bulk;
-    if (waited) pdl_wait();
-    int n_rows, L;
-    if (a.st) {
-        const SeqState* st = a.st + seq;
-        n_rows = st->active ? st->n_rows : 0;
-        L = st->L;
-    } else {
-        n_rows = a.n_rows_fixed;
-        L = a.L_fixed;
-    }
-    if (r_beg >= n_rows) { pdl_wait(); return; }
-    const int r_end = min(r_beg + rows_per_cta, n_rows);
-    // The window: from the smallest T0 of the CTA's rows (every warp looks at every row: at most 128) to the last block row
-    // they name.  In a step a row's ancestors stand before it; the rows of the operator come in any order.
-    int w0 = 0x7fffffff, last = r_end - 1;
-    for (int r = r_beg + lane; r < r_end; r += 32) {
-        w0 = min(w0, tail_start_tc(L + (a.st ? a.st[seq].row_depth[r] : a.depth[seq * RT + r]), a.dcap));
-        if (!a.st) last = max(last, last_set_bit128(a.anc[(size_t)(seq * RT + r) * 2], a.anc[(size_t)(seq * RT + r) * 2 + 1]));
-    }
-    w0 = __reduce_min_sync(0xffffffffu, w0);
-    last = __reduce_max_sync(0xffffffffu, last);
-    const int n_win = min(L + last + 1 - w0, window);
-    {
-        const size_t row0 = ((size_t)(a.kv_shared ? 0 : seq) * a.Hkv + kvh) * a.cap + w0;
-        const __nv_bfloat16* kb = reinterpret_cast<const __nv_bfloat16*>(a.kc) + row0 * HD;
-        const __nv_bfloat16* vb = reinterpret_cast<const __nv_bfloat16*>(a.vc) + row0 * HD;
-        for (int i = threadIdx.x; i < n_win * (HD / 8); i += TM_WARPS * 32) {
-            const int r = i / (HD / 8), j = (i % (HD / 8)) * 8;
-            tm_copy16(s_k + r * TM_LD + j, kb + (size_t)r * HD + j);
-            tm_copy16(s_v + r * TM_LD + j, vb + (size_t)r * HD + j);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncthreads();
-    float* s_q = s_qall + warp * GH * HD;
-    float* s_p = s_pall + warp * 32 * GH;
-    const int sets = group / GH;                     // GH heads of one row = one task of a warp
-    for (int task = warp; task < (r_end - r_beg) * sets; task += TM_WARPS) {
-        PairCtx c;
-        c.r = r_beg + task / sets; c.seq = seq; c.L = L;
-        const int head0 = kvh * group + (task % sets) * GH;
-        if (a.st) {
-            const SeqState* st = a.st + seq;
-            c.depth = st->row_depth[c.r]; c.lo = st->row_anc[c.r][0]; c.hi = st->row_anc[c.r][1];
-        } else {
-            const int i = seq * RT + c.r;
-            c.depth = a.depth[i]; c.lo = a.anc[(size_t)i * 2]; c.hi = a.anc[(size_t)i * 2 + 1];
-        }
-        const int P = L + c.depth, T0 = tail_start_tc(P, a.dcap), n_tail = P - T0 + 1;     // at most 32 keys
-        const __nv_bfloat16* q = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((size_t)(seq * RT + c.r) * a.Hq + head0) * HD;
-#pragma unroll
-        for (int h = 0; h < GH; ++h) {
-            const uint2 qq = __ldcg(reinterpret_cast<const uint2*>(q + h * HD + lane * 4));
-            const __nv_bfloat162 q01 = *reinterpret_cast<const __nv_bfloat162*>(&qq.x), q23 = *reinterpret_cast<const __nv_bfloat162*>(&qq.y);
-            *reinterpret_cast<float4*>(s_q + h * HD + lane * 4) = make_float4(__low2float(q01), __high2float(q01), __low2float(q23), __high2float(q23));
-        }
-        bool valid = lane < n_tail;
-        int slot = w0;
-        if (valid) {
-            const int pos = T0 + lane;
-            if (pos < L) slot = pos;
-            else {
-                const int b = nth_set_bit128(c.lo, c.hi, pos - L);
-                slot = b < 0 ? w0 + n_win : L + b;
-            }
-            if (slot - w0 >= n_win) { set_error(a.err, DEV_E_INDEX); valid = false; slot = w0; }
-        }
-        slot -= w0;
-        __syncwarp();
-        float sc[GH];
-#pragma unroll
-        for (int h = 0; h < GH; ++h) sc[h] = 0.f;
-        const uint4* kr = reinterpret_cast<const uint4*>(s_k + slot * TM_LD);
-#pragma unroll 4
-        for (int d8 = 0; d8 < HD / 8; ++d8) {
-            const uint4 kk = kr[d8];
-            const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kk);
-            float kf[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { kf[2 * i] = __low2float(k2[i]); kf[2 * i + 1] = __high2float(k2[i]); }
-#pragma unroll
-            for (int h = 0; h < GH; ++h) {
-                const float4 qa = *reinterpret_cast<const float4*>(s_q + h * HD + d8 * 8), qb = *reinterpret_cast<const float4*>(s_q + h * HD + d8 * 8 + 4);
-                sc[h] = __fmaf_rn(qa.x, kf[0], sc[h]); sc[h] = __fmaf_rn(qa.y, kf[1], sc[h]);
-                sc[h] = __fmaf_rn(qa.z, kf[2], sc[h]); sc[h] = __fmaf_rn(qa.w, kf[3], sc[h]);
-                sc[h] = __fmaf_rn(qb.x, kf[4], sc[h]); sc[h] = __fmaf_rn(qb.y, kf[5], sc[h]);
-                sc[h] = __fmaf_rn(qb.z, kf[6], sc[h]); sc[h] = __fmaf_rn(qb.w, kf[7], sc[h]);
-            }
-        }
-        TailAcc t[GH];
-#pragma unroll
-        for (int h = 0; h < GH; ++h) {
-            const float s = valid ? __fmul_rn(sc[h], a.scale_log2) : -INFINITY;
-            float cm = s;
-#pragma unroll
-            for (int of = 16; of > 0; of >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, of));
-            const float pe = valid ? exp2f(__fsub_rn(s, cm)) : 0.f;
-            float cl = pe;
-#pragma unroll
-            for (int of = 16; of > 0; of >>= 1) cl = __fadd_rn(cl, __shfl_xor_sync(0xffffffffu, cl, of));
-            s_p[lane * GH + h] = pe;
-            t[h].m = cm; t[h].l = cl;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) t[h].o[i] = 0.f;
-        }
-        __syncwarp();
-        // weighted values, keys in position order
-#pragma unroll 4
-        for (int j = 0; j < n_tail; ++j) {
-            const int sj = __shfl_sync(0xffffffffu, slot, j);
-            const uint2 vv = *reinterpret_cast<const uint2*>(s_v + sj * TM_LD + lane * 4);
-            const __nv_bfloat162 v01 = *reinterpret_cast<const __nv_bfloat162*>(&vv.x), v23 = *reinterpret_cast<const __nv_bfloat162*>(&vv.y);
-            const float v[4] = {__low2float(v01), __high2float(v01), __low2float(v23), __high2float(v23)};
-            float pj[GH];
-#pragma unroll
-            for (int h = 0; h < GH; ++h) pj[h] = s_p[j * GH + h];
-#pragma unroll
-            for (int h = 0; h < GH; ++h)
-                if (pj[h] != 0.f) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) t[h].o[i] = __fmaf_rn(pj[h], v[i], t[h].o[i]);
-                }
-        }
-        // (the warp-per-pair kernel merges its one chunk into an empty running sum: the same values)
-        if (!waited) { pdl_wait(); waited = true; }      // the bulk partials
-        __syncwarp();
-        // Merge: bulk partials in split order, the tail last.  The next split's values of all GH heads are requested
-        // before the current one's are used: a round trip per split, not per split and head.
-        const int n_sp = (T0 + a.split_len - 1) / a.split_len;
-        const size_t base = ((size_t)(seq * RT + c.r) * a.Hq + head0) * a.n_split_max;
-        float m[GH], l[GH], o[GH][4];
-        float2 ml[GH];
-        float4 c4[GH];
-        auto request = [&](int sp) {
-#pragma unroll
-            for (int h = 0; h < GH; ++h) {
-                const size_t i = base + (size_t)h * a.n_split_max + sp;
-                ml[h] = __ldcg(a.part_ml + i);
-                c4[h] = __ldcg(reinterpret_cast<const float4*>(a.part_o + i * HD + lane * 4));
-            }
-        };
-        if (n_sp > 0) request(0);
-#pragma unroll
-        for (int h = 0; h < GH; ++h) {
-            m[h] = -INFINITY; l[h] = 0.f;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) o[h][i] = 0.f;
-        }
-        for (int sp = 0; sp < n_sp; ++sp) {
-            float2 ml0[GH];
-            float4 c40[GH];
-#pragma unroll
-            for (int h = 0; h < GH; ++h) { ml0[h] = ml[h]; c40[h] = c4[h]; }
-            if (sp + 1 < n_sp) request(sp + 1);
-#pragma unroll
-            for (int h = 0; h < GH; ++h) {
-                const float co[4] = {c40[h].x, c40[h].y, c40[h].z, c40[h].w};
-                merge_ml(m[h], l[h], o[h], ml0[h].x, ml0[h].y, co);
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < GH; ++h) {
-            c.head = head0 + h;
-            merge_ml(m[h], l[h], o[h], t[h].m, t[h].l, t[h].o);
-            store_pair(l[h], o[h], a, c, lane);
-        }
-    }
-    if (!waited) pdl_wait();
+    tail_task<4>(t, a, c, lane);
+    if (behind_bulk) pdl_wait();
+    merge_task<4>(t, a, c, lane);
 }
 
 }  // namespace
@@ -837,43 +627,9 @@ int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_la
     // their own wait, so its start-up, and its tail where it fits beside them, overlaps them
     const bool behind_bulk = n_split_launch > 0, tail_pdl = pdl || behind_bulk;
     const int group = a.Hq / a.Hkv;
-    // From 3000 pairs on the kernel that shares keys and values between the rows and heads of a CTA (dcap 16: a row's tail is
-    // one chunk of at most 32 keys and the window fits shared memory).  Below, the warp-per-pair kernel's CTAs fit beside the
-    // bulk CTAs and run their tails there; with more of them most start when the bulk CTAs leave, and what counts is the
-    // work.  Where the two meet depends on the bulk kernel as well: its wave is shorter at 1024 positions than at 4096.
-    // Measured, us, warp per pair / shared.  Operator, KV 4096, 32 heads: 34 rows 29.7 / 33.1, 68 35.2 / 39.8, 94 (3008 pairs)
-    // 37.9 / 41.0, 108 45.1 / 45.1, 2 x 47 45.1 / 39.0, 2 x 68 48.6 / 40.7, 4 x 34 53.8 / 47.4; KV 1024: 34 rows 16.0 / 16.7, 68 21.5 /
-    // 19.3, 120 26.7 / 24.6, 2 x 47 24.9 / 18.5.  Step at 1024 positions, eight 8B layers, four runs: 32 rows 1061 / 1070, 68 1178 to
-    // 1243 / 1187 to 1224, 94 1356 to 1397 / 1359 to 1363, 128 1523 to 1620 / 1489 to 1528, 2 x 47 1520 to 1583 / 1466 to 1512.
-    const long long pairs = (long long)rows_cap * a.Hq * batch;
-    if (a.dcap == TM_DCAP && pairs > TM_MIN_PAIRS) {
-        const int gh = group % 4 == 0 ? 4 : (group % 2 == 0 ? 2 : 1);
-        // row groups: as many as two CTAs per SM take in one wave, none of fewer than 8 rows (one per warp)
-        int groups = 2 * 148 / (a.Hkv * batch);
-        if (groups > (rows_cap + TM_WARPS - 1) / TM_WARPS) groups = (rows_cap + TM_WARPS - 1) / TM_WARPS;
-        if (groups < 1) groups = 1;
-        const int rpc = (rows_cap + groups - 1) / groups;
-        const int window = a.st ? TM_DCAP + 15 + rows_cap : TM_WINDOW;
-        const dim3 grid((rows_cap + rpc - 1) / rpc, a.Hkv, batch);
-#define ESP_TAIL_MANY(GH)                                                                                              \
-        {                                                                                                              \
-            if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_attn_tail_merge_many_tc<GH>), (int)tail_many_smem(TM_WINDOW, GH))) return -1; \
-            return launch_k(k_attn_tail_merge_many_tc<GH>, grid, dim3(TM_WARPS * 32), tail_many_smem(window, GH), s, tail_pdl, a, rpc, window, behind_bulk) == cudaSuccess ? 0 : -1; \
-        }
-        if (gh == 4) ESP_TAIL_MANY(4)
-        if (gh == 2) ESP_TAIL_MANY(2)
-        ESP_TAIL_MANY(1)
-#undef ESP_TAIL_MANY
-    }
-    const dim3 tgrid((rows_cap + 3) / 4, a.Hq, batch);
-    // Deeper trees (dcap > 16) of as many pairs, launched on their own: the lean instance.  Operator at KV 4096, us without ->
-    // with it: dcap 32, 1 x 68 rows x 32 heads 43.4 -> 50.9, 1 x 120 58.9 -> 55.8, 2 x 68 56.3 -> 55.7, 4 x 68 97.8 -> 91.1,
-    // 16 x 68 330 -> 301, 16 x 120 496 -> 442; dcap 48, 1 x 120 62.0 -> 60.6, 2 x 68 59.5 -> 59.6, 16 x 120 549 -> 496.
-    // (Inside a step, where the tail overlaps the bulk kernel, dcap is 16 and each CTA's own latency counts.)
-    const bool lean = behind_bulk && !pdl && pairs > TM_MIN_PAIRS;
-    const cudaError_t e = lean          ? launch_k(k_attn_tail_merge_tc<true, true>, tgrid, dim3(128), 0, s, tail_pdl, a)
-                          : behind_bulk ? launch_k(k_attn_tail_merge_tc<true, false>, tgrid, dim3(128), 0, s, tail_pdl, a)
-                                        : launch_k(k_attn_tail_merge_tc<false, false>, tgrid, dim3(128), 0, s, tail_pdl, a);
+    const int gh = tail_heads(group);
+    const dim3 tgrid((rows_cap + TAIL_ROWS - 1) / TAIL_ROWS, a.Hq / gh, batch);
+    const cudaError_t e = launch_k(k_attn_tail_merge_tc, tgrid, dim3(TAIL_ROWS * 32), 0, s, tail_pdl, a, gh, behind_bulk);
     if (e != cudaSuccess) return -1;
     return 0;
 }

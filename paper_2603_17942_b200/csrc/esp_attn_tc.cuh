@@ -331,7 +331,31 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
     }
 }
 
-// ---- tail + merge: one warp per (row, head) pair
+// ---- tail + merge: one warp per task = up to TG query heads of one row that share a KV head
+// The tail of a row: positions T0..P in position order, in chunks of 32 keys anchored at T0 (one chunk for dcap 16).  Keys
+// below L are cache positions, the others block rows found through the row's ancestor mask, so every row has a key list of
+// its own: a gather, for which the list has to reach registers, and then a contraction of 4 heads x 32 keys x 128 dims
+// that mma.sync takes without staging anything (tcgen05 wants its operands in shared memory, 128 rows at a time).
+//   S = Q K^T   m16n8k16, rows 0..3 and again 4..7 the heads, columns the keys of an 8-key tile; the 128 dims are dealt to
+//               the k-steps so that a lane's 16-byte pieces of Q and K are its fragments as they come from memory;
+//   softmax     a lane holds 8 keys of head (lane / 4) % 4, lanes 4 apart share a row; both copies compute the same;
+//   O = P V     P in three bf16 pieces (hi + mid + lo = the 24 bits of the fp32 weight, products exact): hi in rows 0..3,
+//               mid in rows 4..7, lo in rows 8..11 of ONE A operand; V's 8 x 8 blocks are transposed in registers.
+// Every sum's order follows from the position in the list alone.  What bounded the kernels before this one was their
+// instruction count and a chain of dependent trips: a warp per (row, head) gathered its keys 32 cache lines per load
+// (8.6 us a task), a CTA with the keys in shared memory spent about 1700 instructions per task of four heads.
+constexpr int TG = 4;
+__host__ __device__ constexpr int tail_heads(int group) { return group % 4 == 0 ? 4 : (group % 2 == 0 ? 2 : 1); }
+
+struct TailTask {           // heads head0 .. head0 + gh - 1 (gh <= TG) of one row of one sequence
+    int r, head0, gh, seq, L, depth;
+    unsigned long long lo, hi;   // the row's ancestor-or-self mask over block rows
+};
+// A lane's share: head (lane / 4) % 4 of the task, dims 64 * (lane / 16) + 32 * j + 8 * (lane % 4) + 0..7, j = 0, 1
+struct TailAcc {
+    float m, l, o[16];
+};
+
 __device__ __forceinline__ int nth_set_bit128(unsigned long long lo, unsigned long long hi, int n) {
     int c = __popcll(lo);
     unsigned long long m = lo;
@@ -340,192 +364,223 @@ __device__ __forceinline__ int nth_set_bit128(unsigned long long lo, unsigned lo
     for (int i = 0; i < n; ++i) m &= m - 1;
     return m ? base + __ffsll((long long)m) - 1 : -1;
 }
-// highest set bit of a 128-bit mask, -1 if there is none
-__device__ __forceinline__ int last_set_bit128(unsigned long long lo, unsigned long long hi) {
-    return hi ? 127 - __clzll((long long)hi) : 63 - __clzll((long long)lo);
-}
-__device__ __forceinline__ void merge_ml(float& m, float& l, float (&o)[4], float cm, float cl, const float (&co)[4]) {
+__device__ __forceinline__ void merge_ml(float& m, float& l, float (&o)[16], float cm, float cl, const float (&co)[16]) {
     // products and sums are rounded one by one, so that every instance of the kernel rounds alike
     const float mn = fmaxf(m, cm);
     const float a = exp2f(__fsub_rn(m, mn)), b = exp2f(__fsub_rn(cm, mn));
     l = __fmaf_rn(l, a, __fmul_rn(cl, b));
 #pragma unroll
-    for (int i = 0; i < 4; ++i) o[i] = __fmaf_rn(o[i], a, __fmul_rn(co[i], b));
+    for (int i = 0; i < 16; ++i) o[i] = __fmaf_rn(o[i], a, __fmul_rn(co[i], b));
     m = mn;
 }
-
-struct PairCtx {            // one (row, head) pair of one sequence
-    int r, head, seq, L, depth;
-    unsigned long long lo, hi;   // the row's ancestor-or-self mask over block rows
-};
-struct TailAcc {            // running (max, sum, weighted values) of a key list, this lane's 4 of the 128 dims
-    float m, l, o[4];
-};
-template <int PB>
-struct FirstPartials {      // the first PB split partials of a pair, requested ahead of their use
-    float2 ml[PB];
-    float4 c4[PB];
-};
-__device__ __forceinline__ int pair_splits(const AttnArgs& a, const PairCtx& c) {
-    return (tail_start_tc(c.L + c.depth, a.dcap) + a.split_len - 1) / a.split_len;
+// D += A B, 16 x 8 x 16, bf16 in, fp32 accumulators
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-template <int PB>
-__device__ __forceinline__ void request_partials(FirstPartials<PB>& fp, const AttnArgs& a, const PairCtx& c, int lane) {
-    const int n_sp = pair_splits(a, c);
-    const size_t base = ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * a.n_split_max;
-#pragma unroll
-    for (int u = 0; u < PB; ++u) {
-        if (u < n_sp) {
-            fp.ml[u] = __ldcg(a.part_ml + base + u);
-            fp.c4[u] = __ldcg(reinterpret_cast<const float4*>(a.part_o + (base + u) * HD + lane * 4));
-        }
-    }
+// the warp's 8 x 8 block of 16-bit values (lane l: row l / 4, columns 2 * (l % 4), + 1), transposed
+__device__ __forceinline__ uint32_t transpose8x8(uint32_t x) {
+    uint32_t y;
+    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+    return y;
+}
+__device__ __forceinline__ uint32_t pack_bf16(float x, float y) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(x, y);
+    return *reinterpret_cast<const uint32_t*>(&b);
 }
 
-// The tail: positions T0..P in position order, lane j owns key j of a 32-key chunk (chunk grid anchored at T0);
-// in-flight ancestors are found through the ancestor mask.  s_q: 128 floats of shared memory owned by the warp.
-// What this step wrote shortly before, in another kernel or CTA -- the queries and the keys / values of the block's
-// own rows (slots >= L) -- is read with L2 loads (ld.global.cg), never through L1; cache positions below L were
-// written by earlier steps and go through L1, where the pairs that share a KV head find them again.
-// KB8 / VB: 16-byte key pieces / value rows in flight.
-template <int KB8, int VB>
-__device__ __forceinline__ void tail_pair(TailAcc& t, const AttnArgs& a, const PairCtx& c, float* s_q, int lane) {
-    const int kvh = c.head / (a.Hq / a.Hkv);
+// What this step wrote shortly before, in another kernel or CTA -- the queries and the keys / values of the block's own
+// rows (slots >= L) -- is read with L2 loads (ld.global.cg), never through L1; cache positions below L were written by
+// earlier steps (unless a.cache_in_flight) and go through L1, where the tasks that share a KV head find them again.
+__device__ __forceinline__ uint4 load_kv16(const __nv_bfloat16* p, bool settled) {
+    return settled ? *reinterpret_cast<const uint4*>(p) : __ldcg(reinterpret_cast<const uint4*>(p));
+}
+
+// The slot of key t of the row's list (position T0 + t), -1 if the ancestor mask does not name it.
+__device__ __forceinline__ int tail_slot(const TailTask& c, int pos) {
+    if (pos < c.L) return pos;
+    const int b = nth_set_bit128(c.lo, c.hi, pos - c.L);
+    return b < 0 ? -1 : c.L + b;
+}
+
+// JB: 32-dim columns of the keys, and then of the values, requested at once; 4: all of both ahead of any use (160 registers).
+template <int JB>
+__device__ __forceinline__ void tail_task(TailAcc& t, const AttnArgs& a, const TailTask& c, int lane) {
+    const int kvh = c.head0 / (a.Hq / a.Hkv);
     const int P = c.L + c.depth, T0 = tail_start_tc(P, a.dcap);
     const size_t kv0 = ((size_t)(a.kv_shared ? 0 : c.seq) * a.Hkv + kvh) * a.cap * HD;
-    const __nv_bfloat16* kbase = reinterpret_cast<const __nv_bfloat16*>(a.kc) + kv0;
-    const __nv_bfloat16* vbase = reinterpret_cast<const __nv_bfloat16*>(a.vc) + kv0;
-    const __nv_bfloat16* q = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * HD;
-    {
-        const uint2 qq = __ldcg(reinterpret_cast<const uint2*>(q + lane * 4));
-        const __nv_bfloat162 q01 = *reinterpret_cast<const __nv_bfloat162*>(&qq.x), q23 = *reinterpret_cast<const __nv_bfloat162*>(&qq.y);
-        s_q[lane * 4 + 0] = __low2float(q01); s_q[lane * 4 + 1] = __high2float(q01);
-        s_q[lane * 4 + 2] = __low2float(q23); s_q[lane * 4 + 3] = __high2float(q23);
-    }
-    __syncwarp();
+    const int g = lane >> 2, c4 = lane & 3;
+    const __nv_bfloat16* kbase = reinterpret_cast<const __nv_bfloat16*>(a.kc) + kv0 + c4 * 8;
+    const __nv_bfloat16* vbase = reinterpret_cast<const __nv_bfloat16*>(a.vc) + kv0 + c4 * 8;
+    const int head = c.head0 + min(g & 3, c.gh - 1);
+    const __nv_bfloat16* q = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((size_t)(c.seq * RT + c.r) * a.Hq + head) * HD + c4 * 8;
+    uint4 qf[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) qf[j] = __ldcg(reinterpret_cast<const uint4*>(q + j * 32));
     t.m = -INFINITY; t.l = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) t.o[i] = 0.f;
+    for (int i = 0; i < 16; ++i) t.o[i] = 0.f;
     const int n_tail = P - T0 + 1;
+#pragma unroll 1
     for (int t0 = 0; t0 < n_tail; t0 += 32) {
-        const int tt = t0 + lane;
-        bool valid = tt < n_tail;
-        int slot = 0;
-        if (valid) {
-            const int pos = T0 + tt;
-            if (pos < c.L) slot = pos;
-            else {
-                const int b = nth_set_bit128(c.lo, c.hi, pos - c.L);
-                if (b < 0) { set_error(a.err, DEV_E_INDEX); valid = false; }
-                else slot = c.L + b;
-            }
+        int slot = -1;
+        if (t0 + lane < n_tail) {
+            slot = tail_slot(c, T0 + t0 + lane);
+            if (slot < 0) set_error(a.err, DEV_E_INDEX);
         }
-        float sc = -INFINITY;
-        if (valid) {
-            const uint4* kr = reinterpret_cast<const uint4*>(kbase + (size_t)slot * HD);
-            float acc = 0.f;
+        // a key that is not in the chunk takes the place of one that is, with weight 0: nothing else is read
+        const uint32_t in = __ballot_sync(0xffffffffu, slot >= 0);
+        const int any = in ? __shfl_sync(0xffffffffu, slot, __ffs(in) - 1) : 0;
+        if (slot < 0) slot = any;
+        int sl[4];
 #pragma unroll
-            for (int dh = 0; dh < HD / 8; dh += KB8) {
-                uint4 kreg[KB8];
+        for (int n = 0; n < 4; ++n) sl[n] = __shfl_sync(0xffffffffu, slot, n * 8 + g);
+        auto load4x = [&](uint4 (&f)[4], const __nv_bfloat16* base, int j) {      // column j of this lane's four keys
 #pragma unroll
-                for (int d8 = 0; d8 < KB8; ++d8) kreg[d8] = slot < c.L ? kr[dh + d8] : __ldcg(kr + dh + d8);
+            for (int n = 0; n < 4; ++n) f[n] = load_kv16(base + (size_t)sl[n] * HD + j * 32, sl[n] < c.L && !a.cache_in_flight);
+        };
+        uint4 kf[JB][4], vf[JB][4];
+        float s[4][4];
 #pragma unroll
-                for (int d8 = dh; d8 < dh + KB8; ++d8) {
-                    const uint4 kk = kreg[d8 - dh];
-                    const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kk);
-                    const float4 qa = *reinterpret_cast<const float4*>(s_q + d8 * 8), qb = *reinterpret_cast<const float4*>(s_q + d8 * 8 + 4);
-                    acc = __fmaf_rn(qa.x, __low2float(k2[0]), acc); acc = __fmaf_rn(qa.y, __high2float(k2[0]), acc);
-                    acc = __fmaf_rn(qa.z, __low2float(k2[1]), acc); acc = __fmaf_rn(qa.w, __high2float(k2[1]), acc);
-                    acc = __fmaf_rn(qb.x, __low2float(k2[2]), acc); acc = __fmaf_rn(qb.y, __high2float(k2[2]), acc);
-                    acc = __fmaf_rn(qb.z, __low2float(k2[3]), acc); acc = __fmaf_rn(qb.w, __high2float(k2[3]), acc);
-                }
-            }
-            sc = __fmul_rn(acc, a.scale_log2);
+        for (int n = 0; n < 4; ++n) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s[n][i] = 0.f;
         }
-        float cm = sc;
 #pragma unroll
-        for (int of = 16; of > 0; of >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, of));
-        const float pe = valid ? exp2f(__fsub_rn(sc, cm)) : 0.f;
-        float cl = pe;
+        for (int j0 = 0; j0 < 4; j0 += JB) {
 #pragma unroll
-        for (int of = 16; of > 0; of >>= 1) cl = __fadd_rn(cl, __shfl_xor_sync(0xffffffffu, cl, of));
-        float co[4] = {0.f, 0.f, 0.f, 0.f};
-        // weighted values, keys in position order; the loads of VB keys are issued before their sums
-        // (a key that is not in the chunk reads slot 0 with weight 0 and is skipped)
-        for (int j0 = 0; j0 < 32; j0 += VB) {
-            float pj[VB];
-            uint2 vv[VB];
+            for (int j = 0; j < JB; ++j) load4x(kf[j], kbase, j0 + j);
+            if (JB == 4) {
 #pragma unroll
-            for (int u = 0; u < VB; ++u) {
-                pj[u] = __shfl_sync(0xffffffffu, pe, j0 + u);
-                const int sj = __shfl_sync(0xffffffffu, slot, j0 + u);
-                const uint2* vr = reinterpret_cast<const uint2*>(vbase + (size_t)sj * HD + lane * 4);
-                vv[u] = sj < c.L ? *vr : __ldcg(vr);
+                for (int j = 0; j < JB; ++j) load4x(vf[j], vbase, j);
             }
 #pragma unroll
-            for (int u = 0; u < VB; ++u) {
-                if (pj[u] != 0.f) {
-                    const __nv_bfloat162 v01 = *reinterpret_cast<const __nv_bfloat162*>(&vv[u].x), v23 = *reinterpret_cast<const __nv_bfloat162*>(&vv[u].y);
-                    co[0] = __fmaf_rn(pj[u], __low2float(v01), co[0]); co[1] = __fmaf_rn(pj[u], __high2float(v01), co[1]);
-                    co[2] = __fmaf_rn(pj[u], __low2float(v23), co[2]); co[3] = __fmaf_rn(pj[u], __high2float(v23), co[3]);
+            for (int j = 0; j < JB; ++j)
+#pragma unroll
+                for (int n = 0; n < 4; ++n) {
+                    mma16816(s[n], qf[j0 + j].x, 0u, qf[j0 + j].y, 0u, kf[j][n].x, kf[j][n].y);
+                    mma16816(s[n], qf[j0 + j].z, 0u, qf[j0 + j].w, 0u, kf[j][n].z, kf[j][n].w);
                 }
+        }
+        // softmax over the chunk: this lane's keys are t0 + 8 n + 2 c4 + e
+        float cm = -INFINITY;
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool ok = (in >> (8 * n + 2 * c4 + e)) & 1u;
+                s[n][e] = ok ? __fmul_rn(s[n][e], a.scale_log2) : -INFINITY;
+                cm = fmaxf(cm, s[n][e]);
             }
+        cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 1));
+        cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 2));
+        float cl = 0.f;
+        uint32_t pa[4][2];          // rows g and g + 8 of the A operand: hi and lo pieces (lanes 0..15), mid and nothing (16..31)
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            float hi[2], mid[2], lo[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool ok = (in >> (8 * n + 2 * c4 + e)) & 1u;
+                const float p = ok ? exp2f(__fsub_rn(s[n][e], cm)) : 0.f;
+                cl = __fadd_rn(cl, p);
+                hi[e] = __bfloat162float(__float2bfloat16_rn(p));
+                const float r1 = __fsub_rn(p, hi[e]);
+                mid[e] = __bfloat162float(__float2bfloat16_rn(r1));
+                lo[e] = __fsub_rn(r1, mid[e]);
+            }
+            pa[n][0] = lane < 16 ? pack_bf16(hi[0], hi[1]) : pack_bf16(mid[0], mid[1]);
+            pa[n][1] = lane < 16 ? pack_bf16(lo[0], lo[1]) : 0u;
+        }
+        cl = __fadd_rn(cl, __shfl_xor_sync(0xffffffffu, cl, 1));
+        cl = __fadd_rn(cl, __shfl_xor_sync(0xffffffffu, cl, 2));
+        float co[16];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (JB < 4 && j % JB == 0) {
+#pragma unroll
+                for (int u = 0; u < JB; ++u) load4x(vf[u], vbase, j + u);
+            }
+            float d[4][4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) d[r][i] = 0.f;
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {       // 16 keys per step
+                const uint4 x0 = vf[j % JB][2 * k], x1 = vf[j % JB][2 * k + 1];
+                const uint32_t v0[4] = {x0.x, x0.y, x0.z, x0.w}, v1[4] = {x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    mma16816(d[r], pa[2 * k][0], pa[2 * k][1], pa[2 * k + 1][0], pa[2 * k + 1][1], transpose8x8(v0[r]), transpose8x8(v1[r]));
+            }
+            // d[r]: dims 32 j + 8 c4 + 2 r, + 1; rows g (hi, or mid) and g + 8 (lo).  Lanes 0..15 keep j = 0, 1, the others 2, 3.
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float v = __fadd_rn(d[r][e], d[r][2 + e]);
+                    const float w = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 16));
+                    if ((j >> 1) == 0) { if (lane < 16) co[(j & 1) * 8 + 2 * r + e] = w; }
+                    else { if (lane >= 16) co[(j & 1) * 8 + 2 * r + e] = w; }
+                }
         }
         merge_ml(t.m, t.l, t.o, cm, cl, co);
     }
-    __syncwarp();     // s_q may be rewritten by the warp's next pair
 }
 
-// The output of a pair, o / l, as bf16 and (a.out_lo) its low-order plane; a lane owns 4 of the 128 output dims.
-__device__ __forceinline__ void store_pair(float l, const float (&o)[4], const AttnArgs& a, const PairCtx& c, int lane) {
+// The output of a task, o / l, as bf16 and (a.out_lo) its low-order plane.
+__device__ __forceinline__ void store_task(float l, const float (&o)[16], const AttnArgs& a, const TailTask& c, int lane) {
+    if (((lane >> 2) & 3) >= c.gh) return;
     const float inv = 1.0f / l;
-    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out) + ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * HD + lane * 4;
-    __nv_bfloat16 oh[4], ol[4];
+    const size_t at = ((size_t)(c.seq * RT + c.r) * a.Hq + c.head0 + ((lane >> 2) & 3)) * HD + (lane >> 4) * 64 + (lane & 3) * 8;
+    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out) + at;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float v = __fmul_rn(o[i], inv);
-        oh[i] = __float2bfloat16_rn(v);
-        ol[i] = __float2bfloat16_rn(__fsub_rn(v, __bfloat162float(oh[i])));
+    for (int j = 0; j < 2; ++j) {
+        __align__(16) __nv_bfloat16 oh[8], ol[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float v = __fmul_rn(o[j * 8 + i], inv);
+            oh[i] = __float2bfloat16_rn(v);
+            ol[i] = __float2bfloat16_rn(__fsub_rn(v, __bfloat162float(oh[i])));
+        }
+        *reinterpret_cast<uint4*>(out + j * 32) = *reinterpret_cast<const uint4*>(oh);
+        if (a.out_lo)      // low-order plane for an O projection that reads the output as hi + lo
+            *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.out_lo) + at + j * 32) = *reinterpret_cast<const uint4*>(ol);
     }
-    *reinterpret_cast<uint2*>(out) = *reinterpret_cast<const uint2*>(oh);
-    if (a.out_lo)      // low-order plane for an O projection that reads the output as hi + lo
-        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out_lo) + ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * HD + lane * 4) =
-            *reinterpret_cast<const uint2*>(ol);
 }
 
-// The merge: bulk partials in split order, the tail last; a lane owns 4 of the 128 output dims.
+// The merge: bulk partials in split order, the tail last.  PB splits are requested before they are used.
 template <int PB>
-__device__ __forceinline__ void merge_pair(const FirstPartials<PB>& fp, const TailAcc& t, const AttnArgs& a, const PairCtx& c, int lane) {
-    const int n_sp = pair_splits(a, c);
-    const size_t base = ((size_t)(c.seq * RT + c.r) * a.Hq + c.head) * a.n_split_max;
-    float m = -INFINITY, l = 0.f, o[4] = {0.f, 0.f, 0.f, 0.f};
+__device__ __forceinline__ void merge_task(const TailAcc& t, const AttnArgs& a, const TailTask& c, int lane) {
+    const int n_sp = (tail_start_tc(c.L + c.depth, a.dcap) + a.split_len - 1) / a.split_len;
+    const int head = c.head0 + min((lane >> 2) & 3, c.gh - 1);
+    const size_t base = ((size_t)(c.seq * RT + c.r) * a.Hq + head) * a.n_split_max;
+    const float* po = a.part_o + base * HD + (lane >> 4) * 64 + (lane & 3) * 8;
+    float m = -INFINITY, l = 0.f, o[16];
 #pragma unroll
-    for (int u = 0; u < PB; ++u) {
-        if (u < n_sp) {
-            const float co[4] = {fp.c4[u].x, fp.c4[u].y, fp.c4[u].z, fp.c4[u].w};
-            merge_ml(m, l, o, fp.ml[u].x, fp.ml[u].y, co);
-        }
-    }
-    for (int s0 = PB; s0 < n_sp; s0 += PB) {
+    for (int i = 0; i < 16; ++i) o[i] = 0.f;
+#pragma unroll 1
+    for (int s0 = 0; s0 < n_sp; s0 += PB) {
         float2 ml[PB];
-        float4 c4[PB];
+        float co[PB][16];
 #pragma unroll
         for (int u = 0; u < PB; ++u) {
             if (s0 + u < n_sp) {
                 ml[u] = __ldcg(a.part_ml + base + s0 + u);
-                c4[u] = __ldcg(reinterpret_cast<const float4*>(a.part_o + (base + s0 + u) * HD + lane * 4));
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    *reinterpret_cast<float4*>(&co[u][i * 4]) =
+                        __ldcg(reinterpret_cast<const float4*>(po + (size_t)(s0 + u) * HD + (i >> 1) * 32 + (i & 1) * 4));
             }
         }
 #pragma unroll
-        for (int u = 0; u < PB; ++u) {
-            if (s0 + u < n_sp) {
-                const float co[4] = {c4[u].x, c4[u].y, c4[u].z, c4[u].w};
-                merge_ml(m, l, o, ml[u].x, ml[u].y, co);
-            }
-        }
+        for (int u = 0; u < PB; ++u)
+            if (s0 + u < n_sp) merge_ml(m, l, o, ml[u].x, ml[u].y, co[u]);
     }
     merge_ml(m, l, o, t.m, t.l, t.o);
-    store_pair(l, o, a, c, lane);
+    store_task(l, o, a, c, lane);
 }
 
 }  // namespace attn

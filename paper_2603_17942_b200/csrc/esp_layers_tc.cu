@@ -82,7 +82,7 @@ struct LayersParams {
     // attention
     float* part_o;
     float2* part_ml;
-    int32_t split_len, n_split_max, dcap, group, rows_per_tile;
+    int32_t split_len, n_split_max, dcap, group, rows_per_tile, tail_heads;
     int32_t kv_rows_layer;         // rows of one layer in the K/V maps (batch * Hkv * cap)
     int32_t kv_row_seq;            // first row of this sequence inside a layer
     float scale_log2;
@@ -100,9 +100,8 @@ struct Shared {                    // behind the ring
     int abort_flag, T0max, sync_ok;
     alignas(16) float red[128];
     alignas(16) float xch[2][2 * attn::MP];
-    alignas(16) float s_q[CONS_WARPS][attn::HD];      // read as float4
 };
-static_assert(offsetof(Shared, s_q) % 16 == 0 && offsetof(Shared, full) % 8 == 0, "vector and barrier alignment");
+static_assert(offsetof(Shared, full) % 8 == 0, "barrier alignment");
 constexpr size_t SMEM_BYTES = 1024 + RING_BYTES + sizeof(Shared);
 static_assert(SMEM_BYTES <= 227 * 1024, "dynamic shared memory of one CTA");
 
@@ -453,16 +452,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_layers_tc(const __grid_const
             if (!prefetch_weights(p, sh, ring, rg, G_O, l, pol_w)) { set_error(p.err, DEV_E_WAIT_TIMEOUT); sh.abort_flag = 1; }
         } else if (warp >= 2) {
             aa.kc = kc; aa.vc = vc;
-            const int total = n_rows * p.Hq;
+            const int sets = p.Hq / p.tail_heads, total = n_rows * sets;
             for (int t = cta * CONS_WARPS + cw; t < total; t += G * CONS_WARPS) {
-                attn::PairCtx c;
-                c.r = t / p.Hq; c.head = t % p.Hq; c.seq = 0; c.L = L;
+                attn::TailTask c;
+                c.r = t / sets; c.head0 = t % sets * p.tail_heads; c.gh = p.tail_heads; c.seq = 0; c.L = L;
                 c.depth = st->row_depth[c.r]; c.lo = st->row_anc[c.r][0]; c.hi = st->row_anc[c.r][1];
-                attn::FirstPartials<8> fp;
-                attn::request_partials<8>(fp, aa, c, lane);      // in flight while the tail is computed
                 attn::TailAcc ta;
-                attn::tail_pair<16, 16>(ta, aa, c, sh.s_q[cw], lane);
-                attn::merge_pair<8>(fp, ta, aa, c, lane);
+                attn::tail_task<1>(ta, aa, c, lane);
+                attn::merge_task<2>(ta, aa, c, lane);
             }
         }
         if (!(ok = grid_sync(p, sh, epoch, stamp))) break;
@@ -558,7 +555,7 @@ int layers_tc_create(LayersTc** out, const LayersTcDesc& d) {
     p.n_layers = d.n_layers; p.d = d.d; p.Hq = d.Hq; p.Hkv = d.Hkv; p.F = d.F; p.cap = d.cap; p.qk_norm = d.qk_norm; p.rms_eps = d.rms_eps;
     p.part_o = d.part_o; p.part_ml = d.part_ml;
     p.split_len = d.split_len; p.n_split_max = d.n_split_max; p.dcap = d.dcap;
-    p.group = d.Hq / d.Hkv; p.rows_per_tile = attn::MP / p.group;
+    p.group = d.Hq / d.Hkv; p.rows_per_tile = attn::MP / p.group; p.tail_heads = attn::tail_heads(p.group);
     p.kv_rows_layer = d.batch * d.Hkv * d.cap;
     p.scale_log2 = d.scale_log2;
     p.sync_counter = d.sync_counter; p.err = d.err;
