@@ -73,6 +73,7 @@ __device__ __forceinline__ void resid_norm_row(float* xr, const StreamK& sk, int
     }
     bar();
     float tot = 0.f;
+#pragma unroll 8
     for (int gi = 0; gi < ng; ++gi) tot = __fadd_rn(tot, red[gi]);
     const float rinv = 1.0f / sqrtf(__fadd_rn(tot / (float)d, eps));
     it = 0;
@@ -154,6 +155,7 @@ __device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk
     }
     bar();
     float tot = 0.f;
+#pragma unroll 8
     for (int gi = 0; gi < ng; ++gi) tot = __fadd_rn(tot, red[gi]);
     const float rinv = 1.0f / sqrtf(__fadd_rn(tot / (float)d, eps));
 #pragma unroll
@@ -263,28 +265,59 @@ __device__ __forceinline__ void qkv_finish_task(const QkvPre<HD>& pf, const QkvA
     else dst[0] = o[0];
 }
 
-// ------------------------------------------------------------------ gate/up: eight features of one row per task
+// ------------------------------------------------------------------ gate/up: FPT features of one row per task
 // A tile holds 64 gate features (columns 0..63) and the matching 64 up features (columns 64..127).
 // en: the contributor entry of tile j0 / 64; act_row: the row's [F] activations; sr: row in the partials.
 // act_lo_row (may be NULL): the row of the low-order plane.
+// All loads of PB pieces are requested together: the sums one after the other were a round trip each, 2.8 of the kernel's 3.6
+// to 6 us behind its wait.  A tile of a large matrix has one or two pieces: eight features per thread, two pieces.  Small matrices
+// are cut into up to 15 pieces: four features, eight pieces (the small bf16 decoder: a 64-token request of it 5506 -> 5197 us with the rest of the change).
+template <int FPT, int PB>
 __device__ __forceinline__ void swiglu_task(const StreamK& sk, const SkEntry& en, int sr, __nv_bfloat16* act_row, __nv_bfloat16* act_lo_row,
                                             int j0, int F) {
-    float4 g[2], u[2];
+    constexpr int Q = FPT / 4;
+    const uint32_t w[8] = {en.e0.x, en.e0.y, en.e0.z, en.e0.w, en.e1.x, en.e1.y, en.e1.z, en.e1.w};
+    const int n = (int)(w[0] & 0xffffu);
+    const float* base = sk.partials + (size_t)sr * TILE_N + j0 % 64;     // (the last task's columns beyond F are padding of its tile)
+    float4 g[Q], u[Q];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const int j = j0 + 4 * q, f = j % 64;
-        if (j >= F) { g[q] = u[q] = make_float4(0.f, 0.f, 0.f, 0.f); continue; }
-        g[q] = sk_sum4(sk, en, sr, f);
-        u[q] = sk_sum4(sk, en, sr, 64 + f);
+    for (int q = 0; q < Q; ++q) g[q] = u[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < 15; c += PB) {
+        if (c >= n) break;
+        float4 t[PB][2 * Q];
+#pragma unroll
+        for (int e = 0; e < PB; ++e) {
+            const int hw = c + e + 1;   // halfword holding idx[c + e]
+#pragma unroll
+            for (int i = 0; i < 2 * Q; ++i) t[e][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            // (many pieces: loads without a branch, so that they do go out together; a piece that is not there reads the first)
+            const bool in = hw < 16 && c + e < n;
+            if (PB > 2 || in) {
+                const float* p = base + (size_t)((in ? w[(hw & 15) >> 1] >> ((hw & 1) * 16) : w[0] >> 16) & 0xffffu) * ((size_t)sk.rows * TILE_N);
+#pragma unroll
+                for (int i = 0; i < 2 * Q; ++i) {
+                    const float4 v = __ldcg(reinterpret_cast<const float4*>(p + (i / Q) * 64 + (i % Q) * 4));
+                    if (in) t[e][i] = v;
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < PB; ++e)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                g[q].x += t[e][q].x; g[q].y += t[e][q].y; g[q].z += t[e][q].z; g[q].w += t[e][q].w;
+                u[q].x += t[e][Q + q].x; u[q].y += t[e][Q + q].y; u[q].z += t[e][Q + q].z; u[q].w += t[e][Q + q].w;
+            }
     }
-    __nv_bfloat16 o[8], ol[8];
+    __align__(16) __nv_bfloat16 o[FPT], ol[FPT];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < Q; ++q) {
         const float gv[4] = {g[q].x, g[q].y, g[q].z, g[q].w}, uv[4] = {u[q].x, u[q].y, u[q].z, u[q].w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) split_bf16(__fmul_rn(gv[i] / __fadd_rn(1.0f, expf(-gv[i])), uv[i]), o[4 * q + i], ol[4 * q + i]);
     }
-    if (j0 + 8 <= F) {
+    if (FPT == 8 && j0 + 8 <= F) {
         *reinterpret_cast<uint4*>(act_row + j0) = *reinterpret_cast<const uint4*>(o);
         if (act_lo_row) *reinterpret_cast<uint4*>(act_lo_row + j0) = *reinterpret_cast<const uint4*>(ol);
     } else {

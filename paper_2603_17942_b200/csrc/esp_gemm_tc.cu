@@ -256,6 +256,28 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
             float* part = p.partials + ((size_t)(blockIdx.x * p.slots + sg.slot) * (NQ * NRS)) * TILE_N + f;
             // sequence by sequence: NRS accumulator columns -> that sequence's rows of the partial, or (a whole tile of a
             // fused epilogue) shared memory and the epilogue
+            if constexpr (JOINT) {
+                // 16 rows at a time, hi + lo: 70 registers a thread, so that the kernels on either side of this one fit beside
+                // its CTA -- the consumer's CTAs while it runs, the next GEMM's CTA (whose weight stream then starts early)
+                // beside the consumer's.  (All rows in registers at once: 146, 210 for 128 rows.)
+                const int nr = rows_of(0);
+#pragma unroll 1
+                for (int c = 0; c < NRS / 16; ++c) {
+                    uint32_t hi16[16], lo16[16];
+                    tmem_ld16_issue(taddr + c * 16, hi16);
+                    tmem_ld16_issue(taddr + NRS + c * 16, lo16);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (c == NRS / 16 - 1) {    // everything is in registers: hand the tensor-memory buffer back to the MMA warp
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        mbar_arrive(&tempty[buf]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (c * 16 + j < nr)
+                            __stcg(part + (size_t)(c * 16 + j) * TILE_N, __fadd_rn(__uint_as_float(hi16[j]), __uint_as_float(lo16[j])));
+                }
+                continue;
+            }
 #pragma unroll 1
             for (int sq = 0; sq < NQ; ++sq) {
                 uint32_t v[NRS];
@@ -263,16 +285,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
                 for (int c = 0; c < NRS / 16; ++c)
                     tmem_ld16_issue(taddr + sq * NRS + c * 16, *reinterpret_cast<uint32_t(*)[16]>(&v[c * 16]));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if constexpr (JOINT) {      // + the product with the low-order plane
-#pragma unroll
-                    for (int c = 0; c < NRS / 16; ++c) {
-                        uint32_t lo16[16];
-                        tmem_ld16_issue(taddr + NRS + c * 16, lo16);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) v[c * 16 + j] = __float_as_uint(__fadd_rn(__uint_as_float(v[c * 16 + j]), __uint_as_float(lo16[j])));
-                    }
-                }
                 if (sq == NQ - 1) {         // the accumulator is in registers: hand the tensor-memory buffer back to the MMA warp
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     mbar_arrive(&tempty[buf]);

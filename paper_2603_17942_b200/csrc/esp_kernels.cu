@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(NORM_MANY_WARPS * 32, 3) k_resid_norm_many(con
 // row's position L + depth, q to the query buffer, k and v to cache slot L + row.  One warp per (row, head),
 // a lane owns HD/32 consecutive features; the rotate-half partner (i, i + HD/2) sits 16 lanes away.
 template <int HD>
-__global__ void __launch_bounds__(128) k_qkv_finish(EpiArgs a, StreamK sk) {
+__global__ void __launch_bounds__(128, 16) k_qkv_finish(EpiArgs a, StreamK sk) {
     // let the next kernel start its own preamble (for a GEMM: the first weight tiles) while this one runs; it still
     // waits for this kernel to complete before it touches anything this kernel or its predecessors write
     if (threadIdx.x == 0) pdl_launch_dependents();
@@ -233,21 +233,23 @@ __global__ void __launch_bounds__(128) k_qkv_finish(EpiArgs a, StreamK sk) {
 
 // Consumer of the split gate/up GEMM: a tile holds 64 gate features (columns 0..63) and the matching 64 up
 // features (columns 64..127); sums both over the tile's contributors in CTA order and stores silu(gate) * up.
-__global__ void __launch_bounds__(256) k_swiglu_finish(const SeqState* states, int rows_fixed, StreamK sk, __nv_bfloat16* act,
+constexpr int SWIGLU_THREADS = 128;
+template <int FPT, int PB>
+__global__ void __launch_bounds__(SWIGLU_THREADS) k_swiglu_finish(const SeqState* states, int rows_fixed, StreamK sk, __nv_bfloat16* act,
                                                       __nv_bfloat16* act_lo, int F) {
     // let the next kernel start its own preamble (for a GEMM: the first weight tiles) while this one runs; it still
     // waits for this kernel to complete before it touches anything this kernel or its predecessors write
     if (threadIdx.x == 0) pdl_launch_dependents();
-    // eight features per thread: half the threads, so that the next GEMM's CTA finds registers free beside this
-    // kernel's CTAs and can start its weight stream while they run
-    const int j0 = (blockIdx.x * 256 + threadIdx.x) * 8;
-    SkEntry en;      // fixed since the plan was built: fetched before the wait (the eight features share a tile)
+    // (eight features per thread in large launches: half the threads, so that the next GEMM's CTA finds registers free
+    // beside this kernel's CTAs and can start its weight stream while they run)
+    const int j0 = (blockIdx.x * SWIGLU_THREADS + threadIdx.x) * FPT;
+    SkEntry en;      // fixed since the plan was built: fetched before the wait (a task's features share a tile)
     if (j0 < F) en = sk_entry(sk, j0 / 64);
     const int r = blockIdx.y, seq = blockIdx.z;
     const int n_rows = states ? (states[seq].active ? states[seq].n_rows : 0) : rows_fixed;   // written by an earlier step
     pdl_wait();
     if (r >= n_rows || j0 >= F) return;
-    swiglu_task(sk, en, seq * sk.seq_rows + r, act + (size_t)(seq * RT + r) * F, act_lo ? act_lo + (size_t)(seq * RT + r) * F : nullptr, j0, F);
+    swiglu_task<FPT, PB>(sk, en, seq * sk.seq_rows + r, act + (size_t)(seq * RT + r) * F, act_lo ? act_lo + (size_t)(seq * RT + r) * F : nullptr, j0, F);
 }
 
 // ------------------------------------------------------------------ CUDA-core GEMM
@@ -1459,8 +1461,11 @@ void launch_resid_norm(const SeqState* st, float* hres, const StreamK& sk, const
              (__nv_bfloat16*)y, (__nv_bfloat16*)y_lo, d, eps, copy_out);
 }
 void launch_swiglu_finish(const SeqState* st, const StreamK& sk, void* act, void* act_lo, int F, int nq, cudaStream_t s, bool pdl, int rows_cap) {
-    launch_k(k_swiglu_finish, dim3((F / 8 + 255) / 256, rows_cap, nq), dim3(256), 0, s, pdl, st, 0, sk, (__nv_bfloat16*)act,
-             (__nv_bfloat16*)act_lo, F);
+    // (a tile of a GEMM of fewer tiles than half its CTAs has more than two pieces)
+    const int fpt = sk.G > 2 * sk.n_tiles ? 4 : 8;
+    const dim3 grid(((F + fpt - 1) / fpt + SWIGLU_THREADS - 1) / SWIGLU_THREADS, rows_cap, nq);
+    if (fpt == 4) launch_k(k_swiglu_finish<4, 8>, grid, dim3(SWIGLU_THREADS), 0, s, pdl, st, 0, sk, (__nv_bfloat16*)act, (__nv_bfloat16*)act_lo, F);
+    else launch_k(k_swiglu_finish<8, 2>, grid, dim3(SWIGLU_THREADS), 0, s, pdl, st, 0, sk, (__nv_bfloat16*)act, (__nv_bfloat16*)act_lo, F);
 }
 int launch_qkv_finish(const EpiArgs& a, const StreamK& sk, int nq, cudaStream_t s, bool pdl, int rows_cap) {
     const int n_heads = a.Hq + 2 * a.Hkv;

@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_layers_tc(const __grid_const
             const long long total = (long long)n_rows * groups;
             for (long long t = (long long)cta * CONS_THREADS + (threadIdx.x - 64); t < total; t += (long long)G * CONS_THREADS) {
                 const int r = (int)(t / groups), j0 = (int)(t % groups) * 8;
-                swiglu_task(sk, sk_entry(sk, j0 / 64), r, p.act + (size_t)r * p.F, p.act_lo + (size_t)r * p.F, j0, p.F);
+                swiglu_task<8, 2>(sk, sk_entry(sk, j0 / 64), r, p.act + (size_t)r * p.F, p.act_lo + (size_t)r * p.F, j0, p.F);
             }
         }
         if (!(ok = grid_sync(p, sh, epoch, stamp))) break;
