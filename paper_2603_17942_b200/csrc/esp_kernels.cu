@@ -842,17 +842,21 @@ int launch_attn_simt(int dtype, const AttnArgs& a, int batch, int n_split_launch
 
 // ------------------------------------------------------------------ Top-K' merge over vocabulary tiles
 // One block per row: global Top-K' (value desc, id asc) of the per-tile lists, plus
-// lse = max + log(sum exp) merged over tiles in a fixed order.  The row's per-tile lists are staged in
-// shared memory (when they fit) so the K' selection rounds touch no global memory.
-constexpr int TOPK_THREADS = 256;
+// lse = max + log(sum exp) merged over tiles in a fixed order.
+// What bounds it is the number of dependent trips to L2, so there are two: the heads of all tiles' lists (with the tiles'
+// (max, sum) pairs), then the whole lists of the K' tiles with the best heads -- an entry of any other tile has K' heads
+// before it.  A vocabulary of 1002 tiles, K' = 11, 4 probe rows of 68: 25 -> 17 us (all lists of a row staged in shared
+// memory, K' rounds over all of them).
+constexpr int TOPK_THREADS = 256, TOPK_WARPS = TOPK_THREADS / 32;
 constexpr int TOPK_MAXT = 8;   // tiles per thread (n_tiles <= 2048)
 __global__ void __launch_bounds__(TOPK_THREADS) k_topk_merge(const SeqState* states, const Cand* cand, const float2* cand_ms,
-                                                             int n_tiles, int KP, int batch, Cand* topk, float* lse, int stage,
+                                                             int n_tiles, int KP, int batch, Cand* topk, float* lse,
                                                              uint32_t* cand_floor) {
-    extern __shared__ __align__(16) unsigned char tk_smem[];
-    Cand* s_c = reinterpret_cast<Cand*>(tk_smem);
     __shared__ float s_v[TOPK_THREADS];
     __shared__ int s_i[TOPK_THREADS];
+    __shared__ Cand s_w[TOPK_WARPS * KP_MAX];                         // the best heads of each warp's tiles
+    __shared__ int s_wt[TOPK_WARPS * KP_MAX], s_tile[KP_MAX];         // their tiles; the best of all
+    __shared__ Cand s_l[KP_MAX * (KP_MAX + 1) / 2];                   // what is read of the best tiles' lists
     if (threadIdx.x == 0) pdl_launch_dependents();
     const int seq = blockIdx.y, r = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const SeqState* st = states + seq;
@@ -861,108 +865,107 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_topk_merge(const SeqState* sta
     if (idle) return;
     const int Mtot = batch * RT, grow = seq * RT + r;
     const int kp = probe ? KP : 1;
-    if (stage) {
-        for (int i = tid; i < n_tiles * kp; i += TOPK_THREADS) {
-            const int t = i / kp, q = i - t * kp;
-            s_c[i] = cand[((size_t)t * Mtot + grow) * KP + q];
-        }
-        __syncthreads();
-    }
-    auto entry = [&](int t, int q) -> Cand { return stage ? s_c[t * kp + q] : cand[((size_t)t * Mtot + grow) * KP + q]; };
-    // Two levels, both by (value desc, id asc).  Level 1: each warp merges the sorted lists of its tiles (tile t
-    // belongs to thread t mod 256) into its own top kp -- a round is the lane-local best head, then two warp-wide
-    // integer reductions (largest order-preserving key, smallest id among its holders); no block barrier.
-    // Level 2: warp 0 merges the 8 warp lists the same way, one list per lane.
-    __shared__ Cand s_w[TOPK_THREADS / 32][KP_MAX];
-    unsigned char cur[TOPK_MAXT];
+    // tile t belongs to thread t mod 256
+    Cand head[TOPK_MAXT];
+    float2 ms[TOPK_MAXT];
 #pragma unroll
-    for (int i = 0; i < TOPK_MAXT; ++i) cur[i] = 0;
+    for (int i = 0; i < TOPK_MAXT; ++i) {
+        const int t = tid + TOPK_THREADS * i;
+        head[i].val = -INFINITY; head[i].id = -1;
+        ms[i] = make_float2(-INFINITY, 0.f);
+        if (t < n_tiles) {
+            head[i] = cand[((size_t)t * Mtot + grow) * KP];
+            if (probe) ms[i] = cand_ms[(size_t)t * Mtot + grow];
+        }
+    }
+    if (tid < KP_MAX) s_tile[tid] = -1;
+    // each warp's kp best heads, in order: a round is the lane-local best, then two warp-wide integer reductions (largest
+    // order-preserving key, smallest id among its holders); no block barrier
     for (int j = 0; j < kp; ++j) {
         float bv = -INFINITY;
         int bi = 0x7fffffff, bt = -1;
 #pragma unroll
-        for (int i = 0; i < TOPK_MAXT; ++i) {
-            const int t = tid + TOPK_THREADS * i;
-            if (t < n_tiles && cur[i] < kp) {
-                const Cand c = entry(t, cur[i]);
-                if (c.id >= 0 && cand_before(c.val, c.id, bv, bi)) { bv = c.val; bi = c.id; bt = i; }
-            }
-        }
+        for (int i = 0; i < TOPK_MAXT; ++i)
+            if (head[i].id >= 0 && cand_before(head[i].val, head[i].id, bv, bi)) { bv = head[i].val; bi = head[i].id; bt = i; }
         const uint32_t key = bt >= 0 ? float_order_key(bv) : 0u;
         const uint32_t wkey = __reduce_max_sync(0xffffffffu, key);
         const uint32_t wid = __reduce_min_sync(0xffffffffu, (bt >= 0 && key == wkey) ? (uint32_t)bi : 0xffffffffu);
         if (bt >= 0 && key == wkey && (uint32_t)bi == wid) {   // token ids are unique across tiles: one owner
 #pragma unroll
-            for (int i = 0; i < TOPK_MAXT; ++i) if (i == bt) cur[i]++;
-            s_w[warp][j].val = bv;
-            s_w[warp][j].id = bi;
+            for (int i = 0; i < TOPK_MAXT; ++i) if (i == bt) head[i].id = -1;
+            s_w[warp * kp + j].val = bv;
+            s_w[warp * kp + j].id = bi;
+            s_wt[warp * kp + j] = tid + TOPK_THREADS * bt;
         }
-        if (wkey == 0u && lane == 0) { s_w[warp][j].val = -INFINITY; s_w[warp][j].id = -1; }
+        if (wkey == 0u && lane == 0) { s_w[warp * kp + j].val = -INFINITY; s_w[warp * kp + j].id = -1; }
     }
     __syncthreads();
-    if (warp == 0) {
-        int c2 = 0;     // this lane's cursor into warp list `lane`
-        for (int j = 0; j < kp; ++j) {
-            float bv = -INFINITY;
-            int bi = 0x7fffffff;
-            bool have = false;
-            if (lane < TOPK_THREADS / 32 && c2 < kp) {
-                const Cand c = s_w[lane][c2];
-                if (c.id >= 0) { bv = c.val; bi = c.id; have = true; }
+    // the kp best of the warps' heads, by rank (ids are unique)
+    Cand none;
+    none.val = -INFINITY; none.id = -1;
+    if (tid < TOPK_WARPS * kp) {
+        const Cand c = s_w[tid];
+        if (c.id >= 0) {
+            int rank = 0;
+            for (int o = 0; o < TOPK_WARPS * kp; ++o) rank += s_w[o].id >= 0 && cand_before(s_w[o].val, s_w[o].id, c.val, c.id) ? 1 : 0;
+            if (rank < kp) {
+                s_tile[rank] = s_wt[tid];
+                if (!probe) topk[(size_t)grow * KP_MAX] = c;
             }
-            const uint32_t key = have ? float_order_key(bv) : 0u;
-            const uint32_t wkey = __reduce_max_sync(0xffffffffu, key);
-            const uint32_t wid = __reduce_min_sync(0xffffffffu, (have && key == wkey) ? (uint32_t)bi : 0xffffffffu);
-            if (have && key == wkey && (uint32_t)bi == wid) {
-                ++c2;
-                topk[(size_t)grow * KP_MAX + j].val = bv;
-                topk[(size_t)grow * KP_MAX + j].id = bi;
-            }
-            if (wkey == 0u && lane == 0) { topk[(size_t)grow * KP_MAX + j].val = -INFINITY; topk[(size_t)grow * KP_MAX + j].id = -1; }
         }
     }
     __syncthreads();
-    if (probe) {
-        // thread-strided partial merges in tile order, then a fixed tree over threads
-        float m = -INFINITY, sm = 0.f;
-        for (int t = tid; t < n_tiles; t += TOPK_THREADS) {
-            const float2 ms = cand_ms[(size_t)t * Mtot + grow];
-            const float mn = fmaxf(m, ms.x);
-            sm = sm * expf(m - mn) + ms.y * expf(ms.x - mn);
+    if (!probe) {
+        if (tid == 0 && s_tile[0] < 0) topk[(size_t)grow * KP_MAX] = none;
+        return;
+    }
+    // Their lists: entry q of the tile with the p-th best head has p heads and q entries of its own before it, so only
+    // p + q < kp matter.  The kp best of these by rank.
+    for (int i = tid; i < kp * kp; i += TOPK_THREADS) {
+        const int p = i / kp, q = i % kp;
+        if (p + q < kp) s_l[p * kp - p * (p - 1) / 2 + q] = s_tile[p] >= 0 ? cand[((size_t)s_tile[p] * Mtot + grow) * KP + q] : none;
+    }
+    if (tid < kp) topk[(size_t)grow * KP_MAX + tid] = none;     // (if there are fewer)
+    // thread-strided partial merges in tile order, then a fixed tree over threads
+    float m = -INFINITY, sm = 0.f;
+#pragma unroll
+    for (int i = 0; i < TOPK_MAXT; ++i) {
+        if (tid + TOPK_THREADS * i < n_tiles) {
+            const float mn = fmaxf(m, ms[i].x);
+            sm = sm * expf(m - mn) + ms[i].y * expf(ms[i].x - mn);
             m = mn;
         }
-        float* s_s = reinterpret_cast<float*>(s_i);
-        s_v[tid] = m;
-        s_s[tid] = sm;
-        __syncthreads();
-        for (int o = TOPK_THREADS / 2; o > 0; o >>= 1) {
-            if (tid < o) {
-                const float m1 = s_v[tid], m2 = s_v[tid + o];
-                const float s1 = s_s[tid], s2 = s_s[tid + o];
-                const float mn = fmaxf(m1, m2);
-                const float sn = (m1 == -INFINITY ? 0.f : s1 * expf(m1 - mn)) + (m2 == -INFINITY ? 0.f : s2 * expf(m2 - mn));
-                s_v[tid] = mn;
-                s_s[tid] = sn;
-            }
-            __syncthreads();
-        }
-        if (tid == 0) lse[grow] = s_v[0] + logf(s_s[0]);
-        if (tid < KP_MAX && cand_floor) cand_floor[(size_t)grow * KP_MAX + tid] = 0;     // nothing is known about the next forward's logits
     }
+    float* s_s = reinterpret_cast<float*>(s_i);
+    s_v[tid] = m;
+    s_s[tid] = sm;
+    __syncthreads();
+    const int n_l = kp * (kp + 1) / 2;
+    for (int i = tid; i < n_l; i += TOPK_THREADS) {
+        const Cand c = s_l[i];
+        if (c.id < 0) continue;
+        int rank = 0;
+        for (int o = 0; o < n_l; ++o) rank += s_l[o].id >= 0 && cand_before(s_l[o].val, s_l[o].id, c.val, c.id) ? 1 : 0;
+        if (rank < kp) topk[(size_t)grow * KP_MAX + rank] = c;
+    }
+    for (int o = TOPK_THREADS / 2; o > 0; o >>= 1) {
+        if (tid < o) {
+            const float m1 = s_v[tid], m2 = s_v[tid + o];
+            const float s1 = s_s[tid], s2 = s_s[tid + o];
+            const float mn = fmaxf(m1, m2);
+            const float sn = (m1 == -INFINITY ? 0.f : s1 * expf(m1 - mn)) + (m2 == -INFINITY ? 0.f : s2 * expf(m2 - mn));
+            s_v[tid] = mn;
+            s_s[tid] = sn;
+        }
+        __syncthreads();
+    }
+    if (tid == 0) lse[grow] = s_v[0] + logf(s_s[0]);
+    if (tid < KP_MAX && cand_floor) cand_floor[(size_t)grow * KP_MAX + tid] = 0;     // nothing is known about the next forward's logits
 }
 
 void launch_topk_merge(const SeqState* st, const Cand* cand, const float2* cand_ms, int n_tiles, int KP, int batch,
                        Cand* topk, float* lse, cudaStream_t s, bool pdl, int rows_cap, uint32_t* cand_floor) {
-    dim3 grid(rows_cap, batch);
-    size_t smem = (size_t)n_tiles * KP * sizeof(Cand);
-    int stage = smem <= 160 * 1024 ? 1 : 0;
-    if (!stage) smem = 0;
-    static size_t attr_bytes = 0;
-    if (smem > attr_bytes) {
-        cudaFuncSetAttribute(k_topk_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr_bytes = smem;
-    }
-    launch_k(k_topk_merge, grid, dim3(TOPK_THREADS), smem, s, pdl, st, cand, cand_ms, n_tiles, KP, batch, topk, lse, stage, cand_floor);
+    launch_k(k_topk_merge, dim3(rows_cap, batch), dim3(TOPK_THREADS), 0, s, pdl, st, cand, cand_ms, n_tiles, KP, batch, topk, lse, cand_floor);
 }
 
 // ------------------------------------------------------------------ sampling noise, stand-alone (for checking)
