@@ -978,16 +978,18 @@ void launch_gumbel_noise(uint32_t key0, uint32_t key1, uint32_t position, int n,
 }
 
 // ------------------------------------------------------------------ row-table builders
-__device__ void write_probe_rows(SeqState* st, int N, int k, int first_anchor, int n_anchor_rows) {
+// (depth, anc: those of the tree's rows; threads tid, tid + n_threads, .. take part)
+__device__ void write_probe_rows(SeqState* st, int N, int k, int first_anchor, int n_anchor_rows, const int* depth,
+                                 const unsigned long long (*anc)[2], int tid, int n_threads) {
     // probe j (1-based) of the a-th anchored node sits at row N + a*k + (j-1)
-    for (int i = threadIdx.x; i < n_anchor_rows * k; i += blockDim.x) {
+    for (int i = tid; i < n_anchor_rows * k; i += n_threads) {
         int aidx = i / k, j = i % k + 1;
         int u = first_anchor + aidx;
         int row = N + aidx * k + (j - 1);
         st->row_token[row] = -1;
         st->row_parent[row] = j == 1 ? u : row - 1;
-        st->row_depth[row] = st->row_depth[u] + j;
-        unsigned long long lo = st->row_anc[u][0], hi = st->row_anc[u][1];
+        st->row_depth[row] = depth[u] + j;
+        unsigned long long lo = anc[u][0], hi = anc[u][1];
         for (int jj = 0; jj < j; ++jj) {
             int b = N + aidx * k + jj;
             if (b < 64) lo |= 1ull << b; else hi |= 1ull << (b - 64);
@@ -1030,7 +1032,7 @@ __global__ void k_setup_chain(SeqState* states, int seq, const int32_t* prompt_d
     SeqState* st = states + seq;
     write_chain_rows(st, prompt_dev, off, n);
     __syncthreads();
-    if (last && k > 0) write_probe_rows(st, n, k, n - 1, 1);
+    if (last && k > 0) write_probe_rows(st, n, k, n - 1, 1, st->row_depth, st->row_anc, threadIdx.x, blockDim.x);
     if (threadIdx.x == 0) {
         st->n_nodes = n;
         st->n_rows = n + (last ? k : 0);
@@ -1061,7 +1063,7 @@ __global__ void k_set_tree(SeqState* states, int seq, const int32_t* tokens, con
     }
     __syncthreads();
     int nA = k > 0 ? (n_anchor == 0 ? n : min(n_anchor, n)) : 0;
-    write_probe_rows(st, n, k, 0, nA);
+    write_probe_rows(st, n, k, 0, nA, st->row_depth, st->row_anc, threadIdx.x, blockDim.x);
     if (threadIdx.x == 0) { st->n_rows = n + nA * k; st->mode = 0; st->forced = 1; }
 }
 
@@ -1076,44 +1078,70 @@ __device__ __forceinline__ unsigned long long node_key(float lp, int depth, int 
     return ((unsigned long long)(~u) << 32) | ((unsigned long long)depth << 16) | (unsigned long long)idx;
 }
 
+// What bounds it is one block's chain of short phases: every barrier, every dependent trip to L2 and every loop of dependent
+// shared-memory loads counts.  So the first half of the block does what the next forward pass's rows hang on -- verification,
+// lists, tree, row table -- and the other half compacts the cache and updates the masks meanwhile; keys are ranked from
+// packed arrays, breadth-first places come from bit masks, and counters and the error word are fetched ahead of their use.
+// 64 nodes, K = 10, four probes: 48 -> 32 us for the ranking alone, step of eight 8B layers 1278 -> 1255 us with the halves; 16 nodes, K = 5, three probes: its request 5209 -> 4680 us a step of 35 kernels.
+constexpr int TREE_THREADS = 1024, TREE_BUILD = 512;      // threads; those of them that build the tree
+__device__ __forceinline__ void tree_bar() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
+__device__ __forceinline__ bool tree_bar_or(bool x) {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 512, p;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(r) : "r"((uint32_t)x) : "memory");
+    return r != 0;
+}
+// keys of the n given ones that are smaller
+__device__ __forceinline__ int rank_among(const unsigned long long* keys, int n, unsigned long long key) {
+    int rank = 0;
+#pragma unroll 4
+    for (int o = 0; o + 1 < n; o += 2) {
+        const ulonglong2 k2 = *reinterpret_cast<const ulonglong2*>(keys + o);
+        rank += (k2.x < key ? 1 : 0) + (k2.y < key ? 1 : 0);
+    }
+    if (n & 1) rank += keys[n - 1] < key ? 1 : 0;
+    return rank;
+}
+
 template <typename T>
-__global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
-    extern __shared__ unsigned char smem_raw[];
-    int* c_tok = reinterpret_cast<int*>(smem_raw);
+__global__ void __launch_bounds__(TREE_THREADS) k_tree_step(TreeArgs A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned long long* c_sort = reinterpret_cast<unsigned long long*>(smem_raw);      // [MAX_CAND] keys that are ranked
+    int* c_tok = reinterpret_cast<int*>(c_sort + MAX_CAND);
     int* c_par = c_tok + MAX_CAND;
     int* c_dep = c_par + MAX_CAND;
     float* c_lp = reinterpret_cast<float*>(c_dep + MAX_CAND);
-    int* c_rank = reinterpret_cast<int*>(c_lp + MAX_CAND);
+    int* c_row = reinterpret_cast<int*>(c_lp + MAX_CAND);            // creation index -> new row
     __shared__ int s_path[PROBES_MAX + 2], s_out[PROBES_MAX + 2];
-    __shared__ int s_na, s_ustar, s_delta, s_nexp, s_ncreated, s_abort;
-    __shared__ int s_exp[RT], s_sel[RT], s_new[RT];
-    __shared__ int s_rtok[RT], s_rpar[RT], s_rdep[RT], s_arg[RT];   // this step's row table and per-row argmax
-    __shared__ int s_cnt[3], s_nsurv;
-    __shared__ int s_keep[PROBES_MAX * RT], s_nkeep;                  // per depth, the B-1 best nodes: the only ones the final pick can take
+    __shared__ int s_na, s_ustar, s_delta, s_nexp, s_ncreated, s_nkeep, s_nsurv, s_abort, s_err;
+    __shared__ int s_exp[RT], s_sel[RT];
+    __shared__ int s_rtok[RT], s_rpar[RT], s_rdep[RT], s_arg[RT];     // this step's row table and per-row argmax
+    __shared__ __align__(16) unsigned long long s_keep[PROBES_MAX * RT];      // per depth, the keys of the B-1 best nodes: the only ones the final pick can take
+    __shared__ unsigned long long s_anc[RT][2];                       // the next tree's ancestor masks
+    __shared__ uint32_t s_dmask[PROBES_MAX + 1][RT / 32];             // by depth: which selection ranks stand there
     __shared__ Cand s_list[PROBES_MAX][KP_MAX];                       // Top-K' lists of the probes the next tree uses
     __shared__ float s_lse[PROBES_MAX];
-    unsigned long long* c_key = reinterpret_cast<unsigned long long*>(c_rank + MAX_CAND);   // total-order keys
-    unsigned long long* c_sort = c_key + MAX_CAND;                                           // scratch of the sorts
 
     // Before the wait: the sequence's state and row table, which only this kernel and the set-up of a prefill block (plain
     // launches) write.
     const Dims& D = A.D;
-    const int seq = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+    const int seq = blockIdx.x, tid = threadIdx.x, nt = TREE_THREADS, lane = tid & 31;
     SeqState* st = A.states + seq;
     // where this launch's record goes; every sequence, active or not, counts the handle's decode steps
     const unsigned long long rec_no = st->rec;
     int32_t* rec = A.out_ring + ((size_t)(A.is_step ? (int)(rec_no % NREC) : NREC) * D.batch + seq) * RING;
-    const int active = st->active, mode = st->mode, N0 = st->n_nodes, L0 = st->L;
+    const int active = st->active, mode = st->mode, N0 = st->n_nodes, L0 = st->L, rows0 = st->n_rows;
     for (int r = tid; r < N0 && r < RT; r += nt) {
         s_rtok[r] = st->row_token[r];
         s_rpar[r] = st->row_parent[r];
         s_rdep[r] = st->row_depth[r];
     }
+    if (tid == 0) { s_abort = 0; s_err = 0; s_nsurv = 0; }
     pdl_wait();
+    const int err0 = tid == 0 ? __ldcg(A.err) : 0;       // the error word before this kernel
     __syncthreads();      // every thread has read the counter
     if (A.is_step && tid == 0) st->rec = rec_no + 1;
     if (!active) {
-        if (tid == 0) { rec[0] = 0; rec[RING - 1] = __ldcg(A.err); }
+        if (tid == 0) { rec[0] = 0; rec[RING - 1] = err0; }
         return;
     }
     const int grow0 = seq * RT;
@@ -1122,10 +1150,11 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
         if (tid == 0) st->L = L0 + N0;
         return;
     }
+    auto fail = [&](int code) { set_error(A.err, code); atomicCAS(&s_err, 0, code); };
     for (int r = tid; r < N0; r += nt) {
         const int t = A.topk[(size_t)(grow0 + r) * KP_MAX].id;
         s_arg[r] = t >= 0 ? t : 0;                       // a row of NaN has no arg-max: its token would index the embeddings
-        if (t < 0) set_error(A.err, DEV_E_INDEX);
+        if (t < 0) fail(DEV_E_INDEX);
     }
     __syncthreads();
 
@@ -1156,7 +1185,6 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
         }
         __syncwarp();
         if (tid == 0) {
-            s_abort = 0;
             if (mode != 2) {
                 // deepest anchored node on the accepted path
                 int nA = D.k > 0 ? (D.n_anchor == 0 ? N0 : min(D.n_anchor, N0)) : 0;
@@ -1166,57 +1194,58 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
                 s_delta = a - s_rdep[us];
             }
             s_na = a;
-            st->n_out = n_emit;
-            for (int q = 0; q < n_emit; ++q) st->out_tokens[q] = s_out[q];
-            rec[0] = n_emit;
-            rec[1] = mode == 2 ? L0 + N0 : L0 + a + 1;
-            for (int q = 0; q < n_emit; ++q) rec[2 + q] = s_out[q];
-            if (mode == 0) {
-                const int rows = st->n_rows;
-                st->rows_hist[rows <= 16 ? 0 : (rows <= 32 ? 1 : (rows <= 64 ? 2 : 3))] += 1;
-                st->steps += 1;
-                st->emitted += n_emit;
-                st->accept_hist[a < PROBES_MAX ? a : PROBES_MAX] += 1;
-            }
         }
     }
     __syncthreads();
     const int a_acc = s_na;
     const int n_emit = mode == 2 ? 1 : a_acc + 1;
-
-    // ---- KV compaction: cache slot L+j <- row p_j for the accepted path (row 0 is already at slot L).
-    // Sources sit at or above their destination, so increasing j with a barrier in between is safe.
-    if (mode == 0) {
-        const int vec_per_row = D.h * (int)sizeof(T) / 16;
-        const size_t layer_stride = (size_t)D.batch * D.Hkv * D.cap * D.h;
-        const int per_j = D.n_layers * D.Hkv * 2 * vec_per_row;
-        for (int j = 1; j <= a_acc; ++j) {
-            const int src = L0 + s_path[j], dst = L0 + j;
-            if (src != dst) {
-                for (int i = tid; i < per_j; i += nt) {
-                    int v = i % vec_per_row, rest = i / vec_per_row;
-                    int kv = rest & 1;
-                    rest >>= 1;
-                    int hh = rest % D.Hkv, l = rest / D.Hkv;
-                    T* basep = reinterpret_cast<T*>(kv ? A.vcache : A.kcache) + (size_t)l * layer_stride +
-                               ((size_t)seq * D.Hkv + hh) * D.cap * D.h;
-                    const uint4* s4 = reinterpret_cast<const uint4*>(basep + (size_t)src * D.h) + v;
-                    uint4* d4 = reinterpret_cast<uint4*>(basep + (size_t)dst * D.h) + v;
-                    *d4 = *s4;
-                }
-            }
-            __syncthreads();
-        }
-    }
     const int Lnew = mode == 2 ? L0 + N0 : L0 + a_acc + 1;
 
-    // ---- mask update, Eq. (mask_update_mean): m <- m + lambda (e - m)
-    {
+    if (tid >= TREE_BUILD) {
+        // ================ the other half: record, counters, KV compaction, masks
+        const int ht = tid - TREE_BUILD, hn = TREE_THREADS - TREE_BUILD;
+        if (ht == 0) {
+            st->n_out = n_emit;
+            for (int q = 0; q < n_emit; ++q) st->out_tokens[q] = s_out[q];
+            rec[0] = n_emit;
+            rec[1] = Lnew;
+            for (int q = 0; q < n_emit; ++q) rec[2 + q] = s_out[q];
+            if (mode == 0) {
+                st->rows_hist[rows0 <= 16 ? 0 : (rows0 <= 32 ? 1 : (rows0 <= 64 ? 2 : 3))] += 1;
+                st->steps += 1;
+                st->emitted += n_emit;
+                st->accept_hist[a_acc < PROBES_MAX ? a_acc : PROBES_MAX] += 1;
+            }
+        }
+        // ---- KV compaction: cache slot L+j <- row p_j for the accepted path (row 0 is already at slot L).  A thread moves the
+        // same 16 bytes of every row, all read before the first is written: sources sit at or above their destination, and
+        // nothing a thread reads is written by another.
+        if (mode == 0 && a_acc > 0) {
+            const int vec_per_row = D.h * (int)sizeof(T) / 16;
+            const size_t layer_stride = (size_t)D.batch * D.Hkv * D.cap * D.h;
+            const int per_j = D.n_layers * D.Hkv * 2 * vec_per_row;
+            for (int i = ht; i < per_j; i += hn) {
+                const int v = i % vec_per_row;
+                int rest = i / vec_per_row;
+                const int kv = rest & 1;
+                rest >>= 1;
+                const int hh = rest % D.Hkv, l = rest / D.Hkv;
+                T* basep = reinterpret_cast<T*>(kv ? A.vcache : A.kcache) + (size_t)l * layer_stride + ((size_t)seq * D.Hkv + hh) * D.cap * D.h;
+                uint4 x[PROBES_MAX];
+#pragma unroll
+                for (int j = 1; j <= PROBES_MAX; ++j)
+                    if (j <= a_acc) x[j - 1] = reinterpret_cast<const uint4*>(basep + (size_t)(L0 + s_path[j]) * D.h)[v];
+#pragma unroll
+                for (int j = 1; j <= PROBES_MAX; ++j)
+                    if (j <= a_acc && s_path[j] != j) reinterpret_cast<uint4*>(basep + (size_t)(L0 + j) * D.h)[v] = x[j - 1];
+            }
+        }
+        // ---- mask update, Eq. (mask_update_mean): m <- m + lambda (e - m)
         const T* E = reinterpret_cast<const T*>(A.embed);
         float* m = A.mvec + (size_t)seq * D.mask_slots * D.d;
         // four consecutive elements per thread; every load of a pass is issued before the first store
         const int e0 = D.ema_per_token ? 0 : n_emit - 1;
-        for (int j = tid * 4; j < D.d; j += nt * 4) {
+        for (int j = ht * 4; j < D.d; j += hn * 4) {
             float ev[PROBES_MAX + 2][4];
             float4 mv[PROBES_MAX];
             for (int e = e0; e < n_emit; ++e)
@@ -1244,191 +1273,195 @@ __global__ void __launch_bounds__(1024) k_tree_step(TreeArgs A) {
                 }
             }
         }
+        return;
     }
 
-    // ---- next tree (Algorithm 1 with the pruner).  Depth i draws from probe delta+i of u*.
+    // ================ the first half: next tree (Algorithm 1 with the pruner).  Depth i draws from probe delta+i of u*.
     const int root_tok = s_out[n_emit - 1];
     const int ustar = s_ustar, delta = s_delta;
     const int Dd = D.k - delta > 0 ? D.k - delta : 0;
-    if (tid == 0) {
-        c_tok[0] = root_tok; c_par[0] = -1; c_dep[0] = 0; c_lp[0] = 0.f;
-        s_exp[0] = 0; s_nexp = 1; s_ncreated = 1; s_nkeep = 0;
-    }
     // the probe lists the tree draws from, staged once
-    for (int w = tid; w < Dd * KP_MAX; w += nt) {
+    for (int w = tid; w < Dd * KP_MAX; w += TREE_BUILD) {
         const int i = w / KP_MAX + 1, q = w % KP_MAX;
         const int prow = mode == 2 ? N0 + (i - 1) : N0 + ustar * D.k + (delta + i - 1);
         s_list[i - 1][q] = A.topk[(size_t)(grow0 + prow) * KP_MAX + q];
         if (q == 0) s_lse[i - 1] = A.lse[grow0 + prow];
     }
-    __syncthreads();
+    if (tid == 0) {
+        c_tok[0] = root_tok; c_par[0] = -1; c_dep[0] = 0; c_lp[0] = 0.f; c_row[0] = 0;
+        s_exp[0] = 0; s_nexp = 1; s_ncreated = 1; s_nkeep = 0;
+    }
+    for (int r = tid; r < RT; r += TREE_BUILD) s_sel[r] = -1;
+    tree_bar();
     for (int i = 1; i <= Dd; ++i) {
         // Algorithm 1 draws min(K, B-i) candidates per expanded node; a static tree its fixed width for this depth
         const int pool = D.static_w[0] > 0 ? D.static_w[i - 1] : min(D.K, D.B - i);
         if (pool <= 0) break;
         const Cand* list = s_list[i - 1];
         const float lse_i = s_lse[i - 1];
-        const int base = s_ncreated, n_exp = s_nexp;
+        const int base = s_ncreated, n_exp = s_nexp, keep0 = s_nkeep;
         const int n_new = n_exp * pool;
-        if (base + n_new > MAX_CAND) { if (tid == 0) { set_error(A.err, DEV_E_TREE_OVERFLOW); s_abort = 1; } }
-        __syncthreads();
-        if (s_abort) break;
-        for (int w = tid; w < n_new; w += nt) {
-            const int e = w / pool, j = w % pool;
-            const int p = s_exp[e];
-            const int ptok = c_tok[p];
-            int seen = 0, q = 0;
-            for (; q < D.KP; ++q) {
-                int t = list[q].id;
-                if (D.prune_parent && t == ptok) continue;
-                if (D.prune_root && t == root_tok) continue;
-                if (seen == j) break;
-                ++seen;
-            }
-            const int c = base + w;
-            if (ptok >= 0 && q < D.KP && list[q].id >= 0) {
-                c_tok[c] = list[q].id;
-                c_lp[c] = __fadd_rn(c_lp[p], __fsub_rn(list[q].val, lse_i));
-            } else {  // list exhausted (logits of NaN; K' = K + pruner flags otherwise): neither it nor its children selectable
-                c_tok[c] = -1;
-                c_lp[c] = -INFINITY;
-            }
-            c_par[c] = p;
-            c_dep[c] = i;
-            c_key[c] = node_key(c_lp[c], i, c);
-        }
-        __syncthreads();
+        if (base + n_new > MAX_CAND) { if (tid == 0) fail(DEV_E_TREE_OVERFLOW); break; }
         const int width = D.W == 0 ? D.B - i : min(D.W, D.B - i);
         // Ranks of the new nodes among themselves (same depth: logP desc, creation asc) matter only below
-        // R = max(width, B-1).  With many new nodes, first find by bisection on the keys' high words (the logP
-        // part) the smallest bound that at least R keys do not exceed; only the nodes within it are ranked.
+        // R = max(width, B-1).  The expanded nodes stand in the order of their logP and all draw from one sorted list, of which
+        // the pruner takes at most two entries for each: child j of the e-th node has the children up to j - 2 of every node
+        // before it, and its own j earlier siblings, before it.  Where these are R it need not be ranked.  (Rounding keeps the
+        // order and equal values go by creation; a NaN would break it, then every node is ranked.)  64 nodes, K = 10: 313 of
+        // 620 nodes at the third depth.
         const int R = min(max(width, D.B - 1), RT);
-        const int n_kept = min(min(D.B - 1, RT), n_new), keep0 = s_nkeep;
-        int* surv = reinterpret_cast<int*>(c_sort);     // creation indices of the nodes that may rank below R
-        int n_surv = n_new;
-        if (n_new > 4 * R) {
-            unsigned hk[MAX_CAND / 1024];               // high words of this thread's keys (n_new <= MAX_CAND)
-            bool hv[MAX_CAND / 1024];
-#pragma unroll
-            for (int q = 0; q < MAX_CAND / 1024; ++q) {
-                const int w = tid + q * nt;
-                hv[q] = w < n_new;
-                hk[q] = hv[q] ? (unsigned)(c_key[base + w] >> 32) : 0u;
+        const int n_kept = min(min(D.B - 1, RT), n_new);
+        // the keys to rank, packed (whole warps run along: the places of a warp's keys come from one addition)
+        auto put = [&](bool in, unsigned long long key) {
+            const uint32_t who = __ballot_sync(0xffffffffu, in);
+            int at = 0;
+            if (lane == 0 && who) at = atomicAdd(&s_nsurv, __popc(who));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (in) c_sort[at + __popc(who & ((1u << lane) - 1u))] = key;
+        };
+        bool saw_nan = false;
+        for (int w0 = 0; w0 < n_new; w0 += TREE_BUILD) {
+            const int w = w0 + tid;
+            bool in = false;
+            unsigned long long key = 0;
+            if (w < n_new) {
+                const int e = w / pool, j = w % pool;
+                const int p = s_exp[e];
+                const int ptok = c_tok[p];
+                int seen = 0, q = D.KP;                  // the j-th entry that the pruner leaves
+#pragma unroll 4
+                for (int u = 0; u < D.KP; ++u) {
+                    const int t = list[u].id;
+                    const bool cut = (D.prune_parent && t == ptok) || (D.prune_root && t == root_tok);
+                    if (!cut) {
+                        if (seen == j) q = min(q, u);
+                        ++seen;
+                    }
+                }
+                const int c = base + w;
+                float lp = -INFINITY;
+                int tok = -1;      // list exhausted (logits of NaN; K' = K + pruner flags otherwise): neither it nor its children selectable
+                if (ptok >= 0 && q < D.KP && list[q].id >= 0) {
+                    tok = list[q].id;
+                    lp = __fadd_rn(c_lp[p], __fsub_rn(list[q].val, lse_i));
+                }
+                c_tok[c] = tok;
+                c_lp[c] = lp;
+                c_par[c] = p;
+                c_dep[c] = i;
+                key = node_key(lp, i, c);
+                saw_nan |= isnan(lp);
+                in = e * (j - 1) + j < R;
             }
-            if (tid == 0) { s_cnt[0] = 0; s_cnt[1] = 0; s_cnt[2] = 0; s_nsurv = 0; }
-            __syncthreads();
-            unsigned lo = 0u, hi = 0xffffffffu;         // count(high word <= hi) >= R throughout
-            for (int it = 0; lo < hi; ++it) {
-                const unsigned mid = lo + ((hi - lo) >> 1);
-                if (tid == 0) s_cnt[(it + 1) % 3] = 0;  // last read two barriers ago
-                int mine = 0;
-#pragma unroll
-                for (int q = 0; q < MAX_CAND / 1024; ++q) mine += (hv[q] && hk[q] <= mid) ? 1 : 0;
-                mine = __reduce_add_sync(0xffffffffu, mine);
-                if ((tid & 31) == 0 && mine) atomicAdd(&s_cnt[it % 3], mine);
-                __syncthreads();
-                if (s_cnt[it % 3] >= R) hi = mid; else lo = mid + 1;
-            }
-#pragma unroll
-            for (int q = 0; q < MAX_CAND / 1024; ++q)
-                if (hv[q] && hk[q] <= lo) surv[atomicAdd(&s_nsurv, 1)] = base + tid + q * nt;
-            __syncthreads();
-            n_surv = s_nsurv;
-        } else {
-            for (int w = tid; w < n_new; w += nt) surv[w] = base + w;
-            __syncthreads();
+            put(in, key);
         }
-        for (int w = tid; w < n_surv; w += nt) {
-            const int c = surv[w];
-            const unsigned long long key = c_key[c];
-            int rank = 0;
-            for (int o = 0; o < n_surv; ++o) rank += c_key[surv[o]] < key ? 1 : 0;
-            if (rank < width) s_exp[rank] = c;
+        if (tree_bar_or(saw_nan)) {
+            if (tid == 0) s_nsurv = 0;
+            tree_bar();
+            for (int w0 = 0; w0 < n_new; w0 += TREE_BUILD) {
+                const int w = w0 + tid;
+                put(w < n_new, w < n_new ? node_key(c_lp[base + w], i, base + w) : 0ull);
+            }
+            tree_bar();
+        }
+        const int n_surv = s_nsurv;
+        for (int w = tid; w < n_surv; w += TREE_BUILD) {
+            const unsigned long long key = c_sort[w];
+            const int rank = rank_among(c_sort, n_surv, key);
+            if (rank < width) s_exp[rank] = (int)(key & 0xffffu);          // (the creation index)
             // a node with B-1 or more nodes of its own depth before it cannot be among the B-1 best overall
-            if (rank < n_kept) s_keep[keep0 + rank] = c;
+            if (rank < n_kept) s_keep[keep0 + rank] = key;
         }
-        __syncthreads();
         if (tid == 0) { s_ncreated = base + n_new; s_nexp = min(width, n_new); s_nkeep = keep0 + n_kept; }
-        __syncthreads();
+        tree_bar();
+        if (tid == 0) s_nsurv = 0;      // (the next depth adds to it behind its own first barrier ...)
+        tree_bar();
     }
+    tree_bar();
     // final selection: root + the B-1 best created nodes by (logP desc, depth asc, creation asc)
     // (ranked among the kept nodes only: every node that precedes one of the B-1 best is itself kept)
     const int n_keep = s_nkeep;
-    for (int r = tid; r < RT; r += nt) s_sel[r] = -1;
-    __syncthreads();
-    for (int w = tid; w < n_keep; w += nt) {
-        const int c = s_keep[w];
-        const unsigned long long key = c_key[c];
-        int rank = 0;
-        for (int o = 0; o < n_keep; ++o) rank += c_key[s_keep[o]] < key ? 1 : 0;
-        c_rank[c] = rank;
+    for (int w = tid; w < n_keep; w += TREE_BUILD) {
+        const unsigned long long key = s_keep[w];
+        const int c = (int)(key & 0xffffu), rank = rank_among(s_keep, n_keep, key);
         if (rank < D.B - 1 && c_tok[c] >= 0 && rank < RT) s_sel[rank] = c;
     }
-    __syncthreads();
-    int n_sel = min(D.B - 1, n_keep);
-    // (entries with token -1 rank last because their logP is -inf; drop them)
-    if (tid == 0) {
-        int n = 0;
-        while (n < n_sel && s_sel[n] >= 0) ++n;
-        s_nexp = n;
-    }
-    __syncthreads();
-    n_sel = s_nexp;
-    // breadth-first row order: by depth, ties by selection rank
-    for (int r = tid; r < n_sel; r += nt) {
-        const int c = s_sel[r], dp = c_dep[c];
-        int idx = 1;
-        for (int o = 0; o < n_sel; ++o) {
-            const int d2 = c_dep[s_sel[o]];
-            idx += (d2 < dp || (d2 == dp && o < r)) ? 1 : 0;
+    tree_bar();
+    // Breadth-first row order: by depth, ties by selection rank.  (Entries with token -1 rank last because their logP is -inf:
+    // what is selected ends with the first empty place.)
+    int n_sel = 0, idx = 0;
+    const int c_mine = tid < RT ? s_sel[tid] : -1;
+    {
+        const int most = min(D.B - 1, n_keep);
+        bool open = true;
+        for (int r0 = 0; r0 < RT && open; r0 += 32) {
+            const uint32_t ok = __ballot_sync(0xffffffffu, r0 + lane < most && s_sel[r0 + lane] >= 0);
+            n_sel += ok == 0xffffffffu ? 32 : __ffs(~ok) - 1;
+            open = ok == 0xffffffffu;
         }
-        s_new[r] = idx;
-        c_rank[c] = idx;  // creation index -> new row index
     }
-    if (tid == 0) c_rank[0] = 0;
-    __syncthreads();
+    const int dp = tid < n_sel ? c_dep[c_mine] : 0;
+    if (tid < RT)
+        for (int d = 1; d <= Dd; ++d) {
+            const uint32_t who = __ballot_sync(0xffffffffu, dp == d);
+            if (lane == 0) s_dmask[d][tid >> 5] = who;
+        }
+    tree_bar();
+    if (tid < n_sel) {
+        idx = 1;
+        for (int d = 1; d < dp; ++d)
+#pragma unroll
+            for (int w = 0; w < RT / 32; ++w) idx += __popc(s_dmask[d][w]);
+#pragma unroll
+        for (int w = 0; w < RT / 32; ++w)
+            if (w < (tid >> 5)) idx += __popc(s_dmask[dp][w]);
+        idx += __popc(s_dmask[dp][tid >> 5] & ((1u << lane) - 1u));
+        c_row[c_mine] = idx;
+    }
+    tree_bar();
     const int N = n_sel + 1;
-    for (int r = tid; r < n_sel; r += nt) {
-        const int c = s_sel[r], row = s_new[r];
-        st->row_token[row] = c_tok[c];
-        st->row_parent[row] = c_rank[c_par[c]];
-        st->row_depth[row] = c_dep[c];
-        st->row_logp[row] = c_lp[c];
+    if (tid < n_sel) {
         // ancestor-or-self mask by walking up the creation-time parents
         unsigned long long lo = 0, hi = 0;
-        for (int x = c; x >= 0; x = c_par[x]) {
-            int b = c_rank[x];
+        for (int x = c_mine; x >= 0; x = c_par[x]) {
+            const int b = c_row[x];
             if (b < 64) lo |= 1ull << b; else hi |= 1ull << (b - 64);
         }
-        st->row_anc[row][0] = lo;
-        st->row_anc[row][1] = hi;
+        st->row_token[idx] = c_tok[c_mine];
+        st->row_parent[idx] = c_row[c_par[c_mine]];
+        st->row_depth[idx] = dp;
+        st->row_logp[idx] = c_lp[c_mine];
+        st->row_anc[idx][0] = s_anc[idx][0] = lo;
+        st->row_anc[idx][1] = s_anc[idx][1] = hi;
+        s_rdep[idx] = dp;
     }
-    if (tid == 0) {
+    if (tid == RT) {
         st->row_token[0] = root_tok; st->row_parent[0] = -1; st->row_depth[0] = 0; st->row_logp[0] = 0.f;
-        st->row_anc[0][0] = 1ull; st->row_anc[0][1] = 0ull;
+        st->row_anc[0][0] = s_anc[0][0] = 1ull; st->row_anc[0][1] = s_anc[0][1] = 0ull;
+        s_rdep[0] = 0;
     }
-    __syncthreads();
+    tree_bar();
     const int nA = D.k > 0 ? (D.n_anchor == 0 ? N : min(D.n_anchor, N)) : 0;
-    write_probe_rows(st, N, D.k, 0, nA);
+    write_probe_rows(st, N, D.k, 0, nA, s_rdep, s_anc, tid, TREE_BUILD);
     if (tid == 0) {
         st->n_nodes = N;
         st->n_rows = N + nA * D.k;
         st->L = Lnew;
         st->mode = 0;
         st->forced = 0;
-        if (Lnew + RT > D.cap) set_error(A.err, DEV_E_CAPACITY);
-        rec[RING - 1] = atomicAdd(A.err, 0);       // the error word as this step leaves it
+        if (Lnew + RT > D.cap) fail(DEV_E_CAPACITY);
+        rec[RING - 1] = err0 ? err0 : s_err;       // the error word as this step leaves it
     }
 }
 
 void launch_tree_step(int dtype, const TreeArgs& A, cudaStream_t s, bool pdl) {
-    size_t smem = (size_t)MAX_CAND * 36;
+    size_t smem = (size_t)MAX_CAND * 28;
     if (dtype == 0) {
         ensure_dynamic_smem(reinterpret_cast<const void*>(k_tree_step<float>), (int)smem);
-        launch_k(k_tree_step<float>, dim3(A.D.batch), dim3(1024), smem, s, pdl, A);
+        launch_k(k_tree_step<float>, dim3(A.D.batch), dim3(TREE_THREADS), smem, s, pdl, A);
     } else {
         ensure_dynamic_smem(reinterpret_cast<const void*>(k_tree_step<__nv_bfloat16>), (int)smem);
-        launch_k(k_tree_step<__nv_bfloat16>, dim3(A.D.batch), dim3(1024), smem, s, pdl, A);
+        launch_k(k_tree_step<__nv_bfloat16>, dim3(A.D.batch), dim3(TREE_THREADS), smem, s, pdl, A);
     }
 }
 
