@@ -529,47 +529,92 @@ __device__ __forceinline__ void attn_row_info(const AttnArgs& a, int seq, int r,
     }
 }
 
-// One chunk of up to 32 keys for one (row, head) handled by one warp: lane j owns key j (its row gathered straight
-// from the cache).  Returns the chunk's own (max, sum, weighted values) relative to its own max, in the log2 domain.
-// Every load of a key row, and eight value rows at a time, are in flight together (lanes without a key hold slot 0,
-// whose value row is read and not used).  VEC: the cache starts on 16 bytes.
-template <typename T, int HD, bool VEC>
-__device__ __forceinline__ void warp_chunk(const float* s_q, const T* kbase, const T* vbase, int slot, bool valid,
-                                           float scale_log2, float& cm, float& cl, float (&co)[HD / 32]) {
-    const int lane = threadIdx.x & 31;
-    float s = -INFINITY;
-    if (valid) {
-        const T* kr = kbase + (size_t)slot * HD;
-        float acc = 0.f;
-        if constexpr (VEC) {
+// E consecutive elements as floats, read from L2 (VEC: 16 bytes aligned, or all of them if they are fewer)
+template <typename T, int E, bool VEC>
+__device__ __forceinline__ void load_row(float (&v)[E], const T* p) {
+    if constexpr (!VEC) {
 #pragma unroll
-            for (int d = 0; d < HD; d += 4) {
-                const float4 kv = load_f4(kr + d), qv = load_f4(s_q + d);
-                acc = fmaf(qv.w, kv.w, fmaf(qv.z, kv.z, fmaf(qv.y, kv.y, fmaf(qv.x, kv.x, acc))));
-            }
-        } else {
-#pragma unroll 16
-            for (int d = 0; d < HD; ++d) acc = fmaf(s_q[d], to_f32(kr[d]), acc);
+        for (int i = 0; i < E; ++i) {
+            if constexpr (sizeof(T) == 4) v[i] = __ldcg(p + i);
+            else v[i] = __bfloat162float(__ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p) + i)));
         }
-        s = acc * scale_log2;
+    } else if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int i = 0; i < E; i += 4) {
+            const float4 x = __ldcg(reinterpret_cast<const float4*>(p + i));
+            v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < E; i += 4) {
+            const uint2 x = __ldcg(reinterpret_cast<const uint2*>(p + i));
+            const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&x.x), hi = *reinterpret_cast<const __nv_bfloat162*>(&x.y);
+            v[i] = __low2float(lo); v[i + 1] = __high2float(lo); v[i + 2] = __low2float(hi); v[i + 3] = __high2float(hi);
+        }
     }
-    cm = warp_max(s);
-    float p = valid ? exp2f(s - cm) : 0.f;
-    cl = warp_sum(p);
+}
+
+// One chunk of up to 32 keys for one (row, head) handled by one warp; lane j names the cache slot of key j.  Returns the
+// chunk's own (max, sum, weighted values) relative to its own max, in the log2 domain.
+// Scores: eight lanes per key, HD / 8 dims each, four keys side by side, so that a load touches whole rows (a lane per key
+// touches 32 cache lines per load: 13 us of the tiny decoder's step per layer, now 0.8 behind the cache kernel, its 64-token request 8530 -> 7446 us); values: a lane per dim.
+// Keys, and values, of RB rounds (of VB keys) are in flight together (lanes without a key hold the slot of one that is
+// there; its value row is read and not used).  VEC: the cache starts on 16 bytes.
+template <typename T, int HD, bool VEC>
+__device__ __forceinline__ void warp_chunk(const float (&q)[HD / 8], const T* kbase, const T* vbase, int slot, uint32_t valid,
+                                           float scale_log2, float& cm, float& cl, float (&co)[HD / 32]) {
+    constexpr int E = HD / 8, RB = HD == 128 ? 4 : 8, VB = HD == 128 ? 16 : 32;
+    const int lane = threadIdx.x & 31, kg = lane >> 3;
+    float s[8];
+#pragma unroll
+    for (int u0 = 0; u0 < 8; u0 += RB) {
+        float k[RB][E];
+#pragma unroll
+        for (int u = 0; u < RB; ++u) load_row<T, E, VEC>(k[u], kbase + (size_t)__shfl_sync(0xffffffffu, slot, 4 * (u0 + u) + kg) * HD + (lane & 7) * E);
+#pragma unroll
+        for (int u = 0; u < RB; ++u) {
+            float acc = 0.f;
+#pragma unroll
+            for (int e = 0; e < E; ++e) acc = fmaf(q[e], k[u][e], acc);
+#pragma unroll
+            for (int of = 1; of < 8; of <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, of);
+            s[u0 + u] = acc * scale_log2;
+        }
+    }
+    cm = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        if (!((valid >> (4 * u + kg)) & 1u)) s[u] = -INFINITY;
+        cm = fmaxf(cm, s[u]);
+    }
+    cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 8));
+    cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 16));
+    cl = 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        s[u] = ((valid >> (4 * u + kg)) & 1u) ? exp2f(s[u] - cm) : 0.f;
+        cl += s[u];
+    }
+    cl += __shfl_xor_sync(0xffffffffu, cl, 8);
+    cl += __shfl_xor_sync(0xffffffffu, cl, 16);
 #pragma unroll
     for (int i = 0; i < HD / 32; ++i) co[i] = 0.f;
-#pragma unroll 1
-    for (int j0 = 0; j0 < 32; j0 += 8) {
-        float v[8][HD / 32];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+    for (int j0 = 0; j0 < 32; j0 += VB) {
+        float v[VB][HD / 32];
+#pragma unroll
+        for (int j = 0; j < VB; ++j) {
             const T* vr = vbase + (size_t)__shfl_sync(0xffffffffu, slot, j0 + j) * HD;
 #pragma unroll
-            for (int i = 0; i < HD / 32; ++i) v[j][i] = to_f32(vr[lane + 32 * i]);
+            for (int i = 0; i < HD / 32; ++i) {
+                float x[1];
+                load_row<T, 1, false>(x, vr + lane + 32 * i);
+                v[j][i] = x[0];
+            }
         }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float pj = __shfl_sync(0xffffffffu, p, j0 + j);
+        for (int j = 0; j < VB; ++j) {
+            const float pj = __shfl_sync(0xffffffffu, s[(j0 + j) >> 2], (j & 3) * 8);
             if (pj != 0.f) {
 #pragma unroll
                 for (int i = 0; i < HD / 32; ++i) co[i] = fmaf(pj, v[j][i], co[i]);
@@ -607,7 +652,6 @@ __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_
     T* s_k = reinterpret_cast<T*>(bulk_smem);            // [2][32][LD]
     T* s_v = s_k + 2 * 32 * LD;                          // [2][32][LD]
     float* s_qall = reinterpret_cast<float*>(s_v + 2 * 32 * LD);
-    if (threadIdx.x == 0) pdl_launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int kvh = blockIdx.y, group = a.Hq / a.Hkv;
     const int split = blockIdx.z % n_split_launch, seq = blockIdx.z / n_split_launch;
@@ -626,6 +670,7 @@ __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_
         cta_end = max(cta_end, end[w]);
     }
     pdl_wait();             // (the row table above was written by an earlier step)
+    pdl_launch_dependents();      // the tail kernel computes its tail beside this kernel: queries, keys and values are there
 #pragma unroll
     for (int w = 0; w < BS_PW; ++w)
         if (end[w] > 0) {
@@ -728,9 +773,10 @@ __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_
 }
 
 // Tail + merge: one warp per (row, head).  grid = (ceil(rows/4), Hq, batch).
+// behind_bulk: launched as a dependent of the bulk kernel, whose CTAs release this one after their own wait; the tail is
+// computed while they run (from L2 loads only: nothing another kernel wrote comes from a stale L1 line).
 template <typename T, int HD, bool VEC>
-__global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a) {
-    __shared__ __align__(16) float s_qall[4][HD];
+__global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a, bool behind_bulk) {
     // let the next kernel start its own preamble (for a GEMM: the first weight tiles) while this one runs; it still
     // waits for this kernel to complete before it touches anything this kernel or its predecessors write
     if (threadIdx.x == 0) pdl_launch_dependents();
@@ -739,49 +785,62 @@ __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a) {
     int n_rows, L, depth;
     unsigned long long lo, hi;
     attn_row_info(a, seq, r < RT ? r : 0, n_rows, L, depth, lo, hi);      // (written by an earlier step)
-    pdl_wait();
+    if (!behind_bulk || r >= n_rows) pdl_wait();
     if (r >= n_rows) return;
     const int P = L + depth;
     const int T0 = tail_start(P, a.dcap);
     const int kvh = head / (a.Hq / a.Hkv);
-    const T* q = reinterpret_cast<const T*>(a.q) + ((size_t)(seq * RT + r) * a.Hq + head) * HD;
-    float* s_q = s_qall[warp];
-    for (int d = lane; d < HD; d += 32) s_q[d] = to_f32(q[d]);
-    __syncwarp();
+    float q[HD / 8];
+    load_row<T, HD / 8, false>(q, reinterpret_cast<const T*>(a.q) + ((size_t)(seq * RT + r) * a.Hq + head) * HD + (lane & 7) * (HD / 8));
     const T* kb = reinterpret_cast<const T*>(a.kc) + ((size_t)seq * a.Hkv + kvh) * a.cap * HD;
     const T* vb = reinterpret_cast<const T*>(a.vc) + ((size_t)seq * a.Hkv + kvh) * a.cap * HD;
-    float m = -INFINITY, l = 0.f, o[HD / 32];
-#pragma unroll
-    for (int i = 0; i < HD / 32; ++i) o[i] = 0.f;
-    // bulk partials in split order
-    const int n_sp = (T0 + a.split_len - 1) / a.split_len;
-    const size_t base = ((size_t)(seq * RT + r) * a.Hq + head) * a.n_split_max;
-    for (int s = 0; s < n_sp; ++s) {
-        float2 ml = a.part_ml[base + s];
-        float co[HD / 32];
-#pragma unroll
-        for (int i = 0; i < HD / 32; ++i) co[i] = a.part_o[(base + s) * HD + lane + 32 * i];
-        merge_partial(m, l, o, ml.x, ml.y, co);
-    }
     // tail: positions T0..P in order
     const int n_tail = P - T0 + 1;
+    float tm = -INFINITY, tl = 0.f, to[HD / 32];
+#pragma unroll
+    for (int i = 0; i < HD / 32; ++i) to[i] = 0.f;
+#pragma unroll 1
     for (int t0 = 0; t0 < n_tail; t0 += 32) {
-        int t = t0 + lane;
-        bool valid = t < n_tail;
-        int slot = 0;
-        if (valid) {
-            int pos = T0 + t;
+        int slot = -1;
+        if (t0 + lane < n_tail) {
+            const int pos = T0 + t0 + lane;
             if (pos < L) slot = pos;
             else {
-                int b = nth_set_bit(lo, hi, pos - L);
-                if (b < 0) { set_error(a.err, DEV_E_INDEX); valid = false; }
+                const int b = nth_set_bit(lo, hi, pos - L);
+                if (b < 0) set_error(a.err, DEV_E_INDEX);
                 else slot = L + b;
             }
         }
+        const uint32_t valid = __ballot_sync(0xffffffffu, slot >= 0);
+        const int any = valid ? __shfl_sync(0xffffffffu, slot, __ffs(valid) - 1) : 0;
+        if (slot < 0) slot = any;
         float cm, cl, co[HD / 32];
-        warp_chunk<T, HD, VEC>(s_q, kb, vb, slot, valid, a.scale_log2, cm, cl, co);
-        merge_partial(m, l, o, cm, cl, co);
+        warp_chunk<T, HD, VEC>(q, kb, vb, slot, valid, a.scale_log2, cm, cl, co);
+        merge_partial(tm, tl, to, cm, cl, co);
     }
+    if (behind_bulk) pdl_wait();
+    // bulk partials in split order, MB in flight, then the tail
+    constexpr int MB = 4;
+    float m = -INFINITY, l = 0.f, o[HD / 32];
+#pragma unroll
+    for (int i = 0; i < HD / 32; ++i) o[i] = 0.f;
+    const int n_sp = (T0 + a.split_len - 1) / a.split_len;
+    const size_t base = ((size_t)(seq * RT + r) * a.Hq + head) * a.n_split_max;
+    for (int s0 = 0; s0 < n_sp; s0 += MB) {
+        float2 ml[MB];
+        float co[MB][HD / 32];
+#pragma unroll
+        for (int u = 0; u < MB; ++u)
+            if (s0 + u < n_sp) {
+                ml[u] = __ldcg(a.part_ml + base + s0 + u);
+#pragma unroll
+                for (int i = 0; i < HD / 32; ++i) co[u][i] = __ldcg(a.part_o + (base + s0 + u) * HD + lane + 32 * i);
+            }
+#pragma unroll
+        for (int u = 0; u < MB; ++u)
+            if (s0 + u < n_sp) merge_partial(m, l, o, ml[u].x, ml[u].y, co[u]);
+    }
+    merge_partial(m, l, o, tm, tl, to);
     T* out = reinterpret_cast<T*>(a.out) + ((size_t)(seq * RT + r) * a.Hq + head) * HD;
     const float inv = 1.0f / l;
 #pragma unroll
@@ -801,7 +860,8 @@ __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a) {
 
 template <typename T, int HD, bool VEC>
 static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, bool bulk_too, cudaStream_t s, bool pdl) {
-    if (bulk_too && n_split_launch > 0) {
+    const bool behind_bulk = bulk_too && n_split_launch > 0;
+    if (behind_bulk) {
         const int pairs = a.rows_cap * (a.Hq / a.Hkv);
         const long long ctas4 = (long long)((pairs + 15) / 16) * a.Hkv * n_split_launch * batch;
         // Four-pair warps once their CTAs cover half of the SMs.  Operator with the tail kernel, us, one pair / four pairs per warp:
@@ -817,7 +877,7 @@ static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, 
 #undef ESP_BULK_SIMT
     }
     const dim3 g2((a.rows_cap + 3) / 4, a.Hq, batch);
-    launch_k(k_attn_tail_merge<T, HD, VEC>, g2, dim3(128), 0, s, pdl, a);
+    launch_k(k_attn_tail_merge<T, HD, VEC>, g2, dim3(128), 0, s, pdl || behind_bulk, a, behind_bulk);
     return 0;
 }
 
