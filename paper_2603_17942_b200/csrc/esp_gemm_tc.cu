@@ -40,7 +40,10 @@ namespace {
 
 using namespace tc;
 
-// NRS = rows of a block that take part (80, or 128 for blocks of more than 80 rows); NQ = sequences one launch covers
+// NRS = rows of a block that are loaded and multiplied: 80, or 128 for blocks of more than 80 rows; two-plane plans have
+// instances in between and below (TWO_PLANE_ROWS), the smallest that holds the handle's blocks.  Every 16 KB of weights come
+// with 256 bytes per row of activations from L2, through the same 64 bytes per clock and SM, and rows cost ring stages:
+// step of eight 8B layers at 1k positions, 80 rows loaded -> this: 24-row trees 1154 -> 1046 us, 68-row trees 1256 -> 1241; request with 30-row static trees 20.37 -> 18.70 ms.  (A row's bits do not depend on the instance.)  NQ = sequences one launch covers
 // (the LM head takes up to three): the first NRS rows of their activation blocks ([RT][K] each, consecutive) are gathered by one
 // 3-D TMA box into one B operand of NQ*NRS <= 256 rows, so the weights are streamed once for all.  (The layer GEMMs of
 // several sequences: esp_gemm_wide.cu.)
@@ -51,7 +54,8 @@ using namespace tc;
 // x = hi + lo (hi = bf16(x), lo = bf16(x - hi), stored n_seq blocks apart in the same buffer) and takes every product
 // with both: it then sees the activation to 2^-17 instead of 2^-9, for 10 KB more shared memory per stage.
 __host__ __device__ constexpr int stages_of(int epi, int nq, int nrs, int pl = 1) {
-    return pl == 2 ? (nrs == 80 ? 6 : 4) : (nrs == 80 ? (nq == 3 ? 4 : (nq == 2 ? 5 : 6)) : 4);
+    return pl == 2 ? (nrs <= 16 ? 10 : nrs <= 32 ? 9 : nrs <= 64 ? 7 : nrs <= 80 ? 6 : nrs <= 96 ? 5 : 4)
+                   : (nrs == 80 ? (nq == 3 ? 4 : (nq == 2 ? 5 : 6)) : 4);
 }
 __host__ __device__ constexpr int b_bytes_of(int nq, int nrs) { return nq * nrs * BK * 2; }   // 10240 per 80-row sequence and plane
 __host__ __device__ constexpr int stage_bytes_of(int nq, int nrs, int pl = 1) { return A_BYTES + pl * b_bytes_of(nq, nrs); }
@@ -59,6 +63,7 @@ __host__ __device__ constexpr int stage_bytes_of(int nq, int nrs, int pl = 1) { 
 __host__ __device__ constexpr int acc_cols_of(int nr) { return nr <= 128 ? 128 : 256; }
 constexpr int NUM_THREADS = 192;
 constexpr int MAX_NQ = 3;
+constexpr int TWO_PLANE_ROWS[] = {16, 32, 48, 56, 64, 72, 80, 96, 112, 128};
 __host__ __device__ constexpr int max_nq_of(int nrs, int pl) { return pl == 1 && nrs == 80 ? MAX_NQ : 1; }
 
 struct TcParams {
@@ -70,8 +75,9 @@ struct TcParams {
     int32_t n_tiles, KB, grid, epi;
     int32_t map_swiglu;  // tile = 64 rows of w[0] (gate) + the matching 64 rows of w[1] (up)
     int32_t slots;       // partial slots per CTA
+    int32_t part_rows;   // rows of a partial slot
     const unsigned char* a_packed;  // weights repacked per (tile, k-block) unit, or NULL: read w[] through map_a
-    float* partials;   // [grid][slots][NQ*NRS][TILE_N]
+    float* partials;   // [grid][slots][part_rows][TILE_N]
     int* counters;     // [n_tiles], zero between launches
     int* err;
     EpiArgs a;
@@ -89,7 +95,7 @@ __device__ __forceinline__ void tile_source(const TcParams& p, int tile, int hal
 template <int EPI, int NQ, int NRS, int PL>
 __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constant__ TcParams p) {
     static_assert(NQ == 1 || EPI == EPI_LOGITS, "several sequences per launch: logits");
-    static_assert(PL * NQ * NRS <= 256 && NRS % 16 == 0 && NRS <= RT, "MMA N");
+    static_assert(PL * NQ * NRS <= 256 && (PL * NRS) % 16 == 0 && NRS % 8 == 0 && NRS <= RT, "MMA N");
     static_assert((PL == 2) == (EPI == EPI_PARTIAL), "partials: two activation planes; fused epilogues: one");
     // Two planes: hi and lo rows sit back to back in the stage and form ONE B operand of 2 * NRS
     // rows; the accumulator gets W x_hi in columns [0, NRS) and W x_lo in [NRS, 2 NRS), added by the epilogue.
@@ -240,7 +246,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
         auto rows_of = [&](int sq) { return p.a.st ? (p.a.st[sq].active ? p.a.st[sq].n_rows : 0) : p.a.rows_fixed; };
         StreamK sk;
         sk.partials = p.partials; sk.table = nullptr; sk.n_tiles = p.n_tiles; sk.KB = p.KB; sk.G = p.grid; sk.slots = p.slots;
-        sk.rows = NQ * NRS; sk.seq_rows = NRS;
+        sk.rows = p.part_rows; sk.seq_rows = NRS;
         bool ok = true;
         for (int i = 0; i < rng.n_seg && ok; ++i) {
             const Seg sg = get_seg(rng, i);
@@ -253,7 +259,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t taddr = tmem_base + buf * ACC_COLS + ((uint32_t)(q * 32) << 16);
             const bool direct = EPI != EPI_PARTIAL && sg.whole;
-            float* part = p.partials + ((size_t)(blockIdx.x * p.slots + sg.slot) * (NQ * NRS)) * TILE_N + f;
+            float* part = p.partials + ((size_t)(blockIdx.x * p.slots + sg.slot) * p.part_rows) * TILE_N + f;
             // sequence by sequence: NRS accumulator columns -> that sequence's rows of the partial, or (a whole tile of a
             // fused epilogue) shared memory and the epilogue
             if constexpr (JOINT) {
@@ -262,12 +268,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
                 // beside the consumer's.  (All rows in registers at once: 146, 210 for 128 rows.)
                 const int nr = rows_of(0);
 #pragma unroll 1
-                for (int c = 0; c < NRS / 16; ++c) {
+                for (int c = 0; c < (NRS + 15) / 16; ++c) {      // (8 rows too many where NRS is no multiple of 16: not stored)
                     uint32_t hi16[16], lo16[16];
                     tmem_ld16_issue(taddr + c * 16, hi16);
                     tmem_ld16_issue(taddr + NRS + c * 16, lo16);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (c == NRS / 16 - 1) {    // everything is in registers: hand the tensor-memory buffer back to the MMA warp
+                    if (c == (NRS + 15) / 16 - 1) {    // everything is in registers: hand the tensor-memory buffer back to the MMA warp
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         mbar_arrive(&tempty[buf]);
                     }
@@ -447,9 +453,11 @@ int make_map_b(CUtensorMap* m, const void* base, int n_seq, int K, int box_rows,
 struct TcGemm {
     TcParams p;
     const TileSrc* table = nullptr;
-    CUtensorMap map_b_nq[MAX_NQ];   // activation maps with a box of nrs rows x (i+1) sequences
+    CUtensorMap map_b_nq[MAX_NQ];   // activation maps with a box of `load` rows x (i+1) sequences
+    CUtensorMap map_b_nrs;          // ... of nrs rows (the kernel that runs all layers)
     int nq_max = 1;
-    int nrs = 80;                   // rows of a sequence's block that take part: 80 or RT
+    int nrs = 80;                   // rows of a sequence's block in the partials: 80 or RT
+    int load = 80;                  // rows that are loaded and multiplied: nrs, or (two planes) one of TWO_PLANE_ROWS
     int planes = 1;                 // 2: the activation buffer holds a hi and a lo plane, x_seqs blocks apart
 };
 
@@ -467,12 +475,12 @@ void tc_gemm_geometry(const TcGemm* g, TcGemmGeom* out) {
     out->n_tiles = g->p.n_tiles; out->KB = g->p.KB; out->grid = g->p.grid; out->slots = g->p.slots;
     out->table = g->table; out->packed = g->p.a_packed; out->partials = g->p.partials; out->nrs = g->nrs;
     out->planes = g->planes; out->plane_seqs = g->p.b_plane_seqs;
-    out->map_b = g->map_b_nq[0];
+    out->map_b = g->map_b_nrs;
 }
 
 int tc_gemm_create(TcGemm** out, int epi, bool defer, const void* const w[3], const int32_t rows_w[3], int K, const void* x,
                    int x_seqs, int nrs, int nq_max, void* partials, size_t partial_bytes, int* counters, int n_sm, int* err, TileSrc* table_dev,
-                   int table_entries, void* packed, cudaStream_t stream, int planes) {
+                   int table_entries, void* packed, cudaStream_t stream, int planes, int rows_cap) {
     if (!out || (nrs != 80 && nrs != RT) || (planes != 1 && planes != 2) || nq_max < 1 || nq_max > max_nq_of(nrs, planes) ||
         x_seqs < nq_max || K % 8 || n_sm < 1)
         return -1;
@@ -492,10 +500,14 @@ int tc_gemm_create(TcGemm** out, int epi, bool defer, const void* const w[3], co
             p.map_a[i] = p.map_a[0];
         }
     }
-    for (int i = 0; i < nq_max; ++i)
-        if (make_map_b(&g->map_b_nq[i], x, planes * x_seqs, K, nrs, i + 1)) { delete g; return -1; }
     g->nq_max = nq_max;
-    g->nrs = nrs;
+    g->nrs = g->load = nrs;
+    if (planes == 2)
+        for (int r : TWO_PLANE_ROWS)
+            if (r >= rows_cap && r < g->load) g->load = r;
+    for (int i = 0; i < nq_max; ++i)
+        if (make_map_b(&g->map_b_nq[i], x, planes * x_seqs, K, g->load, i + 1)) { delete g; return -1; }
+    if (make_map_b(&g->map_b_nrs, x, planes * x_seqs, K, nrs, 1)) { delete g; return -1; }
     g->planes = planes;
     p.b_plane_seqs = x_seqs;
     p.map_b = g->map_b_nq[0];
@@ -600,6 +612,7 @@ int tc_gemm_launch(const TcGemm* g, const EpiArgs& a, cudaStream_t s, bool pdl, 
     p.a = a;
     p.map_b = g->map_b_nq[nq - 1];
     p.b_seq0 = b_seq0;
+    p.part_rows = nq * g->nrs;
     cudaError_t e = cudaSuccess;
 #define ESP_TC_CASE(E, Q, N, PLN)                                                                                  \
     {                                                                                                              \
@@ -608,10 +621,20 @@ int tc_gemm_launch(const TcGemm* g, const EpiArgs& a, cudaStream_t s, bool pdl, 
     }
     const bool wide = g->nrs != 80;
     if (g->planes == 2) {
-        if (p.epi != EPI_PARTIAL) return ESP_E_ARG;
-        if (!wide && nq == 1) ESP_TC_CASE(EPI_PARTIAL, 1, 80, 2)
-        else if (wide && nq == 1) ESP_TC_CASE(EPI_PARTIAL, 1, RT, 2)
-        else return ESP_E_ARG;
+        if (p.epi != EPI_PARTIAL || nq != 1) return ESP_E_ARG;
+        switch (g->load) {
+            case 16: ESP_TC_CASE(EPI_PARTIAL, 1, 16, 2) break;
+            case 32: ESP_TC_CASE(EPI_PARTIAL, 1, 32, 2) break;
+            case 48: ESP_TC_CASE(EPI_PARTIAL, 1, 48, 2) break;
+            case 56: ESP_TC_CASE(EPI_PARTIAL, 1, 56, 2) break;
+            case 64: ESP_TC_CASE(EPI_PARTIAL, 1, 64, 2) break;
+            case 72: ESP_TC_CASE(EPI_PARTIAL, 1, 72, 2) break;
+            case 80: ESP_TC_CASE(EPI_PARTIAL, 1, 80, 2) break;
+            case 96: ESP_TC_CASE(EPI_PARTIAL, 1, 96, 2) break;
+            case 112: ESP_TC_CASE(EPI_PARTIAL, 1, 112, 2) break;
+            case 128: ESP_TC_CASE(EPI_PARTIAL, 1, 128, 2) break;
+            default: return ESP_E_ARG;
+        }
     }
     else if (p.epi == EPI_STORE_F32 && !wide) ESP_TC_CASE(EPI_STORE_F32, 1, 80, 1)
     else if (p.epi == EPI_STORE_F32) ESP_TC_CASE(EPI_STORE_F32, 1, RT, 1)

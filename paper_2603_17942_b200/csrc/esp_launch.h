@@ -115,10 +115,11 @@ struct TcGemm;
 // (EPI_PARTIAL) and the caller runs the matching consumer kernel.  x: activations [x_seqs][RT][K]; nrs = rows of a
 // block that take part (80, or RT for blocks of more than 80 rows); an 80-row EPI_LOGITS plan may cover nq_max <= 3
 // sequences per launch, so that the weights are streamed once for them.  Deferred plans have planes = 2: x holds the
-// activations as hi + lo bf16 pairs, [2][x_seqs][RT][K], and every product is taken with both
+// activations as hi + lo bf16 pairs, [2][x_seqs][RT][K], and every product is taken with both; no block of the plan's launches
+// has more than rows_cap rows
 int tc_gemm_create(TcGemm** out, int epi, bool defer, const void* const w[3], const int32_t rows_w[3], int K, const void* x,
                    int x_seqs, int nrs, int nq_max, void* partials, size_t partial_bytes, int* counters, int n_sm, int* err, TileSrc* table_dev,
-                   int table_entries, void* packed, cudaStream_t stream, int planes = 1);
+                   int table_entries, void* packed, cudaStream_t stream, int planes = 1, int rows_cap = RT);
 // bytes of the repacked copy of a weight set (tc_gemm_create's `packed`; NULL there = stream the caller's matrices)
 size_t tc_gemm_packed_bytes(int epi, const int32_t rows_w[3], int K);
 void tc_gemm_destroy(TcGemm* g);

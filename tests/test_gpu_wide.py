@@ -260,3 +260,22 @@ def test_steps_of_a_partly_filled_handle_cost_what_takes_part():
         us.append(best)
         h.close()
     assert us[1] < 0.55 * us[0]
+
+
+def test_rows_have_the_bits_of_the_greedy_handle_in_every_instance(weights):
+    """One sequence: the layer GEMMs load as many rows as the handle's blocks have, in steps of 8 to 16, and 128-row plans take
+    the blocks of more than 80 rows; the split of k is the same in all of them, so the first row of a step has the bits it has in
+    the greedy handle."""
+    prompt = synth.make_prompt(BF16_SMALL.vocab, 150, 4)
+    first = []
+    for nodes in (0, 13, 14, 29, 30, 45, 46, 53, 61, 62, 69, 70, 77, 78, 93, 94, 109, 110, 125):
+        kw = dict(n_probes=0, max_nodes=1) if not nodes else dict(n_probes=3, topk=10, max_nodes=nodes, expand_width=0, n_anchor=1)
+        h, logits = _handle(weights, 400, P.spec_cfg(**kw))
+        h.prefill(prompt)
+        assert h.state()["n_rows"] == (nodes + 3 if nodes else 1)
+        h.step()
+        assert h.stats().device_error == 0
+        first.append(logits[0, 0].clone())
+        h.close()
+    for f in first[1:]:
+        assert torch.equal(f, first[0])
