@@ -52,6 +52,24 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
+// Pairs of floats as one operand of the packed instructions (each element rounded like its scalar form).
+__device__ __forceinline__ uint64_t pack2(float x, float y) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // ---- one 128-key chunk of the online softmax, for one thread = one half (64 keys) of one pair's row.
 // S (raw scores) is read from tensor memory; keys at or beyond T0row are masked; the two threads of a pair
 // exchange their maxima through `xch` ([2 * MP] floats); P goes back to tensor memory as bf16 pairs, over the scores it
@@ -66,19 +84,16 @@ __device__ __forceinline__ bool softmax_chunk(uint32_t s_addr, uint32_t o_addr, 
                                               int hf, uint64_t* p_ready, volatile int* s_abort) {
     uint32_t sv[64];
     tmem_ld64(s_addr, sv);
-    float cmax = -INFINITY;
-    if (__all_sync(0xffffffffu, cbase + 64 <= T0row)) {     // every key of the half is visible to every row of the warp
+    if (!__all_sync(0xffffffffu, cbase + 64 <= T0row)) {     // otherwise every key of the half is visible to every row of the warp
 #pragma unroll
-        for (int i = 0; i < 64; ++i) cmax = fmaxf(cmax, __uint_as_float(sv[i]));
-    } else {
-#pragma unroll
-        for (int i = 0; i < 64; ++i) {
-            const float sc = cbase + i < T0row ? __uint_as_float(sv[i]) : -INFINITY;
-            sv[i] = __float_as_uint(sc);
-            cmax = fmaxf(cmax, sc);
-        }
+        for (int i = 0; i < 64; ++i) sv[i] = cbase + i < T0row ? sv[i] : 0xff800000u;
     }
-    cmax = __fmul_rn(cmax, scale_log2);     // the half's maximum in the log2 domain (scaling is monotone)
+    float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};     // four chains: one takes 64 dependent steps
+#pragma unroll
+    for (int i = 0; i < 64; i += 8)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) m4[j] = fmaxf(fmaxf(m4[j], __uint_as_float(sv[i + 2 * j])), __uint_as_float(sv[i + 2 * j + 1]));
+    float cmax = __fmul_rn(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])), scale_log2);     // in the log2 domain (scaling is monotone)
     // the chunk maximum over both halves
     // (double buffered by exchange parity: a thread can be one exchange ahead of its partner, not two)
     // (one arrival per warp, after the warp's values are in shared memory: 256 single arrivals on one barrier
@@ -97,19 +112,23 @@ __device__ __forceinline__ bool softmax_chunk(uint32_t s_addr, uint32_t o_addr, 
     const float m_new = (m_run == -INFINITY || __fsub_rn(m_max, m_run) > 8.f) ? m_max : m_run;
     const float m_use = m_new == -INFINITY ? 0.f : m_new;
     const float alpha = exp2f(__fsub_rn(m_run, m_use));
-    // probabilities and their sum (key order), packed as bf16 pairs
-    float csum = 0.f;
-    const float neg_m = -m_use;
+    // probabilities, packed as bf16 pairs, and their sums over the even and the odd keys
+    const uint64_t scale2 = pack2(scale_log2, scale_log2), neg_m2 = pack2(-m_use, -m_use);
+    uint64_t csum2 = 0;
     uint32_t pk[32];
 #pragma unroll
     for (int i = 0; i < 64; i += 2) {
-        const float p0 = ex2_approx(__fmaf_rn(__uint_as_float(sv[i]), scale_log2, neg_m));
-        const float p1 = ex2_approx(__fmaf_rn(__uint_as_float(sv[i + 1]), scale_log2, neg_m));
-        csum = __fadd_rn(csum, p0);
-        csum = __fadd_rn(csum, p1);
+        float p0, p1;
+        unpack2(fma2(pack2(__uint_as_float(sv[i]), __uint_as_float(sv[i + 1])), scale2, neg_m2), p0, p1);
+        p0 = ex2_approx(p0);
+        p1 = ex2_approx(p1);
+        csum2 = add2(csum2, pack2(p0, p1));
         const __nv_bfloat162 b2 = __floats2bfloat162_rn(p0, p1);
         pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&b2);
     }
+    float c0, c1;
+    unpack2(csum2, c0, c1);
+    const float csum = __fadd_rn(c0, c1);
     // (the values are pinned here: without it the compiler is free to sink the arithmetic behind the wait)
 #pragma unroll
     for (int i = 0; i < 32; ++i) asm volatile("" : "+r"(pk[i]));
@@ -323,7 +342,9 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
                              ::"l"(a.part_o + idx * HD + hf * 64), "r"(smem_u32(orow)), "r"(64 * 4) : "memory");
             }
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");        // copies complete: shared memory may be released
+            // shared memory may be released when it has been read; the end of the kernel, where there is one, completes the copies
+            if (PDL) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            else asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         } else if (!ok && lane == 0) {
             set_error(a.err, DEV_E_WAIT_TIMEOUT);
             *s_abort = 1;
