@@ -71,16 +71,27 @@ __device__ __forceinline__ void run_epilogue_rows(float* s_acc, float* s_aux, in
             epi_bar(bar_id);
             // rotary embedding at position L + depth, rotate-half pairing (i, i + h/2)
             const int partner = fl < half ? f + half : f - half;
-            for (int r = r0; r < r1; ++r) {
-                const int pos = L + (st ? st->row_depth[r] : r);
-                const float cs = a.rope_cos[(size_t)pos * half + (fl % half)];
-                const float sn = a.rope_sin[(size_t)pos * half + (fl % half)];
-                const float me = s_acc[r * ACC_LD + f], other = s_acc[r * ACC_LD + partner];
-                const float v = fl < half ? me * cs - other * sn : me * cs + other * sn;
-                if (which == 0) {
-                    reinterpret_cast<T*>(a.q_out)[(size_t)(grow0 + r) * dq + head * h + fl] = from_f32<T>(v);
-                } else {
-                    reinterpret_cast<T*>(a.kcache)[(((size_t)seq * a.Hkv + head) * a.cap + (L + r)) * h + fl] = from_f32<T>(v);
+            // (the factors of eight rows are fetched before any is used: row by row each was two dependent trips)
+            for (int rb = r0; rb < r1; rb += 8) {
+                float cs[8], sn[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (rb + i < r1) {
+                        const int pos = L + (st ? __ldg(&st->row_depth[rb + i]) : rb + i);
+                        cs[i] = __ldg(a.rope_cos + (size_t)pos * half + (fl % half));
+                        sn[i] = __ldg(a.rope_sin + (size_t)pos * half + (fl % half));
+                    }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int r = rb + i;
+                    if (r >= r1) break;
+                    const float me = s_acc[r * ACC_LD + f], other = s_acc[r * ACC_LD + partner];
+                    const float v = fl < half ? me * cs[i] - other * sn[i] : me * cs[i] + other * sn[i];
+                    if (which == 0) {
+                        reinterpret_cast<T*>(a.q_out)[(size_t)(grow0 + r) * dq + head * h + fl] = from_f32<T>(v);
+                    } else {
+                        reinterpret_cast<T*>(a.kcache)[(((size_t)seq * a.Hkv + head) * a.cap + (L + r)) * h + fl] = from_f32<T>(v);
+                    }
                 }
             }
         } else {

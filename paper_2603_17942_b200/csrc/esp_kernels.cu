@@ -253,8 +253,7 @@ __global__ void __launch_bounds__(SWIGLU_THREADS) k_swiglu_finish(const SeqState
 }
 
 // ------------------------------------------------------------------ CUDA-core GEMM
-// y[row][n] = sum_k x[row][k] * w[n][k], one running fp32 sum per output with k ascending, one thread per output
-// feature of a 128-feature tile.  Used for fp32 models and as the on-GPU cross-check of the tcgen05 kernel.
+// y[row][n] = sum_k x[row][k] * w[n][k], four running fp32 sums per output with k ascending, added in order.  Used for fp32 models and as the on-GPU cross-check of the tcgen05 kernel.
 // Tile -> weight rows mapping is the same as there: up to three stacked matrices (q|k|v), or gate/up halves
 // interleaved per tile.
 //
@@ -280,6 +279,10 @@ struct SimtGemmArgs {
 };
 constexpr int SIMT_ROWS = 8, SIMT_NORM_K = 1024;
 constexpr int SIMT_KC = 32, SIMT_STAGES = 4;       // whole tile: two CTAs of 84 KB per SM
+// k is dealt to four threads per feature (narrow: to the four warps, each with all 8 rows), whose sums are added in order at
+// the end: one thread per feature and 8 rows, or two rows per warp, was a chain of dependent additions with nothing to hide it
+// (the tiny decoder, 64-token request 7177 -> 6982 us).
+constexpr int SIMT_KS = 4, SIMT_THREADS = 128 * SIMT_KS;
 constexpr int NARROW_F = 32, NARROW_KC = 64, NARROW_STAGES = 6;
 // elements between two rows of a stage: 16 bytes of padding put the eight rows of a quarter-warp's 16-byte loads on
 // different banks
@@ -308,12 +311,12 @@ __device__ __forceinline__ float4 load_f4(const __nv_bfloat16* p) {
 }
 
 // Stage `dst` [n_rows][LD] <- rows 0..n_valid-1 of `src` (K elements apart), elements k0 .. k0+KC-1; zeros outside.
-// All 128 threads take part, 16 bytes each per pass.  VEC: src starts on 16 bytes (its rows then do too, K is a
+// All NT threads take part, 16 bytes each per pass.  VEC: src starts on 16 bytes (its rows then do too, K is a
 // multiple of 8): asynchronous copies.  Otherwise element by element (a caller's matrix needs no more than its
 // type's alignment).
-template <typename T, int KC, int N_ROWS, bool VEC>
+template <typename T, int KC, int N_ROWS, bool VEC, int NT = 128>
 __device__ __forceinline__ void simt_load(T* dst, const T* src, int n_valid, int K, int k0) {
-    constexpr int LD = simt_ld<T>(KC), V = 16 / (int)sizeof(T), PER_ROW = KC / V, STEP = 128 / PER_ROW;
+    constexpr int LD = simt_ld<T>(KC), V = 16 / (int)sizeof(T), PER_ROW = KC / V, STEP = NT / PER_ROW;
     const int j = (threadIdx.x % PER_ROW) * V, first = threadIdx.x / PER_ROW;
     const bool k_ok = k0 + j < K;
     const T* p = src + (size_t)first * K + k0 + j;
@@ -358,15 +361,17 @@ __device__ __forceinline__ void simt_mac_n(float (&acc)[R], const float* w, cons
     }
 }
 
-// NORM: rows r0 .. of the residual stream, normalised, to shared memory ([SIMT_ROWS][K + 4] floats); a warp takes two rows.  The
+// NORM: rows r0 .. of the residual stream, normalised, to shared memory ([SIMT_ROWS][K + 4] floats); a warp takes PER rows.  The
 // sum of squares: per lane over its elements in ascending order, then over the warp.
 __host__ __device__ constexpr int norm_x_ld(int K) { return K + 4; }
+template <int PER>
 __device__ __forceinline__ void norm_rows(float* s_x, const SimtGemmArgs& g, size_t row0, int n_valid, int warp, int lane, bool copy) {
     const float* gain = reinterpret_cast<const float*>(g.gain);
     const int ld = g.K + 4;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int r = warp * 2 + i;
+    for (int i = 0; i < PER; ++i) {
+        const int r = warp * PER + i;
+        if (r >= SIMT_ROWS) return;
         float* d = s_x + r * ld;
         if (r >= n_valid) {
             for (int j = lane * 4; j < g.K; j += 128) *reinterpret_cast<float4*>(d + j) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -393,10 +398,10 @@ __device__ __forceinline__ void norm_rows(float* s_x, const SimtGemmArgs& g, siz
     }
 }
 
-// 8 rows x one 128-feature tile, one thread per feature.  EPI_QKV (the stacked matrices end on tile boundaries) and
+// 8 rows x one 128-feature tile, SIMT_KS threads per feature, each a quarter of every stage's k.  EPI_QKV (the stacked matrices end on tile boundaries) and
 // EPI_LOGITS.
 template <typename T, int EPI, bool VEC, bool NORM>
-__global__ void __launch_bounds__(128) k_gemm_simt(SimtGemmArgs g, EpiArgs a) {
+__global__ void __launch_bounds__(SIMT_THREADS, 2) k_gemm_simt(SimtGemmArgs g, EpiArgs a) {
     static_assert(!NORM || sizeof(T) == 4, "the normalised rows are fp32");
     constexpr int LD = simt_ld<T>(SIMT_KC);
     extern __shared__ __align__(16) unsigned char simt_smem[];
@@ -406,13 +411,13 @@ __global__ void __launch_bounds__(128) k_gemm_simt(SimtGemmArgs g, EpiArgs a) {
     float* s_aux = s_acc + SIMT_ROWS * ACC_LD;                  // RT * 4
     float* s_xn = s_aux + RT * 4;                               // NORM: [ROWS][K + 4]
     if (threadIdx.x == 0) pdl_launch_dependents();
-    const int tile = blockIdx.x, r0 = blockIdx.y * SIMT_ROWS, seq = blockIdx.z, f = threadIdx.x;
+    const int tile = blockIdx.x, r0 = blockIdx.y * SIMT_ROWS, seq = blockIdx.z, f = threadIdx.x % 128, ks = threadIdx.x / 128;
     int m = 0, feat = tile * TILE_N;
     while (m < 2 && feat >= g.rows_w[m]) feat -= g.rows_w[m++];
     const T* w = reinterpret_cast<const T*>(g.w[m]) + (size_t)feat * g.K;
     const int n_feat = g.rows_w[m] - feat < TILE_N ? g.rows_w[m] - feat : TILE_N;
     const int n_chunks = (g.K + SIMT_KC - 1) / SIMT_KC;
-    auto load_w = [&](int c) { simt_load<T, SIMT_KC, TILE_N, VEC>(s_w + (c % SIMT_STAGES) * TILE_N * LD, w, n_feat, g.K, c * SIMT_KC); };
+    auto load_w = [&](int c) { simt_load<T, SIMT_KC, TILE_N, VEC, SIMT_THREADS>(s_w + (c % SIMT_STAGES) * TILE_N * LD, w, n_feat, g.K, c * SIMT_KC); };
     for (int c = 0; c < SIMT_STAGES - 1 && c < n_chunks; ++c) load_w(c);      // (they join the first group below)
     // (the row table was written by an earlier step: read before the wait, like the weights)
     const SeqState* st = a.st ? a.st + seq : nullptr;
@@ -422,13 +427,13 @@ __global__ void __launch_bounds__(128) k_gemm_simt(SimtGemmArgs g, EpiArgs a) {
     const int r1 = r0 + SIMT_ROWS < n_rows ? r0 + SIMT_ROWS : n_rows;
     const T* x = reinterpret_cast<const T*>(g.x) + (size_t)(seq * RT + r0) * g.K;
     auto load_x = [&](int c) {
-        if constexpr (!NORM) simt_load<T, SIMT_KC, SIMT_ROWS, VEC>(s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD, x, r1 - r0, g.K, c * SIMT_KC);
+        if constexpr (!NORM) simt_load<T, SIMT_KC, SIMT_ROWS, VEC, SIMT_THREADS>(s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD, x, r1 - r0, g.K, c * SIMT_KC);
     };
     for (int c = 0; c < SIMT_STAGES - 1; ++c) {
         if (c < n_chunks) load_x(c);
         cp_async_commit();
     }
-    if constexpr (NORM) norm_rows(s_xn, g, (size_t)(seq * RT + r0), r1 - r0, threadIdx.x >> 5, threadIdx.x & 31, g.copy && blockIdx.x == 0);
+    if constexpr (NORM) norm_rows<1>(s_xn, g, (size_t)(seq * RT + r0), r1 - r0, threadIdx.x >> 5, threadIdx.x & 31, g.copy && blockIdx.x == 0);
     float acc[SIMT_ROWS];
 #pragma unroll
     for (int r = 0; r < SIMT_ROWS; ++r) acc[r] = 0.f;
@@ -437,18 +442,31 @@ __global__ void __launch_bounds__(128) k_gemm_simt(SimtGemmArgs g, EpiArgs a) {
         __syncthreads();                                // chunk c has landed, and chunk c - 1's buffer is free
         if (c + SIMT_STAGES - 1 < n_chunks) { load_w(c + SIMT_STAGES - 1); load_x(c + SIMT_STAGES - 1); }
         cp_async_commit();
-        const T* wr = s_w + ((c % SIMT_STAGES) * TILE_N + f) * LD;
-        if constexpr (NORM) simt_mac_n<SIMT_ROWS, SIMT_KC>(acc, wr, s_xn + c * SIMT_KC, norm_x_ld(g.K), g.K - c * SIMT_KC);
-        else simt_mac<SIMT_ROWS, SIMT_KC>(acc, wr, s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD, LD);
+        constexpr int KQ = SIMT_KC / SIMT_KS;
+        const T* wr = s_w + ((c % SIMT_STAGES) * TILE_N + f) * LD + ks * KQ;
+        if constexpr (NORM) simt_mac_n<SIMT_ROWS, KQ>(acc, wr, s_xn + c * SIMT_KC + ks * KQ, norm_x_ld(g.K), g.K - c * SIMT_KC - ks * KQ);
+        else simt_mac<SIMT_ROWS, KQ>(acc, wr, s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD + ks * KQ, LD);
     }
-#pragma unroll
-    for (int r = 0; r < SIMT_ROWS; ++r) s_acc[r * ACC_LD + f] = acc[r];
+    // the quarters' sums, added in order (in the weights' buffers, which nothing reads or writes any more)
     __syncthreads();
+    float* s_part = reinterpret_cast<float*>(s_w);              // [KS][ROWS][128]
+#pragma unroll
+    for (int r = 0; r < SIMT_ROWS; ++r) s_part[(ks * SIMT_ROWS + r) * TILE_N + f] = acc[r];
+    __syncthreads();
+    if (ks) return;
+#pragma unroll
+    for (int r = 0; r < SIMT_ROWS; ++r) {
+        float v = s_part[r * TILE_N + f];
+#pragma unroll
+        for (int q = 1; q < SIMT_KS; ++q) v += s_part[(q * SIMT_ROWS + r) * TILE_N + f];
+        s_acc[r * ACC_LD + f] = v;
+    }
+    epi_bar(1);
     run_epilogue_rows<T, EPI>(s_acc, s_aux, tile, seq, a, f, 1, st, n_rows, r0, r1);
 }
 
-// 8 rows x 32 features (SWIGLU: 16 gate features and the matching 16 up features), a lane per feature, two rows per
-// warp.  EPI_STORE_F32, EPI_RESID, EPI_SWIGLU.
+// 8 rows x 32 features (SWIGLU: 16 gate features and the matching 16 up features), a lane per feature, a quarter of every
+// stage's k per warp.  EPI_STORE_F32, EPI_RESID, EPI_SWIGLU.
 template <typename T, int EPI, bool VEC, bool NORM>
 __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArgs a) {
     constexpr int LD = simt_ld<T>(NARROW_KC), HALF = NARROW_F / 2;
@@ -495,16 +513,31 @@ __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArg
             if (lane < n_feat && r < r1) old[i] = a.hres[(size_t)(seq * RT + r) * a.n_out + n0 + lane];
         }
     }
-    if constexpr (NORM) norm_rows(s_xn, g, (size_t)(seq * RT + r0), r1 - r0, warp, lane, false);
-    float acc[2] = {0.f, 0.f};
+    if constexpr (NORM) norm_rows<2>(s_xn, g, (size_t)(seq * RT + r0), r1 - r0, warp, lane, false);
+    float part[SIMT_ROWS];
+#pragma unroll
+    for (int r = 0; r < SIMT_ROWS; ++r) part[r] = 0.f;
     for (int c = 0; c < n_chunks; ++c) {
         cp_async_wait<NARROW_STAGES - 2>();
         __syncthreads();
         if (c + NARROW_STAGES - 1 < n_chunks) { load_w(c + NARROW_STAGES - 1); load_x(c + NARROW_STAGES - 1); }
         cp_async_commit();
-        const T* wr = s_w + ((c % NARROW_STAGES) * NARROW_F + lane) * LD;
-        if constexpr (NORM) simt_mac_n<2, NARROW_KC>(acc, wr, s_xn + warp * 2 * norm_x_ld(g.K) + c * NARROW_KC, norm_x_ld(g.K), g.K - c * NARROW_KC);
-        else simt_mac<2, NARROW_KC>(acc, wr, s_x + ((c % NARROW_STAGES) * SIMT_ROWS + warp * 2) * LD, LD);
+        constexpr int KQ = NARROW_KC / 4;
+        const T* wr = s_w + ((c % NARROW_STAGES) * NARROW_F + lane) * LD + warp * KQ;
+        if constexpr (NORM) simt_mac_n<SIMT_ROWS, KQ>(part, wr, s_xn + c * NARROW_KC + warp * KQ, norm_x_ld(g.K), g.K - c * NARROW_KC - warp * KQ);
+        else simt_mac<SIMT_ROWS, KQ>(part, wr, s_x + (c % NARROW_STAGES) * SIMT_ROWS * LD + warp * KQ, LD);
+    }
+    // the quarters' sums, added in order: two rows per warp
+    __shared__ float s_part[4][SIMT_ROWS][NARROW_F];
+#pragma unroll
+    for (int r = 0; r < SIMT_ROWS; ++r) s_part[warp][r][lane] = part[r];
+    __syncthreads();
+    float acc[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        acc[i] = s_part[0][warp * 2 + i][lane];
+#pragma unroll
+        for (int q = 1; q < 4; ++q) acc[i] += s_part[q][warp * 2 + i][lane];
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -529,7 +562,7 @@ int launch_gemm_simt_t(int epi, int n_tiles, int batch, const SimtGemmArgs& g, c
     {                                                                                                               \
         if (ensure_dynamic_smem(reinterpret_cast<const void*>(KERNEL<T, E, VEC, NORM>), (int)(SMEM<T>() + (NORM ? sizeof(float) * SIMT_ROWS * norm_x_ld(SIMT_NORM_K) : 0)))) \
             return ESP_E_CUDA;                                                                                      \
-        return launch_k(KERNEL<T, E, VEC, NORM>, dim3(TILES, groups, batch), dim3(128), SMEM<T>() + norm_bytes, s, pdl, g, a) == cudaSuccess ? ESP_OK : ESP_E_CUDA; \
+        return launch_k(KERNEL<T, E, VEC, NORM>, dim3(TILES, groups, batch), dim3((E == EPI_QKV || E == EPI_LOGITS) ? SIMT_THREADS : 128), SMEM<T>() + norm_bytes, s, pdl, g, a) == cudaSuccess ? ESP_OK : ESP_E_CUDA; \
     }
     if constexpr (sizeof(T) == 4) {
         if (g.gain) {
