@@ -281,7 +281,7 @@ constexpr int SIMT_ROWS = 8, SIMT_NORM_K = 1024;
 constexpr int SIMT_KC = 32, SIMT_STAGES = 4;       // whole tile: two CTAs of 84 KB per SM
 // k is dealt to four threads per feature (narrow: to the four warps, each with all 8 rows), whose sums are added in order at
 // the end: one thread per feature and 8 rows, or two rows per warp, was a chain of dependent additions with nothing to hide it
-// (the tiny decoder, 64-token request 7177 -> 6982 us).
+// (64-token request of the tiny decoder 7177 -> 6982 us).
 constexpr int SIMT_KS = 4, SIMT_THREADS = 128 * SIMT_KS;
 constexpr int NARROW_F = 32, NARROW_KC = 64, NARROW_STAGES = 6;
 // elements between two rows of a stage: 16 bytes of padding put the eight rows of a quarter-warp's 16-byte loads on
@@ -756,20 +756,28 @@ __device__ __forceinline__ void merge_partial(float& m, float& l, float (&o)[N],
 // fp32 heads of 64 over 777 positions: 184 us with a warp per (row, head) gathering its keys from L1, 33 us now; one
 // split of 100 positions on its own 13.4 us with four pairs per warp, 7.3 with one.
 // grid = (ceil(rows * group / (4 * BS_PW)), Hkv, n_split * batch).
+// The CTA's warps form bulk_groups() groups that take the split's chunks in turn, each with buffers and running sums of its own,
+// merged in group order at the end (which chunk goes where follows from the position alone): the chain over 256 positions is eight
+// chunks of about 3 us for one group.  Operator, 3 sequences x 35 rows x 4 fp32 heads of 64 over 777 positions: 34.9 -> 23.3 us.
 constexpr int BS_WARPS = 4;
+template <typename T, int HD> __host__ __device__ constexpr int bulk_groups() { return sizeof(T) * HD <= 256 ? 4 : 2; }
 template <typename T, int HD> __host__ __device__ constexpr int bulk_simt_ld() { return HD + 16 / (int)sizeof(T); }
-template <typename T, int HD> constexpr size_t bulk_simt_smem(int pw) { return sizeof(T) * 4 * 32 * bulk_simt_ld<T, HD>() + sizeof(float) * BS_WARPS * pw * HD; }
+template <typename T, int HD> constexpr size_t bulk_simt_smem(int pw) {
+    return bulk_groups<T, HD>() * (sizeof(T) * 4 * 32 * bulk_simt_ld<T, HD>() + sizeof(float) * BS_WARPS * pw * HD);
+}
 template <typename T, int HD, bool VEC, int BS_PW>
-__global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_launch) {
-    constexpr int LD = bulk_simt_ld<T, HD>(), V = 16 / (int)sizeof(T), PER_ROW = HD / V;
+__global__ void __launch_bounds__(128 * bulk_groups<T, HD>()) k_attn_bulk_simt(AttnArgs a, int n_split_launch) {
+    constexpr int LD = bulk_simt_ld<T, HD>(), V = 16 / (int)sizeof(T), PER_ROW = HD / V, KG = bulk_groups<T, HD>();
     extern __shared__ __align__(16) unsigned char bulk_smem[];
-    T* s_k = reinterpret_cast<T*>(bulk_smem);            // [2][32][LD]
-    T* s_v = s_k + 2 * 32 * LD;                          // [2][32][LD]
-    float* s_qall = reinterpret_cast<float*>(s_v + 2 * 32 * LD);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int kg = threadIdx.x >> 7, gt = threadIdx.x & 127;      // key group, thread of the group
+    const int warp = gt >> 5, lane = gt & 31;
+    T* s_k = reinterpret_cast<T*>(bulk_smem) + kg * 4 * 32 * LD;      // [2][32][LD]
+    T* s_v = s_k + 2 * 32 * LD;                                       // [2][32][LD]
+    float* s_qall = reinterpret_cast<float*>(reinterpret_cast<T*>(bulk_smem) + KG * 4 * 32 * LD) + kg * BS_WARPS * BS_PW * HD;
     const int kvh = blockIdx.y, group = a.Hq / a.Hkv;
     const int split = blockIdx.z % n_split_launch, seq = blockIdx.z / n_split_launch;
     const int beg = split * a.split_len;
+    auto group_bar = [&] { asm volatile("bar.sync %0, 128;" ::"r"(1 + kg) : "memory"); };
     int row[BS_PW], end[BS_PW], cta_end = 0;
     const int pair0 = (blockIdx.x * BS_WARPS + warp) * BS_PW;
     float* s_q = s_qall + warp * BS_PW * HD;
@@ -792,7 +800,7 @@ __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_
             for (int d = lane; d < HD; d += 32) s_q[w * HD + d] = to_f32(q[d]);
         }
     __shared__ int s_end[BS_WARPS];
-    if (lane == 0) s_end[warp] = cta_end;
+    if (lane == 0 && kg == 0) s_end[warp] = cta_end;
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < BS_WARPS; ++w) cta_end = max(cta_end, s_end[w]);
@@ -800,7 +808,7 @@ __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_
     const T* kb = reinterpret_cast<const T*>(a.kc) + ((size_t)seq * a.Hkv + kvh) * a.cap * HD;
     const T* vb = reinterpret_cast<const T*>(a.vc) + ((size_t)seq * a.Hkv + kvh) * a.cap * HD;
     auto load = [&](int p0, int buf) {
-        for (int i = threadIdx.x; i < 32 * PER_ROW; i += 128) {
+        for (int i = gt; i < 32 * PER_ROW; i += 128) {
             const int pos = p0 + i / PER_ROW, e0 = (i % PER_ROW) * V;
             const bool ok = pos < cta_end;
             const size_t src = (size_t)(ok ? pos : beg) * HD + e0;
@@ -827,12 +835,12 @@ __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_
 #pragma unroll
         for (int i = 0; i < HD / 32; ++i) o[w][i] = 0.f;
     }
-    load(beg, 0);
-    for (int p0 = beg, buf = 0; p0 < cta_end; p0 += 32, buf ^= 1) {
-        if (p0 + 32 < cta_end) load(p0 + 32, buf ^ 1);
+    if (beg + 32 * kg < cta_end) load(beg + 32 * kg, 0);
+    for (int p0 = beg + 32 * kg, buf = 0; p0 < cta_end; p0 += 32 * KG, buf ^= 1) {
+        if (p0 + 32 * KG < cta_end) load(p0 + 32 * KG, buf ^ 1);
         else cp_async_commit();
         cp_async_wait<1>();
-        __syncthreads();
+        group_bar();
         const T* kr = s_k + (buf * 32 + lane) * LD;
         float acc[BS_PW], p[BS_PW], cm[BS_PW], cl[BS_PW], co[BS_PW][HD / 32];
 #pragma unroll
@@ -874,11 +882,34 @@ __global__ void __launch_bounds__(128) k_attn_bulk_simt(AttnArgs a, int n_split_
 #pragma unroll
         for (int w = 0; w < BS_PW; ++w)
             if (p0 < end[w]) merge_partial(m[w], l[w], o[w], cm[w], cl[w], co[w]);
-        __syncthreads();       // this buffer is loaded again in the next round but one
+        group_bar();           // this buffer is loaded again in the next round but one
     }
+    // the groups' sums meet in the first group's buffers ([group - 1][pair][HD + 2] floats), which it has done with
+    __syncthreads();
+    float* s_m = reinterpret_cast<float*>(bulk_smem);
+    static_assert(sizeof(float) * (KG - 1) * BS_WARPS * BS_PW * (HD + 2) <= KG * sizeof(T) * 4 * 32 * LD, "room for the groups' sums");
+    if (kg > 0) {
+#pragma unroll
+        for (int w = 0; w < BS_PW; ++w) {
+            float* d = s_m + (((kg - 1) * BS_WARPS + warp) * BS_PW + w) * (HD + 2);
+            if (lane == 0) { d[HD] = m[w]; d[HD + 1] = l[w]; }
+#pragma unroll
+            for (int i = 0; i < HD / 32; ++i) d[lane + 32 * i] = o[w][i];
+        }
+    }
+    __syncthreads();
+    if (kg > 0) return;
 #pragma unroll
     for (int w = 0; w < BS_PW; ++w) {
         if (end[w] <= beg) continue;
+#pragma unroll
+        for (int g = 1; g < KG; ++g) {
+            const float* d = s_m + (((g - 1) * BS_WARPS + warp) * BS_PW + w) * (HD + 2);
+            float co[HD / 32];
+#pragma unroll
+            for (int i = 0; i < HD / 32; ++i) co[i] = d[lane + 32 * i];
+            if (beg + 32 * g < end[w]) merge_partial(m[w], l[w], o[w], d[HD], d[HD + 1], co);
+        }
         const size_t idx = ((size_t)(seq * RT + row[w]) * a.Hq + kvh * group + (pair0 + w) % group) * a.n_split_max + split;
         if (lane == 0) a.part_ml[idx] = make_float2(m[w], l[w]);
 #pragma unroll
@@ -984,7 +1015,7 @@ static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, 
 #define ESP_BULK_SIMT(PW)                                                                                              \
         {                                                                                                              \
             if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_attn_bulk_simt<T, HD, VEC, PW>), (int)bulk_simt_smem<T, HD>(PW))) return -1; \
-            launch_k(k_attn_bulk_simt<T, HD, VEC, PW>, dim3((pairs + 4 * PW - 1) / (4 * PW), a.Hkv, n_split_launch * batch), dim3(128),          \
+            launch_k(k_attn_bulk_simt<T, HD, VEC, PW>, dim3((pairs + 4 * PW - 1) / (4 * PW), a.Hkv, n_split_launch * batch), dim3(128 * bulk_groups<T, HD>()), \
                      bulk_simt_smem<T, HD>(PW), s, pdl, a, n_split_launch);                                            \
         }
         if (ctas4 >= 74) ESP_BULK_SIMT(4) else ESP_BULK_SIMT(1)

@@ -331,3 +331,28 @@ def test_tree_attention_with_room_for_the_block_only(dt, h):
     ref = torch.einsum("bhrc,bhcd->brhd", s.softmax(-1), vc.repeat_interleave(2, 1)[:, :, :n_rows].double())
     tol = 2e-5 if dt == "fp32" else 2.0 ** -8 * float(ref.abs().max())      # sums of a few terms; the result's own rounding
     assert (out.double() - ref).abs().max() <= tol
+
+
+@pytest.mark.parametrize("group,n_rows,L,dcap", [(1, 33, 5, 16), (2, 9, 0, 16), (4, 68, 15, 16), (8, 41, 16, 32), (16, 7, 40, 48), (4, 128, 16, 128)])
+def test_tree_attention_tail_alone(group, n_rows, L, dcap):
+    """No row has a position below its T0, so the tail kernel does it all: fewer heads per KV head than a warp takes together,
+    as many, and several times as many; lists of one key, of 32 and one more, of several chunks; keys before, on and behind the
+    end of the cache.  Its weights are exact to fp32, so what is left is the result's own rounding."""
+    Hkv, h, b = 2, 128, 2
+    Hq, cap = Hkv * group, L + R
+    if dcap == 128:
+        depth1, vis = np.arange(n_rows), np.tril(np.ones((n_rows, n_rows), np.uint8))
+    else:
+        _, depth1, vis = _tree_block(n_rows, 0, dcap, n_rows)
+    assert (np.maximum(L + depth1 - dcap, 0) // 16 * 16).max() == 0
+    g = torch.Generator().manual_seed(group)
+    q = torch.randn(b, R, Hq, h, generator=g).bfloat16().cuda()
+    kc, vc = (torch.randn(b, Hkv, cap, h, generator=g).bfloat16().cuda() for _ in range(2))
+    depth = np.zeros((b, R), np.int32)
+    depth[:, :n_rows] = depth1
+    out = _run_attention(1, q, kc, vc, np.stack([_anc_words(vis)] * b), depth, n_rows, L, Hq, Hkv, h, dcap)[:, :n_rows]
+    s = torch.einsum("brhd,bhcd->bhrc", q[:, :n_rows].double(), kc.repeat_interleave(group, 1)[:, :, :L + n_rows].double()) / h ** 0.5
+    hide = torch.zeros(n_rows, L + n_rows, dtype=torch.bool)
+    hide[:, L:] = torch.from_numpy(vis == 0)
+    ref = torch.einsum("bhrc,bhcd->brhd", s.masked_fill_(hide.cuda(), -float("inf")).softmax(-1), vc.repeat_interleave(group, 1)[:, :, :L + n_rows].double())
+    assert (out.double() - ref).abs().max() <= 2.0 ** -8 * float(ref.abs().max())
