@@ -1045,6 +1045,29 @@ int launch_attn_simt(int dtype, const AttnArgs& a, int batch, int n_split_launch
     return -1;
 }
 
+// ------------------------------------------------------------------ ranking by packed keys
+// keys of the n given ones that are smaller
+__device__ __forceinline__ int rank_among(const unsigned long long* keys, int n, unsigned long long key) {
+    int rank = 0;
+#pragma unroll 4
+    for (int o = 0; o + 1 < n; o += 2) {
+        const ulonglong2 k2 = *reinterpret_cast<const ulonglong2*>(keys + o);
+        rank += (k2.x < key ? 1 : 0) + (k2.y < key ? 1 : 0);
+    }
+    if (n & 1) rank += keys[n - 1] < key ? 1 : 0;
+    return rank;
+}
+// A Top-K' entry as a key: by value descending, then id ascending, smaller first (-0 and +0 are equal); none: behind all.
+__device__ __forceinline__ unsigned long long cand_key(float val, int id) {
+    return id < 0 ? ~0ull : ((unsigned long long)(~float_order_key(val)) << 32) | (uint32_t)id;
+}
+__device__ __forceinline__ Cand cand_of(unsigned long long key) {
+    Cand c;
+    c.id = key == ~0ull ? -1 : (int)(uint32_t)key;
+    c.val = key == ~0ull ? -INFINITY : float_from_order_key(~(uint32_t)(key >> 32));
+    return c;
+}
+
 // ------------------------------------------------------------------ Top-K' merge over vocabulary tiles
 // One block per row: global Top-K' (value desc, id asc) of the per-tile lists, plus
 // lse = max + log(sum exp) merged over tiles in a fixed order.
@@ -1059,9 +1082,9 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_topk_merge(const SeqState* sta
                                                              uint32_t* cand_floor) {
     __shared__ float s_v[TOPK_THREADS];
     __shared__ int s_i[TOPK_THREADS];
-    __shared__ Cand s_w[TOPK_WARPS * KP_MAX];                         // the best heads of each warp's tiles
-    __shared__ int s_wt[TOPK_WARPS * KP_MAX], s_tile[KP_MAX];         // their tiles; the best of all
-    __shared__ Cand s_l[KP_MAX * (KP_MAX + 1) / 2];                   // what is read of the best tiles' lists
+    __shared__ __align__(16) unsigned long long s_w[TOPK_WARPS * KP_MAX];      // the best heads of each warp's tiles
+    __shared__ int s_wt[TOPK_WARPS * KP_MAX], s_tile[KP_MAX];                  // their tiles; the best of all
+    __shared__ __align__(16) unsigned long long s_l[KP_MAX * (KP_MAX + 1) / 2];   // what is read of the best tiles' lists
     if (threadIdx.x == 0) pdl_launch_dependents();
     const int seq = blockIdx.y, r = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const SeqState* st = states + seq;
@@ -1071,66 +1094,69 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_topk_merge(const SeqState* sta
     const int Mtot = batch * RT, grow = seq * RT + r;
     const int kp = probe ? KP : 1;
     // tile t belongs to thread t mod 256
-    Cand head[TOPK_MAXT];
+    unsigned long long head[TOPK_MAXT];
     float2 ms[TOPK_MAXT];
+    {
+        Cand c[TOPK_MAXT];
 #pragma unroll
-    for (int i = 0; i < TOPK_MAXT; ++i) {
-        const int t = tid + TOPK_THREADS * i;
-        head[i].val = -INFINITY; head[i].id = -1;
-        ms[i] = make_float2(-INFINITY, 0.f);
-        if (t < n_tiles) {
-            head[i] = cand[((size_t)t * Mtot + grow) * KP];
-            if (probe) ms[i] = cand_ms[(size_t)t * Mtot + grow];
+        for (int i = 0; i < TOPK_MAXT; ++i) {
+            const int t = tid + TOPK_THREADS * i;
+            c[i].val = -INFINITY; c[i].id = -1;
+            ms[i] = make_float2(-INFINITY, 0.f);
+            if (t < n_tiles) {
+                c[i] = cand[((size_t)t * Mtot + grow) * KP];
+                if (probe) ms[i] = cand_ms[(size_t)t * Mtot + grow];
+            }
         }
+#pragma unroll
+        for (int i = 0; i < TOPK_MAXT; ++i) head[i] = cand_key(c[i].val, c[i].id);
     }
     if (tid < KP_MAX) s_tile[tid] = -1;
-    // each warp's kp best heads, in order: a round is the lane-local best, then two warp-wide integer reductions (largest
-    // order-preserving key, smallest id among its holders); no block barrier
+    // each warp's kp best heads, in order: a round is the lane-local best, then two warp-wide integer reductions (the high words,
+    // then the low words -- ids -- of those that share the smallest); no block barrier
     for (int j = 0; j < kp; ++j) {
-        float bv = -INFINITY;
-        int bi = 0x7fffffff, bt = -1;
+        unsigned long long best = head[0];
+        int bt = 0;
 #pragma unroll
-        for (int i = 0; i < TOPK_MAXT; ++i)
-            if (head[i].id >= 0 && cand_before(head[i].val, head[i].id, bv, bi)) { bv = head[i].val; bi = head[i].id; bt = i; }
-        const uint32_t key = bt >= 0 ? float_order_key(bv) : 0u;
-        const uint32_t wkey = __reduce_max_sync(0xffffffffu, key);
-        const uint32_t wid = __reduce_min_sync(0xffffffffu, (bt >= 0 && key == wkey) ? (uint32_t)bi : 0xffffffffu);
-        if (bt >= 0 && key == wkey && (uint32_t)bi == wid) {   // token ids are unique across tiles: one owner
+        for (int i = 1; i < TOPK_MAXT; ++i)
+            if (head[i] < best) { best = head[i]; bt = i; }
+        const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(best >> 32));
+        const uint32_t lo = __reduce_min_sync(0xffffffffu, (uint32_t)(best >> 32) == hi ? (uint32_t)best : 0xffffffffu);
+        const unsigned long long all = ((unsigned long long)hi << 32) | lo;
+        if (all == ~0ull) {          // (no more entries)
+            if (lane == 0) s_w[warp * kp + j] = ~0ull;
+        } else if (best == all) {    // token ids are unique across tiles: one owner
 #pragma unroll
-            for (int i = 0; i < TOPK_MAXT; ++i) if (i == bt) head[i].id = -1;
-            s_w[warp * kp + j].val = bv;
-            s_w[warp * kp + j].id = bi;
+            for (int i = 0; i < TOPK_MAXT; ++i) if (i == bt) head[i] = ~0ull;
+            s_w[warp * kp + j] = best;
             s_wt[warp * kp + j] = tid + TOPK_THREADS * bt;
         }
-        if (wkey == 0u && lane == 0) { s_w[warp * kp + j].val = -INFINITY; s_w[warp * kp + j].id = -1; }
     }
     __syncthreads();
     // the kp best of the warps' heads, by rank (ids are unique)
-    Cand none;
-    none.val = -INFINITY; none.id = -1;
-    if (tid < TOPK_WARPS * kp) {
-        const Cand c = s_w[tid];
-        if (c.id >= 0) {
-            int rank = 0;
-            for (int o = 0; o < TOPK_WARPS * kp; ++o) rank += s_w[o].id >= 0 && cand_before(s_w[o].val, s_w[o].id, c.val, c.id) ? 1 : 0;
-            if (rank < kp) {
-                s_tile[rank] = s_wt[tid];
-                if (!probe) topk[(size_t)grow * KP_MAX] = c;
-            }
+    if (tid < TOPK_WARPS * kp && s_w[tid] != ~0ull) {
+        const int rank = rank_among(s_w, TOPK_WARPS * kp, s_w[tid]);
+        if (rank < kp) {
+            s_tile[rank] = s_wt[tid];
+            if (!probe) topk[(size_t)grow * KP_MAX] = cand_of(s_w[tid]);
         }
     }
     __syncthreads();
     if (!probe) {
-        if (tid == 0 && s_tile[0] < 0) topk[(size_t)grow * KP_MAX] = none;
+        if (tid == 0 && s_tile[0] < 0) topk[(size_t)grow * KP_MAX] = cand_of(~0ull);
         return;
     }
     // Their lists: entry q of the tile with the p-th best head has p heads and q entries of its own before it, so only
     // p + q < kp matter.  The kp best of these by rank.
     for (int i = tid; i < kp * kp; i += TOPK_THREADS) {
         const int p = i / kp, q = i % kp;
-        if (p + q < kp) s_l[p * kp - p * (p - 1) / 2 + q] = s_tile[p] >= 0 ? cand[((size_t)s_tile[p] * Mtot + grow) * KP + q] : none;
+        if (p + q < kp) {
+            Cand c = cand_of(~0ull);
+            if (s_tile[p] >= 0) c = cand[((size_t)s_tile[p] * Mtot + grow) * KP + q];
+            s_l[p * kp - p * (p - 1) / 2 + q] = cand_key(c.val, c.id);
+        }
     }
-    if (tid < kp) topk[(size_t)grow * KP_MAX + tid] = none;     // (if there are fewer)
+    if (tid < kp) topk[(size_t)grow * KP_MAX + tid] = cand_of(~0ull);     // (if there are fewer)
     // thread-strided partial merges in tile order, then a fixed tree over threads
     float m = -INFINITY, sm = 0.f;
 #pragma unroll
@@ -1147,11 +1173,9 @@ __global__ void __launch_bounds__(TOPK_THREADS) k_topk_merge(const SeqState* sta
     __syncthreads();
     const int n_l = kp * (kp + 1) / 2;
     for (int i = tid; i < n_l; i += TOPK_THREADS) {
-        const Cand c = s_l[i];
-        if (c.id < 0) continue;
-        int rank = 0;
-        for (int o = 0; o < n_l; ++o) rank += s_l[o].id >= 0 && cand_before(s_l[o].val, s_l[o].id, c.val, c.id) ? 1 : 0;
-        if (rank < kp) topk[(size_t)grow * KP_MAX + rank] = c;
+        if (s_l[i] == ~0ull) continue;
+        const int rank = rank_among(s_l, n_l, s_l[i]);
+        if (rank < kp) topk[(size_t)grow * KP_MAX + rank] = cand_of(s_l[i]);
     }
     for (int o = TOPK_THREADS / 2; o > 0; o >>= 1) {
         if (tid < o) {
@@ -1295,18 +1319,6 @@ __device__ __forceinline__ bool tree_bar_or(bool x) {
     asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 512, p;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(r) : "r"((uint32_t)x) : "memory");
     return r != 0;
 }
-// keys of the n given ones that are smaller
-__device__ __forceinline__ int rank_among(const unsigned long long* keys, int n, unsigned long long key) {
-    int rank = 0;
-#pragma unroll 4
-    for (int o = 0; o + 1 < n; o += 2) {
-        const ulonglong2 k2 = *reinterpret_cast<const ulonglong2*>(keys + o);
-        rank += (k2.x < key ? 1 : 0) + (k2.y < key ? 1 : 0);
-    }
-    if (n & 1) rank += keys[n - 1] < key ? 1 : 0;
-    return rank;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(TREE_THREADS) k_tree_step(TreeArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
