@@ -324,7 +324,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
+        const bool leader = elect_lane();
+        {
             bool ok = true;
             uint32_t gc = 0, n_it = 0;
             const uint32_t q_addr = smem_u32(sQ);
@@ -339,11 +340,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
 #pragma unroll
                     for (int kk = 0; kk < HD / 16; ++kk) {
                         const uint32_t off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
-                        umma(tmem_s, smem_desc(q_addr + off, 16), smem_desc(k_addr + off, 16), IDESC_QK, kk > 0 ? 1u : 0u);
+                        if (leader) umma(tmem_s, smem_desc(q_addr + off, 16), smem_desc(k_addr + off, 16), IDESC_QK, kk > 0 ? 1u : 0u);
                     }
-                    umma_commit(&s_full[g & 1]);
-                    umma_commit(&k_empty[g & 1]);
-                    if (c == it.n_chunks - 1) umma_commit(q_free);
+                    if (leader) umma_commit(&s_full[g & 1]);
+                    if (leader) umma_commit(&k_empty[g & 1]);
+                    if (leader && c == it.n_chunks - 1) umma_commit(q_free);
                 };
                 ok = mbar_wait(q_full, n_it & 1, s_abort) && mbar_wait(&k_full[gc & 1], (gc >> 1) & 1, s_abort) &&
                      mbar_wait(&o_free[n_it & 1], ((n_it >> 1) & 1) ^ 1, s_abort);   // this O buffer's previous item was read out
@@ -363,12 +364,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
 #pragma unroll
                     for (int kk = 0; kk < CK / 16; ++kk) {
                         const uint32_t v_off = kk * 16 * 128;                              // V: 16 key rows of 128 bytes further
-                        umma_ta(tmem_o, tmem_base + (g & 1) * 128 + kk * 8, smem_desc(v_addr + v_off, HALF_BYTES), IDESC_PV,
+                        if (leader) umma_ta(tmem_o, tmem_base + (g & 1) * 128 + kk * 8, smem_desc(v_addr + v_off, HALF_BYTES), IDESC_PV,
                                 (c > 0 || kk > 0) ? 1u : 0u);
                     }
-                    umma_commit(pv_done);
-                    umma_commit(&v_empty[g & 1]);
-                    if (c == it.n_chunks - 1) umma_commit(&o_full[n_it & 1]);
+                    if (leader) umma_commit(pv_done);
+                    if (leader) umma_commit(&v_empty[g & 1]);
+                    if (leader && c == it.n_chunks - 1) umma_commit(&o_full[n_it & 1]);
                 }
                 gc += it.n_chunks;
                 ++n_it;

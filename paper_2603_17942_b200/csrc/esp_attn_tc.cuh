@@ -245,7 +245,8 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
+        const bool leader = elect_lane();
+        {
             bool ok = true;
             const uint32_t q_addr = smem_u32(sQ);
             auto issue_qk = [&](int c) {
@@ -254,10 +255,10 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
 #pragma unroll
                 for (int kk = 0; kk < HD / 16; ++kk) {
                     const uint32_t off = (kk >> 2) * HALF_BYTES + (kk & 3) * 32;
-                    umma(tmem_s, smem_desc(q_addr + off, 16), smem_desc(k_addr + off, 16), IDESC_QK, kk > 0 ? 1u : 0u);
+                    if (leader) umma(tmem_s, smem_desc(q_addr + off, 16), smem_desc(k_addr + off, 16), IDESC_QK, kk > 0 ? 1u : 0u);
                 }
-                umma_commit(&sm.s_full[c & 1]);
-                umma_commit(&sm.k_empty[c & 1]);
+                if (leader) umma_commit(&sm.s_full[c & 1]);
+                if (leader) umma_commit(&sm.k_empty[c & 1]);
             };
             ok = mbar_wait(sm.q_full, 0, s_abort) && mbar_wait(&sm.k_full[0], 0, s_abort);
             if (ok) {
@@ -276,11 +277,11 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
 #pragma unroll
                 for (int kk = 0; kk < CK / 16; ++kk) {
                     const uint32_t v_off = kk * 16 * 128;                              // V: 16 key rows of 128 bytes further
-                    umma_ta(tmem_base + 256, tmem_base + (c & 1) * 128 + kk * 8, smem_desc(v_addr + v_off, HALF_BYTES), IDESC_PV,
+                    if (leader) umma_ta(tmem_base + 256, tmem_base + (c & 1) * 128 + kk * 8, smem_desc(v_addr + v_off, HALF_BYTES), IDESC_PV,
                             (c > 0 || kk > 0) ? 1u : 0u);
                 }
-                umma_commit(sm.pv_done);
-                umma_commit(&sm.v_empty[c & 1]);
+                if (leader) umma_commit(sm.pv_done);
+                if (leader) umma_commit(&sm.v_empty[c & 1]);
             }
             // the arrivals on the K/V stage barriers are the item's last asynchronous ones: see them land, so that
             // a kernel that runs several items may initialise the barriers again

@@ -210,7 +210,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
+        const bool leader = elect_lane();
+        {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -227,13 +228,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
                     const uint64_t da = smem_desc(sa, 16), db = smem_desc(sa + A_BYTES, 16);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
-                        umma(tmem_d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), IDESC, (kb > sg.kb0 || k > 0) ? 1u : 0u);
+                        if (leader) umma(tmem_d, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), IDESC, (kb > sg.kb0 || k > 0) ? 1u : 0u);
                     }
-                    umma_commit(&empty[stage]);
+                    if (leader) umma_commit(&empty[stage]);
                     if (++stage == STAGES) { stage = 0; phase ^= 1; }
                 }
                 if (!ok) break;
-                umma_commit(&tfull[buf]);
+                if (leader) umma_commit(&tfull[buf]);
             }
             if (!ok) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
         }

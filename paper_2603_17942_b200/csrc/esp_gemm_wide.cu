@@ -173,7 +173,8 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
             if (!ok) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        const bool leader = elect_lane();
+        {
             constexpr uint32_t IDESC = idesc_of(WR);
             bool ok = true;
             int slot = 0, piece = 0;
@@ -202,22 +203,22 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k) {
                             const uint32_t acc = (u > beg || k > 0) ? 1u : 0u;
-                            umma(tmem_base, dw + (uint64_t)(k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
-                            umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
+                            if (leader) umma(tmem_base, dw + (uint64_t)(k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
+                            if (leader) umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
                         }
-                        umma_commit(&empty[sh]);
+                        if (leader) umma_commit(&empty[sh]);
                         if (!mbar_wait(&full[sl], pl, s_abort)) { ok = false; break; }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint64_t dl = smem_desc(smem_u32(ring + sl * SLOT_BYTES), 16);
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k) {
-                            umma(tmem_base, dw + (uint64_t)(k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
-                            umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
+                            if (leader) umma(tmem_base, dw + (uint64_t)(k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
+                            if (leader) umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dl + (uint64_t)(k * 2), IDESC, 1u);
                         }
-                        umma_commit(&empty[sw]);
-                        umma_commit(&empty[sl]);
+                        if (leader) umma_commit(&empty[sw]);
+                        if (leader) umma_commit(&empty[sl]);
                     }
-                    if (ok) umma_commit(tfull);
+                    if (leader && ok) umma_commit(tfull);
                 }
             } while (ok && next_item(w));
             if (!ok) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
@@ -383,7 +384,8 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide_some(const __grid
             if (!ok) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        const bool leader = elect_lane();
+        {
             bool ok = true;
             int st = 0;
             uint32_t phase = 0;
@@ -399,13 +401,13 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide_some(const __grid
                     const uint32_t base = smem_u32(ring + st * p.stage_bytes);
                     const uint64_t dw = smem_desc(base, 16), dh = smem_desc(base + A_BYTES, 16), dl = smem_desc(base + A_BYTES + p.lo_off, 16);
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k) umma(acc, dw + (uint64_t)(k * 2), dh + (uint64_t)(k * 2), idesc, (u > 0 || k > 0) ? 1u : 0u);
+                    for (int k = 0; k < BK / 16; ++k) if (leader) umma(acc, dw + (uint64_t)(k * 2), dh + (uint64_t)(k * 2), idesc, (u > 0 || k > 0) ? 1u : 0u);
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k) umma(acc, dw + (uint64_t)(k * 2), dl + (uint64_t)(k * 2), idesc, 1u);
-                    umma_commit(&empty[st]);
+                    for (int k = 0; k < BK / 16; ++k) if (leader) umma(acc, dw + (uint64_t)(k * 2), dl + (uint64_t)(k * 2), idesc, 1u);
+                    if (leader) umma_commit(&empty[st]);
                     if (++st == p.stages) { st = 0; phase ^= 1; }
                 }
-                if (ok) umma_commit(&tfull[n & 1]);
+                if (leader && ok) umma_commit(&tfull[n & 1]);
             }
             if (!ok) { set_error(p.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
         }

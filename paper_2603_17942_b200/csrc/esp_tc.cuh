@@ -89,6 +89,13 @@ __device__ __forceinline__ void umma_ta(uint32_t tmem_d, uint32_t tmem_a, uint64
         ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// One lane of a warp that issues tensor-core instructions.  The warp walks its loop as a whole and only the instructions are under
+// the lane's predicate: the descriptors are then warp-uniform values (under a lane's branch every one is moved lane by lane).
+__device__ __forceinline__ bool elect_lane() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
