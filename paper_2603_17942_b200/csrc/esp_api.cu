@@ -1236,7 +1236,8 @@ int esp_tree_attention(int32_t dtype, int32_t batch, int32_t n_rows, int32_t L, 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     char* sc = reinterpret_cast<char*>(scratch);
     // the error word starts at zero (the scratch may hold an earlier call's bytes); the partials are written before they are read
-    if (cudaMemsetAsync(sc, 0, 256, s) != cudaSuccess) return ESP_E_CUDA;
+    const int n_split_launch = (L + S - 1) / S;
+    if (n_split_launch == 0 && cudaMemsetAsync(sc, 0, 256, s) != cudaSuccess) return ESP_E_CUDA;
     AttnArgs a;
     memset(&a, 0, sizeof(a));
     a.q = q; a.kc = kcache; a.vc = vcache; a.out = out;
@@ -1250,7 +1251,7 @@ int esp_tree_attention(int32_t dtype, int32_t batch, int32_t n_rows, int32_t L, 
     a.Hq = n_q_heads; a.Hkv = n_kv_heads; a.h = head_dim; a.cap = cap; a.split_len = S; a.n_split_max = (int)ns; a.dcap = dcap;
     a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)head_dim));
     a.err = reinterpret_cast<int*>(sc);
-    const int n_split_launch = (L + S - 1) / S;
+    a.clear_err = n_split_launch > 0;
     const bool mma = dtype == 1 && attn_tc_supported(head_dim, n_q_heads, n_kv_heads);
     if (mma) {
         if (attn_tc_run(q, kcache, vcache, batch, n_q_heads, n_kv_heads, cap, a, n_split_launch, s)) return ESP_E_BADCFG;

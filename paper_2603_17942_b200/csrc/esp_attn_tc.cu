@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(ONCE_THREADS, 1) k_attn_bulk_tc_once(const __g
 
     const AttnArgs& a = p.a;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) attn_clear_error(a);
     BulkItem it;
     it.split = blockIdx.x;
     it.kvh = blockIdx.y / p.n_row_tiles;
@@ -180,6 +181,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
 
     const AttnArgs& a = p.a;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && p.seq0 == 0) attn_clear_error(a);
 
     // Read before pdl_wait(): the sequence state and the cache below T0, both written by earlier steps.
     // The dependent kernel is released by the producer thread once its wait has returned (trigger_after_wait).

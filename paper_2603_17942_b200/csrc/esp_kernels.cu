@@ -774,6 +774,7 @@ __global__ void __launch_bounds__(128 * bulk_groups<T, HD>()) k_attn_bulk_simt(A
     T* s_k = reinterpret_cast<T*>(bulk_smem) + kg * 4 * 32 * LD;      // [2][32][LD]
     T* s_v = s_k + 2 * 32 * LD;                                       // [2][32][LD]
     float* s_qall = reinterpret_cast<float*>(reinterpret_cast<T*>(bulk_smem) + KG * 4 * 32 * LD) + kg * BS_WARPS * BS_PW * HD;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) attn_clear_error(a);
     const int kvh = blockIdx.y, group = a.Hq / a.Hkv;
     const int split = blockIdx.z % n_split_launch, seq = blockIdx.z / n_split_launch;
     const int beg = split * a.split_len;
@@ -792,7 +793,7 @@ __global__ void __launch_bounds__(128 * bulk_groups<T, HD>()) k_attn_bulk_simt(A
         cta_end = max(cta_end, end[w]);
     }
     pdl_wait();             // (the row table above was written by an earlier step)
-    pdl_launch_dependents();      // the tail kernel computes its tail beside this kernel: queries, keys and values are there
+    if (threadIdx.x == 0) pdl_launch_dependents();      // the tail kernel computes its tail beside this kernel: queries, keys and values are there
 #pragma unroll
     for (int w = 0; w < BS_PW; ++w)
         if (end[w] > 0) {
