@@ -108,15 +108,15 @@ __device__ __forceinline__ void resid_norm_row(float* xr, const StreamK& sk, int
 // The same for launches of many rows (d <= 128 * NW * 4): NW warps per row, four groups per warp in registers, the pieces
 // of the four groups requested together.  Sums, products and their order are resid_norm_row's, so are the bits.
 constexpr int NORM_MANY_WARPS = 8, NORM_MANY_D = TILE_N * NORM_MANY_WARPS * 4;
-template <typename T, typename Bar>
+template <typename T, int NW, int NG, int PB, typename Bar>
 __device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk, int sk_row, const T* g, T* yr, T* yr_lo, int d, float eps,
                                                     float* copy_row, float* red, int warp, int lane, Bar bar) {
     const int ng = (d + TILE_N - 1) / TILE_N;
-    float4 x[4], acc[4];
-    int n[4], idx0[4];
+    float4 x[NG], acc[NG];
+    int n[NG], idx0[NG];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int gi = warp + NORM_MANY_WARPS * u, j = gi * TILE_N + lane * 4;
+    for (int u = 0; u < NG; ++u) {
+        const int gi = warp + NW * u, j = gi * TILE_N + lane * 4;
         x[u] = acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         n[u] = 0;
         idx0[u] = gi;
@@ -125,24 +125,28 @@ __device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk
             if (sk.partials) n[u] = __ldg(&sk.table[gi].n);
         }
     }
-    int most = n[0] > n[1] ? n[0] : n[1];
-    most = max(most, max(n[2], n[3]));
+    int most = 0;
+#pragma unroll
+    for (int u = 0; u < NG; ++u) most = max(most, n[u]);
     const float* base = sk.partials + (size_t)sk_row * TILE_N + lane * 4;
     const size_t piece = (size_t)sk.rows * TILE_N;
-#pragma unroll 2
-    for (int c = 0; c < most; ++c) {          // pieces in ascending order, as sk_sum4 adds them
-        float4 t[4];
+    for (int c0 = 0; c0 < most; c0 += PB) {          // pieces in ascending order, as sk_sum4 adds them
+        float4 t[PB][NG];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            t[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c < n[u]) t[u] = __ldcg(reinterpret_cast<const float4*>(base + (size_t)__ldg(&sk.table[idx0[u]].idx[c]) * piece));
-        }
+        for (int c = 0; c < PB; ++c)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) { acc[u].x += t[u].x; acc[u].y += t[u].y; acc[u].z += t[u].z; acc[u].w += t[u].w; }
+            for (int u = 0; u < NG; ++u) {
+                t[c][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (c0 + c < n[u]) t[c][u] = __ldcg(reinterpret_cast<const float4*>(base + (size_t)__ldg(&sk.table[idx0[u]].idx[c0 + c]) * piece));
+            }
+#pragma unroll
+        for (int c = 0; c < PB; ++c)
+#pragma unroll
+            for (int u = 0; u < NG; ++u) { acc[u].x += t[c][u].x; acc[u].y += t[c][u].y; acc[u].z += t[c][u].z; acc[u].w += t[c][u].w; }
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int gi = warp + NORM_MANY_WARPS * u, j = gi * TILE_N + lane * 4;
+    for (int u = 0; u < NG; ++u) {
+        const int gi = warp + NW * u, j = gi * TILE_N + lane * 4;
         if (gi >= ng) break;
         if (sk.partials && j < d) {
             x[u].x = __fadd_rn(x[u].x, acc[u].x); x[u].y = __fadd_rn(x[u].y, acc[u].y);
@@ -159,8 +163,8 @@ __device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk
     for (int gi = 0; gi < ng; ++gi) tot = __fadd_rn(tot, red[gi]);
     const float rinv = 1.0f / sqrtf(__fadd_rn(tot / (float)d, eps));
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int j = (warp + NORM_MANY_WARPS * u) * TILE_N + lane * 4;
+    for (int u = 0; u < NG; ++u) {
+        const int j = (warp + NW * u) * TILE_N + lane * 4;
         if (j >= d) break;
         const float xv[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
         T gg[4], o[4], ol[4];
