@@ -61,7 +61,7 @@ constexpr int ONCE_THREADS = 320;          // producer warp, MMA warp, 8 softmax
 constexpr int ONCE_OFF_BAR = ITEM_BYTES;
 constexpr size_t ONCE_SMEM_BYTES = 1024 + ONCE_OFF_BAR + 256;
 
-__global__ void __launch_bounds__(ONCE_THREADS, 1) k_attn_bulk_tc_once(const __grid_constant__ BulkParams p) {
+__device__ __forceinline__ void bulk_once(const BulkParams& p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ int s_T0max;
     __shared__ float s_xchg[2][2 * MP];   // [exchange parity][half][pair]
@@ -151,6 +151,11 @@ __global__ void __launch_bounds__(ONCE_THREADS, 1) k_attn_bulk_tc_once(const __g
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
     }
 }
+__global__ void __launch_bounds__(ONCE_THREADS, 1) k_attn_bulk_tc_once(const __grid_constant__ BulkParams p) { bulk_once(p); }
+// The same with 112 registers: its CTA then fits on an SM with up to seven CTAs of the q/k/v finish kernel in front, where the one
+// above, with 126, starts only when these have ended (from six on).  Step of sixteen 8B layers, 68 rows: 2197 -> 2165 us; where
+// there is nothing to gain its spills cost (120-row blocks 1547 -> 1557).
+__global__ void __maxnreg__(112) k_attn_bulk_tc_once_slim(const __grid_constant__ BulkParams p) { bulk_once(p); }
 
 // ---- persistent CTAs: used when the launch has clearly more items than SMs.
 // One work item = (split of the cache, KV head, row tile, sequence); what a role needs to know about it.
@@ -609,9 +614,12 @@ int attn_tc_launch(const AttnTc* t, const AttnArgs& a, int batch, int n_split_la
             // (nearly) every CTA runs once: one item per CTA.  Measured crossover: the persistent kernel wins from
             // about 1.2 waves when timed alone, a little later inside a step, where its larger register and
             // shared-memory footprint delays its start behind the kernel before it
-            if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_attn_bulk_tc_once), (int)ONCE_SMEM_BYTES)) return -1;
+            // (CTAs of four warps of the q/k/v finish kernel per SM: a warp per row and head)
+            const long long finish = ((long long)rows_cap * ((a.Hq + 2 * a.Hkv + 3) / 4) * batch + n_sm - 1) / n_sm;
+            const auto kernel = pdl && finish >= 6 && finish <= 7 ? k_attn_bulk_tc_once_slim : k_attn_bulk_tc_once;
+            if (ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), (int)ONCE_SMEM_BYTES)) return -1;
             dim3 grid(n_split_launch, a.Hkv * p.n_row_tiles, batch);
-            if (launch_k(k_attn_bulk_tc_once, grid, dim3(ONCE_THREADS), ONCE_SMEM_BYTES, s, pdl, p) != cudaSuccess) return -1;
+            if (launch_k(kernel, grid, dim3(ONCE_THREADS), ONCE_SMEM_BYTES, s, pdl, p) != cudaSuccess) return -1;
         } else {
             // persistent CTAs, one per SM, walk the (split, KV head, row tile, sequence) items round-robin
             if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_attn_bulk_tc), (int)SMEM_BYTES)) return -1;
