@@ -1,9 +1,9 @@
 // Small-M bf16 GEMM for the decode-and-verify step on the Blackwell tensor
-// cores: y[row][n] = sum_k x[row][k] * w[n][k] for at most 80 rows.
+// cores: y[row][n] = sum_k x[row][k] * w[n][k] for at most 128 rows.
 //
 // The weight matrix is the MMA "A" operand (128 output features on the MMA-M
-// dimension), the token rows are the "B" operand (MMA-N = 80), so the large
-// operand fills the tensor core and the 80 rows cost no padding.  Both
+// dimension), the token rows are the "B" operand (MMA-N = the rows), so the
+// large operand fills the tensor core and the rows cost little padding.  Both
 // operands are K-major and arrive through TMA with the 128-byte swizzle;
 // tcgen05.mma accumulates fp32 in tensor memory; four epilogue warps read it
 // back with tcgen05.ld.
@@ -13,11 +13,11 @@
 // equal contiguous ranges to one persistent CTA per SM.  A tile whose k-range
 // is split over several CTAs is summed from fp32 partials in CTA order (a
 // fixed order, independent of arrival order and of the number of rows):
-//   * EPI_PARTIAL (QKV, O, down: every tile is split): the kernel only stores
-//     partials; the kernel that consumes the result (RoPE/cache write,
-//     residual add + RMSNorm) sums them, fully parallel and off this kernel's
+//   * EPI_PARTIAL (every layer GEMM): the kernel only stores partials; the
+//     kernel that consumes the result (RoPE/cache write, residual add +
+//     RMSNorm, SiLU*up) sums them, fully parallel and off this kernel's
 //     critical path;
-//   * fused epilogues (gate/up with SiLU*up, LM head with Top-K'): whichever
+//   * fused epilogue (LM head with Top-K'): whichever
 //     contributor of a split tile arrives last sums and finishes it.  Each CTA
 //     does its split pieces first and its whole tiles after, so this happens
 //     while the weight stream of the whole tiles is running.
@@ -43,8 +43,9 @@ using namespace tc;
 // NRS = rows of a block that are loaded and multiplied: 80, or 128 for blocks of more than 80 rows; two-plane plans have
 // instances in between and below (TWO_PLANE_ROWS), the smallest that holds the handle's blocks.  Every 16 KB of weights come
 // with 256 bytes per row of activations from L2, through the same 64 bytes per clock and SM, and rows cost ring stages:
-// step of eight 8B layers at 1k positions, 80 rows loaded -> this: 24-row trees 1154 -> 1046 us, 68-row trees 1256 -> 1241; request with 30-row static trees 20.37 -> 18.70 ms.  (A row's bits do not depend on the instance.)  NQ = sequences one launch covers
-// (the LM head takes up to three): the first NRS rows of their activation blocks ([RT][K] each, consecutive) are gathered by one
+// step of eight 8B layers at 1k positions, 80 rows loaded -> this: 24-row trees 1154 -> 1046 us, 68-row trees 1256 -> 1241;
+// request with 30-row static trees 20.37 -> 18.70 ms.  (A row's bits do not depend on the instance.)  NQ = sequences one
+// launch covers (the LM head takes up to three): the first NRS rows of their activation blocks ([RT][K] each, consecutive) are gathered by one
 // 3-D TMA box into one B operand of NQ*NRS <= 256 rows, so the weights are streamed once for all.  (The layer GEMMs of
 // several sequences: esp_gemm_wide.cu.)
 //

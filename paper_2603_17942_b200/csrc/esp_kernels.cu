@@ -185,8 +185,9 @@ __global__ void __launch_bounds__(1024) k_resid_norm(const SeqState* states, flo
                           copy_out ? copy_out + row : nullptr, red, pf, warp, lane, [] { __syncthreads(); });
 }
 
-// The same, 512 threads per row: the next GEMM's block fits beside it and starts its weight stream meanwhile.  Rows of more than 2048 and up to 4096
-// elements; step of sixteen 8B layers 2158 -> 2148 us, with 120-row blocks (eight layers) 1554 -> 1541.
+// The same, 512 threads per row: the next GEMM's block fits beside it and starts its weight stream meanwhile.  Rows of
+// more than 2048 and up to 4096 elements; step of sixteen 8B layers 2158 -> 2148 us, with 120-row blocks (eight layers)
+// 1554 -> 1541.
 constexpr int NORM_HALF_WARPS = 16, NORM_HALF_D = TILE_N * NORM_HALF_WARPS * 2;
 __global__ void __launch_bounds__(NORM_HALF_WARPS * 32, 1) k_resid_norm_half(const SeqState* states, float* hres, StreamK sk, const __nv_bfloat16* g,
                                                                           __nv_bfloat16* y, __nv_bfloat16* y_lo, int d, float eps, float* copy_out) {
@@ -1092,8 +1093,8 @@ __device__ __forceinline__ Cand cand_of(unsigned long long key) {
 // lse = max + log(sum exp) merged over tiles in a fixed order.
 // What bounds it is the number of dependent trips to L2, so there are two: the heads of all tiles' lists (with the tiles'
 // (max, sum) pairs), then the whole lists of the K' tiles with the best heads -- an entry of any other tile has K' heads
-// before it.  A vocabulary of 1002 tiles, K' = 11, 4 probe rows of 68: 25 -> 17 us (all lists of a row staged in shared
-// memory, K' rounds over all of them).
+// before it.  A vocabulary of 1002 tiles, K' = 11, 4 probe rows of 68: 25 us with all lists of a row staged in
+// shared memory and K' rounds over them, 17 with these two trips, 12.7 with the entries ranked as packed keys.
 constexpr int TOPK_THREADS = 256, TOPK_WARPS = TOPK_THREADS / 32;
 constexpr int TOPK_MAXT = 8;   // tiles per thread (n_tiles <= 2048)
 __global__ void __launch_bounds__(TOPK_THREADS) k_topk_merge(const SeqState* states, const Cand* cand, const float2* cand_ms,
@@ -1330,7 +1331,8 @@ __device__ __forceinline__ unsigned long long node_key(float lp, int depth, int 
 // shared-memory loads counts.  So the first half of the block does what the next forward pass's rows hang on -- verification,
 // lists, tree, row table -- and the other half compacts the cache and updates the masks meanwhile; keys are ranked from
 // packed arrays, breadth-first places come from bit masks, and counters and the error word are fetched ahead of their use.
-// 64 nodes, K = 10, four probes: 48 -> 32 us for the ranking alone, step of eight 8B layers 1278 -> 1255 us with the halves; 16 nodes, K = 5, three probes: its request 5209 -> 4680 us a step of 35 kernels.
+// 64 nodes, K = 10, four probes: 48 -> 32 us with the packed ranking, 26 with the halves (step of eight 8B layers
+// 1278 -> 1255 us).  16 nodes, K = 5, three probes: 8.4 us (a request of 32 small steps 5209 -> 4680 us).
 constexpr int TREE_THREADS = 1024, TREE_BUILD = 512;      // threads; those of them that build the tree
 __device__ __forceinline__ void tree_bar() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 __device__ __forceinline__ bool tree_bar_or(bool x) {
