@@ -107,10 +107,36 @@ __device__ __forceinline__ void resid_norm_row(float* xr, const StreamK& sk, int
 
 // The same for launches of many rows (d <= 128 * NW * 4): NW warps per row, four groups per warp in registers, the pieces
 // of the four groups requested together.  Sums, products and their order are resid_norm_row's, so are the bits.
+// put(group, sum) hands a group's sum of squares to every warp of the row, bar() waits for all of them.
+// `ahead` is what a warp has fetched before the partials exist: counts, the first seven places and the norm weights.
 constexpr int NORM_MANY_WARPS = 8, NORM_MANY_D = TILE_N * NORM_MANY_WARPS * 4;
-template <typename T, int NW, int NG, int PB, typename Bar>
+template <int NG>
+struct NormAhead {
+    uint32_t e[NG][4];        // first half of the group's entry: count, then places, a halfword each
+    uint2 g[NG];
+};
+
+template <int NW, int NG>
+__device__ __forceinline__ void norm_prefetch_many(NormAhead<NG>& ah, const StreamK& sk, const __nv_bfloat16* g, int d, int warp, int lane) {
+#pragma unroll
+    for (int u = 0; u < NG; ++u) {
+        const int gi = warp + NW * u, j = gi * TILE_N + lane * 4;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ah.e[u][i] = 0;
+        ah.g[u] = make_uint2(0, 0);
+        if (j < d) {
+            if (sk.partials) {
+                const uint4 e = __ldg(reinterpret_cast<const uint4*>(sk.table + gi));
+                ah.e[u][0] = e.x; ah.e[u][1] = e.y; ah.e[u][2] = e.z; ah.e[u][3] = e.w;
+            }
+            ah.g[u] = __ldg(reinterpret_cast<const uint2*>(g + j));
+        }
+    }
+}
+
+template <typename T, int NW, int NG, int PB, typename Put, typename Bar>
 __device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk, int sk_row, const T* g, T* yr, T* yr_lo, int d, float eps,
-                                                    float* copy_row, float* red, int warp, int lane, Bar bar) {
+                                                    float* copy_row, float* red, const NormAhead<NG>* ahead, int warp, int lane, Put put, Bar bar) {
     const int ng = (d + TILE_N - 1) / TILE_N;
     float4 x[NG], acc[NG];
     int n[NG], idx0[NG];
@@ -122,7 +148,7 @@ __device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk
         idx0[u] = gi;
         if (gi < ng && j < d) {
             x[u] = __ldcg(reinterpret_cast<const float4*>(xr + j));
-            if (sk.partials) n[u] = __ldg(&sk.table[gi].n);
+            if (sk.partials) n[u] = ahead ? (int)(ahead->e[u][0] & 0xffffu) : (int)__ldg(&sk.table[gi].n);
         }
     }
     int most = 0;
@@ -130,7 +156,25 @@ __device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk
     for (int u = 0; u < NG; ++u) most = max(most, n[u]);
     const float* base = sk.partials + (size_t)sk_row * TILE_N + lane * 4;
     const size_t piece = (size_t)sk.rows * TILE_N;
-    for (int c0 = 0; c0 < most; c0 += PB) {          // pieces in ascending order, as sk_sum4 adds them
+    int c0 = 0;
+    if (ahead) {                                     // the first batch without a trip to the table
+        static_assert(PB <= 7, "places of the first batch");
+        float4 t[PB][NG];
+#pragma unroll
+        for (int c = 0; c < PB; ++c)
+#pragma unroll
+            for (int u = 0; u < NG; ++u) {
+                t[c][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                const uint32_t at = (ahead->e[u][(c + 1) >> 1] >> (((c + 1) & 1) * 16)) & 0xffffu;
+                if (c < n[u]) t[c][u] = __ldcg(reinterpret_cast<const float4*>(base + (size_t)at * piece));
+            }
+#pragma unroll
+        for (int c = 0; c < PB; ++c)
+#pragma unroll
+            for (int u = 0; u < NG; ++u) { acc[u].x += t[c][u].x; acc[u].y += t[c][u].y; acc[u].z += t[c][u].z; acc[u].w += t[c][u].w; }
+        c0 = PB;
+    }
+    for (; c0 < most; c0 += PB) {          // pieces in ascending order, as sk_sum4 adds them
         float4 t[PB][NG];
 #pragma unroll
         for (int c = 0; c < PB; ++c)
@@ -155,7 +199,7 @@ __device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk
         }
         float ss = __fmaf_rn(x[u].w, x[u].w, __fmaf_rn(x[u].z, x[u].z, __fmaf_rn(x[u].y, x[u].y, __fmul_rn(x[u].x, x[u].x))));
         ss = warp_sum(ss);
-        if (lane == 0) red[gi] = ss;
+        if (lane == 0) put(gi, ss);
     }
     bar();
     float tot = 0.f;
@@ -167,8 +211,10 @@ __device__ __forceinline__ void resid_norm_row_many(float* xr, const StreamK& sk
         const int j = (warp + NW * u) * TILE_N + lane * 4;
         if (j >= d) break;
         const float xv[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
-        T gg[4], o[4], ol[4];
-        load4(gg, g + j);
+        __align__(8) T gg[4];
+        T o[4], ol[4];
+        if (ahead) *reinterpret_cast<uint2*>(gg) = ahead->g[u];
+        else load4(gg, g + j);
 #pragma unroll
         for (int i = 0; i < 4; ++i) split_bf16(__fmul_rn(__fmul_rn(xv[i], rinv), to_f32(gg[i])), o[i], ol[i]);
         *reinterpret_cast<uint2*>(yr + j) = *reinterpret_cast<const uint2*>(o);

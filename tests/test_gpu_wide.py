@@ -279,3 +279,27 @@ def test_rows_have_the_bits_of_the_greedy_handle_in_every_instance(weights):
         h.close()
     for f in first[1:]:
         assert torch.equal(f, first[0])
+
+
+@pytest.mark.parametrize("d", [2056, 2944, 4096])
+def test_a_row_normed_by_two_blocks_has_the_bits_of_one_block(d):
+    """Rows of more than 2048 features: up to 74 of them are normed by a pair of blocks each, 75 by one block each (17, 23 and
+    32 groups of 128; the first row of the step, bit for bit)."""
+    shape = BF16_SMALL.replace(name="bf16-wide-rows", d_model=d, n_layers=2, n_q_heads=16, n_kv_heads=4, d_ffn=1376)
+    w = synth.make_weights(shape, seed=4, device="cuda", gain_jitter=True, std=0.03)
+    prompt = synth.make_prompt(shape.vocab, 60, 4)
+    first = []
+    for nodes in (72, 71, 13, 0):
+        kw = dict(n_probes=0, max_nodes=1) if not nodes else dict(n_probes=3, topk=10, max_nodes=nodes, expand_width=0, n_anchor=1)
+        h = P.Handle(shape, P.spec_cfg(**kw), w, max_seq_len=300, max_batch=1)
+        logits = torch.zeros(1, R, shape.vocab, dtype=torch.float32, device="cuda")
+        P.esp_debug_capture(h.h, logits)
+        h.prefill(prompt)
+        assert h.state()["n_rows"] == (nodes + 3 if nodes else 1)
+        h.step()
+        assert h.stats().device_error == 0 and torch.isfinite(logits[0, 0]).all()
+        first.append(logits[0, 0].clone())
+        h.close()
+    assert first[0].abs().max() > 0
+    for f in first[1:]:
+        assert torch.equal(f, first[0])
