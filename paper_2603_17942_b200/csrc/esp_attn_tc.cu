@@ -353,19 +353,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_attn_bulk_tc(const __grid_co
                     if (leader) umma_commit(&k_empty[g & 1]);
                     if (leader && c == it.n_chunks - 1) umma_commit(q_free);
                 };
-                ok = mbar_wait(q_full, n_it & 1, s_abort) && mbar_wait(&k_full[gc & 1], (gc >> 1) & 1, s_abort) &&
-                     mbar_wait(&o_free[n_it & 1], ((n_it >> 1) & 1) ^ 1, s_abort);   // this O buffer's previous item was read out
+                ok = __all_sync(0xffffffffu, mbar_wait(q_full, n_it & 1, s_abort) && mbar_wait(&k_full[gc & 1], (gc >> 1) & 1, s_abort) &&
+                                                  mbar_wait(&o_free[n_it & 1], ((n_it >> 1) & 1) ^ 1, s_abort));   // this O buffer's previous item was read out
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 issue_qk(0);
                 for (int c = 0; c < it.n_chunks && ok; ++c) {
                     const uint32_t g = gc + c;
                     if (c + 1 < it.n_chunks) {     // S of the next chunk while the softmax of this one runs
-                        if (!mbar_wait(&k_full[(g + 1) & 1], ((g + 1) >> 1) & 1, s_abort)) { ok = false; break; }
+                        if (!__all_sync(0xffffffffu, mbar_wait(&k_full[(g + 1) & 1], ((g + 1) >> 1) & 1, s_abort))) { ok = false; break; }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         issue_qk(c + 1);
                     }
-                    if (!mbar_wait(p_ready, g & 1, s_abort) || !mbar_wait(&v_full[g & 1], (g >> 1) & 1, s_abort)) { ok = false; break; }
+                    if (!__all_sync(0xffffffffu, mbar_wait(p_ready, g & 1, s_abort) && mbar_wait(&v_full[g & 1], (g >> 1) & 1, s_abort))) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t v_addr = smem_u32(smem + OFF_KV + (g & 1) * KV_STAGE + K_BYTES);
 #pragma unroll

@@ -260,18 +260,18 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
                 if (leader) umma_commit(&sm.s_full[c & 1]);
                 if (leader) umma_commit(&sm.k_empty[c & 1]);
             };
-            ok = mbar_wait(sm.q_full, 0, s_abort) && mbar_wait(&sm.k_full[0], 0, s_abort);
+            ok = __all_sync(0xffffffffu, mbar_wait(sm.q_full, 0, s_abort) && mbar_wait(&sm.k_full[0], 0, s_abort));
             if (ok) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 issue_qk(0);
             }
             for (int c = 0; c < it.n_chunks && ok; ++c) {
                 if (c + 1 < it.n_chunks) {     // S of the next chunk while the softmax of this one runs
-                    if (!mbar_wait(&sm.k_full[(c + 1) & 1], ((c + 1) >> 1) & 1, s_abort)) { ok = false; break; }
+                    if (!__all_sync(0xffffffffu, mbar_wait(&sm.k_full[(c + 1) & 1], ((c + 1) >> 1) & 1, s_abort))) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     issue_qk(c + 1);
                 }
-                if (!mbar_wait(sm.p_ready, c & 1, s_abort) || !mbar_wait(&sm.v_full[c & 1], (c >> 1) & 1, s_abort)) { ok = false; break; }
+                if (!__all_sync(0xffffffffu, mbar_wait(sm.p_ready, c & 1, s_abort) && mbar_wait(&sm.v_full[c & 1], (c >> 1) & 1, s_abort))) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t v_addr = smem_u32(smem + OFF_KV + (c & 1) * KV_STAGE + K_BYTES);
 #pragma unroll
@@ -286,7 +286,7 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
             // the arrivals on the K/V stage barriers are the item's last asynchronous ones: see them land, so that
             // a kernel that runs several items may initialise the barriers again
             for (int c = it.n_chunks - 2 < 0 ? 0 : it.n_chunks - 2; c < it.n_chunks && ok; ++c)
-                ok = mbar_wait(&sm.k_empty[c & 1], (c >> 1) & 1, s_abort) && mbar_wait(&sm.v_empty[c & 1], (c >> 1) & 1, s_abort);
+                ok = __all_sync(0xffffffffu, mbar_wait(&sm.k_empty[c & 1], (c >> 1) & 1, s_abort) && mbar_wait(&sm.v_empty[c & 1], (c >> 1) & 1, s_abort));
             if (!ok) { set_error(a.err, DEV_E_WAIT_TIMEOUT); *s_abort = 1; }
         }
     } else if (warp < 10) {

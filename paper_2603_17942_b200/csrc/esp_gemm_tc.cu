@@ -219,11 +219,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
             for (int i = 0; i < rng.n_seg && ok; ++i) {
                 const Seg sg = get_seg(rng, i);
                 const int buf = i & 1;
-                if (!mbar_wait(&tempty[buf], ((i >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
+                if (!__all_sync(0xffffffffu, mbar_wait(&tempty[buf], ((i >> 1) & 1) ^ 1, s_abort))) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t tmem_d = tmem_base + buf * ACC_COLS;
                 for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-                    if (!mbar_wait(&full[stage], phase, s_abort)) { ok = false; break; }
+                    if (!__all_sync(0xffffffffu, mbar_wait(&full[stage], phase, s_abort))) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t sa = smem_u32(stages + stage * STAGE_BYTES);
                     const uint64_t da = smem_desc(sa, 16), db = smem_desc(sa + A_BYTES, 16);

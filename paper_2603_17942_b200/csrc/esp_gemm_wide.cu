@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
             do {
                 for (int u = u0; u < u1 && ok; ++piece) {
                     const int end = (u / p.KB + 1) * p.KB < u1 ? (u / p.KB + 1) * p.KB : u1;
-                    if (!mbar_wait(tempty, (piece & 1) ^ 1, s_abort)) { ok = false; break; }     // (a fresh barrier passes parity 1)
+                    if (!__all_sync(0xffffffffu, mbar_wait(tempty, (piece & 1) ^ 1, s_abort))) { ok = false; break; }     // (a fresh barrier passes parity 1)
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     for (const int beg = u; u < end; ++u) {
                         const int sw = slot;
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
                         const int sl = slot;
                         const uint32_t pl = phase;
                         next(slot, phase);
-                        if (!mbar_wait(&full[sw], pw, s_abort) || !mbar_wait(&full[sh], ph, s_abort)) { ok = false; break; }
+                        if (!__all_sync(0xffffffffu, mbar_wait(&full[sw], pw, s_abort) && mbar_wait(&full[sh], ph, s_abort))) { ok = false; break; }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint64_t dw = smem_desc(smem_u32(ring + sw * SLOT_BYTES), 16);
                         const uint64_t dh = smem_desc(smem_u32(ring + sh * SLOT_BYTES), 16);
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide(const __grid_cons
                             if (leader) umma(tmem_base + 256, dw + (uint64_t)((A_BYTES >> 4) + k * 2), dh + (uint64_t)(k * 2), IDESC, acc);
                         }
                         if (leader) umma_commit(&empty[sh]);
-                        if (!mbar_wait(&full[sl], pl, s_abort)) { ok = false; break; }
+                        if (!__all_sync(0xffffffffu, mbar_wait(&full[sl], pl, s_abort))) { ok = false; break; }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint64_t dl = smem_desc(smem_u32(ring + sl * SLOT_BYTES), 16);
 #pragma unroll
@@ -393,10 +393,10 @@ __global__ void __launch_bounds__(WIDE_THREADS, 1) k_gemm_wide_some(const __grid
                 const WideItem it = item(i0 + n);
                 const uint32_t idesc = idesc_of((p.tile0[it.rt + 1] - p.tile0[it.rt]) * WB);
                 const uint32_t acc = tmem_base + (n & 1) * 256;
-                if (!mbar_wait(&tempty[n & 1], ((n >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }     // (a fresh barrier passes parity 1)
+                if (!__all_sync(0xffffffffu, mbar_wait(&tempty[n & 1], ((n >> 1) & 1) ^ 1, s_abort))) { ok = false; break; }     // (a fresh barrier passes parity 1)
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int u = 0; u < it.len; ++u) {
-                    if (!mbar_wait(&full[st], phase, s_abort)) { ok = false; break; }
+                    if (!__all_sync(0xffffffffu, mbar_wait(&full[st], phase, s_abort))) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t base = smem_u32(ring + st * p.stage_bytes);
                     const uint64_t dw = smem_desc(base, 16), dh = smem_desc(base + A_BYTES, 16), dl = smem_desc(base + A_BYTES + p.lo_off, 16);
