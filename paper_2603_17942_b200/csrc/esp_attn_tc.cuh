@@ -567,7 +567,9 @@ __device__ __forceinline__ void store_task(float l, const float (&o)[16], const 
             oh[i] = __float2bfloat16_rn(v);
             ol[i] = __float2bfloat16_rn(__fsub_rn(v, __bfloat162float(oh[i])));
         }
-        *reinterpret_cast<uint4*>(out + j * 32) = *reinterpret_cast<const uint4*>(oh);
+        // (a caller's `out` needs no more than 8 bytes; queries and cache are under the tensor maps' 16)
+        *reinterpret_cast<uint2*>(out + j * 32) = *reinterpret_cast<const uint2*>(oh);
+        *reinterpret_cast<uint2*>(out + j * 32 + 4) = *reinterpret_cast<const uint2*>(oh + 4);
         if (a.out_lo)      // low-order plane for an O projection that reads the output as hi + lo
             *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.out_lo) + at + j * 32) = *reinterpret_cast<const uint4*>(ol);
     }

@@ -356,3 +356,27 @@ def test_tree_attention_tail_alone(group, n_rows, L, dcap):
     hide[:, L:] = torch.from_numpy(vis == 0)
     ref = torch.einsum("bhrc,bhcd->brhd", s.masked_fill_(hide.cuda(), -float("inf")).softmax(-1), vc.repeat_interleave(group, 1)[:, :, :L + n_rows].double())
     assert (out.double() - ref).abs().max() <= 2.0 ** -8 * float(ref.abs().max())
+
+
+@pytest.mark.parametrize("dt,h,offset", [("bf16", 128, 4), ("bf16", 64, 1), ("fp32", 64, 1)])
+def test_tree_attention_output_of_the_stores_own_alignment(dt, h, offset):
+    """`out` may start on any 8 bytes (tensor-core path), or on any element (CUDA-core path): the same bits, and nothing beside
+    them is written.  L = 200: the cache and the tail both take part."""
+    dtype = torch.float32 if dt == "fp32" else torch.bfloat16
+    b, Hq, Hkv, n_rows, L = 1, 8, 2, 21, 200
+    g = torch.Generator().manual_seed(5)
+    q = torch.randn(b, R, Hq, h, generator=g).to(dtype).cuda()
+    kc, vc = (torch.randn(b, Hkv, L + R, h, generator=g).to(dtype).cuda() for _ in range(2))
+    _, depth1, vis = _tree_block(n_rows, 0, 6, 8)
+    depth = np.zeros((b, R), np.int32)
+    depth[:, :n_rows] = depth1
+    ref = _run_attention(int(dt == "bf16"), q, kc, vc, _anc_words(vis)[None], depth, n_rows, L, Hq, Hkv, h)
+    flat = torch.full((q.numel() + 16,), 7.0, dtype=dtype, device="cuda")
+    out = flat[offset:offset + q.numel()].view_as(q)
+    nb = P.esp_tree_attention_scratch_bytes(b, Hq, h, L + R)
+    scratch = torch.zeros(nb, dtype=torch.uint8, device="cuda")
+    P.esp_tree_attention(int(dt == "bf16"), b, n_rows, L, L + R, Hq, Hkv, h, 16, q, kc, vc, torch.from_numpy(_anc_words(vis)[None].view(np.int64)).cuda(),
+                         torch.from_numpy(depth).cuda(), out, scratch, nb)
+    assert P.esp_tree_attention_status(scratch) == 0
+    assert torch.equal(out[:, :n_rows], ref[:, :n_rows])
+    assert (out[:, n_rows:] == 7).all() and (flat[:offset] == 7).all() and (flat[offset + q.numel():] == 7).all()
