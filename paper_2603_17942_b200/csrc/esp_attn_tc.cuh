@@ -548,6 +548,35 @@ __device__ __forceinline__ void tail_task(TailAcc& t, const AttnArgs& a, const T
                     else { if (lane >= 16) co[(j & 1) * 8 + 2 * r + e] = w; }
                 }
         }
+        // A piece of weight 0 times an infinite value is a NaN that the whole weight would not have given: sums that are not finite are
+        // taken again, key by key with the whole weight (hi + mid + lo, exact), keys without weight (below 2^-133, the least of bf16)
+        // left out.
+        float odd = 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) odd = __fmaf_rn(co[i], 0.f, odd);       // 0 x inf and 0 x NaN are NaN
+        if (__any_sync(0xffffffffu, odd != 0.f)) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) co[i] = 0.f;
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+#pragma unroll 1
+                for (int k = 0; k < 8; ++k) {
+                    const int from = (lane & 12) | (k >> 1), sh = 16 * (k & 1);      // who holds key 8 n + k of this lane's head
+                    const uint32_t hi = __shfl_sync(0xffffffffu, pa[n][0], from) >> sh, mid = __shfl_sync(0xffffffffu, pa[n][0], 16 + from) >> sh,
+                                   lo = __shfl_sync(0xffffffffu, pa[n][1], from) >> sh;
+                    const float p = __fadd_rn(__fadd_rn(__uint_as_float(hi << 16), __uint_as_float(mid << 16)), __uint_as_float(lo << 16));
+                    const __nv_bfloat16* vr = vbase + (size_t)__shfl_sync(0xffffffffu, slot, 8 * n + k) * HD + (lane >> 4) * 64;
+                    if (p != 0.f) {
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const uint4 x = __ldcg(reinterpret_cast<const uint4*>(vr + j * 32));
+                            const uint32_t v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) co[j * 8 + i] = __fmaf_rn(p, __uint_as_float(i & 1 ? v[i >> 1] & 0xffff0000u : v[i >> 1] << 16), co[j * 8 + i]);
+                        }
+                    }
+                }
+        }
         merge_ml(t.m, t.l, t.o, cm, cl, co);
     }
 }

@@ -380,3 +380,47 @@ def test_tree_attention_output_of_the_stores_own_alignment(dt, h, offset):
     assert P.esp_tree_attention_status(scratch) == 0
     assert torch.equal(out[:, :n_rows], ref[:, :n_rows])
     assert (out[:, n_rows:] == 7).all() and (flat[:offset] == 7).all() and (flat[offset + q.numel():] == 7).all()
+
+
+@pytest.mark.parametrize("group", [1, 2, 4])
+@pytest.mark.parametrize("L,dcap", [(0, 16), (9, 48)])
+def test_tree_attention_infinite_values_in_the_tail(group, L, dcap):
+    """A value that is not finite reaches the dimensions of the rows that give its key a weight, as one product with the whole weight
+    does: infinite where the sum is, NaN only where opposite infinities or a NaN meet; a key whose weight underflows leaves nothing
+    behind.  Keys: the one with the largest weight, an ordinary one, one of weight 0, one that only some rows see."""
+    Hkv, h, b, n_rows = 2, 128, 1, 40
+    Hq, inf = Hkv * group, float("inf")
+    _, depth1, vis = _tree_block(n_rows, 0, dcap, 3)
+    g = torch.Generator().manual_seed(group)
+    q = torch.randn(b, R, Hq, h, generator=g)
+    kc, vc = (torch.randn(b, Hkv, L + R, h, generator=g) for _ in range(2))
+    q[..., 0] = 8.0
+    kc[..., 0] = 0.0
+    kc[:, :, L, 0] = 40.0                     # the root: weight 1 in every row
+    far = L + 1
+    kc[:, :, far, 0] = -400.0                 # its weight underflows
+    vc[:, :, L, 0], vc[:, :, L, 1] = inf, -inf
+    vc[:, :, far, 2], vc[:, :, far, 3] = inf, float("nan")
+    vc[:, :, L + 2, 4], vc[:, :, L + 2, 5] = inf, float("nan")
+    vc[:, :, L + 5, 0], vc[:, :, L + 5, 1] = -inf, -inf       # meets the root's +inf where it is visible
+    q, kc, vc = q.bfloat16().cuda(), kc.bfloat16().cuda(), vc.bfloat16().cuda()
+    depth = np.zeros((b, R), np.int32)
+    depth[:, :n_rows] = depth1
+    assert (np.maximum(L + depth1 - dcap, 0) // 16 * 16).max() == 0        # the tail does it all
+    out = _run_attention(1, q, kc, vc, _anc_words(vis)[None], depth, n_rows, L, Hq, Hkv, h, dcap)[0, :n_rows].double().cpu()
+    k, v = (t[0].repeat_interleave(group, 0)[:, :L + n_rows].double().cpu() for t in (kc, vc))
+    s = torch.einsum("rhd,hcd->rhc", q[0, :n_rows].double().cpu(), k) / h ** 0.5
+    hide = torch.zeros(n_rows, 1, L + n_rows, dtype=torch.bool)
+    hide[:, 0, L:] = torch.from_numpy(vis == 0)
+    s = s.masked_fill(hide, -inf)
+    p = torch.exp(s - s.max(-1, keepdim=True).values)
+    p[p < 2.0 ** -140] = 0.0
+    assert (p[..., far] == 0).all()
+    terms = torch.where(p[..., None] > 0, p[..., None] * v[None], torch.zeros(()).double())
+    ref = terms.sum(2) / p.sum(-1, keepdim=True)
+    assert torch.equal(torch.isnan(out), torch.isnan(ref)) and torch.equal(torch.isinf(out), torch.isinf(ref))
+    assert torch.isinf(ref[..., :2]).any() and torch.isnan(ref[..., 0]).any() and torch.isfinite(ref[:, :, 2:4]).all()
+    odd = torch.isinf(ref)
+    assert torch.equal(out[odd], ref[odd])
+    fin = torch.isfinite(ref)
+    assert (out[fin] - ref[fin]).abs().max() <= 2.0 ** -8 * float(ref[fin].abs().max())
