@@ -77,7 +77,7 @@ void launch_topk_merge(const SeqState* st, const Cand* cand, const float2* cand_
 void launch_tree_step(int dtype, const TreeArgs& A, cudaStream_t s, bool pdl);
 
 // CUDA-core GEMM (fp32 models; on-GPU cross-check for bf16)
-// (rows_cap: no block has more rows; sizes the grid.  With a.norm_gain, fp32 and K <= 1024, the GEMM takes the RMSNorm in front of it along.)
+// (rows_cap: no block has more rows; sizes the grid)
 int launch_gemm_simt(int dtype, int epi, int n_tiles, int batch, const void* const w[3], const int32_t rows_w[3],
                      const void* x, int K, const EpiArgs& a, int rows_cap, cudaStream_t s, bool pdl);
 

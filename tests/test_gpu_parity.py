@@ -94,6 +94,61 @@ def test_tiny_fp32_nontrivial_stream(pu):
     run.close()
 
 
+@pytest.mark.parametrize("d,F", [(8, 40), (136, 72), (264, 200), (520, 304), (1016, 136), (1024, 136), (1032, 136)])
+def test_fp32_widths_parity(pu, d, F):
+    """fp32 models of other widths than the tiny one's: k that is no multiple of the GEMMs' stages of 32 and 64, norms whose row does not
+    fill a warp, the largest row that one warp norms and the first one beyond it.  ESP equals greedy there, and the captured residual
+    stream gives the captured logits."""
+    import paper_2603_17942_b200 as P
+    shape = synth.TINY.replace(name="fp32-widths", d_model=d, n_q_heads=4, n_kv_heads=4, head_dim=32, d_ffn=F, vocab=515, tied=False)
+    w = synth.make_weights(shape, seed=6, gain_jitter=True, std=0.3)
+    prompt = synth.make_prompt(shape.vocab, 131, 4)
+    spec = O.SpecCfg(n_probes=3, topk=4, max_nodes=20, expand_width=0, n_anchor=1)
+    run = pu.ParityRun(shape, w, spec, prompt, 12, TOL_FP32)
+    out = run.run()
+    assert len(set(out)) > 3
+    hidden = torch.zeros(P.ESP_MAX_ROWS, d, device="cuda")
+    P.esp_debug_capture(run.h.h, run.logits, hidden)
+    n_rows = run.h.state()["n_rows"]
+    run.h.step()
+    x = hidden[:n_rows].double().cpu()
+    x = x / (x.pow(2).mean(-1, keepdim=True) + shape.rms_eps).sqrt() * w["final_norm"].double()
+    ref = x @ w["lm_head"].double().T
+    # (the norm and a sum of d products in fp32: a few 2^-24 each)
+    assert n_rows > 16 and (run.logits[:n_rows].double().cpu() - ref).abs().max() <= 2e-5 * float(ref.abs().max())
+    g, _ = pu.gpu_generate(shape, run.wd, pu.GREEDY, prompt, 12)
+    assert g == out[:12]
+    run.close()
+
+
+def test_fp32_weights_on_any_element_have_the_same_bits(pu):
+    """Matrices and gains that start on 4 bytes only are read element by element: the bits of the aligned copies."""
+    import paper_2603_17942_b200 as P
+    shape = synth.TINY.replace(name="fp32-odd", d_model=264, d_ffn=200, vocab=515, tied=False)
+    wd = pu.to_device(synth.make_weights(shape, seed=6, gain_jitter=True, std=0.3))
+
+    def odd(t):
+        flat = torch.zeros(t.numel() + 4, device="cuda")
+        out = flat[1:1 + t.numel()].view(t.shape)
+        out.copy_(t)
+        assert out.data_ptr() % 16 == 4
+        return out
+
+    moved = {k: v if k == "embed" else [odd(t) for t in v] if isinstance(v, list) else odd(v) for k, v in wd.items()}
+    torch.cuda.synchronize()
+    prompt = synth.make_prompt(shape.vocab, 50, 4)
+    got = []
+    for ww in (wd, moved):
+        h = P.Handle(shape, P.spec_cfg(n_probes=3, topk=4, max_nodes=20, expand_width=0, n_anchor=1), ww, max_seq_len=128)
+        logits = torch.zeros(P.ESP_MAX_ROWS, shape.vocab, device="cuda")
+        P.esp_debug_capture(h.h, logits)
+        h.prefill(prompt)
+        toks = [h.step() for _ in range(3)]
+        got.append((toks, logits[:h.state()["n_rows"]].clone()))
+        h.close()
+    assert got[0][0] == got[1][0] and torch.equal(got[0][1], got[1][1]) and got[0][1].abs().max() > 0
+
+
 def test_forced_drafts_are_accepted_and_compacted(pu):
     """Drive acceptance lengths random-init models never reach: the tree is set to contain the true
     continuation (found by GPU greedy decoding), so several nodes are accepted and their KV rows move."""
