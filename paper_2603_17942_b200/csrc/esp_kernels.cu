@@ -653,25 +653,27 @@ __device__ __forceinline__ void attn_row_info(const AttnArgs& a, int seq, int r,
     }
 }
 
-// E consecutive elements as floats, read from L2 (VEC: 16 bytes aligned, or all of them if they are fewer)
+template <typename V>
+__device__ __forceinline__ V load_l2_or_l1(const V* p, bool l1) { return l1 ? *p : __ldcg(p); }
+// E consecutive elements as floats, read from L2, or (l1) through L1 (VEC: 16 bytes aligned, or all of them if they are fewer)
 template <typename T, int E, bool VEC>
-__device__ __forceinline__ void load_row(float (&v)[E], const T* p) {
+__device__ __forceinline__ void load_row(float (&v)[E], const T* p, bool l1 = false) {
     if constexpr (!VEC) {
 #pragma unroll
         for (int i = 0; i < E; ++i) {
-            if constexpr (sizeof(T) == 4) v[i] = __ldcg(p + i);
-            else v[i] = __bfloat162float(__ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p) + i)));
+            if constexpr (sizeof(T) == 4) v[i] = load_l2_or_l1(p + i, l1);
+            else v[i] = __bfloat162float(__ushort_as_bfloat16(load_l2_or_l1(reinterpret_cast<const unsigned short*>(p) + i, l1)));
         }
     } else if constexpr (sizeof(T) == 4) {
 #pragma unroll
         for (int i = 0; i < E; i += 4) {
-            const float4 x = __ldcg(reinterpret_cast<const float4*>(p + i));
+            const float4 x = load_l2_or_l1(reinterpret_cast<const float4*>(p + i), l1);
             v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
         }
     } else {
 #pragma unroll
         for (int i = 0; i < E; i += 4) {
-            const uint2 x = __ldcg(reinterpret_cast<const uint2*>(p + i));
+            const uint2 x = load_l2_or_l1(reinterpret_cast<const uint2*>(p + i), l1);
             const __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&x.x), hi = *reinterpret_cast<const __nv_bfloat162*>(&x.y);
             v[i] = __low2float(lo); v[i + 1] = __high2float(lo); v[i + 2] = __low2float(hi); v[i + 3] = __high2float(hi);
         }
@@ -683,9 +685,10 @@ __device__ __forceinline__ void load_row(float (&v)[E], const T* p) {
 // Scores: eight lanes per key, HD / 8 dims each, four keys side by side, so that a load touches whole rows (a lane per key
 // touches 32 cache lines per load: 13 us of the tiny decoder's step per layer, now 0.8 behind the cache kernel, its 64-token request 8530 -> 7446 us); values: a lane per dim.
 // Keys, and values, of RB rounds (of VB keys) are in flight together (lanes without a key hold the slot of one that is
-// there; its value row is read and not used).  VEC: the cache starts on 16 bytes.
+// there; its value row is read and not used).  Slots below n_l1 go through L1, where the warps that share a KV head find them
+// again; what this step wrote is read from L2.  VEC: the cache starts on 16 bytes.
 template <typename T, int HD, bool VEC>
-__device__ __forceinline__ void warp_chunk(const float (&q)[HD / 8], const T* kbase, const T* vbase, int slot, uint32_t valid,
+__device__ __forceinline__ void warp_chunk(const float (&q)[HD / 8], const T* kbase, const T* vbase, int slot, int n_l1, uint32_t valid,
                                            float scale_log2, float& cm, float& cl, float (&co)[HD / 32]) {
     constexpr int E = HD / 8, RB = HD == 128 ? 4 : 8, VB = HD == 128 ? 16 : 32;
     const int lane = threadIdx.x & 31, kg = lane >> 3;
@@ -694,7 +697,10 @@ __device__ __forceinline__ void warp_chunk(const float (&q)[HD / 8], const T* kb
     for (int u0 = 0; u0 < 8; u0 += RB) {
         float k[RB][E];
 #pragma unroll
-        for (int u = 0; u < RB; ++u) load_row<T, E, VEC>(k[u], kbase + (size_t)__shfl_sync(0xffffffffu, slot, 4 * (u0 + u) + kg) * HD + (lane & 7) * E);
+        for (int u = 0; u < RB; ++u) {
+            const int sl = __shfl_sync(0xffffffffu, slot, 4 * (u0 + u) + kg);
+            load_row<T, E, VEC>(k[u], kbase + (size_t)sl * HD + (lane & 7) * E, sl < n_l1);
+        }
 #pragma unroll
         for (int u = 0; u < RB; ++u) {
             float acc = 0.f;
@@ -728,11 +734,12 @@ __device__ __forceinline__ void warp_chunk(const float (&q)[HD / 8], const T* kb
         float v[VB][HD / 32];
 #pragma unroll
         for (int j = 0; j < VB; ++j) {
-            const T* vr = vbase + (size_t)__shfl_sync(0xffffffffu, slot, j0 + j) * HD;
+            const int sl = __shfl_sync(0xffffffffu, slot, j0 + j);
+            const T* vr = vbase + (size_t)sl * HD;
 #pragma unroll
             for (int i = 0; i < HD / 32; ++i) {
                 float x[1];
-                load_row<T, 1, false>(x, vr + lane + 32 * i);
+                load_row<T, 1, false>(x, vr + lane + 32 * i, sl < n_l1);
                 v[j][i] = x[0];
             }
         }
@@ -751,9 +758,9 @@ template <int N>
 __device__ __forceinline__ void merge_partial(float& m, float& l, float (&o)[N], float cm, float cl, const float (&co)[N]) {
     float mn = fmaxf(m, cm);
     float a = exp2f(m - mn), b = exp2f(cm - mn);
-    l = l * a + cl * b;
+    l = __fmaf_rn(l, a, __fmul_rn(cl, b));      // (spelled out: every kernel that merges rounds alike)
 #pragma unroll
-    for (int i = 0; i < N; ++i) o[i] = o[i] * a + co[i] * b;
+    for (int i = 0; i < N; ++i) o[i] = __fmaf_rn(o[i], a, __fmul_rn(co[i], b));
     m = mn;
 }
 
@@ -762,28 +769,31 @@ __device__ __forceinline__ void merge_partial(float& m, float& l, float (&o)[N],
 // loading (16-byte asynchronous copies) while the current one is used.  What bounds it is a warp's serial chain over
 // the split: with four pairs a warp shares every key and value read from shared memory between them and the CTA reads
 // the split from L2 for 16 pairs; with one pair the chain is a third as long, which is what counts while the four-pair
-// CTAs would leave SMs idle (launch_attn_simt_t).  Measured with the tail kernel behind it, 3 sequences x 35 rows x 4
-// fp32 heads of 64 over 777 positions: 184 us with a warp per (row, head) gathering its keys from L1, 33 us now; one
-// split of 100 positions on its own 13.4 us with four pairs per warp, 7.3 with one.
+// CTAs would leave SMs idle (launch_attn_simt_t).
 // grid = (ceil(rows * group / (4 * BS_PW)), Hkv, n_split * batch).
-// The CTA's warps form bulk_groups() groups that take the split's chunks in turn, each with buffers and running sums of its own,
-// merged in group order at the end (which chunk goes where follows from the position alone): the chain over 256 positions is eight
-// chunks of about 3 us for one group.  Operator, 3 sequences x 35 rows x 4 fp32 heads of 64 over 777 positions: 34.9 -> 23.3 us.
+// The chunks of a split go in turn to bulk_groups() groups, each with running sums of its own, merged in group order at the end; which
+// chunk goes where follows from the position alone, and so do a row's bits.  KS = bulk_groups(): a group of warps with buffers of its
+// own for each, so that the chain over 256 positions is two or four chunks long instead of eight of about 3 us each.  KS = 1: one group
+// of warps takes the groups' chunks one group after the other.  Its CTAs need a quarter or half of the shared memory, which counts
+// where there are more CTAs than fit anyway.
 constexpr int BS_WARPS = 4;
 template <typename T, int HD> __host__ __device__ constexpr int bulk_groups() { return sizeof(T) * HD <= 256 ? 4 : 2; }
+// one group of warps: where the sums of the chunk groups already done wait (fp32 heads of 128: three CTAs leave no shared memory for them)
+template <typename T, int HD> __host__ __device__ constexpr bool bulk_sums_in_regs() { return sizeof(T) * HD > 256; }
 template <typename T, int HD> __host__ __device__ constexpr int bulk_simt_ld() { return HD + 16 / (int)sizeof(T); }
-template <typename T, int HD> constexpr size_t bulk_simt_smem(int pw) {
-    return bulk_groups<T, HD>() * (sizeof(T) * 4 * 32 * bulk_simt_ld<T, HD>() + sizeof(float) * BS_WARPS * pw * HD);
+template <typename T, int HD> constexpr size_t bulk_simt_smem(int pw, int ks) {
+    return ks * (sizeof(T) * 4 * 32 * bulk_simt_ld<T, HD>() + sizeof(float) * BS_WARPS * pw * HD) + (ks == 1 && !bulk_sums_in_regs<T, HD>() ? sizeof(float) * BS_WARPS * pw * (HD + 2) : 0);
 }
-template <typename T, int HD, bool VEC, int BS_PW>
-__global__ void __launch_bounds__(128 * bulk_groups<T, HD>()) k_attn_bulk_simt(AttnArgs a, int n_split_launch) {
+template <typename T, int HD, bool VEC, int BS_PW, int KS>
+__device__ __forceinline__ void attn_bulk_simt(const AttnArgs& a, int n_split_launch) {
     constexpr int LD = bulk_simt_ld<T, HD>(), V = 16 / (int)sizeof(T), PER_ROW = HD / V, KG = bulk_groups<T, HD>();
+    static_assert(KS == KG || KS == 1, "a group of warps per group of chunks, or one for all");
     extern __shared__ __align__(16) unsigned char bulk_smem[];
     const int kg = threadIdx.x >> 7, gt = threadIdx.x & 127;      // key group, thread of the group
     const int warp = gt >> 5, lane = gt & 31;
     T* s_k = reinterpret_cast<T*>(bulk_smem) + kg * 4 * 32 * LD;      // [2][32][LD]
     T* s_v = s_k + 2 * 32 * LD;                                       // [2][32][LD]
-    float* s_qall = reinterpret_cast<float*>(reinterpret_cast<T*>(bulk_smem) + KG * 4 * 32 * LD) + kg * BS_WARPS * BS_PW * HD;
+    float* s_qall = reinterpret_cast<float*>(reinterpret_cast<T*>(bulk_smem) + KS * 4 * 32 * LD) + kg * BS_WARPS * BS_PW * HD;
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) attn_clear_error(a);
     const int kvh = blockIdx.y, group = a.Hq / a.Hkv;
     const int split = blockIdx.z % n_split_launch, seq = blockIdx.z / n_split_launch;
@@ -839,16 +849,48 @@ __global__ void __launch_bounds__(128 * bulk_groups<T, HD>()) k_attn_bulk_simt(A
         cp_async_commit();
     };
     float m[BS_PW], l[BS_PW], o[BS_PW][HD / 32];
+    auto reset = [&] {
 #pragma unroll
-    for (int w = 0; w < BS_PW; ++w) {
-        m[w] = -INFINITY;
-        l[w] = 0.f;
+        for (int w = 0; w < BS_PW; ++w) {
+            m[w] = -INFINITY;
+            l[w] = 0.f;
 #pragma unroll
-        for (int i = 0; i < HD / 32; ++i) o[w][i] = 0.f;
-    }
-    if (beg + 32 * kg < cta_end) load(beg + 32 * kg, 0);
-    for (int p0 = beg + 32 * kg, buf = 0; p0 < cta_end; p0 += 32 * KG, buf ^= 1) {
-        if (p0 + 32 * KG < cta_end) load(p0 + 32 * KG, buf ^ 1);
+            for (int i = 0; i < HD / 32; ++i) o[w][i] = 0.f;
+        }
+    };
+    reset();
+    // KS == 1: the sums of the groups done so far, [pair][HD + 2] per warp
+    constexpr bool SUMS_REG = bulk_sums_in_regs<T, HD>();
+    float* s_sum = s_qall + (KS == 1 ? BS_WARPS * BS_PW * HD : 0) + warp * BS_PW * (HD + 2);
+    float r_sum[BS_PW][HD / 32 + 2];
+    auto put_sum = [&](int w) {
+        if constexpr (SUMS_REG) {
+            r_sum[w][HD / 32] = m[w]; r_sum[w][HD / 32 + 1] = l[w];
+#pragma unroll
+            for (int i = 0; i < HD / 32; ++i) r_sum[w][i] = o[w][i];
+        } else {
+            float* d = s_sum + w * (HD + 2);
+            if (lane == 0) { d[HD] = m[w]; d[HD + 1] = l[w]; }
+#pragma unroll
+            for (int i = 0; i < HD / 32; ++i) d[lane + 32 * i] = o[w][i];
+        }
+    };
+    auto get_sum = [&](int w, float& md, float& ld, float (&od)[HD / 32]) {
+        const float* d = s_sum + w * (HD + 2);
+        md = SUMS_REG ? r_sum[w][HD / 32] : d[HD];
+        ld = SUMS_REG ? r_sum[w][HD / 32 + 1] : d[HD + 1];
+#pragma unroll
+        for (int i = 0; i < HD / 32; ++i) od[i] = SUMS_REG ? r_sum[w][i] : d[lane + 32 * i];
+    };
+    int g = kg, p0 = beg + 32 * kg;
+    bool more = p0 < cta_end;
+    if (more) load(p0, 0);
+    for (int buf = 0; more; buf ^= 1) {
+        // the next chunk: of this group, or (one group of warps) the first of the next group
+        int g_next = g, p_next = p0 + 32 * KG;
+        if (KS == 1 && p_next >= cta_end) { g_next = g + 1; p_next = g_next < KG ? beg + 32 * g_next : cta_end; }
+        more = p_next < cta_end;
+        if (more) load(p_next, buf ^ 1);
         else cp_async_commit();
         cp_async_wait<1>();
         group_bar();
@@ -894,6 +936,37 @@ __global__ void __launch_bounds__(128 * bulk_groups<T, HD>()) k_attn_bulk_simt(A
         for (int w = 0; w < BS_PW; ++w)
             if (p0 < end[w]) merge_partial(m[w], l[w], o[w], cm[w], cl[w], co[w]);
         group_bar();           // this buffer is loaded again in the next round but one
+        if (KS == 1 && (!more || g_next != g)) {        // the group is done
+#pragma unroll
+            for (int w = 0; w < BS_PW; ++w) {
+                if (g > 0) {
+                    float md, ld, od[HD / 32];
+                    get_sum(w, md, ld, od);
+                    if (beg + 32 * g < end[w]) merge_partial(md, ld, od, m[w], l[w], o[w]);
+                    m[w] = md; l[w] = ld;
+#pragma unroll
+                    for (int i = 0; i < HD / 32; ++i) o[w][i] = od[i];
+                    __syncwarp();
+                }
+                if (more) put_sum(w);
+            }
+            __syncwarp();
+            if (more) reset();
+        }
+        g = g_next;
+        p0 = p_next;
+    }
+    auto store = [&](int w) {
+        const size_t idx = ((size_t)(seq * RT + row[w]) * a.Hq + kvh * group + (pair0 + w) % group) * a.n_split_max + split;
+        if (lane == 0) a.part_ml[idx] = make_float2(m[w], l[w]);
+#pragma unroll
+        for (int i = 0; i < HD / 32; ++i) a.part_o[idx * HD + lane + 32 * i] = o[w][i];
+    };
+    if constexpr (KS == 1) {
+#pragma unroll
+        for (int w = 0; w < BS_PW; ++w)
+            if (end[w] > beg) store(w);
+        return;
     }
     // the groups' sums meet in the first group's buffers ([group - 1][pair][HD + 2] floats), which it has done with
     __syncthreads();
@@ -921,16 +994,24 @@ __global__ void __launch_bounds__(128 * bulk_groups<T, HD>()) k_attn_bulk_simt(A
             for (int i = 0; i < HD / 32; ++i) co[i] = d[lane + 32 * i];
             if (beg + 32 * g < end[w]) merge_partial(m[w], l[w], o[w], d[HD], d[HD + 1], co);
         }
-        const size_t idx = ((size_t)(seq * RT + row[w]) * a.Hq + kvh * group + (pair0 + w) % group) * a.n_split_max + split;
-        if (lane == 0) a.part_ml[idx] = make_float2(m[w], l[w]);
-#pragma unroll
-        for (int i = 0; i < HD / 32; ++i) a.part_o[idx * HD + lane + 32 * i] = o[w][i];
+        store(w);
     }
+}
+
+template <typename T, int HD, bool VEC, int BS_PW>
+__global__ void __launch_bounds__(128 * bulk_groups<T, HD>()) k_attn_bulk_simt(AttnArgs a, int n_split_launch) {
+    attn_bulk_simt<T, HD, VEC, BS_PW, bulk_groups<T, HD>()>(a, n_split_launch);
+}
+// (Blocks per SM: as many as shared memory holds with fp32 heads of 64 and 128.  Heads of 32 and 64 with 6 to 8 blocks: spills and less
+// in flight, 1.2 to 1.6 times as long; with 3, 1.1 to 1.4.)
+template <typename T, int HD, bool VEC>
+__global__ void __launch_bounds__(128, sizeof(T) * HD > 256 ? 3 : 5) k_attn_bulk_simt_serial(AttnArgs a, int n_split_launch) {
+    attn_bulk_simt<T, HD, VEC, 4, 1>(a, n_split_launch);
 }
 
 // Tail + merge: one warp per (row, head).  grid = (ceil(rows/4), Hq, batch).
 // behind_bulk: launched as a dependent of the bulk kernel, whose CTAs release this one after their own wait; the tail is
-// computed while they run (from L2 loads only: nothing another kernel wrote comes from a stale L1 line).
+// computed while they run (what the step wrote from L2 only: nothing of it comes from a stale L1 line).
 template <typename T, int HD, bool VEC>
 __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a, bool behind_bulk) {
     // let the next kernel start its own preamble (for a GEMM: the first weight tiles) while this one runs; it still
@@ -950,6 +1031,7 @@ __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a, bool behind
     load_row<T, HD / 8, false>(q, reinterpret_cast<const T*>(a.q) + ((size_t)(seq * RT + r) * a.Hq + head) * HD + (lane & 7) * (HD / 8));
     const T* kb = reinterpret_cast<const T*>(a.kc) + ((size_t)seq * a.Hkv + kvh) * a.cap * HD;
     const T* vb = reinterpret_cast<const T*>(a.vc) + ((size_t)seq * a.Hkv + kvh) * a.cap * HD;
+    const int n_l1 = a.cache_in_flight ? 0 : L;      // cache positions below L were written by earlier steps
     // tail: positions T0..P in order
     const int n_tail = P - T0 + 1;
     float tm = -INFINITY, tl = 0.f, to[HD / 32];
@@ -971,7 +1053,7 @@ __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a, bool behind
         const int any = valid ? __shfl_sync(0xffffffffu, slot, __ffs(valid) - 1) : 0;
         if (slot < 0) slot = any;
         float cm, cl, co[HD / 32];
-        warp_chunk<T, HD, VEC>(q, kb, vb, slot, valid, a.scale_log2, cm, cl, co);
+        warp_chunk<T, HD, VEC>(q, kb, vb, slot, n_l1, valid, a.scale_log2, cm, cl, co);
         merge_partial(tm, tl, to, cm, cl, co);
     }
     if (behind_bulk) pdl_wait();
@@ -1020,16 +1102,24 @@ static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, 
     if (behind_bulk) {
         const int pairs = a.rows_cap * (a.Hq / a.Hkv);
         const long long ctas4 = (long long)((pairs + 15) / 16) * a.Hkv * n_split_launch * batch;
-        // Four-pair warps once their CTAs cover half of the SMs.  Operator with the tail kernel, us, one pair / four pairs per warp:
-        // fp32, heads of 128: 36 CTAs 31 / 41, 72 39 / 43, 80 45 / 43, 128 47 / 45 and 66 / 43, 144 69 / 42, 480 147 / 88; heads of 64, whose
-        // chain is half as long, meet later: fp32 40 28 / 35, 80 31 / 35, 120 33 / 35, 240 50 / 41, bf16 128 31 / 35, 216 38 / 40, 480 66 / 53.
-#define ESP_BULK_SIMT(PW)                                                                                              \
+        // One pair per warp while its CTAs, four times as many, find room at once (one per SM with fp32 heads of 64 and 128, two
+        // otherwise); four pairs with a group of warps per group of chunks up to one and a half CTAs per SM; then one group of warps.
+        // Operator with its tail kernel, 32/8 or 4/2 heads, us, one pair / four / four with one group of warps, at CTAs of four pairs:
+        // fp32, heads of 32: 20 13.7 / 16.8 / 22, 72 14.1 / 16.9 / 23, 144 20.8 / 17.9 / 23, 288 50 / 47 / 41, 544 52 / 54 / 35, 4096 1107 / 1045 /
+        // 684 (656 with one chain per split); of 64: 32 14.0 / 18.7 / 25, 48 20.8 / 20.1 / 25, 72 20.9 / 18.7 / 25, 192 66 / 51.5 / 52.5, 272 50 / 31 /
+        // 28, 544 112 / 62 / 49, 4096 2522 / 1229 / 990; of 128: 36 20.8 / 26.9 / 31, 48 34 / 28.8 / 32, 144 64 / 29 / 33, 288 223 / 88 / 93, 352 1051 /
+        // 459 / 389, 4096 5813 / 2174 / 1716.  bf16, heads of 32: 72 12.7 / 16.7 / 21, 144 20.7 / 17.7 / 21, 544 55 / 39 / 35, 4096 1071 / 709 / 654;
+        // of 64: 72 16.5 / 18.1 / 24, 144 24.9 / 18.8 / 25, 288 70 / 55.6 / 51, 4096 1637 / 1087 / 930.
+#define ESP_BULK_SIMT(KERNEL, PW, KS)                                                                                  \
         {                                                                                                              \
-            if (ensure_dynamic_smem(reinterpret_cast<const void*>(k_attn_bulk_simt<T, HD, VEC, PW>), (int)bulk_simt_smem<T, HD>(PW))) return -1; \
-            launch_k(k_attn_bulk_simt<T, HD, VEC, PW>, dim3((pairs + 4 * PW - 1) / (4 * PW), a.Hkv, n_split_launch * batch), dim3(128 * bulk_groups<T, HD>()), \
-                     bulk_simt_smem<T, HD>(PW), s, pdl, a, n_split_launch);                                            \
+            const auto kernel = KERNEL;                                                                                \
+            if (ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), (int)bulk_simt_smem<T, HD>(PW, KS))) return -1; \
+            launch_k(kernel, dim3((pairs + 4 * PW - 1) / (4 * PW), a.Hkv, n_split_launch * batch), dim3(128 * KS), bulk_simt_smem<T, HD>(PW, KS), s, pdl, a, n_split_launch); \
         }
-        if (ctas4 >= 74) ESP_BULK_SIMT(4) else ESP_BULK_SIMT(1)
+        constexpr int KG = bulk_groups<T, HD>(), one_pair = sizeof(T) * HD >= 256 ? 37 : 74;
+        if (ctas4 < one_pair) ESP_BULK_SIMT((k_attn_bulk_simt<T, HD, VEC, 1>), 1, KG)
+        else if (ctas4 <= 222) ESP_BULK_SIMT((k_attn_bulk_simt<T, HD, VEC, 4>), 4, KG)
+        else ESP_BULK_SIMT((k_attn_bulk_simt_serial<T, HD, VEC>), 4, 1)
 #undef ESP_BULK_SIMT
     }
     const dim3 g2((a.rows_cap + 3) / 4, a.Hq, batch);

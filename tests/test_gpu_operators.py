@@ -424,3 +424,30 @@ def test_tree_attention_infinite_values_in_the_tail(group, L, dcap):
     assert torch.equal(out[odd], ref[odd])
     fin = torch.isfinite(ref)
     assert (out[fin] - ref[fin]).abs().max() <= 2.0 ** -8 * float(ref[fin].abs().max())
+
+
+@pytest.mark.parametrize("odd", [False, True])
+@pytest.mark.parametrize("L", [33, 301, 1111])
+@pytest.mark.parametrize("dt,h", [("fp32", 32), ("fp32", 64), ("fp32", 128), ("bf16", 32), ("bf16", 64)])
+def test_cuda_core_attention_has_the_same_bits_in_launches_of_every_size(dt, h, L, odd):
+    """The CUDA-core kernel over the cache takes one or four pairs to a warp and several groups of warps or one by the size of the launch;
+    the first rows of a block have the same bits whichever runs, and with a cache that starts on any element.  Splits that end in the
+    middle of a chunk, with fewer chunks than groups, and full ones."""
+    dtype = torch.float32 if dt == "fp32" else torch.bfloat16
+    Hq, Hkv, cap = 32, 8, L + R
+    g = torch.Generator().manual_seed(h + L)
+    q = torch.randn(1, R, Hq, h, generator=g).to(dtype).cuda()
+    kc, vc = (torch.randn(1, Hkv, cap, h, generator=g).to(dtype).cuda() for _ in range(2))
+    if odd:
+        kc, vc = (torch.cat([t.new_zeros(1), t.flatten()])[1:].view_as(t) for t in (kc, vc))
+        assert kc.data_ptr() % 16 == kc.element_size()
+    _, depth1, vis = _tree_block(R, 0, 12, 5)
+    outs = [_run_attention(int(dt == "bf16"), q, kc, vc, _anc_words(vis)[None], depth1[None], n, L, Hq, Hkv, h)[0] for n in (1, 5, 16, 44, R)]
+    for n, o in zip((1, 5, 16, 44), outs):
+        assert torch.equal(o[:n], outs[-1][:n])
+    s = torch.einsum("rhd,hcd->rhc", q[0].double(), kc[0].repeat_interleave(4, 0).double()) / h ** 0.5
+    hide = torch.zeros(R, 1, cap, dtype=torch.bool)
+    hide[:, 0, L:] = torch.from_numpy(vis == 0)
+    ref = torch.einsum("rhc,hcd->rhd", s.masked_fill_(hide.cuda(), -float("inf")).softmax(-1), vc[0].repeat_interleave(4, 0).double())
+    # (fp32: sums of up to 1239 terms; bf16: the result's own rounding)
+    assert (outs[-1].double() - ref).abs().max() <= (1e-5 if dt == "fp32" else 2.0 ** -8) * float(ref.abs().max())
