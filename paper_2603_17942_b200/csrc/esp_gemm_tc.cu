@@ -50,12 +50,16 @@ using namespace tc;
 // several sequences: esp_gemm_wide.cu.)
 //
 // Ring depth.  The bytes in flight per SM (depth x 16 KB of weights) over the load round trip bound the stream rate,
-// and the ring is also what is requested before the preceding kernel has finished: deeper is better.
+// and the ring is also what is requested before the preceding kernel has finished.  So deep is good, as long as the SM keeps room for
+// the blocks of the kernels in front and behind, which run beside this one's.  Steps of eight 8B layers, us, one stage fewer -> the depth
+// taken: 24 rows (9) 969 -> 963, 32 (9) 983 -> 970, 40 (7, eight in 227 KB) 1045 -> 1011 with eight -> seven, 48 1051 -> 1029; 56 and 64 rows
+// with seven stages, which leave 2 KB, -> six: 56 1068 -> 1057, 60 1104 -> 1087, 64 1119 -> 1099; 72 rows (6) and 112 rows (4 or 5) make no
+// difference; 80 rows with six or five 1193 to 1208.
 // Planes (PL).  The activations reach the tensor cores as bf16.  A plan with two planes reads them as a pair
 // x = hi + lo (hi = bf16(x), lo = bf16(x - hi), stored n_seq blocks apart in the same buffer) and takes every product
 // with both: it then sees the activation to 2^-17 instead of 2^-9, for 10 KB more shared memory per stage.
 __host__ __device__ constexpr int stages_of(int epi, int nq, int nrs, int pl = 1) {
-    return pl == 2 ? (nrs <= 16 ? 10 : nrs <= 32 ? 9 : nrs <= 64 ? 7 : nrs <= 80 ? 6 : nrs <= 96 ? 5 : 4)
+    return pl == 2 ? (nrs <= 16 ? 10 : nrs <= 32 ? 9 : nrs <= 48 ? 7 : nrs <= 80 ? 6 : nrs <= 96 ? 5 : 4)
                    : (nrs == 80 ? (nq == 3 ? 4 : (nq == 2 ? 5 : 6)) : 4);
 }
 __host__ __device__ constexpr int b_bytes_of(int nq, int nrs) { return nq * nrs * BK * 2; }   // 10240 per 80-row sequence and plane
@@ -64,6 +68,8 @@ __host__ __device__ constexpr int stage_bytes_of(int nq, int nrs, int pl = 1) { 
 __host__ __device__ constexpr int acc_cols_of(int nr) { return nr <= 128 ? 128 : 256; }
 constexpr int NUM_THREADS = 192;
 constexpr int MAX_NQ = 3;
+// Steps of 16 rows, of 8 between 48 and 80, where trees of 48 and 64 nodes with their probes lie.  (Any multiple of 8 is possible: 24, 40,
+// 88, 104 and 120 would give such blocks about 1 to 2 % of a step each.)
 constexpr int TWO_PLANE_ROWS[] = {16, 32, 48, 56, 64, 72, 80, 96, 112, 128};
 __host__ __device__ constexpr int max_nq_of(int nrs, int pl) { return pl == 1 && nrs == 80 ? MAX_NQ : 1; }
 
@@ -265,7 +271,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) k_gemm_tc(const __grid_constan
             // sequence by sequence: NRS accumulator columns -> that sequence's rows of the partial, or (a whole tile of a
             // fused epilogue) shared memory and the epilogue
             if constexpr (JOINT) {
-                // 16 rows at a time, hi + lo: 70 registers a thread, so that the kernels on either side of this one fit beside
+                // 16 rows at a time, hi + lo: 54 to 62 registers a thread, so that the kernels on either side of this one fit beside
                 // its CTA -- the consumer's CTAs while it runs, the next GEMM's CTA (whose weight stream then starts early)
                 // beside the consumer's.  (All rows in registers at once: 146, 210 for 128 rows.)
                 const int nr = rows_of(0);
