@@ -464,7 +464,7 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
                 if (attn_tc_launch(h->p_attn[(size_t)l * D.batch + s0], a, nb, n_split_launch, s, pdl)) return ESP_E_BADCFG;
                 h->launches += n_split_launch > 0 ? 2 : 1;
             } else {
-                if (launch_attn_simt(h->dtype, a, nb, n_split_launch, true, s, pdl)) return ESP_E_BADCFG;
+                if (launch_attn_simt(h->dtype, a, nb, n_split_launch, s, pdl)) return ESP_E_BADCFG;
                 h->launches += n_split_launch > 0 ? 2 : 1;
             }
             mark(h, KIND_ATTN);
@@ -1249,7 +1249,7 @@ int esp_tree_attention(int32_t dtype, int32_t batch, int32_t n_rows, int32_t L, 
     const bool mma = dtype == 1 && attn_tc_supported(head_dim, n_q_heads, n_kv_heads);
     if (mma) {
         if (attn_tc_run(q, kcache, vcache, batch, n_q_heads, n_kv_heads, cap, a, n_split_launch, s)) return ESP_E_BADCFG;
-    } else if (launch_attn_simt(dtype, a, batch, n_split_launch, true, s, false)) {
+    } else if (launch_attn_simt(dtype, a, batch, n_split_launch, s, false)) {
         return ESP_E_BADCFG;
     }
     return cuda_ok(cudaGetLastError());

@@ -153,8 +153,9 @@ __device__ __forceinline__ void bulk_once(const BulkParams& p) {
 }
 __global__ void __launch_bounds__(ONCE_THREADS, 1) k_attn_bulk_tc_once(const __grid_constant__ BulkParams p) { bulk_once(p); }
 // The same with 112 registers: its CTA then fits on an SM with up to seven CTAs of the q/k/v finish kernel in front, where the one
-// above, with 126, starts only when these have ended (from six on).  Step of sixteen 8B layers, 68 rows: 2197 -> 2165 us; where
-// there is nothing to gain its spills cost (120-row blocks 1547 -> 1557).
+// above, with 126, starts only when these have ended (from six on).  Steps of eight 8B layers, us, without -> with it where six or
+// seven are in front: 62 rows 1089 -> 1095, 64 1105 -> 1107, 66 1161 -> 1137, 68 1152 -> 1135, 72 1171 -> 1143, 76 1220 -> 1197, 80 1205 -> 1181,
+// 84 1410 -> 1414, 86 1424 -> 1408; with more in front its spills cost (120 rows 1547 -> 1557).
 __global__ void __maxnreg__(112) k_attn_bulk_tc_once_slim(const __grid_constant__ BulkParams p) { bulk_once(p); }
 
 // ---- persistent CTAs: used when the launch has clearly more items than SMs.

@@ -363,7 +363,11 @@ __device__ __forceinline__ void bulk_item_roles(const BulkMaps& mp, const AttnAr
 //   softmax     a lane holds 8 keys of head (lane / 4) % 4, lanes 4 apart share a row; both copies compute the same;
 //   O = P V     P in three bf16 pieces (hi + mid + lo = the 24 bits of the fp32 weight, products exact): hi in rows 0..3,
 //               mid in rows 4..7, lo in rows 8..11 of ONE A operand; V's 8 x 8 blocks are transposed in registers.
-// Every sum's order follows from the position in the list alone.  What bounded the kernels before this one was their
+// Every sum's order follows from the position in the list alone.  (The additions inside one mma.sync are not rounded one by one as a chain
+// of multiply-adds is.  Error of o / l against 64 bits, 2-norm, chain / this: scores of deviation 0.3 1.19 / 0.81e-7, 1 1.66 / 1.57e-7, 3 2.48 /
+// 2.29e-7, 10 3.60 / 2.82e-7; values all positive 0.98 / 0.81, 1.43 / 1.81 and 2.15 / 2.07e-7 at deviations 1, 3 and 10.)
+// A KV head of a single query head leaves three of the four places empty: launches of more than 12000 (row, head) pairs then take
+// 1.05 to 1.3 times as long as the kernel before this one, smaller ones and deep trees less.  What bounded the kernels before this one was their
 // instruction count and a chain of dependent trips: a warp per (row, head) gathered its keys 32 cache lines per load
 // (8.6 us a task), a CTA with the keys in shared memory spent about 1700 instructions per task of four heads.
 constexpr int TG = 4;

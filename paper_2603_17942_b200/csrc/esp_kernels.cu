@@ -1097,8 +1097,8 @@ __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a, bool behind
 }
 
 template <typename T, int HD, bool VEC>
-static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, bool bulk_too, cudaStream_t s, bool pdl) {
-    const bool behind_bulk = bulk_too && n_split_launch > 0;
+static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, cudaStream_t s, bool pdl) {
+    const bool behind_bulk = n_split_launch > 0;
     if (behind_bulk) {
         const int pairs = a.rows_cap * (a.Hq / a.Hkv);
         const long long ctas4 = (long long)((pairs + 15) / 16) * a.Hkv * n_split_launch * batch;
@@ -1127,12 +1127,12 @@ static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, 
     return 0;
 }
 
-int launch_attn_simt(int dtype, const AttnArgs& a, int batch, int n_split_launch, bool bulk_too, cudaStream_t s, bool pdl) {
+int launch_attn_simt(int dtype, const AttnArgs& a, int batch, int n_split_launch, cudaStream_t s, bool pdl) {
     // 16-byte loads where the caches start on 16 bytes (their rows then do too)
     const bool vec = (reinterpret_cast<uintptr_t>(a.kc) | reinterpret_cast<uintptr_t>(a.vc)) % 16 == 0;
 #define ESP_ATTN_CASE(TT, H)                                                              \
-    return vec ? launch_attn_simt_t<TT, H, true>(a, batch, n_split_launch, bulk_too, s, pdl) \
-               : launch_attn_simt_t<TT, H, false>(a, batch, n_split_launch, bulk_too, s, pdl);
+    return vec ? launch_attn_simt_t<TT, H, true>(a, batch, n_split_launch, s, pdl) \
+               : launch_attn_simt_t<TT, H, false>(a, batch, n_split_launch, s, pdl);
     if (dtype == 0) {
         if (a.h == 32) { ESP_ATTN_CASE(float, 32) }
         if (a.h == 64) { ESP_ATTN_CASE(float, 64) }
@@ -1431,7 +1431,7 @@ __global__ void __launch_bounds__(TREE_THREADS) k_tree_step(TreeArgs A) {
     float* c_lp = reinterpret_cast<float*>(c_dep + MAX_CAND);
     int* c_row = reinterpret_cast<int*>(c_lp + MAX_CAND);            // creation index -> new row
     __shared__ int s_path[PROBES_MAX + 2], s_out[PROBES_MAX + 2];
-    __shared__ int s_na, s_ustar, s_delta, s_nexp, s_ncreated, s_nkeep, s_nsurv, s_abort, s_err;
+    __shared__ int s_na, s_ustar, s_delta, s_nexp, s_ncreated, s_nkeep, s_nsurv, s_err;
     __shared__ int s_exp[RT], s_sel[RT];
     __shared__ int s_rtok[RT], s_rpar[RT], s_rdep[RT], s_arg[RT];     // this step's row table and per-row argmax
     __shared__ __align__(16) unsigned long long s_keep[PROBES_MAX * RT];      // per depth, the keys of the B-1 best nodes: the only ones the final pick can take
@@ -1454,7 +1454,7 @@ __global__ void __launch_bounds__(TREE_THREADS) k_tree_step(TreeArgs A) {
         s_rpar[r] = st->row_parent[r];
         s_rdep[r] = st->row_depth[r];
     }
-    if (tid == 0) { s_abort = 0; s_err = 0; s_nsurv = 0; }
+    if (tid == 0) { s_err = 0; s_nsurv = 0; }
     pdl_wait();
     const int err0 = tid == 0 ? __ldcg(A.err) : 0;       // the error word before this kernel
     __syncthreads();      // every thread has read the counter

@@ -83,7 +83,7 @@ int launch_gemm_simt(int dtype, int epi, int n_tiles, int batch, const void* con
 
 // position-canonical attention: CUDA-core bulk (+ tail/merge), or tail/merge only when the
 // tensor-core bulk kernel already produced the split partials
-int launch_attn_simt(int dtype, const AttnArgs& a, int batch, int n_split_launch, bool bulk_too, cudaStream_t s, bool pdl);
+int launch_attn_simt(int dtype, const AttnArgs& a, int batch, int n_split_launch, cudaStream_t s, bool pdl);
 // bf16, head_dim 128: tcgen05 bulk kernel over the cache below each row's T0, then tail + merge (esp_attn_tc.cu).
 // A plan holds the TMA descriptors of one query buffer and one layer's KV cache.
 struct AttnTc;
