@@ -337,7 +337,8 @@ def test_tree_attention_with_room_for_the_block_only(dt, h):
 def test_tree_attention_tail_alone(group, n_rows, L, dcap):
     """No row has a position below its T0, so the tail kernel does it all: fewer heads per KV head than a warp takes together,
     as many, and several times as many; lists of one key, of 32 and one more, of several chunks; keys before, on and behind the
-    end of the cache.  Its weights are exact to fp32, so what is left is the result's own rounding."""
+    end of the cache.  The bound is the result's own rounding; that the weights keep their bits is seen by
+    test_tree_attention_tail_weights_keep_their_24_bits."""
     Hkv, h, b = 2, 128, 2
     Hq, cap = Hkv * group, L + R
     if dcap == 128:
@@ -451,3 +452,60 @@ def test_cuda_core_attention_has_the_same_bits_in_launches_of_every_size(dt, h, 
     ref = torch.einsum("rhc,hcd->rhd", s.masked_fill_(hide.cuda(), -float("inf")).softmax(-1), vc[0].repeat_interleave(4, 0).double())
     # (fp32: sums of up to 1239 terms; bf16: the result's own rounding)
     assert (outs[-1].double() - ref).abs().max() <= (1e-5 if dt == "fp32" else 2.0 ** -8) * float(ref.abs().max())
+
+
+@pytest.mark.parametrize("group,n_rows,L,dcap", [(1, 33, 5, 16), (2, 9, 0, 16), (4, 68, 15, 16), (8, 41, 16, 32), (16, 7, 40, 48), (4, 128, 3, 128)])
+def test_tree_attention_tail_weights_keep_their_24_bits(group, n_rows, L, dcap):
+    """Three keys have weight, and their values nearly cancel in a dimension of each (row, head): what is left is far below the result's
+    bf16 rounding of any one product, so a weight that lost bits shows.  Scores are single products (exact), so a weight's error is
+    that of its scaled exponent (below 4, 2^-22) and of the exponential: 2^-21 of sum(p |v|), twice that allowed beside the result's own
+    rounding.  Weights of 16 bits, and of 8, must fail the same bound."""
+    Hkv, h = 2, 128
+    Hq, cap = Hkv * group, L + R
+    parents = np.minimum(np.arange(n_rows) - 1, 2)                 # a trunk of three nodes, the others behind it
+    vis = np.zeros((n_rows, n_rows), np.uint8)
+    depth = np.zeros((1, R), np.int32)
+    for r in range(n_rows):
+        vis[r, r] = 1
+        if r:
+            vis[r] |= vis[parents[r]]
+            depth[0, r] = depth[0, parents[r]] + 1
+    rng = np.random.default_rng(group * 1000 + n_rows)
+
+    def bf(x):
+        return torch.from_numpy(np.asarray(x, np.float32)).bfloat16().double().numpy()
+
+    c = bf(rng.uniform(1, 4, (n_rows, Hq)))                        # queries and keys: one dimension each
+    key = np.full((Hkv, L + n_rows), -2048.0)                      # weight 0
+    key[:, L:L + 3] = bf([[0.0, -2.7, -5.2], [-4.1, 0.0, -1.9]])
+    head_kv = np.repeat(np.arange(Hkv), group)
+    s = c[:, :, None] * key[head_kv][None] / h ** 0.5
+    s = np.where(np.concatenate([np.ones((n_rows, L)), vis], 1)[:, None] > 0, s, -np.inf)
+    p = np.exp(s - s.max(-1, keepdims=True))
+    p[p < 2.0 ** -149] = 0.0
+    assert np.array_equal((p[2:] > 0).sum(-1), np.full((n_rows - 2, Hq), 3))
+    # dimension d of a KV head: values of the trunk that cancel for one (row, head)
+    v = np.zeros((Hkv, L + n_rows, h))
+    v[:, L] = bf(rng.uniform(500, 2000, (Hkv, h)))
+    for kv in range(Hkv):
+        for d in range(h):
+            w = p[2 + d % (n_rows - 2), kv * group + d % group, L:L + 3]
+            v[kv, L + 1, d] = bf(-v[kv, L, d] * w[0] / w[1])
+            v[kv, L + 2, d] = bf(-(v[kv, L, d] * w[0] + v[kv, L + 1, d] * w[1]) / w[2])
+
+    def out_of(pp):
+        return np.einsum("rhc,hcd->rhd", pp, v[head_kv]) / p.sum(-1)[..., None]
+
+    ref = out_of(p)
+    tol = 2.0 ** -8 * np.abs(ref) + 2.0 ** -20 * np.einsum("rhc,hcd->rhd", p, np.abs(v[head_kv])) / p.sum(-1)[..., None]
+    hi = bf(p)
+    mid = bf(p - hi)
+    assert (np.abs(out_of(hi) - ref) > tol).any() and (np.abs(out_of(hi + mid) - ref) > tol).any()
+    assert (np.abs(out_of(hi + mid + bf(p - hi - mid)) - ref) <= tol / 4).all()
+    q = torch.zeros(1, R, Hq, h)
+    q[0, :n_rows, :, 7] = torch.from_numpy(c)
+    kc, vc = torch.zeros(1, Hkv, cap, h), torch.zeros(1, Hkv, cap, h)
+    kc[0, :, :L + n_rows, 7] = torch.from_numpy(key)
+    vc[0, :, :L + n_rows] = torch.from_numpy(v)
+    out = _run_attention(1, q.bfloat16().cuda(), kc.bfloat16().cuda(), vc.bfloat16().cuda(), _anc_words(vis)[None], depth, n_rows, L, Hq, Hkv, h, dcap)
+    assert (np.abs(out[0, :n_rows].double().cpu().numpy() - ref) <= tol).all()

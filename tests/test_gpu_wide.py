@@ -303,3 +303,27 @@ def test_a_row_normed_by_two_blocks_has_the_bits_of_one_block(d):
     assert first[0].abs().max() > 0
     for f in first[1:]:
         assert torch.equal(f, first[0])
+
+
+def test_rows_of_two_sequences_normed_by_pairs_of_blocks():
+    """Two sequences of up to 37 rows have their norms taken by a pair of blocks per row, of 38 by one block per row: the root rows' bits
+    of both sequences are those of the greedy handle of as many sequences."""
+    shape = BF16_SMALL.replace(name="bf16-wide-rows", d_model=2944, n_layers=2, n_q_heads=16, n_kv_heads=4, d_ffn=1376)
+    w = synth.make_weights(shape, seed=4, device="cuda", gain_jitter=True, std=0.03)
+    torch.cuda.synchronize()
+    first = []
+    for nodes in (0, 13, 34, 35):
+        kw = dict(n_probes=0, max_nodes=1) if not nodes else dict(n_probes=3, topk=10, max_nodes=nodes, expand_width=0, n_anchor=1)
+        h = P.Handle(shape, P.spec_cfg(**kw), w, max_seq_len=300, max_batch=2)
+        logits = torch.zeros(2, R, shape.vocab, dtype=torch.float32, device="cuda")
+        P.esp_debug_capture(h.h, logits)
+        for i in range(2):
+            h.prefill(synth.make_prompt(shape.vocab, 60 + i, 4 + i), i)
+        assert all(h.state(i)["n_rows"] == (nodes + 3 if nodes else 1) for i in range(2))
+        h.step()
+        assert h.stats().device_error == 0 and torch.isfinite(logits[:, 0]).all()
+        first.append(logits[:, 0].clone())
+        h.close()
+    assert (first[0][0] != first[0][1]).any()
+    for f in first[1:]:
+        assert torch.equal(f, first[0])
