@@ -40,9 +40,9 @@ if ROOT not in sys.path:
 METRIC = "esp_accepted_tokens_per_s"
 UNIT = "tok/s"
 
-# DRAM bytes (read + written) of one gate/up GEMM launch from the ncu capture summarised under profiles/
-# (Llama-3-8B shape, 68 rows, one sequence); None for workloads without a capture of the current kernel.
-GATEUP_DRAM_TRAFFIC = {"llama3-8b": 242.9e6}
+# DRAM bytes (read + written) of one gate/up GEMM launch (k_gemm_tc<5, 1, 72, 2>, Llama-3-8B shape, 68 rows, one sequence; ncu, the
+# counters summarised in profiles/launch_list_llama3-8b_step.md); None for workloads without a capture of the current kernel.
+GATEUP_DRAM_TRAFFIC = {"llama3-8b": 241.1e6}
 
 GEN_TOKENS = 256          # new tokens per request of the two model workloads
 GEN_TOKENS_SWEEP = 128    # ... of the batch / long-context sweep (--batch, --prompt-len)
