@@ -408,6 +408,11 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
     auto pieces = [&](int kind, const TcGemm* one) -> StreamK { return multi ? wide_gemm_streamk(h->p_batch[kind], nb, pass, live) : tc_gemm_streamk(one); };
     launch_assemble(h->dtype, st0, h->embed, mvec0, b.hres, D.d, D.mask_slots, nb, s, false, rc_rows);
     h->launches++;
+    // fp32 models: a small GEMM behind a norm takes it along
+    const bool norm_qkv = gemm_simt_takes_norm(h->dtype, EPI_QKV, D.d, dq + 2 * dkv, rc_rows, D.batch);
+    const bool norm_gu = gemm_simt_takes_norm(h->dtype, EPI_SWIGLU, D.d, D.F, rc_rows, D.batch);
+    const bool norm_lm = gemm_simt_takes_norm(h->dtype, EPI_LOGITS, D.d, D.V, rc_rows, D.batch);
+    auto x_of = [&](bool in_gemm) { return in_gemm ? static_cast<const void*>(b.hres) : static_cast<const void*>(b.xn); };
     // One sequence, a block of at most 80 rows, bf16: every layer in one persistent launch (same bits as the
     // kernel-per-operation path below, which serves batches, prefill blocks and larger blocks).
     const bool fused = tc && nb == 1 && !prefill && h->p_layers && h->use_layers;
@@ -423,8 +428,8 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
     }
     for (int l = 0; l < D.n_layers && !fused; ++l) {
         if (tc) launch_resid_norm(st0, b.hres, pending, h->na[l], b.xn, b.xn_lo, D.d, D.rms_eps, nullptr, nb, s, pdl, rc_rows);
-        else launch_rmsnorm(h->dtype, st0, b.hres, h->na[l], b.xn, D.d, D.rms_eps, nb, nullptr, s, pdl, rc_rows);
-        h->launches++;
+        else if (!norm_qkv) launch_rmsnorm(h->dtype, st0, b.hres, h->na[l], b.xn, D.d, D.rms_eps, nb, nullptr, s, pdl, rc_rows);
+        h->launches += norm_qkv ? 0 : 1;
         mark(h, KIND_MISC);
         {
             EpiArgs a = base_epi(h, dq + 2 * dkv, s0, nb);
@@ -433,9 +438,10 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             a.vcache = reinterpret_cast<char*>(layer_ptr(b.vcache, h->layer_kv_stride, l)) + kv_seq_off;
             a.q_norm = D.qk_norm ? h->qn[l] : nullptr;
             a.k_norm = D.qk_norm ? h->kn[l] : nullptr;
+            if (norm_qkv) a.norm_gain = h->na[l];
             const void* w[3] = {h->wq[l], h->wk[l], h->wv[l]};
             const int32_t rows[3] = {dq, dkv, dkv};
-            int rc = gemm(0, tc ? plan(h->p_qkv, h->p_qkv_w, l) : nullptr, l, EPI_QKV, (dq + 2 * dkv) / TILE_N, w, rows, b.xn, D.d, a);
+            int rc = gemm(0, tc ? plan(h->p_qkv, h->p_qkv_w, l) : nullptr, l, EPI_QKV, (dq + 2 * dkv) / TILE_N, w, rows, x_of(norm_qkv), D.d, a);
             if (rc) return rc;
             mark(h, KIND_QKV);
             if (tc) {
@@ -479,15 +485,16 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             mark(h, KIND_O);
         }
         if (tc) launch_resid_norm(st0, b.hres, pieces(1, plan(h->p_o, h->p_o_w, l)), h->nf[l], b.xn, b.xn_lo, D.d, D.rms_eps, nullptr, nb, s, pdl, rc_rows);
-        else launch_rmsnorm(h->dtype, st0, b.hres, h->nf[l], b.xn, D.d, D.rms_eps, nb, nullptr, s, pdl, rc_rows);
-        h->launches++;
+        else if (!norm_gu) launch_rmsnorm(h->dtype, st0, b.hres, h->nf[l], b.xn, D.d, D.rms_eps, nb, nullptr, s, pdl, rc_rows);
+        h->launches += norm_gu ? 0 : 1;
         mark(h, KIND_MISC);
         {
             EpiArgs a = base_epi(h, D.F, s0, nb);
             a.act_out = b.act;
+            if (norm_gu) a.norm_gain = h->nf[l];
             const void* w[3] = {h->wg[l], h->wu[l], nullptr};
             const int32_t rows[3] = {D.F, D.F, 0};
-            int rc = gemm(2, tc ? plan(h->p_gu, h->p_gu_w, l) : nullptr, l, EPI_SWIGLU, (D.F + 63) / 64, w, rows, b.xn, D.d, a);
+            int rc = gemm(2, tc ? plan(h->p_gu, h->p_gu_w, l) : nullptr, l, EPI_SWIGLU, (D.F + 63) / 64, w, rows, x_of(norm_gu), D.d, a);
             if (rc) return rc;
             mark(h, KIND_GATEUP);
             if (tc) {
@@ -510,8 +517,8 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
     if (with_lm) {
         float* dbg_hidden = h->dbg_hidden ? h->dbg_hidden + (size_t)s0 * RT * D.d : nullptr;
         if (tc) launch_resid_norm(st0, b.hres, pending, h->final_norm, b.xn, nullptr, D.d, D.rms_eps, dbg_hidden, nb, s, pdl, rc_rows);   // the LM head reads one plane
-        else launch_rmsnorm(h->dtype, st0, b.hres, h->final_norm, b.xn, D.d, D.rms_eps, nb, dbg_hidden, s, pdl, rc_rows);
-        h->launches++;
+        else if (!norm_lm) launch_rmsnorm(h->dtype, st0, b.hres, h->final_norm, b.xn, D.d, D.rms_eps, nb, dbg_hidden, s, pdl, rc_rows);
+        h->launches += norm_lm ? 0 : 1;
         mark(h, KIND_MISC);
         const int n_tiles = (D.V + TILE_N - 1) / TILE_N;
         // tensor-core path: the sequences of a pass share the LM head's weight stream too (128-row plans: one at a time; the
@@ -526,9 +533,10 @@ int forward_pass(esp_handle* h, bool with_lm, int dcap, int s0, int nb, bool tc,
             EpiArgs a = base_epi(h, D.V, sq, per);
             a.cand = b.cand; a.cand_ms = b.cand_ms; a.cand_floor = b.cand_floor; a.n_tiles = n_tiles;
             a.logits_dump = h->dbg_logits ? h->dbg_logits + (size_t)sq * RT * D.V : nullptr;
+            if (norm_lm) { a.norm_gain = h->final_norm; a.norm_copy = dbg_hidden; }
             const void* w[3] = {h->lm_head, nullptr, nullptr};
             const int32_t rows[3] = {D.V, 0, 0};
-            int rc = run_gemm(h, wide ? h->p_lm_w : h->p_lm, EPI_LOGITS, n_tiles, w, rows, b.xn, D.d, a, tc, pdl, rc_rows, per, q);
+            int rc = run_gemm(h, wide ? h->p_lm_w : h->p_lm, EPI_LOGITS, n_tiles, w, rows, x_of(norm_lm), D.d, a, tc, pdl, rc_rows, per, q);
             if (rc) return rc;
             mark(h, KIND_LMHEAD);
             launch_topk_merge(b.states + sq, b.cand, b.cand_ms, n_tiles, D.KP, per, b.topk + (size_t)sq * RT * KP_MAX, b.lse + (size_t)sq * RT, s, pdl, rc_rows, b.cand_floor);

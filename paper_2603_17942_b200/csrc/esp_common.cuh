@@ -189,6 +189,9 @@ struct EpiArgs {
     int32_t Hq, Hkv, h, cap, qk_norm;
     int32_t kv_shared;        // 1: every block of the launch writes the first sequence's cache (prefill blocks of one prompt)
     float rms_eps;
+    // CUDA-core GEMMs of fp32 models: the gain of the norm in front; the GEMM's x is then the residual stream
+    const void* norm_gain;
+    float* norm_copy;         // optional: the residual stream is copied there
     // EPI_SWIGLU
     void* act_out;            // [batch*RT][F] T
     // EPI_LOGITS

@@ -159,39 +159,41 @@ __global__ void __launch_bounds__(256) k_rmsnorm(const SeqState* states, const f
         for (int j = threadIdx.x; j < d; j += 256) copy_out[(size_t)(seq * RT + r) * d + j] = xr[j];
 }
 
-// The same for fp32 rows of up to 1024 elements, a warp per row: no barrier, and the whole row requested at once.  The sum of squares:
-// per lane over its elements in ascending order, then over the warp.
-// (Built and taken back: the blocks of the GEMM behind the norm normalise their own eight rows.  That saves a launch, which the kernel
-// here hides as well, and repeats the norm in every block.  Steps of fp32 models, us, in the GEMM / here: d 256, vocabulary 4096, 1 row
-// 80 / 80, 35 rows 120 / 122, 128 rows 171 / 153; d 512, 35 rows 191 / 175; d 1024, vocabulary 32000, 35 rows 524 / 435, four sequences
-// of 128 rows 5031 / 3309.)
+// One fp32 row of up to MAX elements by a warp: y = x * rsqrt(mean(x^2) + eps) * g.  The whole row is requested at once.  The sum of
+// squares: per lane over its elements in ascending order, then over the warp; the same bits wherever the norm is taken.
+template <int MAX>
+__device__ __forceinline__ void norm_row(float* y, const float* x, const float* g, int d, float eps, int lane, float* copy) {
+    float4 v[MAX / 128];
+    float ss = 0.f;
+#pragma unroll
+    for (int q = 0; q < MAX / 128; ++q)
+        if (lane * 4 + 128 * q < d) v[q] = __ldcg(reinterpret_cast<const float4*>(x + lane * 4 + 128 * q));
+#pragma unroll
+    for (int q = 0; q < MAX / 128; ++q)
+        if (lane * 4 + 128 * q < d) ss = fmaf(v[q].w, v[q].w, fmaf(v[q].z, v[q].z, fmaf(v[q].y, v[q].y, fmaf(v[q].x, v[q].x, ss))));
+    const float rinv = 1.0f / sqrtf(warp_sum(ss) / (float)d + eps);
+#pragma unroll
+    for (int q = 0; q < MAX / 128; ++q) {
+        const int j = lane * 4 + 128 * q;
+        if (j < d) {
+            if (copy) *reinterpret_cast<float4*>(copy + j) = v[q];
+            *reinterpret_cast<float4*>(y + j) = make_float4(v[q].x * rinv * g[j], v[q].y * rinv * g[j + 1], v[q].z * rinv * g[j + 2], v[q].w * rinv * g[j + 3]);
+        }
+    }
+}
+
+// fp32 rows of up to 1024 elements, a warp per row
 constexpr int NORM_ROWS_WARPS = 4, NORM_ROWS_D = 1024;
 __global__ void __launch_bounds__(NORM_ROWS_WARPS * 32) k_rmsnorm_rows(const SeqState* states, const float* x, const float* g, float* y, int d,
                                                                        float eps, float* copy_out) {
     if (threadIdx.x == 0) pdl_launch_dependents();
-    const int seq = blockIdx.y, r = blockIdx.x * NORM_ROWS_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int seq = blockIdx.y, r = blockIdx.x * NORM_ROWS_WARPS + (threadIdx.x >> 5);
     const SeqState* st = states + seq;
     const bool idle = !st->active || r >= st->n_rows;     // the row table was written by an earlier step
     pdl_wait();
     if (idle) return;
     const size_t row = (size_t)(seq * RT + r) * d;
-    float4 v[NORM_ROWS_D / 128];
-    float ss = 0.f;
-#pragma unroll
-    for (int q = 0; q < NORM_ROWS_D / 128; ++q)
-        if (lane * 4 + 128 * q < d) v[q] = __ldcg(reinterpret_cast<const float4*>(x + row + lane * 4 + 128 * q));
-#pragma unroll
-    for (int q = 0; q < NORM_ROWS_D / 128; ++q)
-        if (lane * 4 + 128 * q < d) ss = fmaf(v[q].w, v[q].w, fmaf(v[q].z, v[q].z, fmaf(v[q].y, v[q].y, fmaf(v[q].x, v[q].x, ss))));
-    const float rinv = 1.0f / sqrtf(warp_sum(ss) / (float)d + eps);
-#pragma unroll
-    for (int q = 0; q < NORM_ROWS_D / 128; ++q) {
-        const int j = lane * 4 + 128 * q;
-        if (j < d) {
-            if (copy_out) *reinterpret_cast<float4*>(copy_out + row + j) = v[q];
-            *reinterpret_cast<float4*>(y + row + j) = make_float4(v[q].x * rinv * g[j], v[q].y * rinv * g[j + 1], v[q].z * rinv * g[j + 2], v[q].w * rinv * g[j + 3]);
-        }
-    }
+    norm_row<NORM_ROWS_D>(y + row, x + row, g, d, eps, threadIdx.x & 31, copy_out ? copy_out + row : nullptr);
 }
 
 // Consumer of a split GEMM (O or down projection) fused with the residual add and the next RMSNorm:
@@ -353,16 +355,21 @@ __global__ void __launch_bounds__(SWIGLU_THREADS) k_swiglu_finish(const SeqState
 // A CTA takes 8 rows; where the epilogue works feature by feature (residual add, SiLU*up, plain store) also only 32
 // features (k_gemm_simt_narrow), elsewhere -- rotary pairs and head norms, per-tile selection -- the whole 128-feature
 // tile.  Weights and rows arrive by asynchronous copies several stages ahead, the weights of the first stages
-// requested before the wait for the preceding kernel.  Measured on the tiny fp32 decoder (d_model 256, 35 rows; device
+// requested before the wait for the preceding kernel.  Small GEMMs behind a norm (QKV, gate/up, LM head) take it along (NORM): every CTA
+// normalises its own 8 rows, which saves a launch in a chain of dependent launches and repeats the norm in every block of columns
+// (gemm_simt_takes_norm).  Measured on the tiny fp32 decoder (d_model 256, 35 rows; device
 // time of a launch on its own): QKV 11, O and down 9, gate/up 7, LM head (vocabulary 4096) 13 us, where one CTA per
 // 128-feature tile with all rows took 140 to 240; its 64-token request 103 -> 9.9 ms.
 struct SimtGemmArgs {
     const void* w[3];   // stacked matrices (rows_w[i] rows each); SWIGLU: w[0]=gate, w[1]=up
     int32_t rows_w[3];
-    const void* x;      // [batch*RT][K]
+    const void* x;      // [batch*RT][K]; NORM: the residual stream (fp32)
     int32_t K;
+    const void* gain;   // NORM: [K]
+    float eps;
+    float* copy;        // NORM, optional: the residual stream is copied there
 };
-constexpr int SIMT_ROWS = 8;
+constexpr int SIMT_ROWS = 8, SIMT_NORM_K = 256;
 constexpr int SIMT_KC = 32, SIMT_STAGES = 4;       // whole tile: two CTAs of 84 KB per SM
 // k is dealt to four threads per feature (narrow: to the four warps, each with all 8 rows), whose sums are added in order at
 // the end: one thread per feature and 8 rows, or two rows per warp, was a chain of dependent additions with nothing to hide it
@@ -432,16 +439,50 @@ __device__ __forceinline__ void simt_mac(float (&acc)[R], const T* w, const T* x
     }
 }
 
+// the same from whole rows of x, of which `left` (a multiple of 4) elements remain
+template <int R, int KC>
+__device__ __forceinline__ void simt_mac_n(float (&acc)[R], const float* w, const float* x, int ld, int left) {
+    if (left >= KC) { simt_mac<R, KC>(acc, w, x, ld); return; }
+    for (int k = 0; k < left; k += 4) {
+        const float4 wv = load_f4(w + k);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4 xv = load_f4(x + r * ld + k);
+            acc[r] = fmaf(xv.w, wv.w, fmaf(xv.z, wv.z, fmaf(xv.y, wv.y, fmaf(xv.x, wv.x, acc[r]))));
+        }
+    }
+}
+
+// NORM: rows r0 .. of the residual stream, normalised, to shared memory ([SIMT_ROWS][K + 4] floats); a warp takes PER rows.
+__host__ __device__ constexpr int norm_x_ld(int K) { return K + 4; }
+template <int PER>
+__device__ __forceinline__ void norm_rows(float* s_x, const SimtGemmArgs& g, size_t row0, int n_valid, int warp, int lane, bool copy) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int r = warp * PER + i;
+        if (r >= SIMT_ROWS) return;
+        float* d = s_x + r * norm_x_ld(g.K);
+        if (r < n_valid) {
+            norm_row<SIMT_NORM_K>(d, reinterpret_cast<const float*>(g.x) + (row0 + r) * g.K, reinterpret_cast<const float*>(g.gain), g.K, g.eps, lane,
+                                  copy ? g.copy + (row0 + r) * g.K : nullptr);
+        } else {
+            for (int j = lane * 4; j < g.K; j += 128) *reinterpret_cast<float4*>(d + j) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+}
+
 // 8 rows x one 128-feature tile, SIMT_KS threads per feature, each a quarter of every stage's k.  EPI_QKV (the stacked matrices end on tile boundaries) and
 // EPI_LOGITS.
-template <typename T, int EPI, bool VEC>
+template <typename T, int EPI, bool VEC, bool NORM>
 __global__ void __launch_bounds__(SIMT_THREADS, 2) k_gemm_simt(SimtGemmArgs g, EpiArgs a) {
+    static_assert(!NORM || sizeof(T) == 4, "the normalised rows are fp32");
     constexpr int LD = simt_ld<T>(SIMT_KC);
     extern __shared__ __align__(16) unsigned char simt_smem[];
     T* s_w = reinterpret_cast<T*>(simt_smem);                   // [STAGES][128][LD]
     T* s_x = s_w + SIMT_STAGES * TILE_N * LD;                   // [STAGES][ROWS][LD]
     float* s_acc = reinterpret_cast<float*>(s_x + SIMT_STAGES * SIMT_ROWS * LD);   // [ROWS][ACC_LD]
     float* s_aux = s_acc + SIMT_ROWS * ACC_LD;                  // RT * 4
+    float* s_xn = s_aux + RT * 4;                               // NORM: [ROWS][K + 4]
     if (threadIdx.x == 0) pdl_launch_dependents();
     const int tile = blockIdx.x, r0 = blockIdx.y * SIMT_ROWS, seq = blockIdx.z, f = threadIdx.x % 128, ks = threadIdx.x / 128;
     int m = 0, feat = tile * TILE_N;
@@ -458,11 +499,14 @@ __global__ void __launch_bounds__(SIMT_THREADS, 2) k_gemm_simt(SimtGemmArgs g, E
     if (r0 >= n_rows) { cp_async_wait<0>(); return; }
     const int r1 = r0 + SIMT_ROWS < n_rows ? r0 + SIMT_ROWS : n_rows;
     const T* x = reinterpret_cast<const T*>(g.x) + (size_t)(seq * RT + r0) * g.K;
-    auto load_x = [&](int c) { simt_load<T, SIMT_KC, SIMT_ROWS, VEC, SIMT_THREADS>(s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD, x, r1 - r0, g.K, c * SIMT_KC); };
+    auto load_x = [&](int c) {
+        if constexpr (!NORM) simt_load<T, SIMT_KC, SIMT_ROWS, VEC, SIMT_THREADS>(s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD, x, r1 - r0, g.K, c * SIMT_KC);
+    };
     for (int c = 0; c < SIMT_STAGES - 1; ++c) {
         if (c < n_chunks) load_x(c);
         cp_async_commit();
     }
+    if constexpr (NORM) norm_rows<1>(s_xn, g, (size_t)(seq * RT + r0), r1 - r0, threadIdx.x >> 5, threadIdx.x & 31, g.copy && blockIdx.x == 0);
     float acc[SIMT_ROWS];
 #pragma unroll
     for (int r = 0; r < SIMT_ROWS; ++r) acc[r] = 0.f;
@@ -473,7 +517,8 @@ __global__ void __launch_bounds__(SIMT_THREADS, 2) k_gemm_simt(SimtGemmArgs g, E
         cp_async_commit();
         constexpr int KQ = SIMT_KC / SIMT_KS;
         const T* wr = s_w + ((c % SIMT_STAGES) * TILE_N + f) * LD + ks * KQ;
-        simt_mac<SIMT_ROWS, KQ>(acc, wr, s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD + ks * KQ, LD);
+        if constexpr (NORM) simt_mac_n<SIMT_ROWS, KQ>(acc, wr, s_xn + c * SIMT_KC + ks * KQ, norm_x_ld(g.K), g.K - c * SIMT_KC - ks * KQ);
+        else simt_mac<SIMT_ROWS, KQ>(acc, wr, s_x + (c % SIMT_STAGES) * SIMT_ROWS * LD + ks * KQ, LD);
     }
     // the quarters' sums, added in order (in the weights' buffers, which nothing reads or writes any more)
     __syncthreads();
@@ -495,12 +540,13 @@ __global__ void __launch_bounds__(SIMT_THREADS, 2) k_gemm_simt(SimtGemmArgs g, E
 
 // 8 rows x 32 features (SWIGLU: 16 gate features and the matching 16 up features), a lane per feature, a quarter of every
 // stage's k per warp.  EPI_STORE_F32, EPI_RESID, EPI_SWIGLU.
-template <typename T, int EPI, bool VEC>
+template <typename T, int EPI, bool VEC, bool NORM>
 __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArgs a) {
     constexpr int LD = simt_ld<T>(NARROW_KC), HALF = NARROW_F / 2;
     extern __shared__ __align__(16) unsigned char simt_smem[];
     T* s_w = reinterpret_cast<T*>(simt_smem);                   // [STAGES][32][LD]
     T* s_x = s_w + NARROW_STAGES * NARROW_F * LD;               // [STAGES][ROWS][LD]
+    float* s_xn = reinterpret_cast<float*>(s_x + NARROW_STAGES * SIMT_ROWS * LD);      // NORM: [ROWS][K + 4]
     if (threadIdx.x == 0) pdl_launch_dependents();
     const int r0 = blockIdx.y * SIMT_ROWS, seq = blockIdx.z, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n0 = blockIdx.x * (EPI == EPI_SWIGLU ? HALF : NARROW_F);
@@ -525,7 +571,9 @@ __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArg
     if (r0 >= n_rows) { cp_async_wait<0>(); return; }
     const int r1 = r0 + SIMT_ROWS < n_rows ? r0 + SIMT_ROWS : n_rows;
     const T* x = reinterpret_cast<const T*>(g.x) + (size_t)(seq * RT + r0) * g.K;
-    auto load_x = [&](int c) { simt_load<T, NARROW_KC, SIMT_ROWS, VEC>(s_x + (c % NARROW_STAGES) * SIMT_ROWS * LD, x, r1 - r0, g.K, c * NARROW_KC); };
+    auto load_x = [&](int c) {
+        if constexpr (!NORM) simt_load<T, NARROW_KC, SIMT_ROWS, VEC>(s_x + (c % NARROW_STAGES) * SIMT_ROWS * LD, x, r1 - r0, g.K, c * NARROW_KC);
+    };
     for (int c = 0; c < NARROW_STAGES - 1; ++c) {
         if (c < n_chunks) load_x(c);
         cp_async_commit();
@@ -538,6 +586,7 @@ __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArg
             if (lane < n_feat && r < r1) old[i] = a.hres[(size_t)(seq * RT + r) * a.n_out + n0 + lane];
         }
     }
+    if constexpr (NORM) norm_rows<2>(s_xn, g, (size_t)(seq * RT + r0), r1 - r0, warp, lane, false);
     float part[SIMT_ROWS];
 #pragma unroll
     for (int r = 0; r < SIMT_ROWS; ++r) part[r] = 0.f;
@@ -548,7 +597,8 @@ __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArg
         cp_async_commit();
         constexpr int KQ = NARROW_KC / 4;
         const T* wr = s_w + ((c % NARROW_STAGES) * NARROW_F + lane) * LD + warp * KQ;
-        simt_mac<SIMT_ROWS, KQ>(part, wr, s_x + (c % NARROW_STAGES) * SIMT_ROWS * LD + warp * KQ, LD);
+        if constexpr (NORM) simt_mac_n<SIMT_ROWS, KQ>(part, wr, s_xn + c * NARROW_KC + warp * KQ, norm_x_ld(g.K), g.K - c * NARROW_KC - warp * KQ);
+        else simt_mac<SIMT_ROWS, KQ>(part, wr, s_x + (c % NARROW_STAGES) * SIMT_ROWS * LD + warp * KQ, LD);
     }
     // the quarters' sums, added in order: two rows per warp
     __shared__ float s_part[4][SIMT_ROWS][NARROW_F];
@@ -577,19 +627,40 @@ __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArg
     }
 }
 
+// Whether a GEMM takes the norm in front of it along: K of at most 256 and no more CTAs than two per SM.  Same bits either way.
+// Steps of fp32 models, us, norms in all GEMMs / as launches of a warp per row: d 256, vocabulary 4096, 35 rows 120 / 122, 128 rows (QKV 64
+// CTAs, LM head 512, gate/up 688) 171 / 153; a request of 64 synchronous steps of 35 rows 6926 / 7316; d 512, 1 row 124 / 111, 35 rows
+// 191 / 175; d 1024, vocabulary 32000, 35 rows 524 / 435, four sequences of 128 rows 5031 / 3309.
+bool gemm_simt_takes_norm(int dtype, int epi, int K, int n_out, int rows_cap, int batch) {
+    const int cols = epi == EPI_SWIGLU ? NARROW_F / 2 : TILE_N;
+    return dtype == 0 && K <= SIMT_NORM_K && (long long)((n_out + cols - 1) / cols) * ((rows_cap + SIMT_ROWS - 1) / SIMT_ROWS) * batch <= 2 * 148;
+}
+
 template <typename T, bool VEC>
 int launch_gemm_simt_t(int epi, int n_tiles, int batch, const SimtGemmArgs& g, const EpiArgs& a, int rows_cap, cudaStream_t s, bool pdl) {
     const int groups = (rows_cap + SIMT_ROWS - 1) / SIMT_ROWS;
-#define ESP_SIMT_CASE(E, KERNEL, TILES, SMEM)                                                                       \
-    case E:                                                                                                         \
-        if (ensure_dynamic_smem(reinterpret_cast<const void*>(KERNEL<T, E, VEC>), (int)SMEM<T>())) return ESP_E_CUDA; \
-        return launch_k(KERNEL<T, E, VEC>, dim3(TILES, groups, batch), dim3((E == EPI_QKV || E == EPI_LOGITS) ? SIMT_THREADS : 128), SMEM<T>(), s, pdl, g, a) == cudaSuccess ? ESP_OK : ESP_E_CUDA;
+    const size_t norm_bytes = g.gain ? sizeof(float) * SIMT_ROWS * norm_x_ld(g.K) : 0;
+#define ESP_SIMT_CASE(E, KERNEL, TILES, SMEM, NORM)                                                                 \
+    {                                                                                                               \
+        if (ensure_dynamic_smem(reinterpret_cast<const void*>(KERNEL<T, E, VEC, NORM>), (int)(SMEM<T>() + (NORM ? sizeof(float) * SIMT_ROWS * norm_x_ld(SIMT_NORM_K) : 0)))) \
+            return ESP_E_CUDA;                                                                                      \
+        return launch_k(KERNEL<T, E, VEC, NORM>, dim3(TILES, groups, batch), dim3((E == EPI_QKV || E == EPI_LOGITS) ? SIMT_THREADS : 128), SMEM<T>() + norm_bytes, s, pdl, g, a) == cudaSuccess ? ESP_OK : ESP_E_CUDA; \
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (g.gain) {
+            if (g.K > SIMT_NORM_K || g.K % 4) return ESP_E_ARG;
+            if (epi == EPI_SWIGLU) ESP_SIMT_CASE(EPI_SWIGLU, k_gemm_simt_narrow, (a.n_out + NARROW_F / 2 - 1) / (NARROW_F / 2), narrow_smem_bytes, true)
+            if (epi == EPI_QKV) ESP_SIMT_CASE(EPI_QKV, k_gemm_simt, n_tiles, simt_smem_bytes, true)
+            if (epi == EPI_LOGITS) ESP_SIMT_CASE(EPI_LOGITS, k_gemm_simt, n_tiles, simt_smem_bytes, true)
+            return ESP_E_ARG;
+        }
+    }
     switch (epi) {
-        ESP_SIMT_CASE(EPI_STORE_F32, k_gemm_simt_narrow, (a.n_out + NARROW_F - 1) / NARROW_F, narrow_smem_bytes)
-        ESP_SIMT_CASE(EPI_RESID, k_gemm_simt_narrow, (a.n_out + NARROW_F - 1) / NARROW_F, narrow_smem_bytes)
-        ESP_SIMT_CASE(EPI_SWIGLU, k_gemm_simt_narrow, (a.n_out + NARROW_F / 2 - 1) / (NARROW_F / 2), narrow_smem_bytes)
-        ESP_SIMT_CASE(EPI_QKV, k_gemm_simt, n_tiles, simt_smem_bytes)
-        ESP_SIMT_CASE(EPI_LOGITS, k_gemm_simt, n_tiles, simt_smem_bytes)
+        case EPI_STORE_F32: ESP_SIMT_CASE(EPI_STORE_F32, k_gemm_simt_narrow, (a.n_out + NARROW_F - 1) / NARROW_F, narrow_smem_bytes, false)
+        case EPI_RESID: ESP_SIMT_CASE(EPI_RESID, k_gemm_simt_narrow, (a.n_out + NARROW_F - 1) / NARROW_F, narrow_smem_bytes, false)
+        case EPI_SWIGLU: ESP_SIMT_CASE(EPI_SWIGLU, k_gemm_simt_narrow, (a.n_out + NARROW_F / 2 - 1) / (NARROW_F / 2), narrow_smem_bytes, false)
+        case EPI_QKV: ESP_SIMT_CASE(EPI_QKV, k_gemm_simt, n_tiles, simt_smem_bytes, false)
+        case EPI_LOGITS: ESP_SIMT_CASE(EPI_LOGITS, k_gemm_simt, n_tiles, simt_smem_bytes, false)
     }
 #undef ESP_SIMT_CASE
     return ESP_E_ARG;
@@ -606,6 +677,7 @@ int launch_gemm_simt(int dtype, int epi, int n_tiles, int batch, const void* con
     }
     g.x = x;
     g.K = K;
+    g.gain = a.norm_gain; g.eps = a.rms_eps; g.copy = a.norm_copy;
     if (dtype == 0) return vec ? launch_gemm_simt_t<float, true>(epi, n_tiles, batch, g, a, rows_cap, s, pdl)
                                : launch_gemm_simt_t<float, false>(epi, n_tiles, batch, g, a, rows_cap, s, pdl);
     return vec ? launch_gemm_simt_t<__nv_bfloat16, true>(epi, n_tiles, batch, g, a, rows_cap, s, pdl)

@@ -77,7 +77,9 @@ void launch_topk_merge(const SeqState* st, const Cand* cand, const float2* cand_
 void launch_tree_step(int dtype, const TreeArgs& A, cudaStream_t s, bool pdl);
 
 // CUDA-core GEMM (fp32 models; on-GPU cross-check for bf16)
-// (rows_cap: no block has more rows; sizes the grid)
+// (rows_cap: no block has more rows; sizes the grid.  With a.norm_gain the GEMM takes the RMSNorm in front of it along,
+// x being the residual stream: where gemm_simt_takes_norm says so.)
+bool gemm_simt_takes_norm(int dtype, int epi, int K, int n_out, int rows_cap, int batch);
 int launch_gemm_simt(int dtype, int epi, int n_tiles, int batch, const void* const w[3], const int32_t rows_w[3],
                      const void* x, int K, const EpiArgs& a, int rows_cap, cudaStream_t s, bool pdl);
 

@@ -97,7 +97,7 @@ def test_tiny_fp32_nontrivial_stream(pu):
 @pytest.mark.parametrize("d,F", [(8, 40), (136, 72), (264, 200), (520, 304), (1016, 136), (1024, 136), (1032, 136)])
 def test_fp32_widths_parity(pu, d, F):
     """fp32 models of other widths than the tiny one's: k that is no multiple of the GEMMs' stages of 32 and 64, norms whose row does not
-    fill a warp, the largest row that one warp norms and the first one beyond it.  ESP equals greedy there, and the captured residual
+    fill a warp, norms inside the GEMM behind them (up to 256) and before it, the largest row that one warp norms and the first beyond it.  ESP equals greedy there, and the captured residual
     stream gives the captured logits."""
     import paper_2603_17942_b200 as P
     shape = synth.TINY.replace(name="fp32-widths", d_model=d, n_q_heads=4, n_kv_heads=4, head_dim=32, d_ffn=F, vocab=515, tied=False)
@@ -119,6 +119,33 @@ def test_fp32_widths_parity(pu, d, F):
     g, _ = pu.gpu_generate(shape, run.wd, pu.GREEDY, prompt, 12)
     assert g == out[:12]
     run.close()
+
+
+def test_fp32_rows_have_the_bits_of_the_greedy_handle_in_blocks_of_every_size(pu):
+    """The norm is taken inside a GEMM or in front of it by the size of the launch: the first row of a step has the bits it has in the
+    greedy handle, in blocks with all three norms inside, some of them, and only that of the QKV GEMM, and in a handle of several
+    sequences of the same two sizes."""
+    import paper_2603_17942_b200 as P
+    shape = synth.TINY
+    wd = pu.to_device(synth.make_weights(shape, seed=3, gain_jitter=True, std=0.3))
+    prompt = synth.make_prompt(shape.vocab, 77, 4)
+    for batch, sizes in ((1, (0, 32, 53, 69, 125)), (3, (0, 17, 125))):
+        first = []
+        for nodes in sizes:
+            kw = dict(n_probes=0, max_nodes=1) if not nodes else dict(n_probes=3, topk=10, max_nodes=nodes, expand_width=0, n_anchor=1)
+            h = P.Handle(shape, P.spec_cfg(**kw), wd, max_seq_len=200, max_batch=batch)
+            logits = torch.zeros(batch, P.ESP_MAX_ROWS, shape.vocab, device="cuda")
+            P.esp_debug_capture(h.h, logits)
+            for i in range(batch):
+                h.prefill(prompt, i)
+            assert h.state()["n_rows"] == (nodes + 3 if nodes else 1)
+            h.step()
+            assert h.stats().device_error == 0
+            first.append(logits[batch - 1, 0].clone())
+            h.close()
+        assert first[0].abs().max() > 0
+        for f in first[1:]:
+            assert torch.equal(f, first[0])
 
 
 def test_fp32_weights_on_any_element_have_the_same_bits(pu):
