@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(128) k_gemm_simt_narrow(SimtGemmArgs g, EpiArg
 
 // Whether a GEMM takes the norm in front of it along: K of at most 256 and no more CTAs than two per SM.  Same bits either way.
 // Steps of fp32 models, us, norms in all GEMMs / as launches of a warp per row: d 256, vocabulary 4096, 35 rows 120 / 122, 128 rows (QKV 64
-// CTAs, LM head 512, gate/up 688) 171 / 153; a request of 64 synchronous steps of 35 rows 6926 / 7316; d 512, 1 row 124 / 111, 35 rows
+// CTAs, LM head 512, gate/up 688) 171 / 153; d 512, 1 row 124 / 111, 35 rows
 // 191 / 175; d 1024, vocabulary 32000, 35 rows 524 / 435, four sequences of 128 rows 5031 / 3309.
 bool gemm_simt_takes_norm(int dtype, int epi, int K, int n_out, int rows_cap, int batch) {
     const int cols = epi == EPI_SWIGLU ? NARROW_F / 2 : TILE_N;
@@ -757,9 +757,9 @@ __device__ __forceinline__ void load_row(float (&v)[E], const T* p, bool l1 = fa
 // Scores: eight lanes per key, HD / 8 dims each, four keys side by side, so that a load touches whole rows (a lane per key
 // touches 32 cache lines per load: 13 us of the tiny decoder's step per layer, now 0.8 behind the cache kernel, its 64-token request 8530 -> 7446 us); values: a lane per dim.
 // Keys, and values, of RB rounds (of VB keys) are in flight together (lanes without a key hold the slot of one that is
-// there; its value row is read and not used).  Slots below n_l1 go through L1, where the warps that share a KV head find them
-// again; what this step wrote is read from L2.  VEC: the cache starts on 16 bytes.
-template <typename T, int HD, bool VEC>
+// there; its value row is read and not used).  L1: slots below n_l1 go through L1, where the warps that share a KV head find them again;
+// everything else is read from L2.  VEC: the cache starts on 16 bytes.
+template <typename T, int HD, bool VEC, bool L1>
 __device__ __forceinline__ void warp_chunk(const float (&q)[HD / 8], const T* kbase, const T* vbase, int slot, int n_l1, uint32_t valid,
                                            float scale_log2, float& cm, float& cl, float (&co)[HD / 32]) {
     constexpr int E = HD / 8, RB = HD == 128 ? 4 : 8, VB = HD == 128 ? 16 : 32;
@@ -771,7 +771,7 @@ __device__ __forceinline__ void warp_chunk(const float (&q)[HD / 8], const T* kb
 #pragma unroll
         for (int u = 0; u < RB; ++u) {
             const int sl = __shfl_sync(0xffffffffu, slot, 4 * (u0 + u) + kg);
-            load_row<T, E, VEC>(k[u], kbase + (size_t)sl * HD + (lane & 7) * E, sl < n_l1);
+            load_row<T, E, VEC>(k[u], kbase + (size_t)sl * HD + (lane & 7) * E, L1 && sl < n_l1);
         }
 #pragma unroll
         for (int u = 0; u < RB; ++u) {
@@ -811,7 +811,7 @@ __device__ __forceinline__ void warp_chunk(const float (&q)[HD / 8], const T* kb
 #pragma unroll
             for (int i = 0; i < HD / 32; ++i) {
                 float x[1];
-                load_row<T, 1, false>(x, vr + lane + 32 * i, sl < n_l1);
+                load_row<T, 1, false>(x, vr + lane + 32 * i, L1 && sl < n_l1);
                 v[j][i] = x[0];
             }
         }
@@ -1084,7 +1084,7 @@ __global__ void __launch_bounds__(128, sizeof(T) * HD > 256 ? 3 : 5) k_attn_bulk
 // Tail + merge: one warp per (row, head).  grid = (ceil(rows/4), Hq, batch).
 // behind_bulk: launched as a dependent of the bulk kernel, whose CTAs release this one after their own wait; the tail is
 // computed while they run (what the step wrote from L2 only: nothing of it comes from a stale L1 line).
-template <typename T, int HD, bool VEC>
+template <typename T, int HD, bool VEC, bool L1>
 __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a, bool behind_bulk) {
     // let the next kernel start its own preamble (for a GEMM: the first weight tiles) while this one runs; it still
     // waits for this kernel to complete before it touches anything this kernel or its predecessors write
@@ -1125,7 +1125,7 @@ __global__ void __launch_bounds__(128) k_attn_tail_merge(AttnArgs a, bool behind
         const int any = valid ? __shfl_sync(0xffffffffu, slot, __ffs(valid) - 1) : 0;
         if (slot < 0) slot = any;
         float cm, cl, co[HD / 32];
-        warp_chunk<T, HD, VEC>(q, kb, vb, slot, n_l1, valid, a.scale_log2, cm, cl, co);
+        warp_chunk<T, HD, VEC, L1>(q, kb, vb, slot, n_l1, valid, a.scale_log2, cm, cl, co);
         merge_partial(tm, tl, to, cm, cl, co);
     }
     if (behind_bulk) pdl_wait();
@@ -1195,7 +1195,11 @@ static int launch_attn_simt_t(const AttnArgs& a, int batch, int n_split_launch, 
 #undef ESP_BULK_SIMT
     }
     const dim3 g2((a.rows_cap + 3) / 4, a.Hq, batch);
-    launch_k(k_attn_tail_merge<T, HD, VEC>, g2, dim3(128), 0, s, pdl || behind_bulk, a, behind_bulk);
+    // Through L1 from 4000 (row, head) pairs on: telling the two kinds of slots apart costs every load, which is what counts in a small
+    // launch.  Tail alone, fp32, 32 heads, us, L2 / L1: heads of 128, 35 rows 16.9 / 17.2, 4 x 44 39.6 / 36.8, 4 x 128 88 / 77; of 64 12.9 / 13.8,
+    // 20.8 / 20.8, 50 / 39; of 32 13.0 / 13.5, 16.6 / 14.8, 32 / 28.  A step of the tiny decoder (35 rows x 4 heads) 106 / 111.
+    if ((long long)a.rows_cap * a.Hq * batch >= 4000) launch_k(k_attn_tail_merge<T, HD, VEC, true>, g2, dim3(128), 0, s, pdl || behind_bulk, a, behind_bulk);
+    else launch_k(k_attn_tail_merge<T, HD, VEC, false>, g2, dim3(128), 0, s, pdl || behind_bulk, a, behind_bulk);
     return 0;
 }
 
