@@ -256,7 +256,7 @@ void esp_free(esp_handle* h);
  *            row i's key/value sit at position L+i (the caller writes them there)
  *   anc      [batch][ESP_MAX_ROWS][2] uint64 ancestor-or-self bitmask over block rows
  *   depth    [batch][ESP_MAX_ROWS] int32, position of the row minus L
- *   out      [batch][ESP_MAX_ROWS][n_q_heads][head_dim]
+ *   out      [batch][ESP_MAX_ROWS][n_q_heads][head_dim], on 8 bytes (bf16 heads of 128) or on any element
  *   scratch  esp_tree_attention_scratch_bytes bytes
  * dtype as in esp_model_cfg; n_rows <= ESP_MAX_ROWS rows are real; L + ESP_MAX_ROWS <= cap.
  * The tensor-core path reads the cache in chunks of 128 positions that may reach up to position
